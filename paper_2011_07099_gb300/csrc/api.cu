@@ -124,7 +124,11 @@ void free_plan(Plan* P) {
     cudaFree(P->F64[l]);
     cudaFree(P->M64[l]);
     cudaFree(P->offsets[l]);
+    cudaFree(P->spec_K[l]);
+    cudaFree(P->spec_M[l]);
+    cudaFree(P->spec_P[l]);
   }
+  cudaFree(P->spec_tw);
   cudaFree(P->near_tab);
   cudaFree(P->nz_K);
   cudaFree(P->nz_M);
@@ -163,6 +167,63 @@ bool dev_alloc(T** ptr, size_t count) {
   return cudaMalloc(reinterpret_cast<void**>(ptr), sizeof(T) * count) == cudaSuccess;
 }
 
+// Buffers of the spectral M2L (m2l_spec.cu) for every level of orders >= 2
+// whose spectra take at most kSpecMaxBytes; a level that has none, or whose
+// allocation fails (the dense kernels need ~20 times less memory), keeps the
+// dense contraction.
+constexpr size_t kSpecMaxBytes = (size_t)64 << 30;
+
+// (cos, sin) of 2 pi j / (2 points - 1) as (hi, lo) FP32 pairs.
+int make_twiddles(int points, float4** out) {
+  const int nm = 2 * points - 1;
+  std::vector<float4> tw((size_t)nm);
+  for (int j = 0; j < nm; ++j) {
+    const double a = 2.0 * 3.14159265358979323846 * j / nm, c = std::cos(a), s = std::sin(a);
+    tw[j] = make_float4((float)c, (float)(c - (double)(float)c), (float)s, (float)(s - (double)(float)s));
+  }
+  if (!dev_alloc(out, tw.size())) return FMM_ERR_ALLOC;
+  return cudaMemcpy(*out, tw.data(), tw.size() * sizeof(float4), cudaMemcpyHostToDevice) == cudaSuccess ? FMM_OK
+                                                                                                      : FMM_ERR_CUDA;
+}
+
+int alloc_spec(Plan& P) {
+  if (P.p < 2) return FMM_OK;
+  const int rc = make_twiddles(P.p, &P.spec_tw);
+  if (rc != FMM_OK) return rc;
+  for (int l = 2; l <= P.L; ++l) {
+    const size_t nk = fmm::spec_kernel_bytes(P, l), ns = fmm::spec_source_bytes(P, l),
+                 nt = fmm::spec_target_bytes(P, l);
+    if (nk + ns + nt > kSpecMaxBytes) continue;
+    if (cudaMalloc(&P.spec_K[l], nk) != cudaSuccess || cudaMalloc(&P.spec_M[l], ns) != cudaSuccess ||
+        cudaMalloc(&P.spec_P[l], nt) != cudaSuccess) {
+      cudaFree(P.spec_K[l]);
+      cudaFree(P.spec_M[l]);
+      cudaFree(P.spec_P[l]);
+      P.spec_K[l] = P.spec_M[l] = P.spec_P[l] = nullptr;
+      (void)cudaGetLastError();
+      continue;
+    }
+    // the padding frequencies, and the all-zero spectrum of out-of-box nodes
+    if (cudaMemset(P.spec_K[l], 0, nk) != cudaSuccess || cudaMemset(P.spec_M[l], 0, ns) != cudaSuccess)
+      return FMM_ERR_CUDA;
+  }
+  return FMM_OK;
+}
+
+// Scratch for the offset-range partials of the dense wide levels.
+int alloc_m2l_part(Plan& P) {
+  size_t part = 0;
+  const size_t p3 = (size_t)P.p * P.p * P.p;
+  for (int l = 2; l <= P.L; ++l) {
+    if (!fmm::wide_level(P, l) || P.spec_K[l]) continue;
+    const size_t need = 2 * (size_t)fmm::m2l_fp32_splits(P, l) * ((size_t)1 << (3 * l)) * 4 * p3;
+    if (need > part) part = need;
+  }
+  cudaFree(P.m2l_part);
+  P.m2l_part = nullptr;
+  return !part || dev_alloc(&P.m2l_part, part) ? FMM_OK : FMM_ERR_ALLOC;
+}
+
 // Re-tabulate every table form from G_S1 plus the plan's corrections (MLP,
 // grid), synchronously.  Returns an FMM_* code.
 int retabulate(Plan& P) {
@@ -176,6 +237,8 @@ int retabulate(Plan& P) {
     }
   }
   if (P.near_fft && fmm::launch_near_fft_kernels(P, 0) != cudaSuccess) return FMM_ERR_CUDA;
+  for (int l = 2; l <= P.L; ++l)
+    if (P.spec_K[l] && fmm::launch_spec_kernels(P, l, 0) != cudaSuccess) return FMM_ERR_CUDA;
   if (P.tc_ready) {
     for (int l = fmm::kTcMinLevel; l <= P.L; ++l) {
       if (!P.Apre[l]) continue;
@@ -280,9 +343,7 @@ fmm_plan* fmm_plan_create(int N, int L, int order) {
     const size_t E = 8 * p - 1;
     ok = dev_alloc(&P->M[l], nodes * p3) && dev_alloc(&P->F[l], nodes * 4 * p3) &&
          dev_alloc(&P->tab[l], E * E * E);
-    // split tables for the coarse levels, and for every wide level of the high orders
-    if (ok && (l <= fmm::kExtTopLevel || (p >= fmm::kWideOrder && l < L) || S >= fmm::kWideLeaf))
-      ok = dev_alloc(&P->tab_lo[l], E * E * E);
+    ok = ok && dev_alloc(&P->tab_lo[l], E * E * E);   // low halves: v - fl32(v)
     // FP64 gridlet masses at every level at high order (the leaf copy feeds M2M:
     // the coarse far-field sums cancel ~1000-fold there, so FP32 rounding of
     // the leaf masses alone would cost ~1e-6)
@@ -331,24 +392,20 @@ fmm_plan* fmm_plan_create(int N, int L, int order) {
   }
   {
     // scratch for the offset-range partials of the coarse FP32 M2L levels
-    size_t part = 0;
-    for (int l = 2; l <= L; ++l) {
-      if (!fmm::wide_level(*P, l)) continue;
-      const int ns = fmm::m2l_fp32_splits(*P, l);
-      const size_t need = 2 * (size_t)ns * ((size_t)1 << (3 * l)) * 4 * p3;
-      if (need > part) part = need;
-      if (!dev_alloc(&P->F64[l], ((size_t)1 << (3 * l)) * 4 * p3)) part = 0;
-    }
-    if (!part || !dev_alloc(&P->m2l_part, part)) {
+    bool fok = true;
+    for (int l = 2; l <= L && fok; ++l)
+      if (fmm::wide_level(*P, l)) fok = dev_alloc(&P->F64[l], ((size_t)1 << (3 * l)) * 4 * p3);
+    int rc = fok ? alloc_spec(*P) : FMM_ERR_ALLOC;
+    if (rc != FMM_OK || alloc_m2l_part(*P) != FMM_OK) {
       free_plan(P);
-      set_err(FMM_ERR_ALLOC);
+      set_err(rc != FMM_OK ? rc : FMM_ERR_ALLOC);
       return nullptr;
     }
   }
   if (fmm::setup_upward(*P) != cudaSuccess || fmm::setup_m2l_fp32(*P) != cudaSuccess ||
       fmm::setup_m2l_tc(*P) != cudaSuccess || fmm::setup_learn() != cudaSuccess ||
       fmm::setup_downward(*P) != cudaSuccess || fmm::setup_p2p(*P) != cudaSuccess ||
-      fmm::launch_tables(*P, 0) != cudaSuccess || cudaDeviceSynchronize() != cudaSuccess) {
+      fmm::setup_m2l_spec(*P) != cudaSuccess || retabulate(*P) != FMM_OK) {
     free_plan(P);
     set_err(FMM_ERR_CUDA);
     return nullptr;
@@ -381,7 +438,7 @@ int prepare_tc(Plan& P) {
   const size_t E = 8 * P.p - 1;
   bool made = false;
   for (int l = fmm::tc_first_level(P); l <= P.L; ++l) {
-    if (P.Apre[l]) continue;
+    if (P.Apre[l] || !fmm::tc_level(P, l)) continue;
     const bool wide = fmm::tc_wide(P, l);   // wide modes: tiles from tab + tab_lo, no BF16 table
     if ((!wide && !P.tab_bf[l] && !dev_alloc(&P.tab_bf[l], E * E * E)) ||
         (!P.Mbf_hi[l] && cudaMalloc(&P.Mbf_hi[l], fmm::tc_bsplit_bytes(P.p, l, fmm::tc_splits(P, l))) != cudaSuccess) ||
@@ -436,16 +493,8 @@ int fmm_plan_set_boundary(fmm_plan* plan, int boundary) {
   P.n_off[2] = count;
   P.iso = iso;
   // the offset-range scratch of the coarse levels follows the list length
-  size_t part = 0;
-  const size_t p3 = (size_t)P.p * P.p * P.p;
-  for (int l = 2; l <= P.L; ++l)
-    if (fmm::wide_level(P, l)) {
-      const size_t need = 2 * (size_t)fmm::m2l_fp32_splits(P, l) * ((size_t)1 << (3 * l)) * 4 * p3;
-      if (need > part) part = need;
-    }
-  cudaFree(P.m2l_part);
-  P.m2l_part = nullptr;
-  if (!dev_alloc(&P.m2l_part, part)) return set_err(FMM_ERR_ALLOC);
+  const int rc = alloc_m2l_part(P);
+  if (rc != FMM_OK) return set_err(rc);
   return set_err(retabulate(P));
 }
 
@@ -747,18 +796,14 @@ int fmm_solve(fmm_plan* plan, const float* density, float* potential, float* acc
     FMM_CUDA_TRY(fmm::launch_mean(P, density, s));
   FMM_CUDA_TRY(mark(FMM_TIME_MEAN, 1));
   const bool tc = P.prec != FMM_PREC_FP32 && P.tc_ready;
-  auto on_tc = [&](int l) { return !fmm::fft_level(P, l) && tc && l >= fmm::tc_first_level(P); };
-  // Untimed solves of the tensor-core forms overlap independent stages: the
-  // near zone's source spectra need only the density and its mean (second
-  // auxiliary stream, from the mean on); the M2L levels are independent of
-  // one another until the downward pass, so the CUDA-core levels run on the
-  // first auxiliary stream beside the tensor-core levels on `s` (issued
-  // first).  Measured at 256^3 p = 6: 9.82 -> 9.67 ms; the two kernels
-  // share few SMs (a tensor-core CTA and a CUDA-core CTA together exceed
-  // one SM's shared memory or registers, and capping either cost more).
-  // Timed solves stay serial, so that each stage's events bracket it alone.
-  const bool overlap = !t && tc;
-  const bool fwd_apart = overlap && P.near_fft;
+  auto on_tc = [&](int l) { return !fmm::fft_level(P, l) && tc && fmm::tc_level(P, l); };
+  // Untimed solves overlap independent stages: the near zone's source spectra
+  // need only the density and its mean (second auxiliary stream, from the mean
+  // on); the M2L levels are independent of one another until the downward
+  // pass, so the double-float levels run on the first auxiliary stream beside
+  // the FP32 and tensor-core levels on `s`.  Timed solves stay serial, so that
+  // each stage's events bracket it alone.
+  const bool fwd_apart = !t && P.near_fft;
   if (fwd_apart) {
     FMM_CUDA_TRY(cudaEventRecord(P.fev[0], s));
     FMM_CUDA_TRY(cudaStreamWaitEvent(P.aux[1], P.fev[0], 0));
@@ -772,34 +817,47 @@ int fmm_solve(fmm_plan* plan, const float* density, float* potential, float* acc
   for (int l = P.L - 1; l >= 2; --l) FMM_CUDA_TRY(fmm::launch_m2m(P, l, s));
   FMM_CUDA_TRY(mark(FMM_TIME_M2M, 1));
   FMM_CUDA_TRY(mark(FMM_TIME_M2L, 0));
-  if (overlap) {
-    FMM_CUDA_TRY(cudaEventRecord(P.fev[2], s));
-    for (int l = P.L; l >= 2; --l) {
-      if (!on_tc(l)) continue;
-      FMM_CUDA_TRY(fmm::launch_split_bf16(P, l, s));
-      FMM_CUDA_TRY(fmm::launch_m2l_tc(P, l, P.prec, s));
-    }
-    FMM_CUDA_TRY(cudaStreamWaitEvent(P.aux[0], P.fev[2], 0));
+  auto on_spec = [&](int l) { return !fmm::fft_level(P, l) && !on_tc(l) && P.spec_K[l]; };
+  // one level on its own: FFT ablation, tensor cores or the dense CUDA-core kernels
+  auto m2l_level = [&](int l, cudaStream_t q) -> cudaError_t {
+    if (fmm::fft_level(P, l)) return fmm::launch_m2l_fft(P, l, q);
+    if (!on_tc(l)) return fmm::launch_m2l_fp32(P, l, q);
+    const cudaError_t e = fmm::launch_split_bf16(P, l, q);
+    return e != cudaSuccess ? e : fmm::launch_m2l_tc(P, l, P.prec, q);
+  };
+  if (!t) {
+    // `s`: tensor-core levels, then the FP32 spectral levels; the first
+    // auxiliary stream: the double-float spectral levels and the rest
+    bool side = false, main = false;
     for (int l = 2; l <= P.L; ++l) {
-      if (on_tc(l)) continue;
-      if (fmm::fft_level(P, l))
-        FMM_CUDA_TRY(fmm::launch_m2l_fft(P, l, P.aux[0]));
-      else
-        FMM_CUDA_TRY(fmm::launch_m2l_fp32(P, l, P.aux[0]));
+      if (on_tc(l) || (on_spec(l) && !fmm::wide_level(P, l))) main = true;
+      else side = true;
     }
-    FMM_CUDA_TRY(cudaEventRecord(P.fev[3], P.aux[0]));
-    FMM_CUDA_TRY(cudaStreamWaitEvent(s, P.fev[3], 0));
+    const bool fork = side && main;
+    cudaStream_t q = fork ? P.aux[0] : s;
+    if (fork) FMM_CUDA_TRY(cudaEventRecord(P.fev[2], s));
+    for (int l = P.L; l >= 2; --l)
+      if (on_tc(l)) FMM_CUDA_TRY(m2l_level(l, s));
+    int f0 = P.L + 1, f1 = 1, d0 = P.L + 1, d1 = 1;   // spectral levels: wide_level and on_tc split them by depth
+    for (int l = 2; l <= P.L; ++l) {
+      if (!on_spec(l)) continue;
+      int &lo = fmm::wide_level(P, l) ? d0 : f0, &hi = fmm::wide_level(P, l) ? d1 : f1;
+      lo = l < lo ? l : lo;
+      hi = l;
+    }
+    if (f0 <= f1) FMM_CUDA_TRY(fmm::launch_m2l_spec(P, false, f0, f1, s));
+    if (fork) FMM_CUDA_TRY(cudaStreamWaitEvent(q, P.fev[2], 0));
+    if (d0 <= d1) FMM_CUDA_TRY(fmm::launch_m2l_spec(P, true, d0, d1, q));
+    for (int l = 2; l <= P.L; ++l)
+      if (!on_tc(l) && !on_spec(l)) FMM_CUDA_TRY(m2l_level(l, q));
+    if (fork) {
+      FMM_CUDA_TRY(cudaEventRecord(P.fev[3], q));
+      FMM_CUDA_TRY(cudaStreamWaitEvent(s, P.fev[3], 0));
+    }
   } else {
     for (int l = 2; l <= P.L; ++l) {
       FMM_CUDA_TRY(mark(FMM_TIME_M2L_LEVEL0 + l, 0));
-      if (fmm::fft_level(P, l)) {
-        FMM_CUDA_TRY(fmm::launch_m2l_fft(P, l, s));
-      } else if (on_tc(l)) {
-        FMM_CUDA_TRY(fmm::launch_split_bf16(P, l, s));
-        FMM_CUDA_TRY(fmm::launch_m2l_tc(P, l, P.prec, s));
-      } else {
-        FMM_CUDA_TRY(fmm::launch_m2l_fp32(P, l, s));
-      }
+      FMM_CUDA_TRY(on_spec(l) ? fmm::launch_m2l_spec(P, fmm::wide_level(P, l), l, l, s) : m2l_level(l, s));
       FMM_CUDA_TRY(mark(FMM_TIME_M2L_LEVEL0 + l, 1));
     }
   }

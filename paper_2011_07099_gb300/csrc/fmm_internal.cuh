@@ -94,6 +94,12 @@ struct Plan {
   float2* w_p2m = nullptr;          // Lagrange weights [p][S] as (hi, lo): gridlet s at cell c
   float2* w_m2m = nullptr;          // Lagrange weights [p][2p] as (hi, lo): parent s at child point u
   int8_t* offsets[kMaxLevel + 1] = {};  // per level: [8 child types][n_off][3] (dx, dy, dz) = T - S
+  // spectral M2L (m2l_spec.cu), the levels that have its buffers: kernel
+  // spectra, source spectra and target spectra of the level, and the DFT twiddles
+  void* spec_K[kMaxLevel + 1] = {};
+  void* spec_M[kMaxLevel + 1] = {};
+  void* spec_P[kMaxLevel + 1] = {};
+  float4* spec_tw = nullptr;
   // tensor-core M2L (levels >= kTcMinLevel, allocated on the first mixed-precision solve)
   uint4* tab_bf[kMaxLevel + 1] = {};       // per table entry, per field: bf16 hi | bf16 lo << 16
   void* Mbf_hi[kMaxLevel + 1] = {};        // gridlet masses split into BF16 parts (2; 3 at bf16x6 levels), per parity class with a halo
@@ -177,6 +183,21 @@ inline int tc_first_level(const Plan& P) {
   return P.tc_min_level > wide_first ? P.tc_min_level : wide_first;
 }
 
+// The levels of the mixed forms that run the dense tensor-core contraction:
+// the wide ones (bf16x6; in double-float spectral products level 5 of 512^3
+// order 8 takes 74 ms against 94 ms, but the mixed form's results would then
+// differ from bf16x6's by its own 1e-3 of the rms at the cells around the
+// heaviest clumps), the low orders, and a level without spectral buffers.  From
+// kSpecOrder on the FP32 levels take the spectral products (m2l_spec.cu),
+// whose 16x (p = 6) to 36x (p = 8) fewer terms beat the tensor pipe's three
+// BF16 products per term: measured 256^3 p = 6 levels 4 + 5 4.78 -> 4.46 ms,
+// 512^3 p = 8 level 6 281 -> 77 ms; at p = 4 (5x fewer terms) the tensor
+// cores keep level 5 of 128^3 (0.83 against 1.30 ms).
+constexpr int kSpecOrder = 5;
+inline bool tc_level(const Plan& P, int l) {
+  return l >= tc_first_level(P) && (wide_level(P, l) || P.p < kSpecOrder || !P.spec_K[l]);
+}
+
 cudaError_t setup_m2l_fp32(const Plan& P);
 // Number of offset ranges the FP32 M2L of a level is split into (1 = none).
 int m2l_fp32_splits(const Plan& P, int level);
@@ -200,6 +221,17 @@ bool fft_level(const Plan& P, int level);
 int prepare_fft(Plan& P);
 cudaError_t launch_m2l_fft(Plan& P, int level, cudaStream_t s);
 void free_fft(Plan& P);
+// Spectral M2L (m2l_spec.cu): buffer sizes of a level, function attributes,
+// the plan-time kernel spectra (after every re-tabulation), and the M2L of
+// every spectral level in l0..l1 with FP64 (df) or FP32 local fields.
+size_t spec_kernel_bytes(const Plan& P, int level);
+size_t spec_source_bytes(const Plan& P, int level);
+size_t spec_target_bytes(const Plan& P, int level);
+cudaError_t setup_m2l_spec(const Plan& P);
+cudaError_t launch_spec_kernels(Plan& P, int level, cudaStream_t s);
+// FP32 spectra of `blocks` order-p gridlets, [chunk][blocks + 1][16].
+cudaError_t launch_spec_fwd(Plan& P, const float* src, void* dst, size_t blocks, cudaStream_t s);
+cudaError_t launch_m2l_spec(Plan& P, bool df, int l0, int l1, cudaStream_t s);
 cudaError_t launch_l2l(Plan& P, int level, cudaStream_t s);       // F[level] -> F[level+1] (adds)
 // near_fwd_done: the FFT near zone's source spectra were already taken (launch_near_fft_fwd).
 cudaError_t launch_p2p(Plan& P, const float* rho, float* phi, float* acc, cudaStream_t s,
