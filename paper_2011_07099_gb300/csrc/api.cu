@@ -135,6 +135,13 @@ void free_plan(Plan* P) {
   cudaFree(P->nz_P);
   cudaFree(P->d_err);
   cudaFree(P->corr_w);
+  cudaFree(P->corr_samples);
+  cudaFree(P->corr_val);
+  cudaFree(P->corr_up);
+  cudaFree(P->tg_la);
+  cudaFree(P->tg_mh);
+  cudaFree(P->tg_gh);
+  cudaFree(P->tg_gl);
   cudaFree(P->train_out);
   cudaFree(P->lam_cells);
   cudaFree(P->dT_all);
@@ -263,6 +270,17 @@ int table_gradient(Plan& P, const float* density, const float* target_phi, const
               dev_alloc(&P.grad_partials, (size_t)fmm::mlp_backward_blocks(P) * fmm::mlp::kParams);
     for (int l = 2; l <= P.L && ok; ++l) ok = dev_alloc(&P.lam[l], ((size_t)1 << (3 * l)) * 4 * p3);
     if (!ok) return FMM_ERR_ALLOC;
+    size_t la, mh, gh, gl;
+    fmm::tg_bytes(P, la, mh, gh, gl);
+    if (P.p >= 2 && la + mh + gh + gl <= kSpecMaxBytes &&
+        (cudaMalloc(&P.tg_mh, mh) != cudaSuccess || cudaMalloc(&P.tg_gh, gh) != cudaSuccess ||
+         cudaMalloc(&P.tg_gl, gl) != cudaSuccess || cudaMalloc(&P.tg_la, la) != cudaSuccess)) {
+      for (void** b : {&P.tg_la, &P.tg_mh, &P.tg_gh, &P.tg_gl}) {   // no room: the direct sums
+        cudaFree(*b);
+        *b = nullptr;
+      }
+      (void)cudaGetLastError();
+    }
     for (int l = 2; l <= P.L; ++l) P.dT[l] = P.dT_all + (size_t)(l - 2) * E * E * E * 4;
   }
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
@@ -404,6 +422,7 @@ fmm_plan* fmm_plan_create(int N, int L, int order) {
   }
   if (fmm::setup_upward(*P) != cudaSuccess || fmm::setup_m2l_fp32(*P) != cudaSuccess ||
       fmm::setup_m2l_tc(*P) != cudaSuccess || fmm::setup_learn() != cudaSuccess ||
+      fmm::setup_learn_spec(*P) != cudaSuccess ||
       fmm::setup_downward(*P) != cudaSuccess || fmm::setup_p2p(*P) != cudaSuccess ||
       fmm::setup_m2l_spec(*P) != cudaSuccess || retabulate(*P) != FMM_OK) {
     free_plan(P);
@@ -666,7 +685,16 @@ int fmm_plan_set_correction(fmm_plan* plan, const float* weights, size_t n) {
   Plan& P = *reinterpret_cast<Plan*>(plan);
   if (weights) {
     if (n != (size_t)fmm::mlp::kParams) return set_err(FMM_ERR_ARG);
-    if (!P.corr_w && !dev_alloc(&P.corr_w, (size_t)fmm::mlp::kParams)) return set_err(FMM_ERR_ALLOC);
+    if (!P.corr_w) {
+      const std::vector<uint32_t> samples = fmm::corr_samples(P.p);
+      if ((!P.corr_samples && !dev_alloc(&P.corr_samples, samples.size())) ||
+          (!P.corr_val && !dev_alloc(&P.corr_val, fmm::corr_values(P))) ||
+          (!P.corr_up && !dev_alloc(&P.corr_up, (size_t)(P.L - 1) * samples.size())))
+        return set_err(FMM_ERR_ALLOC);
+      FMM_CUDA_TRY(cudaMemcpy(P.corr_samples, samples.data(), samples.size() * sizeof(uint32_t), cudaMemcpyHostToDevice));
+      P.n_corr = (int)samples.size();
+      if (!dev_alloc(&P.corr_w, (size_t)fmm::mlp::kParams)) return set_err(FMM_ERR_ALLOC);
+    }
     FMM_CUDA_TRY(cudaMemcpy(P.corr_w, weights, n * sizeof(float), cudaMemcpyDefault));
     P.has_corr = 1;
   } else {

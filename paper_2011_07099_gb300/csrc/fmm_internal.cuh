@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <cstdint>
 #include <cstddef>
+#include <vector>
 
 #include "../../include/fmm.h"
 #include "green_s1.cuh"
@@ -122,6 +123,17 @@ struct Plan {
   float* corr_w = nullptr;                 // mlp::kParams weights (device) or unset
   int has_corr = 0;
   int corr_fp32 = 0;                       // 0: BF16 inference (default), 1: FP32
+  // distinct network inputs of the plan's tables, the network's values there
+  // ([level - 2][class][4p]^3) and their upstream gradients (learn_spec.cu)
+  uint32_t* corr_samples = nullptr;
+  int n_corr = 0;
+  float* corr_val = nullptr;
+  float* corr_up = nullptr;
+  // scratch of the spectral table gradient: spectra of lam and M, offset spectra and lags
+  void* tg_la = nullptr;
+  void* tg_mh = nullptr;
+  void* tg_gh = nullptr;
+  void* tg_gl = nullptr;
   float* train_out = nullptr;              // 4 N^3: the solve's outputs during training
   float* lam_cells = nullptr;              // 4 N^3: cell residual adjoint
   float* lam[kMaxLevel + 1] = {};          // adjoint of the local fields, 8^l x 4 x p^3
@@ -247,6 +259,14 @@ cudaError_t launch_near_fft_fwd(Plan& P, const float* rho, cudaStream_t s);
 cudaError_t launch_near_fft(Plan& P, const float* rho, float* phi, float* acc, cudaStream_t s, bool fwd_done);
 cudaError_t setup_m2l_tc(const Plan& P);
 cudaError_t setup_learn();
+// Distinct inputs of the learned correction and the spectral table gradient (learn_spec.cu).
+std::vector<uint32_t> corr_samples(int p);
+size_t corr_values(const Plan& P);
+cudaError_t setup_learn_spec(const Plan& P);
+cudaError_t launch_corr_eval(Plan& P, cudaStream_t s);
+cudaError_t launch_corr_fold(Plan& P, cudaStream_t s);
+void tg_bytes(const Plan& P, size_t& la, size_t& mh, size_t& gh, size_t& gl);
+cudaError_t launch_table_grad_spec(Plan& P, int level, cudaStream_t s);
 cudaError_t launch_residual(const float* phi, const float* acc, const float* tphi, const float* tacc, size_t n3,
                             float w_phi, float w_g, float* lam, float* loss, int sms, cudaStream_t s);
 cudaError_t launch_adjoint_and_table_grad(Plan& P, const float* lam_cells, cudaStream_t s);

@@ -89,6 +89,8 @@ __global__ void k_adj_l2l(const float* __restrict__ lamc, int p, const float2* _
 }
 
 // ------------------------------------------------------ table gradient
+// Direct sums: isolated plans, order 1, and levels whose spectra have no
+// buffers (the others: learn_spec.cu).
 // CTA (offset index io, child type c, field f): for every d in [-(p-1), p-1]^3,
 //   g[d] = sum over targets T of type c, sum_r lam[T][f][r] M[T - o][r - d],
 // added to dT[o p + d][f].  Targets are staged 32 at a time in shared memory.
@@ -160,75 +162,76 @@ __global__ void k_table_grad(const float* __restrict__ lam, const float* __restr
 }
 
 // ----------------------------------------------------------- MLP backward
-// Samples are the table entries (level, n, f); the upstream gradient of the
-// MLP output of a sample is dT * scale * sign (mlp::features).  One block of
-// kBwdTile threads processes tiles of kBwdTile samples (one per thread) and
-// accumulates the parameter gradient in shared memory (each thread owns a
-// fixed set of parameters); per-block partials are summed by k_grad_reduce.
+// Samples are the distinct network inputs of every level (learn_spec.cu) with
+// their folded upstream gradients.  One block of kBwdTile threads processes
+// tiles of kBwdTile samples (one per thread) and accumulates the parameter
+// gradient in shared memory (each thread owns a fixed set of parameters);
+// per-block partials are summed by k_grad_reduce.  Activation rows are padded
+// to 65 floats: a thread walks its own row, so rows 64 apart would put a
+// warp's 32 reads on one bank.  Measured at p = 6, L = 3: 16.4 ms for the
+// 830 600 table entries one by one.
 constexpr int kBwdTile = 64;
 constexpr int kPerThread = (mlp::kParams + kBwdTile - 1) / kBwdTile;   // 138
+constexpr int kRow = mlp::kH + 1;
 
-__global__ void __launch_bounds__(kBwdTile) k_mlp_backward(const float* __restrict__ w, const float* __restrict__ dT,
-                                                          int lmin, int lmax, int p, float* __restrict__ partials) {
+__global__ void __launch_bounds__(kBwdTile) k_mlp_backward(const float* __restrict__ w, const float* __restrict__ up,
+                                                          const uint32_t* __restrict__ samples, int ns, int lmax, int p,
+                                                          float* __restrict__ partials) {
   using namespace mlp;
   extern __shared__ float smf[];
   float* sw = smf;                               // kParams
   float* X = sw + kParams;                       // tile x kIn
-  float* Z1 = X + kBwdTile * kIn;                // tile x kH (pre-activations)
-  float* Z2 = Z1 + kBwdTile * kH;
-  float* Z3 = Z2 + kBwdTile * kH;
-  float* H1 = Z3 + kBwdTile * kH;                // post-activations
-  float* H2 = H1 + kBwdTile * kH;
-  float* G = H2 + kBwdTile * kH;                 // tile x kH (backprop buffer)
-  float* GO = G + kBwdTile * kH;                 // tile (upstream gradient)
+  float* Z1 = X + kBwdTile * kIn;                // tile x kRow (pre-activations)
+  float* Z2 = Z1 + kBwdTile * kRow;
+  float* Z3 = Z2 + kBwdTile * kRow;
+  float* H1 = Z3 + kBwdTile * kRow;              // post-activations
+  float* H2 = H1 + kBwdTile * kRow;
+  float* G = H2 + kBwdTile * kRow;               // tile x kRow (backprop buffer)
+  float* GO = G + kBwdTile * kRow;               // tile (upstream gradient)
   float* gacc = GO + kBwdTile;                   // kParams: this block's gradient
   const int tid = threadIdx.x;
   for (int i = tid; i < kParams; i += kBwdTile) {
     sw[i] = w[i];
     gacc[i] = 0.f;
   }
-  const int E = 8 * p - 1;
-  const long E3 = (long)E * E * E;
-  const long total = (long)(lmax - lmin + 1) * E3 * 4;
+  const int total = (lmax - 1) * ns;
   __syncthreads();
-  for (long base = (long)blockIdx.x * kBwdTile; base < total; base += (long)gridDim.x * kBwdTile) {
+  for (int base = blockIdx.x * kBwdTile; base < total; base += gridDim.x * kBwdTile) {
     // forward for sample base + tid
     {
-      const long sidx = base + tid;
+      const int sidx = base + tid;
       float x[kIn] = {0.f, 0.f, 0.f, 0.f, 0.f};
       float go = 0.f;
       if (sidx < total) {
-        const int f = (int)(sidx % 4);
-        const long e = (sidx / 4) % E3;
-        const int level = lmin + (int)(sidx / (4 * E3));
-        const int hw = 4 * p - 1;
-        const int nx = (int)(e % E) - hw, ny = (int)((e / E) % E) - hw, nz = (int)(e / ((long)E * E)) - hw;
-        float sign;
-        double scale;
-        features(nx, ny, nz, f, level, p, x, sign, scale);
-        const float g = dT[((size_t)(level - lmin) * E3 + e) * 4 + f];
-        go = (nx | ny | nz) ? (float)(g * scale) * sign : 0.f;
+        const uint32_t q = samples[sidx % ns];
+        const float inv = 1.f / (4.f * p);
+        x[0] = (int)((q >> 16) & 255) * inv;
+        x[1] = (int)((q >> 8) & 255) * inv;
+        x[2] = (int)(q & 255) * inv;
+        x[3] = (2 + sidx / ns) * 0.125f;
+        x[4] = (float)(q >> 24);
+        go = up[sidx];
       }
       GO[tid] = go;
       for (int j = 0; j < kIn; ++j) X[tid * kIn + j] = x[j];
       for (int i = 0; i < kH; ++i) {
         float z = sw[kOffB1 + i];
         for (int j = 0; j < kIn; ++j) z = fmaf(sw[kOffW1 + i * kIn + j], x[j], z);
-        Z1[tid * kH + i] = z;
-        H1[tid * kH + i] = gelu(z);
+        Z1[tid * kRow + i] = z;
+        H1[tid * kRow + i] = gelu(z);
       }
       for (int i = 0; i < kH; ++i) {
         float z = sw[kOffB2 + i];
-        for (int j = 0; j < kH; ++j) z = fmaf(sw[kOffW2 + i * kH + j], H1[tid * kH + j], z);
-        Z2[tid * kH + i] = z;
-        H2[tid * kH + i] = gelu(z);
+        for (int j = 0; j < kH; ++j) z = fmaf(sw[kOffW2 + i * kH + j], H1[tid * kRow + j], z);
+        Z2[tid * kRow + i] = z;
+        H2[tid * kRow + i] = gelu(z);
       }
       for (int i = 0; i < kH; ++i) {
         float z = sw[kOffB3 + i];
-        for (int j = 0; j < kH; ++j) z = fmaf(sw[kOffW3 + i * kH + j], H2[tid * kH + j], z);
-        Z3[tid * kH + i] = z;
+        for (int j = 0; j < kH; ++j) z = fmaf(sw[kOffW3 + i * kH + j], H2[tid * kRow + j], z);
+        Z3[tid * kRow + i] = z;
         // dz3 = go * W4 * gelu'(z3)
-        G[tid * kH + i] = go * sw[kOffW4 + i] * gelu_grad(z);
+        G[tid * kRow + i] = go * sw[kOffW4 + i] * gelu_grad(z);
       }
     }
     __syncthreads();
@@ -239,13 +242,13 @@ __global__ void __launch_bounds__(kBwdTile) k_mlp_backward(const float* __restri
         float a = 0.f;
         if (q < kOffB3) {
           const int i = (q - kOffW3) / kH, j = (q - kOffW3) % kH;
-          for (int s = 0; s < kBwdTile; ++s) a = fmaf(G[s * kH + i], H2[s * kH + j], a);
+          for (int s = 0; s < kBwdTile; ++s) a = fmaf(G[s * kRow + i], H2[s * kRow + j], a);
         } else if (q < kOffW4) {
           const int i = q - kOffB3;
-          for (int s = 0; s < kBwdTile; ++s) a += G[s * kH + i];
+          for (int s = 0; s < kBwdTile; ++s) a += G[s * kRow + i];
         } else if (q < kOffB4) {
           const int i = q - kOffW4;
-          for (int s = 0; s < kBwdTile; ++s) a = fmaf(GO[s], gelu(Z3[s * kH + i]), a);
+          for (int s = 0; s < kBwdTile; ++s) a = fmaf(GO[s], gelu(Z3[s * kRow + i]), a);
         } else {
           for (int s = 0; s < kBwdTile; ++s) a += GO[s];
         }
@@ -258,10 +261,10 @@ __global__ void __launch_bounds__(kBwdTile) k_mlp_backward(const float* __restri
       float d2[kH];
       for (int j = 0; j < kH; ++j) d2[j] = 0.f;
       for (int i = 0; i < kH; ++i) {
-        const float g3 = G[tid * kH + i];
+        const float g3 = G[tid * kRow + i];
         for (int j = 0; j < kH; ++j) d2[j] = fmaf(sw[kOffW3 + i * kH + j], g3, d2[j]);
       }
-      for (int j = 0; j < kH; ++j) Z3[tid * kH + j] = d2[j] * gelu_grad(Z2[tid * kH + j]);
+      for (int j = 0; j < kH; ++j) Z3[tid * kRow + j] = d2[j] * gelu_grad(Z2[tid * kRow + j]);
     }
     __syncthreads();
     for (int k = 0; k < kPerThread; ++k) {
@@ -270,10 +273,10 @@ __global__ void __launch_bounds__(kBwdTile) k_mlp_backward(const float* __restri
         float a = 0.f;
         if (q < kOffB2) {
           const int i = (q - kOffW2) / kH, j = (q - kOffW2) % kH;
-          for (int s = 0; s < kBwdTile; ++s) a = fmaf(Z3[s * kH + i], H1[s * kH + j], a);
+          for (int s = 0; s < kBwdTile; ++s) a = fmaf(Z3[s * kRow + i], H1[s * kRow + j], a);
         } else {
           const int i = q - kOffB2;
-          for (int s = 0; s < kBwdTile; ++s) a += Z3[s * kH + i];
+          for (int s = 0; s < kBwdTile; ++s) a += Z3[s * kRow + i];
         }
         gacc[q] += a;
       }
@@ -284,10 +287,10 @@ __global__ void __launch_bounds__(kBwdTile) k_mlp_backward(const float* __restri
       float d1[kH];
       for (int j = 0; j < kH; ++j) d1[j] = 0.f;
       for (int i = 0; i < kH; ++i) {
-        const float g2 = Z3[tid * kH + i];
+        const float g2 = Z3[tid * kRow + i];
         for (int j = 0; j < kH; ++j) d1[j] = fmaf(sw[kOffW2 + i * kH + j], g2, d1[j]);
       }
-      for (int j = 0; j < kH; ++j) G[tid * kH + j] = d1[j] * gelu_grad(Z1[tid * kH + j]);
+      for (int j = 0; j < kH; ++j) G[tid * kRow + j] = d1[j] * gelu_grad(Z1[tid * kRow + j]);
     }
     __syncthreads();
     for (int k = 0; k < kPerThread; ++k) {
@@ -296,10 +299,10 @@ __global__ void __launch_bounds__(kBwdTile) k_mlp_backward(const float* __restri
         float a = 0.f;
         if (q < kOffB1) {
           const int i = q / kIn, j = q % kIn;
-          for (int s = 0; s < kBwdTile; ++s) a = fmaf(G[s * kH + i], X[s * kIn + j], a);
+          for (int s = 0; s < kBwdTile; ++s) a = fmaf(G[s * kRow + i], X[s * kIn + j], a);
         } else {
           const int i = q - kOffB1;
-          for (int s = 0; s < kBwdTile; ++s) a += G[s * kH + i];
+          for (int s = 0; s < kBwdTile; ++s) a += G[s * kRow + i];
         }
         gacc[q] += a;
       }
@@ -407,6 +410,11 @@ cudaError_t launch_adjoint_and_table_grad(Plan& P, const float* lam_cells, cudaS
   }
   const size_t E = 8 * p - 1;
   for (int l = 2; l <= P.L; ++l) {
+    if (P.tg_la && !P.iso) {
+      const cudaError_t e = launch_table_grad_spec(P, l, s);
+      if (e != cudaSuccess) return e;
+      continue;
+    }
     cudaError_t e = cudaMemsetAsync(P.dT[l], 0, sizeof(float) * E * E * E * 4, s);
     if (e != cudaSuccess) return e;
     const size_t smem = sizeof(float) * 2 * kTgChunk * p3;
@@ -419,7 +427,7 @@ cudaError_t launch_adjoint_and_table_grad(Plan& P, const float* lam_cells, cudaS
 }
 
 size_t mlp_backward_smem() {
-  return sizeof(float) * (2 * mlp::kParams + kBwdTile * mlp::kIn + 6 * kBwdTile * mlp::kH + kBwdTile);
+  return sizeof(float) * (2 * mlp::kParams + kBwdTile * mlp::kIn + 6 * kBwdTile * kRow + kBwdTile);
 }
 
 int mlp_backward_blocks(const Plan& P) { return 2 * P.num_sms; }
@@ -435,10 +443,12 @@ cudaError_t setup_learn() {
 }
 
 cudaError_t launch_mlp_backward(Plan& P, const float* w, float* grad, cudaStream_t s) {
-  // dT of levels 2..L are contiguous per level in P.dT_all
+  cudaError_t e = launch_corr_fold(P, s);
+  if (e != cudaSuccess) return e;
   const int nb = mlp_backward_blocks(P);
-  k_mlp_backward<<<nb, kBwdTile, mlp_backward_smem(), s>>>(w, P.dT_all, 2, P.L, P.p, P.grad_partials);
-  cudaError_t e = cudaGetLastError();
+  k_mlp_backward<<<nb, kBwdTile, mlp_backward_smem(), s>>>(w, P.corr_up, P.corr_samples, P.n_corr, P.L, P.p,
+                                                          P.grad_partials);
+  e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   k_grad_reduce<<<(mlp::kParams + 255) / 256, 256, 0, s>>>(P.grad_partials, nb, grad);
   return cudaGetLastError();

@@ -45,14 +45,15 @@ __host__ __device__ inline int wrap_offset(int v, int period) {
   return v;
 }
 
-__host__ __device__ inline void features(int nx, int ny, int nz, int f, int level, int p, float x[kIn], float& sign,
-                                         double& scale) {
+// Table entry n, field f as a network input: the integer components (a, b, c)
+// and the sign and scale its output is applied with.
+__host__ __device__ inline void sample_of(int nx, int ny, int nz, int f, int level, int p, int& a, int& b, int& c,
+                                          float& sign, double& scale) {
   const int period = (1 << level) * p;
   nx = wrap_offset(nx, period);
   ny = wrap_offset(ny, period);
   nz = wrap_offset(nz, period);
   const int ax = nx < 0 ? -nx : nx, ay = ny < 0 ? -ny : ny, az = nz < 0 ? -nz : nz;
-  int a, b, c;
   sign = 1.f;
   if (f == 0) {
     a = ax; b = ay; c = az;
@@ -66,12 +67,6 @@ __host__ __device__ inline void features(int nx, int ny, int nz, int f, int leve
     // odd and periodic: zero at n_i = 0 and at half the box, as grad G_S1
     sign = (2 * own == period) ? 0.f : (s > 0 ? 1.f : (s < 0 ? -1.f : 0.f));
   }
-  const float inv = 1.f / (4.f * p);
-  x[0] = a * inv;
-  x[1] = b * inv;
-  x[2] = c * inv;
-  x[3] = level * 0.125f;
-  x[4] = f == 0 ? 0.f : 1.f;
   const double base = (double)(1 << level) * p;
   scale = kKappa * (f == 0 ? base : base * base) / (4.0 * 3.14159265358979323846);
 }
@@ -83,38 +78,6 @@ __device__ __forceinline__ float gelu_grad(float z) {
 }
 
 __device__ __forceinline__ float round_bf16(float v) { return __bfloat162float(__float2bfloat16_rn(v)); }
-
-// Forward pass for one sample.  BF16 = true rounds the weights and the
-// activations to BF16 (FP32 accumulation): the inference form.
-template <bool BF16>
-__device__ inline float forward(const float* __restrict__ w, const float x[kIn]) {
-  float h1[kH], h2[kH];
-#pragma unroll 4
-  for (int i = 0; i < kH; ++i) {
-    float z = w[kOffB1 + i];
-#pragma unroll
-    for (int j = 0; j < kIn; ++j) {
-      const float wij = BF16 ? round_bf16(w[kOffW1 + i * kIn + j]) : w[kOffW1 + i * kIn + j];
-      z = fmaf(wij, BF16 ? round_bf16(x[j]) : x[j], z);
-    }
-    h1[i] = BF16 ? round_bf16(gelu(z)) : gelu(z);
-  }
-#pragma unroll 2
-  for (int i = 0; i < kH; ++i) {
-    float z = w[kOffB2 + i];
-    for (int j = 0; j < kH; ++j) z = fmaf(BF16 ? round_bf16(w[kOffW2 + i * kH + j]) : w[kOffW2 + i * kH + j], h1[j], z);
-    h2[i] = BF16 ? round_bf16(gelu(z)) : gelu(z);
-  }
-  float out = w[kOffB4];
-#pragma unroll 2
-  for (int i = 0; i < kH; ++i) {
-    float z = w[kOffB3 + i];
-    for (int j = 0; j < kH; ++j) z = fmaf(BF16 ? round_bf16(w[kOffW3 + i * kH + j]) : w[kOffW3 + i * kH + j], h2[j], z);
-    const float h3 = BF16 ? round_bf16(gelu(z)) : gelu(z);
-    out = fmaf(BF16 ? round_bf16(w[kOffW4 + i]) : w[kOffW4 + i], h3, out);
-  }
-  return out;
-}
 
 }  // namespace mlp
 }  // namespace fmm

@@ -14,16 +14,19 @@ namespace {
 using green::cube_mean_inv_r;
 using green::kPi;
 
-// Learned correction of one table entry (all four fields), if weights are set.
-__device__ inline void add_correction(double v[4], int ix, int iy, int iz, int level, int p, const float* mlp, int fp32) {
-  if (!mlp || !(ix | iy | iz)) return;
+// Learned correction of one table entry (all four fields): the network's
+// value at the entry's distinct input (k_corr_eval, learn_spec.cu), `corr` the
+// level's [2 classes][4p]^3 block.
+__device__ inline void add_correction(double v[4], int ix, int iy, int iz, int level, int p, const float* corr) {
+  if (!corr || !(ix | iy | iz)) return;
+  const int G = 4 * p;
   for (int f = 0; f < 4; ++f) {
-    float x[mlp::kIn], sign;
+    int a, b, c;
+    float sign;
     double scale;
-    mlp::features(ix, iy, iz, f, level, p, x, sign, scale);
+    mlp::sample_of(ix, iy, iz, f, level, p, a, b, c, sign, scale);
     if (sign == 0.f) continue;
-    const float o = fp32 ? mlp::forward<false>(mlp, x) : mlp::forward<true>(mlp, x);
-    v[f] += (double)o * (double)sign * scale;
+    v[f] += (double)__ldg(corr + (((size_t)(f ? 1 : 0) * G + a) * G + b) * G + c) * (double)sign * scale;
   }
 }
 
@@ -76,15 +79,15 @@ __device__ inline void table_value(const green::Spec& gs, const double* mesh, in
   }
 }
 
-__global__ void k_tab_m2l(float4* __restrict__ out, float4* __restrict__ lo, int p, int level, const float* mlp,
-                          int fp32, const float* grid, green::Spec gs, const double* mesh, int N) {
+__global__ void k_tab_m2l(float4* __restrict__ out, float4* __restrict__ lo, int p, int level, const float* corr,
+                          const float* grid, green::Spec gs, const double* mesh, int N) {
   const int hw = 4 * p - 1, E = 8 * p - 1;
   const long total = (long)E * E * E;
   for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < total; i += (long)gridDim.x * blockDim.x) {
     const int ix = (int)(i % E) - hw, iy = (int)((i / E) % E) - hw, iz = (int)(i / ((long)E * E)) - hw;
     double v[4] = {0.0, 0.0, 0.0, 0.0};
     if (ix | iy | iz) table_value(gs, mesh, N, level, p, ix, iy, iz, v);
-    add_correction(v, ix, iy, iz, level, p, mlp, fp32);
+    add_correction(v, ix, iy, iz, level, p, corr);
     add_grid(v, ix, iy, iz, level, p, grid);
     out[i] = make_float4((float)v[0], (float)v[1], (float)v[2], (float)v[3]);
     if (lo)
@@ -120,7 +123,7 @@ __global__ void k_tab_near(float4* __restrict__ out, int S, int N, green::Spec g
 // The same level table split into BF16 hi + lo per field for the tensor-core
 // M2L: each uint32 holds hi in its low half and lo = bf16(v - hi) in its high
 // half, the four fields in the four words of a uint4.
-__global__ void k_tab_bf16(uint4* __restrict__ out, int p, int level, const float* mlp, int fp32, const float* grid,
+__global__ void k_tab_bf16(uint4* __restrict__ out, int p, int level, const float* corr, const float* grid,
                            green::Spec gs, const double* mesh, int N) {
   const int hw = 4 * p - 1, E = 8 * p - 1;
   const long total = (long)E * E * E;
@@ -128,7 +131,7 @@ __global__ void k_tab_bf16(uint4* __restrict__ out, int p, int level, const floa
     const int ix = (int)(i % E) - hw, iy = (int)((i / E) % E) - hw, iz = (int)(i / ((long)E * E)) - hw;
     double v[4] = {0.0, 0.0, 0.0, 0.0};
     if (ix | iy | iz) table_value(gs, mesh, N, level, p, ix, iy, iz, v);
-    add_correction(v, ix, iy, iz, level, p, mlp, fp32);
+    add_correction(v, ix, iy, iz, level, p, corr);
     add_grid(v, ix, iy, iz, level, p, grid);
     uint32_t w[4];
     for (int f = 0; f < 4; ++f) {
@@ -173,7 +176,9 @@ bool plain_gs1(const Plan& P) { return P.gspec.kind == 0 && !P.iso; }
 const float* grid_of(const Plan& P, int level) {
   return P.has_grid && plain_gs1(P) ? P.grid + (size_t)(level - 2) * grid_level_size(P.p) : nullptr;
 }
-const float* mlp_of(const Plan& P) { return P.has_corr && plain_gs1(P) ? P.corr_w : nullptr; }
+const float* corr_of(const Plan& P, int level) {
+  return P.has_corr && plain_gs1(P) ? P.corr_val + (size_t)(level - 2) * 2 * 64 * P.p * P.p * P.p : nullptr;
+}
 // The function the tables hold: G_0 in the isolated problem.
 green::Spec spec_of(const Plan& P) {
   if (!P.iso) return P.gspec;
@@ -194,14 +199,18 @@ cudaError_t launch_grid_grad(Plan& P, float* grad, cudaStream_t s) {
 }
 
 cudaError_t launch_tab_bf16(Plan& P, int level, cudaStream_t s) {
-  k_tab_bf16<<<4 * P.num_sms, 256, 0, s>>>(P.tab_bf[level], P.p, level, mlp_of(P), P.corr_fp32, grid_of(P, level),
+  k_tab_bf16<<<4 * P.num_sms, 256, 0, s>>>(P.tab_bf[level], P.p, level, corr_of(P, level), grid_of(P, level),
                                            spec_of(P), P.gmesh, P.N);
   return cudaGetLastError();
 }
 
 cudaError_t launch_tables(Plan& P, cudaStream_t s) {
+  if (P.has_corr && plain_gs1(P)) {
+    const cudaError_t e = launch_corr_eval(P, s);
+    if (e != cudaSuccess) return e;
+  }
   for (int l = 2; l <= P.L; ++l) {
-    k_tab_m2l<<<4 * P.num_sms, 256, 0, s>>>(P.tab[l], P.tab_lo[l], P.p, l, mlp_of(P), P.corr_fp32, grid_of(P, l),
+    k_tab_m2l<<<4 * P.num_sms, 256, 0, s>>>(P.tab[l], P.tab_lo[l], P.p, l, corr_of(P, l), grid_of(P, l),
                                             spec_of(P), P.gmesh, P.N);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;

@@ -78,3 +78,37 @@ def test_levels_in_one_launch_equal_levels_one_by_one_bitwise(B):
     for p in (4, 7):
         a, b = _solve(B, rho, 5, p), _solve(B, rho, 5, p, timing=True)
         assert np.array_equal(a[0], b[0]) and np.array_equal(a[1], b[1])
+
+
+@pytest.mark.parametrize("N,L,p", [(8, 2, 4), (8, 3, 3), (8, 3, 5), (16, 4, 2)])
+def test_spectral_table_gradient_matches_oracle_differences(B, N, L, p):
+    # the loss is quadratic in the table values, so central differences of the
+    # FP64 oracle are exact up to its rounding; entries at window edges
+    # (components that are multiples of p, and the largest 4p - 1), inside
+    # windows and on the axes.  FP32 residual, adjoint and sums: rounding of
+    # ~1e-5 of the largest gradient; bound 1e-3 of it.
+    from oracle import learn as olearn
+    rho = inputs.lognormal(N, sigma=0.8, seed=N + p)
+    n, G = olearn.grid_size(L, p), 4 * p
+    theta = np.zeros(n)
+    tphi, tg = (np.asarray(x) * 1.3 for x in olearn.pm_target(rho))
+    w_phi, w_g = 1.0 / np.sum(tphi ** 2), 1.0 / np.sum(tg ** 2)
+    plan = B.Plan(N, L, p)
+    grad = torch.zeros(n, dtype=torch.float32, device="cuda")
+    loss = torch.zeros(1, dtype=torch.float32, device="cuda")
+    f32 = lambda a: torch.from_numpy(np.ascontiguousarray(a, dtype=np.float32)).cuda()
+    B.fmm_table_grid_grad(plan.handle, f32(rho), f32(tphi), f32(tg), w_phi, w_g, grad, loss)
+    got = grad.cpu().numpy().astype(np.float64)
+    plan.close()
+    for lev in range(2, L + 1):
+        blk = got[(lev - 2) * 4 * G ** 3:(lev - 1) * 4 * G ** 3]
+        for f, a in [(0, (0, 0, 2 * p)), (0, (p, 2 * p - 1, 3)), (1, (2 * p - 1, p, 0)), (2, (1, 2 * p - 1, 2 * p - 1)),
+                     (3, (0, min(p + 1, 2 * p - 1), 2 * p - 1)), (0, (min(4 * p - 1, 2 ** lev * p // 2), 1, 0))]:
+            i = (lev - 2) * 4 * G ** 3 + ((f * G + a[2]) * G + a[1]) * G + a[0]
+            h = 1e-2 * 2.0 ** lev * p
+            tp_, tm_ = theta.copy(), theta.copy()
+            tp_[i] += h
+            tm_[i] -= h
+            fd = (olearn.grid_loss(tp_, rho, L, p, tphi, tg, w_phi, w_g)
+                  - olearn.grid_loss(tm_, rho, L, p, tphi, tg, w_phi, w_g)) / (2 * h)
+            assert abs(got[i] - fd) <= 1e-3 * np.abs(blk).max(), (lev, f, a, got[i], fd, np.abs(blk).max())
