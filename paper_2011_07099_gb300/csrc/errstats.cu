@@ -8,7 +8,8 @@
 // acceleration over those cells is the result.
 //
 // Arithmetic: per-axis xi(d/N), xi'(d/N) in FP64 (green_s1.cuh) rounded to
-// FP32; each pair's (G, -grad G) in FP32; masses and sums in FP64.
+// FP32; each pair's (G, -grad G) in FP32; masses, their products with the pair
+// values and the sums in double-float (fmm_internal.cuh).
 #include <cuda_runtime.h>
 
 #include "fmm_internal.cuh"
@@ -20,21 +21,32 @@ namespace {
 constexpr int kEsThreads = 256;   // one target cell per thread
 constexpr int kEsChunk = 2048;    // source cells staged in shared memory per step
 
+// (s, c) += (mh + ml) g: exact product by FMA, TwoSum, the errors in c
+__device__ __forceinline__ void es_mac(float2& a, float mh, float ml, float g) {
+  const float pr = __fmul_rn(mh, g);
+  const float pe = fmaf(mh, g, -pr);
+  const float2 t = df_two_sum(a.x, pr);
+  a.x = t.x;
+  a.y = fmaf(ml, g, __fadd_rn(a.y, __fadd_rn(pe, t.y)));
+}
+
 // partials[(blockIdx.x * T + t) * 4 + f]: block blockIdx.x's share of the
 // direct sum (Phi, g_x, g_y, g_z) at target t, over the source chunks
-// blockIdx.x, blockIdx.x + gridDim.x, ...
+// blockIdx.x, blockIdx.x + gridDim.x, ...  Bound by FP32 issue, ~55
+// instructions per pair: G = -1/(4 pi |xhat|) and c = G / |xhat|^2 come from
+// one reciprocal square root (one Newton step behind rsqrtf); along a row
+// g_y and g_z differ from the sum of c m by row constants only, so one
+// double-float sum serves both.  With FP64 sums, at 1/64 of the FP32 rate, it
+// took 8.97 ms for 256 targets of a 128^3 mesh.
 __global__ void __launch_bounds__(kEsThreads) k_es_direct(const float* __restrict__ rho,
                                                           const double* __restrict__ mean, int N,
                                                           const unsigned long long* __restrict__ targets, int T,
                                                           double* __restrict__ partials) {
   extern __shared__ __align__(16) unsigned char es_smem[];
-  double* sm = reinterpret_cast<double*>(es_smem);                 // kEsChunk masses
-  float* sxi = reinterpret_cast<float*>(sm + kEsChunk);           // N values xi(d/N)
-  float* sdxi = sxi + N;                                          // N values xi'(d/N)
-  for (int d = threadIdx.x; d < N; d += blockDim.x) {
-    sxi[d] = (float)green::xi_s1((double)d / N);
-    sdxi[d] = (float)green::dxi_s1((double)d / N);
-  }
+  float2* sm = reinterpret_cast<float2*>(es_smem);                 // kEsChunk masses (hi, lo)
+  float2* sx = reinterpret_cast<float2*>(sm + kEsChunk);           // N pairs (xi, xi')(d/N)
+  for (int d = threadIdx.x; d < N; d += blockDim.x)
+    sx[d] = make_float2((float)green::xi_s1((double)d / N), (float)green::dxi_s1((double)d / N));
   const size_t n3 = (size_t)N * N * N;
   const double inv_n3 = 1.0 / (double)n3;
   const double mu = *mean;
@@ -49,11 +61,11 @@ __global__ void __launch_bounds__(kEsThreads) k_es_direct(const float* __restric
   }
   const float inv4pi = (float)(1.0 / (4.0 * green::kPi));
   const float self = (float)(-green::cube_mean_inv_r() * N / (4.0 * green::kPi));
-  double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
+  float2 a[4] = {};
   for (size_t c0 = (size_t)blockIdx.x * kEsChunk; c0 < n3; c0 += (size_t)gridDim.x * kEsChunk) {
     const int cnt = (int)((n3 - c0) < (size_t)kEsChunk ? (n3 - c0) : (size_t)kEsChunk);
     __syncthreads();
-    for (int k = threadIdx.x; k < cnt; k += blockDim.x) sm[k] = ((double)rho[c0 + k] - mu) * inv_n3;
+    for (int k = threadIdx.x; k < cnt; k += blockDim.x) sm[k] = df_from_double(((double)rho[c0 + k] - mu) * inv_n3);
     __syncthreads();
     if (!valid) continue;
     // offsets d = (t - j) mod N per axis, stepped along the chunk (x fastest)
@@ -63,25 +75,32 @@ __global__ void __launch_bounds__(kEsThreads) k_es_direct(const float* __restric
     dx += dx < 0 ? N : 0;
     dy += dy < 0 ? N : 0;
     dz += dz < 0 ? N : 0;
-    float hy = sxi[dy], gy = sdxi[dy], hz = sxi[dz], gz = sdxi[dz];
-    float ryz2 = hy * hy + hz * hz;
-    for (int k = 0; k < cnt; ++k) {
-      const double mj = sm[k];
-      if ((dx | dy | dz) == 0) {
-        a0 = fma(mj, (double)self, a0);   // self term; grad G(0) = 0
-      } else {
-        const float hx = sxi[dx];
-        const float r2 = fmaf(hx, hx, ryz2);
-        const float r = sqrtf(r2);
-        const float G = -inv4pi / r;
-        const float c = G / r2;           // -1 / (4 pi |xhat|^3)
-        a0 = fma(mj, (double)G, a0);
-        a1 = fma(mj, (double)(c * hx * sdxi[dx]), a1);
-        a2 = fma(mj, (double)(c * hy * gy), a2);
-        a3 = fma(mj, (double)(c * hz * gz), a3);
+    for (int k = 0; k < cnt;) {
+      // the sources of one row
+      const int run = N - jx < cnt - k ? N - jx : cnt - k;
+      const float2 vy = sx[dy], vz = sx[dz];
+      const float ryz2 = vy.x * vy.x + vz.x * vz.x;
+      const bool on_row = (dy | dz) == 0;
+      float2 sc = make_float2(0.f, 0.f);
+      for (int q = 0; q < run; ++q) {
+        const float2 mj = sm[k + q];
+        const float2 vx = sx[dx];
+        const float r2 = fmaf(vx.x, vx.x, ryz2);
+        const bool at0 = on_row && dx == 0;             // self term; grad G(0) = 0
+        float ir = rsqrtf(at0 ? 1.f : r2);
+        ir = fmaf(0.5f * ir, fmaf(-r2 * ir, ir, 1.f), ir);
+        const float G = at0 ? self : -inv4pi * ir;
+        const float c = at0 ? 0.f : G * (ir * ir);      // -1 / (4 pi |xhat|^3)
+        es_mac(a[0], mj.x, mj.y, G);
+        es_mac(a[1], mj.x, mj.y, c * (vx.x * vx.y));
+        es_mac(sc, mj.x, mj.y, c);
+        dx = dx == 0 ? N - 1 : dx - 1;
       }
-      dx = dx == 0 ? N - 1 : dx - 1;
-      if (++jx == N) {                    // next row: x restarts, y advances
+      es_mac(a[2], sc.x, sc.y, vy.x * vy.y);
+      es_mac(a[3], sc.x, sc.y, vz.x * vz.y);
+      k += run;
+      jx += run;
+      if (jx == N) {                      // next row: x restarts, y advances
         jx = 0;
         dx = tx;
         dy = dy == 0 ? N - 1 : dy - 1;
@@ -89,21 +108,13 @@ __global__ void __launch_bounds__(kEsThreads) k_es_direct(const float* __restric
           jy = 0;
           dy = ty;
           dz = dz == 0 ? N - 1 : dz - 1;
-          hz = sxi[dz];
-          gz = sdxi[dz];
         }
-        hy = sxi[dy];
-        gy = sdxi[dy];
-        ryz2 = hy * hy + hz * hz;
       }
     }
   }
   if (valid) {
     double* o = partials + ((size_t)blockIdx.x * T + ti) * 4;
-    o[0] = a0;
-    o[1] = a1;
-    o[2] = a2;
-    o[3] = a3;
+    for (int f = 0; f < 4; ++f) o[f] = df_to_double(a[f]);
   }
 }
 
@@ -162,7 +173,7 @@ cudaError_t launch_error_stats(Plan& P, const float* rho, const float* phi, cons
   if (e != cudaSuccess) return e;
   const int gx = error_stats_grid_x(P, T);
   const dim3 grid(gx, (T + kEsThreads - 1) / kEsThreads);
-  const size_t smem = sizeof(double) * kEsChunk + 2 * sizeof(float) * (size_t)P.N;
+  const size_t smem = sizeof(float2) * (size_t)kEsChunk + sizeof(float2) * (size_t)P.N;
   k_es_direct<<<grid, kEsThreads, smem, s>>>(rho, mean, P.N, targets, T, partials);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
