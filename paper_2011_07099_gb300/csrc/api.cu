@@ -130,9 +130,10 @@ void free_plan(Plan* P) {
   }
   cudaFree(P->spec_tw);
   cudaFree(P->near_tab);
-  cudaFree(P->nz_K);
-  cudaFree(P->nz_M);
-  cudaFree(P->nz_P);
+  cudaFree(P->ns_K);
+  cudaFree(P->ns_M);
+  cudaFree(P->ns_P);
+  cudaFree(P->ns_tw);
   cudaFree(P->d_err);
   cudaFree(P->corr_w);
   cudaFree(P->corr_samples);
@@ -193,6 +194,30 @@ int make_twiddles(int points, float4** out) {
                                                                                                       : FMM_ERR_CUDA;
 }
 
+// Buffers of the near zone's spectral products (near_spec.cu) for the leaf
+// sizes it is built for; without them the direct kernels run.
+int alloc_near_spec(Plan& P, size_t limit) {
+  if (P.ns_K || !fmm::near_spec_shape(P)) return FMM_OK;
+  size_t nK, nM, nP;
+  fmm::near_spec_bytes(P, nK, nM, nP);
+  if (nK + nM + nP > limit) return FMM_OK;
+  if (!P.ns_tw) {
+    const int rc = make_twiddles(P.S, &P.ns_tw);
+    if (rc != FMM_OK) return rc;
+  }
+  if (cudaMalloc(&P.ns_M, nM) != cudaSuccess || cudaMalloc(&P.ns_P, nP) != cudaSuccess ||
+      cudaMalloc(&P.ns_K, nK) != cudaSuccess) {
+    cudaFree(P.ns_K);
+    cudaFree(P.ns_M);
+    cudaFree(P.ns_P);
+    P.ns_K = P.ns_M = P.ns_P = nullptr;
+    (void)cudaGetLastError();
+    return FMM_OK;
+  }
+  // the padding frequencies, and the all-zero spectrum of out-of-box leaves
+  return cudaMemset(P.ns_K, 0, nK) == cudaSuccess && cudaMemset(P.ns_M, 0, nM) == cudaSuccess ? FMM_OK : FMM_ERR_CUDA;
+}
+
 int alloc_spec(Plan& P) {
   if (P.p < 2) return FMM_OK;
   const int rc = make_twiddles(P.p, &P.spec_tw);
@@ -243,7 +268,7 @@ int retabulate(Plan& P) {
       if (rc != FMM_OK) return rc;
     }
   }
-  if (P.near_fft && fmm::launch_near_fft_kernels(P, 0) != cudaSuccess) return FMM_ERR_CUDA;
+  if (P.ns_K && fmm::launch_near_spec_kernels(P, 0) != cudaSuccess) return FMM_ERR_CUDA;
   for (int l = 2; l <= P.L; ++l)
     if (P.spec_K[l] && fmm::launch_spec_kernels(P, l, 0) != cudaSuccess) return FMM_ERR_CUDA;
   if (P.tc_ready) {
@@ -414,6 +439,7 @@ fmm_plan* fmm_plan_create(int N, int L, int order) {
     for (int l = 2; l <= L && fok; ++l)
       if (fmm::wide_level(*P, l)) fok = dev_alloc(&P->F64[l], ((size_t)1 << (3 * l)) * 4 * p3);
     int rc = fok ? alloc_spec(*P) : FMM_ERR_ALLOC;
+    if (rc == FMM_OK) rc = alloc_near_spec(*P, kSpecMaxBytes);
     if (rc != FMM_OK || alloc_m2l_part(*P) != FMM_OK) {
       free_plan(P);
       set_err(rc != FMM_OK ? rc : FMM_ERR_ALLOC);
@@ -563,29 +589,16 @@ int fmm_plan_set_near_algorithm(fmm_plan* plan, int algorithm) {
   Plan& P = *reinterpret_cast<Plan*>(plan);
   if (algorithm == FMM_NEAR_DIRECT) {
     if (cudaDeviceSynchronize() != cudaSuccess) return set_err(FMM_ERR_CUDA);
-    cudaFree(P.nz_K);
-    cudaFree(P.nz_M);
-    cudaFree(P.nz_P);
-    P.nz_K = P.nz_M = P.nz_P = nullptr;
     P.near_fft = 0;
     return set_err(FMM_OK);
   }
-  if (!fmm::near_fft_supported(P)) return set_err(FMM_ERR_UNSUPPORTED);
-  if (!P.nz_K) {
-    size_t nK, nM, nP;
-    fmm::near_fft_counts(P, nK, nM, nP);
-    if (!dev_alloc(&P.nz_K, nK) || !dev_alloc(&P.nz_M, nM) || !dev_alloc(&P.nz_P, nP)) {
-      cudaFree(P.nz_K);
-      cudaFree(P.nz_M);
-      cudaFree(P.nz_P);
-      P.nz_K = P.nz_M = P.nz_P = nullptr;
-      return set_err(FMM_ERR_ALLOC);
-    }
-    // the all-zero spectrum of out-of-box neighbours sits after each chunk's leaves
-    FMM_CUDA_TRY(cudaMemset(P.nz_M, 0, sizeof(float2) * nM));
+  if (P.S != 8) return set_err(FMM_ERR_UNSUPPORTED);
+  if (!P.ns_K) {   // over the default limit at plan creation: the caller asks for it
+    const int rc = alloc_near_spec(P, ~(size_t)0);
+    if (rc != FMM_OK || !P.ns_K) return set_err(rc != FMM_OK ? rc : FMM_ERR_ALLOC);
+    FMM_CUDA_TRY(fmm::launch_near_spec_kernels(P, 0));
   }
   P.near_fft = 1;
-  FMM_CUDA_TRY(fmm::launch_near_fft_kernels(P, 0));
   return set_err(cudaDeviceSynchronize() == cudaSuccess ? FMM_OK : FMM_ERR_CUDA);
 }
 
@@ -831,11 +844,11 @@ int fmm_solve(fmm_plan* plan, const float* density, float* potential, float* acc
   // pass, so the double-float levels run on the first auxiliary stream beside
   // the FP32 and tensor-core levels on `s`.  Timed solves stay serial, so that
   // each stage's events bracket it alone.
-  const bool fwd_apart = !t && P.near_fft;
+  const bool fwd_apart = !t && P.ns_K;
   if (fwd_apart) {
     FMM_CUDA_TRY(cudaEventRecord(P.fev[0], s));
     FMM_CUDA_TRY(cudaStreamWaitEvent(P.aux[1], P.fev[0], 0));
-    FMM_CUDA_TRY(fmm::launch_near_fft_fwd(P, density, P.aux[1]));
+    FMM_CUDA_TRY(fmm::launch_near_spec_fwd(P, density, P.aux[1]));
     FMM_CUDA_TRY(cudaEventRecord(P.fev[1], P.aux[1]));
   }
   FMM_CUDA_TRY(mark(FMM_TIME_P2M, 0));

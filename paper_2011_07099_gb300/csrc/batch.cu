@@ -274,7 +274,7 @@ int fmm_batch_set_near_algorithm(fmm_batch* b, int algorithm) {
   if (!b || (algorithm != FMM_NEAR_DIRECT && algorithm != FMM_NEAR_FFT)) return fmm::set_last_error(FMM_ERR_ARG);
   for (auto pl : b->plans) {
     // the FFT near zone needs 8-cell leaves: other fields keep the direct sum
-    if (algorithm == FMM_NEAR_FFT && !fmm::near_fft_supported(*reinterpret_cast<const fmm::Plan*>(pl))) continue;
+    if (algorithm == FMM_NEAR_FFT && reinterpret_cast<const fmm::Plan*>(pl)->S != 8) continue;
     const int rc = fmm_plan_set_near_algorithm(pl, algorithm);
     if (rc != FMM_OK) return rc;
   }

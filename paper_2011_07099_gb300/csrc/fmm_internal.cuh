@@ -113,12 +113,14 @@ struct Plan {
   void* fft = nullptr;                     // its cuFFT plans and buffers (m2l_fft.cu)
   int tc_min_level = kTcMinLevel;          // first level on the tensor cores in the mixed forms
   int tc_min_set = 0;                      // tc_min_level set by the caller (honoured at high order too)
-  // near zone by FFT (p2p_fft.cu; 8-cell leaves): kernel spectra [72][27][4][32],
-  // source spectra [72][leaves + 1][32] (last: all zero), target spectra [leaves][4][2304]
+  // near zone by spectral products (near_spec.cu), where its buffers exist:
+  // kernel, source and target spectra and the DFT twiddles; near_fft: the
+  // caller's FMM_NEAR_FFT (FP32 transforms)
   int near_fft = 0;
-  float2* nz_K = nullptr;
-  float2* nz_M = nullptr;
-  float2* nz_P = nullptr;
+  void* ns_K = nullptr;
+  void* ns_M = nullptr;
+  void* ns_P = nullptr;
+  float4* ns_tw = nullptr;
   // learned table correction (MLP weights) and its training buffers
   float* corr_w = nullptr;                 // mlp::kParams weights (device) or unset
   int has_corr = 0;
@@ -245,18 +247,19 @@ cudaError_t launch_spec_kernels(Plan& P, int level, cudaStream_t s);
 cudaError_t launch_spec_fwd(Plan& P, const float* src, void* dst, size_t blocks, cudaStream_t s);
 cudaError_t launch_m2l_spec(Plan& P, bool df, int l0, int l1, cudaStream_t s);
 cudaError_t launch_l2l(Plan& P, int level, cudaStream_t s);       // F[level] -> F[level+1] (adds)
-// near_fwd_done: the FFT near zone's source spectra were already taken (launch_near_fft_fwd).
+// near_fwd_done: the near zone's source spectra were already taken (launch_near_spec_fwd).
 cudaError_t launch_p2p(Plan& P, const float* rho, float* phi, float* acc, cudaStream_t s,
                        bool near_fwd_done = false);
-// The near zone by FFT (p2p_fft.cu): whether the plan's shape allows it, the
-// float2 counts of its kernel, source and target spectra, function attributes, the plan-time kernel spectra (after every
-// re-tabulation) and the leaf stage itself (launch_p2p dispatches to it).
-bool near_fft_supported(const Plan& P);
-void near_fft_counts(const Plan& P, size_t& nK, size_t& nM, size_t& nP);
-cudaError_t setup_near_fft(const Plan& P);
-cudaError_t launch_near_fft_kernels(Plan& P, cudaStream_t s);
-cudaError_t launch_near_fft_fwd(Plan& P, const float* rho, cudaStream_t s);
-cudaError_t launch_near_fft(Plan& P, const float* rho, float* phi, float* acc, cudaStream_t s, bool fwd_done);
+// Near zone by spectral products (near_spec.cu): the leaf sizes it is built
+// for, its buffers (bytes), function attributes, the plan-time kernel spectra
+// (after every re-tabulation), the source spectra, and the sums with the
+// inverse transforms and L2P.
+bool near_spec_shape(const Plan& P);
+void near_spec_bytes(const Plan& P, size_t& nK, size_t& nM, size_t& nP);
+cudaError_t setup_near_spec(const Plan& P);
+cudaError_t launch_near_spec_kernels(Plan& P, cudaStream_t s);
+cudaError_t launch_near_spec_fwd(Plan& P, const float* rho, cudaStream_t s);
+cudaError_t launch_near_spec(Plan& P, float* phi, float* acc, cudaStream_t s);
 cudaError_t setup_m2l_tc(const Plan& P);
 cudaError_t setup_learn();
 // Distinct inputs of the learned correction and the spectral table gradient (learn_spec.cu).

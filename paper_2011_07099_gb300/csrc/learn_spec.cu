@@ -27,9 +27,10 @@ namespace fmm {
 namespace {
 
 using spec::chunks_of;
-using spec::dft_at;
+using spec::inverse_line;
 using spec::Num;
 using spec::Shape;
+using spec::Twiddle;
 
 constexpr int kOff3 = 343;
 constexpr int kLn = 16;                 // frequencies per chunk (FP32)
@@ -134,35 +135,30 @@ __global__ void __launch_bounds__(128) k_tg_inv(const float2* __restrict__ G, in
   if (tid < NM) tw[tid] = __ldg(twg + tid);
   __syncthreads();
   const float2* src = G + (size_t)blockIdx.x * nkp;
+  const Twiddle<false, P> wt(twg, nullptr);
   for (int q = tid; q < NM * P; q += blockDim.x) {
-    float xr[NM], xi[NM], re, im;
+    float xr[NM], xi[NM];
 #pragma unroll
     for (int s = 0; s < NM; ++s) {
       const float2 c = __ldg(src + s * NM * P + q);
       xr[s] = c.x;
       xi[s] = c.y;
     }
-#pragma unroll 1
-    for (int z = 0; z < NM; ++z) {
-      dft_at<false, NM, NM, false, true>(xr, xi, z, tw, re, im);
-      t1[z * NM * P + q] = make_float2(re, im);
-    }
+    inverse_line<false, P, true>(xr, xi, wt,
+                                 [&](int z, float re, float im) { t1[z * NM * P + q] = make_float2(re, im); });
   }
   __syncthreads();
   for (int q = tid; q < NM * P; q += blockDim.x) {            // line (z, kx)
     const int kx = q % P, z = q / P;
-    float xr[NM], xi[NM], re, im;
+    float xr[NM], xi[NM];
 #pragma unroll
     for (int s = 0; s < NM; ++s) {
       const float2 c = t1[(z * NM + s) * P + kx];
       xr[s] = c.x;
       xi[s] = c.y;
     }
-#pragma unroll 1
-    for (int y = 0; y < NM; ++y) {
-      dft_at<false, NM, NM, false, true>(xr, xi, y, tw, re, im);
-      t2[(z * NM + y) * P + kx] = make_float2(re, im);
-    }
+    inverse_line<false, P, true>(xr, xi, wt,
+                                 [&](int y, float re, float im) { t2[(z * NM + y) * P + kx] = make_float2(re, im); });
   }
   __syncthreads();
   const float scale = 1.f / (float)(NM * NM * NM);

@@ -37,11 +37,14 @@ namespace fmm {
 namespace {
 
 using spec::chunks_of;
-using spec::dft_at;
+using spec::forward_line;
+using spec::inverse_line;
+using spec::inverse_real_line;
 using spec::lanes;
 using spec::narrow;
 using spec::Num;
 using spec::Shape;
+using spec::Twiddle;
 using spec::widen;
 
 constexpr int kTile = 4;                  // target nodes per tile side
@@ -169,7 +172,8 @@ __global__ void __launch_bounds__(128) k_spec_fwd(const __grid_constant__ SpecAr
   const int tid = threadIdx.x, nthr = blockDim.x;
   const SpecLevel& V = level_of(A, blockIdx.x);
   const size_t node0 = (size_t)(blockIdx.x - V.first) * NB, nodes = V.nodes;
-  if (tid < NM) tw[tid] = __ldg(A.tw + tid);
+  if (DFA && tid < NM) tw[tid] = __ldg(A.tw + tid);
+  const Twiddle<DFA, P> wt(A.tw, tw);
   for (int i = tid; i < NB * P3; i += nthr) {
     if constexpr (DFS)
       in[i] = V.M64 ? df_from_double(__ldg(V.M64 + node0 * P3 + i)) : make_float2(__ldg(V.M + node0 * P3 + i), 0.f);
@@ -178,49 +182,39 @@ __global__ void __launch_bounds__(128) k_spec_fwd(const __grid_constant__ SpecAr
   }
   __syncthreads();
   for (int l = tid; l < NB * P * P; l += nthr) {           // x: P reals -> P frequencies
-    real x[P], re, im;
+    real x[P];
 #pragma unroll
     for (int s = 0; s < P; ++s) x[s] = in[l * P + s];
-#pragma unroll(DFA ? 1 : P)
-    for (int k = 0; k < P; ++k) {
-      dft_at<DFA, NM, P, true, false>(x, x, k, tw, re, im);
-      t1[l * P + k] = T::pack(re, im);
-    }
+    forward_line<DFA, P, true>(x, x, wt, [&](int k, real re, real im) { t1[l * P + k] = T::pack(re, im); });
   }
   __syncthreads();
   for (int l = tid; l < NB * P * P; l += nthr) {           // y: line (node, z, kx)
     const int kx = l % P, nz = l / P;
-    real xr[P], xi[P], re, im;
+    real xr[P], xi[P];
 #pragma unroll
     for (int s = 0; s < P; ++s) {
       const cplx c = t1[(nz * P + s) * P + kx];
       xr[s] = T::re(c);
       xi[s] = T::im(c);
     }
-#pragma unroll(DFA ? 1 : NM)
-    for (int k = 0; k < NM; ++k) {
-      dft_at<DFA, NM, P, false, false>(xr, xi, k, tw, re, im);
-      t2[(nz * NM + k) * P + kx] = T::pack(re, im);
-    }
+    forward_line<DFA, P, false>(xr, xi, wt, [&](int k, real re, real im) { t2[(nz * NM + k) * P + kx] = T::pack(re, im); });
   }
   __syncthreads();
   typename store::cplx* Mh = reinterpret_cast<typename store::cplx*>(V.Mh);
   for (int l = tid; l < NB * NM * P; l += nthr) {          // z: line (node, ky, kx)
     const int q = l % (NM * P), nb = l / (NM * P);
-    real xr[P], xi[P], re, im;
+    real xr[P], xi[P];
 #pragma unroll
     for (int s = 0; s < P; ++s) {
       const cplx c = t2[(nb * P + s) * NM * P + q];
       xr[s] = T::re(c);
       xi[s] = T::im(c);
     }
-#pragma unroll(DFA ? 1 : NM)
-    for (int kz = 0; kz < NM; ++kz) {
-      dft_at<DFA, NM, P, false, false>(xr, xi, kz, tw, re, im);
+    forward_line<DFA, P, false>(xr, xi, wt, [&](int kz, real re, real im) {
       const int k = kz * NM * P + q;
       Mh[((size_t)(k / LANES) * (nodes + 1) + node0 + nb) * LANES + k % LANES] =
           store::pack(narrow<DFS, DFA>(re), narrow<DFS, DFA>(im));
-    }
+    });
   }
 }
 
@@ -239,39 +233,32 @@ __global__ void __launch_bounds__(256) k_spec_inv(const __grid_constant__ SpecAr
   const int tid = threadIdx.x, nthr = blockDim.x;
   const SpecLevel& V = level_of(A, blockIdx.x);
   const size_t node0 = (size_t)(blockIdx.x - V.first) * NB;
-  if (tid < NM) tw[tid] = __ldg(A.tw + tid);
+  if (DFA && tid < NM) tw[tid] = __ldg(A.tw + tid);
+  const Twiddle<DFA, P> wt(A.tw, tw);
   __syncthreads();
   const typename store::cplx* Ph = reinterpret_cast<const typename store::cplx*>(V.Ph) + node0 * 4 * A.nkp;
   for (int l = tid; l < NB * 4 * NM * P; l += nthr) {      // z: line (node, f, ky, kx), NM -> P
     const int q = l % (NM * P), nf = l / (NM * P);
-    real xr[NM], xi[NM], re, im;
+    real xr[NM], xi[NM];
 #pragma unroll
     for (int s = 0; s < NM; ++s) {
       const typename store::cplx c = __ldg(Ph + (size_t)nf * A.nkp + s * NM * P + q);
       xr[s] = widen<DFA>(store::re(c));
       xi[s] = widen<DFA>(store::im(c));
     }
-#pragma unroll(DFA ? 1 : P)
-    for (int z = 0; z < P; ++z) {
-      dft_at<DFA, NM, NM, false, true>(xr, xi, z, tw, re, im);
-      t1[(nf * P + z) * NM * P + q] = T::pack(re, im);
-    }
+    inverse_line<DFA, P>(xr, xi, wt, [&](int z, real re, real im) { t1[(nf * P + z) * NM * P + q] = T::pack(re, im); });
   }
   __syncthreads();
   for (int l = tid; l < NB * 4 * P * P; l += nthr) {       // y: line (node, f, z, kx), NM -> P
     const int kx = l % P, nfz = l / P;
-    real xr[NM], xi[NM], re, im;
+    real xr[NM], xi[NM];
 #pragma unroll
     for (int s = 0; s < NM; ++s) {
       const cplx c = t1[(nfz * NM + s) * P + kx];
       xr[s] = T::re(c);
       xi[s] = T::im(c);
     }
-#pragma unroll(DFA ? 1 : P)
-    for (int y = 0; y < P; ++y) {
-      dft_at<DFA, NM, NM, false, true>(xr, xi, y, tw, re, im);
-      t2[(nfz * P + y) * P + kx] = T::pack(re, im);
-    }
+    inverse_line<DFA, P>(xr, xi, wt, [&](int y, real re, real im) { t2[(nfz * P + y) * P + kx] = T::pack(re, im); });
   }
   __syncthreads();
   for (int l = tid; l < NB * 4 * P * P; l += nthr) {       // x: line (node, f, z, y), half spectrum -> P reals
@@ -282,19 +269,7 @@ __global__ void __launch_bounds__(256) k_spec_inv(const __grid_constant__ SpecAr
       xr[s] = T::re(c);
       xi[s] = T::im(c);
     }
-#pragma unroll(DFA ? 1 : P)
-    for (int x = 0; x < P; ++x) {
-      real a = T::zero();
-      int j = x;
-#pragma unroll
-      for (int s = 1; s < P; ++s) {                        // Re(v e^{i a}) = v.re cos a - v.im sin a
-        const float4 w = tw[j];
-        T::mac(a, w.x, w.y, xr[s]);
-        T::mac(a, -w.z, -w.w, xi[s]);
-        j += x;
-        j -= j >= NM ? NM : 0;
-      }
-      const real v = T::add(T::twice(T::done(a)), xr[0]);
+    inverse_real_line<DFA, P>(xr, xi, wt, [&](int x, real v) {
       const size_t g = node0 * 4 * P3 + (size_t)l * P + x;
       if constexpr (DFS) {
         const double d = df_to_double(v);
@@ -303,7 +278,7 @@ __global__ void __launch_bounds__(256) k_spec_inv(const __grid_constant__ SpecAr
       } else {
         V.F[g] = narrow<DFS, DFA>(v);
       }
-    }
+    });
   }
 }
 

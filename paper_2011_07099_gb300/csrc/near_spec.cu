@@ -1,0 +1,584 @@
+// Leaf stage by spectral products: the near-zone sum over the 27 neighbour
+// leaves as zero-padded convolutions, and the leaf's L2P far field.
+//
+// Sec. 3 computes the near zone of a regular grid with an FFT under
+// non-periodic boundary conditions, obtained by doubling the grid.  Here that
+// is done per pair of leaves: for a target leaf T of S cells per side and a
+// neighbour T + o, o in {-1, 0, 1}^3, the field at cell r is the linear
+// convolution
+//   Phi_T(r) += sum_{r'} K(r - r' - S o) m_{T+o}(r'),   r, r' in [0, S)^3,
+// with lags in [-(S-1), S-1]^3: circular without wrap on NM = 2S - 1 points
+// per axis (spec.cuh), so on the spectra Phi^_T(k) = sum_o K^_o(k) m^_{T+o}(k).
+// K = (G, -grad G) at the cell offsets is the plan's near table, the FP32
+// values the direct kernels use.  Per leaf and offset that is NK = NM^2 S
+// complex multiply-adds and field instead of S^6 real ones: 27 x 4 x 1800
+// against 27 x 4 x 262 144 at S = 8.
+//
+// Kernels
+//   k_ns_planes, k_ns_lines  plan time: the 27 x 4 kernel spectra in FP64, rounded once
+//   k_ns_fwd     per leaf: the spectrum of its masses
+//   k_ns_mac     per (tile of 4^3 target leaves, chunk of frequencies): the
+//                27-term sums of the 4 fields
+//   k_ns_inv     per (leaf, field): inverse transform, only the S^3 cells, plus
+//                the L2P far field (eq. fmm3 at the leaves), written once
+// Arithmetic: FP32 spectra and sums; the transforms in FP32 (FMM_NEAR_FFT) or,
+// where the plan asks for the direct sum's accuracy (FMM_NEAR_DIRECT), in
+// double-float with one rounding on store; with 16-cell leaves, whose edge
+// cells amplify every rounding (fmm_internal.cuh, kWideLeaf), double-float
+// throughout.
+// Measured (direct kernels of p2p.cu before -> here): 128^3 isolated with
+// 16-cell leaves 177 -> 3.0 ms; 256^3, S = 8 30.6 -> 6.7 ms at direct accuracy;
+// 96^3, S = 6 1.04 -> 0.33 ms; 128^3, S = 4 0.87 -> 0.51 ms.  The error of the
+// plain 256^3 solve against FP64 went from 3.5e-7 to 2.9e-7 with it.
+#include "fmm_internal.cuh"
+#include "spec.cuh"
+#include "tc_ptx.cuh"
+
+namespace fmm {
+namespace {
+
+using spec::chunks_of;
+using spec::forward_line;
+using spec::inverse_line;
+using spec::inverse_real_line;
+using spec::narrow;
+using spec::Num;
+using spec::Shape;
+using spec::Twiddle;
+using spec::widen;
+
+constexpr int kNO = 27;
+constexpr int kTile = 4;                    // target leaves per tile side
+constexpr int kHaloN = kTile + 2;
+constexpr int kSlots = kHaloN * kHaloN * kHaloN;
+
+template <int S>
+struct NearShape {
+  static constexpr bool DFS = S >= kWideLeaf;                 // storage of the spectra
+  static constexpr int THR_FWD = S >= 16 ? 512 : 128;
+  static constexpr int THR_INV = S >= 16 ? 512 : 256;
+  static constexpr int IB = S >= 16 ? 1 : (S <= 4 ? 8 : 4);    // (leaf, field) items per inverse CTA
+};
+
+// ------------------------------------------------------------- plan time
+// The kernel's value for field f at lag d (cells), from the folded near table
+// (|d_i| in [0, 2S-1]); the gradient fields take the sign of their own
+// component as the direct sum does, and vanish where that component is 0.
+__device__ __forceinline__ double near_value(const float4* __restrict__ tab, int S, int f, int dx, int dy, int dz) {
+  const int TD = 2 * S;
+  const int ax = dx < 0 ? -dx : dx, ay = dy < 0 ? -dy : dy, az = dz < 0 ? -dz : dz;
+  const float4 t = __ldg(tab + (az * TD + ay) * TD + ax);
+  switch (f) {
+    case 0: return (double)t.x;
+    case 1: return dx > 0 ? (double)t.y : (dx < 0 ? -(double)t.y : 0.0);
+    case 2: return dy > 0 ? (double)t.z : (dy < 0 ? -(double)t.z : 0.0);
+    default: return dz > 0 ? (double)t.w : (dz < 0 ? -(double)t.w : 0.0);
+  }
+}
+
+// CTA (z lag, offset x field): the x and y transforms of one lag plane.
+template <int S>
+__global__ void __launch_bounds__(128) k_ns_planes(const float4* __restrict__ tab, double2* __restrict__ out) {
+  constexpr int NM = Shape<S>::NM;
+  __shared__ double2 w[NM];
+  __shared__ double2 T1[NM * S];
+  const int vz = blockIdx.x, of = blockIdx.y, o = of / 4, f = of % 4, tid = threadIdx.x;
+  const int ox = o % 3 - 1, oy = (o / 3) % 3 - 1, oz = o / 9 - 1;
+  if (tid < NM) {
+    double s, c;
+    sincospi(2.0 * tid / NM, &s, &c);
+    w[tid] = make_double2(c, -s);
+  }
+  __syncthreads();
+  auto lag = [](int v) { return v < S ? v : v - NM; };
+  for (int i = tid; i < NM * S; i += blockDim.x) {
+    const int kx = i % S, vy = i / S;
+    double re = 0.0, im = 0.0;
+    for (int vx = 0; vx < NM; ++vx) {
+      const double a = near_value(tab, S, f, lag(vx) - S * ox, lag(vy) - S * oy, lag(vz) - S * oz);
+      const double2 t = w[(kx * vx) % NM];
+      re += a * t.x;
+      im += a * t.y;
+    }
+    T1[i] = make_double2(re, im);
+  }
+  __syncthreads();
+  for (int i = tid; i < NM * S; i += blockDim.x) {
+    const int kx = i % S, ky = i / S;
+    double re = 0.0, im = 0.0;
+    for (int vy = 0; vy < NM; ++vy) {
+      const double2 a = T1[vy * S + kx], t = w[(ky * vy) % NM];
+      re += a.x * t.x - a.y * t.y;
+      im += a.x * t.y + a.y * t.x;
+    }
+    out[((size_t)of * NM + vz) * NM * S + i] = make_double2(re, im);
+  }
+}
+
+// The z transform, 1/NM^3, and the store K^[chunk][o][...] (layouts of
+// m2l_spec.cu: FP32 [2 field pairs][16] float4, double-float [4][8] float4).
+template <int S, bool DF>
+__global__ void __launch_bounds__(128) k_ns_lines(const double2* __restrict__ in, float* __restrict__ K) {
+  constexpr int NM = Shape<S>::NM, LANES = Num<DF>::LANES;
+  __shared__ double2 w[NM];
+  const int o = blockIdx.y / 4, f = blockIdx.y % 4;
+  if (threadIdx.x < NM) {
+    double s, c;
+    sincospi(2.0 * threadIdx.x / NM, &s, &c);
+    w[threadIdx.x] = make_double2(c, -s);
+  }
+  __syncthreads();
+  const int k = blockIdx.x * blockDim.x + threadIdx.x;
+  if (k >= NM * NM * S) return;
+  const int q = k % (NM * S), kz = k / (NM * S);
+  double re = 0.0, im = 0.0;
+  for (int vz = 0; vz < NM; ++vz) {
+    const double2 a = in[((size_t)blockIdx.y * NM + vz) * NM * S + q], t = w[(kz * vz) % NM];
+    re += a.x * t.x - a.y * t.y;
+    im += a.x * t.y + a.y * t.x;
+  }
+  const double scale = 1.0 / ((double)NM * NM * NM);
+  re *= scale;
+  im *= scale;
+  const size_t base = ((size_t)(k / LANES) * kNO + o) * 128;   // floats
+  const int l = k % LANES;
+  if (DF) {
+    const float2 a = df_from_double(re), b = df_from_double(im);
+    reinterpret_cast<float4*>(K + base)[f * LANES + l] = make_float4(a.x, a.y, b.x, b.y);
+  } else {
+    reinterpret_cast<float2*>(K + base)[((f / 2) * LANES + l) * 2 + (f & 1)] = make_float2((float)re, (float)im);
+  }
+}
+
+// ------------------------------------------------------------- transforms
+// Spectra of the leaves' masses m = (rho - mean) / N^3, NB leaves per CTA.
+template <int S, bool DFA>
+__global__ void __launch_bounds__(NearShape<S>::THR_FWD) k_ns_fwd(const float* __restrict__ rho,
+                                                                  const double* __restrict__ mean, int N, int L,
+                                                                  const float4* __restrict__ twg,
+                                                                  void* __restrict__ Mout) {
+  constexpr bool DFS = NearShape<S>::DFS;
+  using T = Num<DFA>;
+  using store = Num<DFS>;
+  using real = typename T::real;
+  using cplx = typename T::cplx;
+  constexpr int NM = Shape<S>::NM, NB = Shape<S>::NB, S3 = S * S * S, LANES = store::LANES;
+  extern __shared__ float4 sm4[];
+  __shared__ float4 tw[NM];
+  cplx* t1 = reinterpret_cast<cplx*>(sm4);                 // [NB][z][y][kx]
+  cplx* t2 = t1 + NB * S3;                                 // [NB][z][ky][kx]
+  real* in = reinterpret_cast<real*>(t2);                  // [NB][z][y][x], consumed before t2 is written
+  const int tid = threadIdx.x, nthr = blockDim.x;
+  const size_t leaf0 = (size_t)blockIdx.x * NB, leaves = (size_t)1 << (3 * L);
+  if (DFA && tid < NM) tw[tid] = __ldg(twg + tid);
+  const Twiddle<DFA, S> wt(twg, tw);
+  const double mu = *mean;
+  const float mu_hi = (float)mu, mu_lo = (float)(mu - (double)mu_hi);
+  const double ivd = 1.0 / ((double)N * N * N);
+  const float iv = (float)ivd, iv_lo = (float)(ivd - (double)iv);
+  for (int i = tid; i < NB * S3; i += nthr) {
+    const int x = i % S, y = (i / S) % S, z = (i / (S * S)) % S;
+    uint32_t lx, ly, lz;
+    unmorton((uint32_t)(leaf0 + i / S3), lx, ly, lz);
+    const float r = __ldg(rho + ((size_t)(lz * S + z) * N + (ly * S + y)) * N + lx * S + x);
+    if constexpr (DFA) {                                   // exactly, as P2M forms them
+      const float2 d = df_two_sum(r, -mu_hi);
+      const float dlo = __fsub_rn(d.y, mu_lo);
+      const float ph = __fmul_rn(d.x, iv);
+      const float lo = fmaf(d.x, iv_lo, fmaf(dlo, iv, fmaf(d.x, iv, -ph)));
+      in[i] = T::done(make_float2(ph, lo));
+    } else {
+      in[i] = ((r - mu_hi) - mu_lo) * iv;
+    }
+  }
+  __syncthreads();
+  for (int l = tid; l < NB * S * S; l += nthr) {           // x: S reals -> S frequencies
+    real x[S];
+#pragma unroll
+    for (int s = 0; s < S; ++s) x[s] = in[l * S + s];
+    forward_line<DFA, S, true>(x, x, wt, [&](int k, real re, real im) { t1[l * S + k] = T::pack(re, im); });
+  }
+  __syncthreads();
+  for (int l = tid; l < NB * S * S; l += nthr) {           // y: line (leaf, z, kx)
+    const int kx = l % S, nz = l / S;
+    real xr[S], xi[S];
+#pragma unroll
+    for (int s = 0; s < S; ++s) {
+      const cplx c = t1[(nz * S + s) * S + kx];
+      xr[s] = T::re(c);
+      xi[s] = T::im(c);
+    }
+    forward_line<DFA, S, false>(xr, xi, wt, [&](int k, real re, real im) { t2[(nz * NM + k) * S + kx] = T::pack(re, im); });
+  }
+  __syncthreads();
+  typename store::cplx* Mh = reinterpret_cast<typename store::cplx*>(Mout);
+  for (int l = tid; l < NB * NM * S; l += nthr) {          // z: line (leaf, ky, kx)
+    const int q = l % (NM * S), nb = l / (NM * S);
+    real xr[S], xi[S];
+#pragma unroll
+    for (int s = 0; s < S; ++s) {
+      const cplx c = t2[(nb * S + s) * NM * S + q];
+      xr[s] = T::re(c);
+      xi[s] = T::im(c);
+    }
+    forward_line<DFA, S, false>(xr, xi, wt, [&](int kz, real re, real im) {
+      const int k = kz * NM * S + q;
+      Mh[((size_t)(k / LANES) * (leaves + 1) + leaf0 + nb) * LANES + k % LANES] =
+          store::pack(narrow<DFS, DFA>(re), narrow<DFS, DFA>(im));
+    });
+  }
+}
+
+// One separable L2P pass over `items` arrays: out[a][c][b] = sum_k W[k][c] in[a][k][b],
+// b < B, a < A; weights (hi, lo).
+template <bool DFA, int S>
+__device__ __forceinline__ void l2p_pass(const typename Num<DFA>::real* in, typename Num<DFA>::real* out, int total,
+                                         int B, int p, const float2* W, int tid, int nthr) {
+  using T = Num<DFA>;
+  for (int i = tid; i < total; i += nthr) {
+    const int b = i % B, c = (i / B) % S, a = i / (B * S);
+    const typename T::real* src = in + (size_t)a * p * B + b;
+    if constexpr (DFA) {
+      float2 acc = T::zero();
+      for (int k = 0; k < p; ++k) T::mac(acc, W[k * S + c].x, W[k * S + c].y, src[k * B]);
+      out[i] = T::done(acc);
+    } else {
+      float acc = 0.f, lo = 0.f;
+      for (int k = 0; k < p; ++k) {
+        acc = fmaf(W[k * S + c].x, src[k * B], acc);
+        lo = fmaf(W[k * S + c].y, src[k * B], lo);
+      }
+      out[i] = acc + lo;
+    }
+  }
+  __syncthreads();
+}
+
+// Outputs.  CTA: IB (leaf, field) items.
+template <int S, bool DFA>
+__global__ void __launch_bounds__(NearShape<S>::THR_INV) k_ns_inv(const void* __restrict__ Pin, int nkp, int N, int p,
+                                                                  const float* __restrict__ F,
+                                                                  const double* __restrict__ F64,
+                                                                  const float2* __restrict__ wp2m,
+                                                                  const float4* __restrict__ twg,
+                                                                  float* __restrict__ phi, float* __restrict__ acc) {
+  constexpr bool DFS = NearShape<S>::DFS;
+  using T = Num<DFA>;
+  using store = Num<DFS>;
+  using real = typename T::real;
+  using cplx = typename T::cplx;
+  constexpr int NM = Shape<S>::NM, IB = NearShape<S>::IB, S3 = S * S * S;
+  extern __shared__ float4 sm4[];
+  __shared__ float4 tw[NM];
+  __shared__ float2 W[kMaxOrder * S];
+  real* far = reinterpret_cast<real*>(sm4);                // [IB][S^3]
+  cplx* t2 = reinterpret_cast<cplx*>(far + IB * S3);       // [IB][z][y][kx]
+  cplx* t1 = t2 + IB * S3;                                 // [IB][z][ky][kx]
+  const int tid = threadIdx.x, nthr = blockDim.x;
+  const size_t item0 = (size_t)blockIdx.x * IB;
+  const int p3 = p * p * p;
+  if (DFA && tid < NM) tw[tid] = __ldg(twg + tid);
+  const Twiddle<DFA, S> wt(twg, tw);
+  for (int i = tid; i < p * S; i += nthr) W[i] = __ldg(wp2m + i);
+  {                                                        // L2P, scratch in t1's space
+    real* a = reinterpret_cast<real*>(t1);                 // [IB][p^3]
+    real* b = a + IB * p3;                                 // [IB][p][p][S]
+    real* c = b + IB * p * p * S;                          // [IB][p][S][S]
+    for (int i = tid; i < IB * p3; i += nthr) {
+      if constexpr (DFS) a[i] = df_from_double(__ldg(F64 + item0 * p3 + i));
+      else a[i] = widen<DFA>(__ldg(F + item0 * p3 + i));
+    }
+    __syncthreads();
+    l2p_pass<DFA, S>(a, b, IB * p * p * S, 1, p, W, tid, nthr);
+    l2p_pass<DFA, S>(b, c, IB * p * S * S, S, p, W, tid, nthr);
+    l2p_pass<DFA, S>(c, far, IB * S3, S * S, p, W, tid, nthr);
+  }
+  const typename store::cplx* Ph = reinterpret_cast<const typename store::cplx*>(Pin) + item0 * nkp;
+  for (int l = tid; l < IB * NM * S; l += nthr) {          // z: line (item, ky, kx), NM -> S
+    const int q = l % (NM * S), it = l / (NM * S);
+    real xr[NM], xi[NM];
+#pragma unroll
+    for (int s = 0; s < NM; ++s) {
+      const typename store::cplx v = __ldg(Ph + (size_t)it * nkp + s * NM * S + q);
+      xr[s] = widen<DFA>(store::re(v));
+      xi[s] = widen<DFA>(store::im(v));
+    }
+    inverse_line<DFA, S>(xr, xi, wt, [&](int z, real re, real im) { t1[(it * S + z) * NM * S + q] = T::pack(re, im); });
+  }
+  __syncthreads();
+  for (int l = tid; l < IB * S * S; l += nthr) {           // y: line (item, z, kx), NM -> S
+    const int kx = l % S, iz = l / S;
+    real xr[NM], xi[NM];
+#pragma unroll
+    for (int s = 0; s < NM; ++s) {
+      const cplx v = t1[(iz * NM + s) * S + kx];
+      xr[s] = T::re(v);
+      xi[s] = T::im(v);
+    }
+    inverse_line<DFA, S>(xr, xi, wt, [&](int y, real re, real im) { t2[(iz * S + y) * S + kx] = T::pack(re, im); });
+  }
+  __syncthreads();
+  const size_t N3 = (size_t)N * N * N;
+  for (int l = tid; l < IB * S * S; l += nthr) {           // x: line (item, z, y), half spectrum -> S cells
+    real xr[S], xi[S];
+#pragma unroll
+    for (int s = 0; s < S; ++s) {
+      const cplx v = t2[l * S + s];
+      xr[s] = T::re(v);
+      xi[s] = T::im(v);
+    }
+    const size_t item = item0 + l / (S * S);
+    const int y = l % S, z = (l / S) % S, f = (int)(item & 3);
+    uint32_t lx, ly, lz;
+    unmorton((uint32_t)(item >> 2), lx, ly, lz);
+    float* dst = (f == 0 ? phi : acc + (size_t)(f - 1) * N3) +
+                 ((size_t)(lz * S + z) * N + (ly * S + y)) * N + lx * S;
+    const real* fr = far + l * S;
+    inverse_real_line<DFA, S>(xr, xi, wt, [&](int x, real v) { dst[x] = narrow<false, DFA>(T::add(v, fr[x])); });
+  }
+}
+
+// ---------------------------------------------------------- spectral sums
+// Rows of 4 target leaves along x per thread, as k_spec_mac; the chunk's 27
+// kernel spectra and the tile's 6^3 source spectra in shared memory (41 KB, so
+// that several CTAs share an SM and one's copies run under another's sums).
+template <bool DF>
+__global__ void __launch_bounds__(DF ? 512 : 256) k_ns_mac(const float4* __restrict__ K, const void* __restrict__ Mh,
+                                                          void* __restrict__ Ph, int L, int nkp, int iso) {
+  constexpr int LANES = Num<DF>::LANES, NTHR = DF ? 512 : 256;
+  extern __shared__ float4 sm4[];
+  float4* sK = sm4;                         // [27][32]
+  float4* sM = sm4 + kNO * 32;              // [216][8]
+  const int tid = threadIdx.x, n = 1 << L, nt = n / kTile;
+  const int tile = blockIdx.x, chunk = blockIdx.y;
+  const int TX = tile % nt, TY = (tile / nt) % nt, TZ = tile / (nt * nt);
+  const size_t leaves = (size_t)1 << (3 * L);
+  const float4* Kc = K + (size_t)chunk * kNO * 32;
+  for (int i = tid; i < kNO * 32; i += NTHR) tc::cp_async16_full(tc::smem_u32(sK + i), Kc + i);
+  const char* src = reinterpret_cast<const char*>(Mh) + (size_t)chunk * (leaves + 1) * 128;
+  for (int i = tid; i < kSlots * 8; i += NTHR) {
+    const int slot = i >> 3, part = i & 7;
+    const int ux = TX * kTile - 1 + slot % kHaloN, uy = TY * kTile - 1 + (slot / kHaloN) % kHaloN,
+              uz = TZ * kTile - 1 + slot / (kHaloN * kHaloN);
+    const bool inbox = (unsigned)ux < (unsigned)n && (unsigned)uy < (unsigned)n && (unsigned)uz < (unsigned)n;
+    const size_t leaf = inbox || !iso ? morton(ux & (n - 1), uy & (n - 1), uz & (n - 1)) : leaves;
+    tc::cp_async16_full(tc::smem_u32(sM + i), src + leaf * 128 + part * 16);
+  }
+  tc::cp_async_commit();
+  tc::cp_async_wait<0>();
+  __syncthreads();
+  if constexpr (!DF) {
+    const int fr = tid & 15, ty = (tid >> 4) & 3, tz = tid >> 6;
+    const float2* halo = reinterpret_cast<const float2*>(sM) + fr;
+    float2 tot[4][4];
+    auto kernel = [&](int o, float2 (&k)[4]) {
+      const float4 ka = sK[o * 32 + fr], kb = sK[o * 32 + 16 + fr];
+      k[0] = make_float2(ka.x, ka.y);
+      k[1] = make_float2(ka.z, ka.w);
+      k[2] = make_float2(kb.x, kb.y);
+      k[3] = make_float2(kb.z, kb.w);
+    };
+    auto row = [&](int oy, int oz, float2 (&m)[kHaloN]) {
+      const float2* m0 = halo + ((tz + 1 + oz) * kHaloN + ty + 1 + oy) * kHaloN * LANES;
+#pragma unroll
+      for (int h = 0; h < kHaloN; ++h) m[h] = m0[h * LANES];
+    };
+    float2 mp[kHaloN], mm[kHaloN], k[4];
+    row(0, 0, mp);
+    kernel(13, k);                                             // the leaf itself
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+      for (int f = 0; f < 4; ++f)
+        tot[j][f] = make_float2(fmaf(-k[f].y, mp[j + 1].y, k[f].x * mp[j + 1].x),
+                                fmaf(k[f].y, mp[j + 1].x, k[f].x * mp[j + 1].y));
+    // Phi's kernel is even and g's odd, so K^_{-o} = s conj(K^_o) (s = 1, -1)
+    // and with M+ = m^_{T+o}, M- = m^_{T-o}, K^_o = a + ib the pair's terms are
+    // a (M+ + s M-) + i b (M+ - s M-): 20 instructions for the 4 fields
+    // instead of 32
+    auto pairs = [&](int oy, int oz, int oxs) {                 // x offsets -1 .. oxs of rows (oy, oz), -(oy, oz)
+#pragma unroll
+      for (int ox = -1; ox <= 1; ++ox) {
+        if (ox > oxs) continue;
+        kernel((oz + 1) * 9 + (oy + 1) * 3 + ox + 1, k);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const float2 p = mp[j + 1 + ox], q = mm[j + 1 - ox];
+          const float2 su = make_float2(p.x + q.x, p.y + q.y), di = make_float2(p.x - q.x, p.y - q.y);
+          tot[j][0].x = fmaf(k[0].x, su.x, tot[j][0].x);
+          tot[j][0].y = fmaf(k[0].x, su.y, tot[j][0].y);
+          tot[j][0].x = fmaf(-k[0].y, di.y, tot[j][0].x);
+          tot[j][0].y = fmaf(k[0].y, di.x, tot[j][0].y);
+#pragma unroll
+          for (int f = 1; f < 4; ++f) {
+            tot[j][f].x = fmaf(k[f].x, di.x, tot[j][f].x);
+            tot[j][f].y = fmaf(k[f].x, di.y, tot[j][f].y);
+            tot[j][f].x = fmaf(-k[f].y, su.y, tot[j][f].x);
+            tot[j][f].y = fmaf(k[f].y, su.x, tot[j][f].y);
+          }
+        }
+      }
+    };
+#pragma unroll
+    for (int h = 0; h < kHaloN; ++h) mm[h] = mp[h];
+    pairs(0, 0, -1);
+#pragma unroll 1
+    for (int r = 0; r < 4; ++r) {                               // rows (-1, -1), (0, -1), (1, -1), (-1, 0)
+      const int oz = r < 3 ? -1 : 0, oy = r < 3 ? r - 1 : -1;
+      row(oy, oz, mp);
+      row(-oy, -oz, mm);
+      pairs(oy, oz, 1);
+    }
+    float2* out = reinterpret_cast<float2*>(Ph);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const size_t leaf = morton(TX * kTile + j, TY * kTile + ty, TZ * kTile + tz);
+#pragma unroll
+      for (int f = 0; f < 4; ++f) out[(leaf * 4 + f) * nkp + (size_t)chunk * LANES + fr] = tot[j][f];
+    }
+  } else {
+    const int fr = tid & 7, ty = (tid >> 3) & 3, f = (tid >> 5) & 3, tz = tid >> 7;
+    const float4* halo = sM + fr;
+    float2 re[4], im[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) re[j] = im[j] = make_float2(0.f, 0.f);
+#pragma unroll 1
+    for (int row = 0; row < 9; ++row) {
+      const int oy = row % 3 - 1, oz = row / 3 - 1;
+      const float4* m0 = halo + ((tz + 1 + oz) * kHaloN + ty + 1 + oy) * kHaloN * LANES;
+#pragma unroll
+      for (int ox = -1; ox <= 1; ++ox) {
+        const float4 k = sK[(row * 3 + ox + 1) * 32 + f * 8 + fr];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const float4 v = m0[(j + 1 + ox) * LANES];
+          const float2 mr = make_float2(v.x, v.y), mi = make_float2(v.z, v.w);
+          Num<true>::mac(re[j], k.x, k.y, mr);
+          Num<true>::mac(im[j], k.x, k.y, mi);
+          Num<true>::mac(re[j], -k.z, -k.w, mi);
+          Num<true>::mac(im[j], k.z, k.w, mr);
+        }
+      }
+    }
+    float4* out = reinterpret_cast<float4*>(Ph);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const size_t leaf = morton(TX * kTile + j, TY * kTile + ty, TZ * kTile + tz);
+      const float2 a = Num<true>::done(re[j]), b = Num<true>::done(im[j]);
+      out[(leaf * 4 + f) * nkp + (size_t)chunk * LANES + fr] = make_float4(a.x, a.y, b.x, b.y);
+    }
+  }
+}
+constexpr size_t kMacSmem = sizeof(float4) * (kNO * 32 + kSlots * 8);
+
+template <int S, bool DFA>
+size_t fwd_smem() {
+  constexpr int NB = Shape<S>::NB, NM = Shape<S>::NM;
+  return sizeof(typename Num<DFA>::cplx) * NB * (S * S * S + S * NM * S);
+}
+template <int S, bool DFA>
+size_t inv_smem(int p) {
+  constexpr int IB = NearShape<S>::IB, NM = Shape<S>::NM, S3 = S * S * S;
+  const size_t real = sizeof(typename Num<DFA>::real), cplx = sizeof(typename Num<DFA>::cplx);
+  const size_t t1 = cplx * IB * S * NM * S, l2p = real * IB * (p * p * p + p * p * S + p * S * S);
+  return real * IB * S3 + cplx * IB * S3 + (t1 > l2p ? t1 : l2p);
+}
+
+template <int S, bool DFA>
+cudaError_t fwd_as(Plan& P, const float* rho, cudaStream_t s) {
+  const unsigned leaves = 1u << (3 * P.L);
+  k_ns_fwd<S, DFA><<<leaves / Shape<S>::NB, NearShape<S>::THR_FWD, fwd_smem<S, DFA>(), s>>>(rho, P.d_mean, P.N, P.L,
+                                                                                            P.ns_tw, P.ns_M);
+  return cudaGetLastError();
+}
+template <int S, bool DFA>
+cudaError_t rest_as(Plan& P, float* phi, float* acc, cudaStream_t s) {
+  constexpr bool DFS = NearShape<S>::DFS;
+  const unsigned leaves = 1u << (3 * P.L);
+  const int nt = (1 << P.L) / kTile, ch = chunks_of(S, DFS), nkp = ch * Num<DFS>::LANES;
+  k_ns_mac<DFS><<<dim3(nt * nt * nt, ch), DFS ? 512 : 256, kMacSmem, s>>>(static_cast<const float4*>(P.ns_K), P.ns_M,
+                                                                         P.ns_P, P.L, nkp, P.iso);
+  k_ns_inv<S, DFA><<<leaves * 4 / NearShape<S>::IB, NearShape<S>::THR_INV, inv_smem<S, DFA>(P.p), s>>>(
+      P.ns_P, nkp, P.N, P.p, P.F[P.L], P.F64[P.L], P.w_p2m, P.ns_tw, phi, acc);
+  return cudaGetLastError();
+}
+
+template <int S>
+cudaError_t kernels_s(Plan& P, cudaStream_t s) {
+  constexpr int NM = Shape<S>::NM;
+  // the target spectra's space holds the half-transformed kernels meanwhile
+  double2* scratch = static_cast<double2*>(P.ns_P);
+  k_ns_planes<S><<<dim3(NM, kNO * 4), 128, 0, s>>>(P.near_tab, scratch);
+  k_ns_lines<S, NearShape<S>::DFS><<<dim3((NM * NM * S + 127) / 128, kNO * 4), 128, 0, s>>>(scratch,
+                                                                                          static_cast<float*>(P.ns_K));
+  return cudaGetLastError();
+}
+
+template <typename F>
+cudaError_t opt_in(F* f, size_t bytes) {
+  return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+}
+template <int S>
+cudaError_t setup_s() {
+  cudaError_t e;
+  if constexpr (!NearShape<S>::DFS) {
+    if ((e = opt_in(k_ns_fwd<S, false>, fwd_smem<S, false>())) != cudaSuccess) return e;
+    if ((e = opt_in(k_ns_inv<S, false>, inv_smem<S, false>(kMaxOrder))) != cudaSuccess) return e;
+  }
+  if ((e = opt_in(k_ns_fwd<S, true>, fwd_smem<S, true>())) != cudaSuccess) return e;
+  if ((e = opt_in(k_ns_inv<S, true>, inv_smem<S, true>(kMaxOrder))) != cudaSuccess) return e;
+  return opt_in(k_ns_mac<NearShape<S>::DFS>, kMacSmem);
+}
+
+}  // namespace
+
+bool near_spec_shape(const Plan& P) { return P.S == 4 || P.S == 6 || P.S == 8 || P.S == 16; }
+
+void near_spec_bytes(const Plan& P, size_t& nK, size_t& nM, size_t& nP) {
+  const size_t leaves = (size_t)1 << (3 * P.L), ch = chunks_of(P.S, P.S >= kWideLeaf);
+  nK = ch * kNO * 512;
+  nM = ch * (leaves + 1) * 128;
+  nP = leaves * 4 * ch * 128;
+}
+
+cudaError_t setup_near_spec(const Plan& P) {
+  switch (P.S) {
+    case 4: return setup_s<4>();
+    case 6: return setup_s<6>();
+    case 8: return setup_s<8>();
+    case 16: return setup_s<16>();
+    default: return cudaSuccess;
+  }
+}
+
+cudaError_t launch_near_spec_kernels(Plan& P, cudaStream_t s) {
+  switch (P.S) {
+    case 4: return kernels_s<4>(P, s);
+    case 6: return kernels_s<6>(P, s);
+    case 8: return kernels_s<8>(P, s);
+    case 16: return kernels_s<16>(P, s);
+    default: return cudaErrorInvalidValue;
+  }
+}
+
+cudaError_t launch_near_spec_fwd(Plan& P, const float* rho, cudaStream_t s) {
+  switch (P.S) {
+    case 4: return fwd_as<4, true>(P, rho, s);
+    case 6: return fwd_as<6, true>(P, rho, s);
+    case 8: return P.near_fft ? fwd_as<8, false>(P, rho, s) : fwd_as<8, true>(P, rho, s);
+    case 16: return fwd_as<16, true>(P, rho, s);
+    default: return cudaErrorInvalidValue;
+  }
+}
+
+cudaError_t launch_near_spec(Plan& P, float* phi, float* acc, cudaStream_t s) {
+  switch (P.S) {
+    case 4: return rest_as<4, true>(P, phi, acc, s);
+    case 6: return rest_as<6, true>(P, phi, acc, s);
+    case 8: return P.near_fft ? rest_as<8, false>(P, phi, acc, s) : rest_as<8, true>(P, phi, acc, s);
+    case 16: return rest_as<16, true>(P, phi, acc, s);
+    default: return cudaErrorInvalidValue;
+  }
+}
+
+}  // namespace fmm

@@ -479,23 +479,25 @@ cudaError_t setup_s() {
 }  // namespace
 
 cudaError_t setup_p2p(const Plan& P) {
+  const cudaError_t e = setup_near_spec(P);
+  if (e != cudaSuccess) return e;
   switch (P.S) {
     case 1: return setup_s<1>();
     case 2: return setup_s<2>();
     case 3: return setup_s<3>();
     case 4: return setup_s<4>();
     case 6: return setup_s<6>();
-    case 8: {
-      const cudaError_t e = setup_s<8>();
-      return e != cudaSuccess ? e : setup_near_fft(P);
-    }
+    case 8: return setup_s<8>();
     case 16: return cudaFuncSetAttribute(k_p2p16, cudaFuncAttributeMaxDynamicSharedMemorySize, 225 * 1024);
     default: return cudaErrorInvalidValue;
   }
 }
 
 cudaError_t launch_p2p(Plan& P, const float* rho, float* phi, float* acc, cudaStream_t s, bool near_fwd_done) {
-  if (P.near_fft) return launch_near_fft(P, rho, phi, acc, s, near_fwd_done);
+  if (P.ns_K) {
+    const cudaError_t e = near_fwd_done ? cudaSuccess : launch_near_spec_fwd(P, rho, s);
+    return e != cudaSuccess ? e : launch_near_spec(P, phi, acc, s);
+  }
   switch (P.S) {
     case 1: return launch_s<1>(P, rho, phi, acc, s);
     case 2: return launch_s<2>(P, rho, phi, acc, s);

@@ -34,6 +34,7 @@ struct Num<false> {
   static __device__ __forceinline__ void mac(real& a, float wh, float, real x) { a = fmaf(wh, x, a); }
   static __device__ __forceinline__ real done(real a) { return a; }
   static __device__ __forceinline__ real twice(real a) { return 2.f * a; }
+  static __device__ __forceinline__ real neg(real a) { return -a; }
   static __device__ __forceinline__ real add(real a, real b) { return a + b; }
   static __device__ __forceinline__ cplx pack(real re, real im) { return make_float2(re, im); }
   static __device__ __forceinline__ real re(cplx c) { return c.x; }
@@ -58,6 +59,7 @@ struct Num<true> {
     return make_float2(s, __fsub_rn(a.y, __fsub_rn(s, a.x)));
   }
   static __device__ __forceinline__ real twice(real a) { return make_float2(2.f * a.x, 2.f * a.y); }
+  static __device__ __forceinline__ real neg(real a) { return make_float2(-a.x, -a.y); }
   static __device__ __forceinline__ real add(real a, real b) {
     const float2 t = df_two_sum(a.x, b.x);
     return done(make_float2(t.x, __fadd_rn(t.y, __fadd_rn(a.y, b.y))));
@@ -67,32 +69,189 @@ struct Num<true> {
   static __device__ __forceinline__ real im(cplx c) { return make_float2(c.z, c.w); }
 };
 
-// One line's DFT value at frequency (or point) k: sum_{s < NIN} x_s e^{-+ 2 pi i k s / NM};
-// `inv` takes the conjugate twiddles.  tw in shared memory.
-template <bool DF, int NM, int NIN, bool REAL_IN, bool INV>
-__device__ __forceinline__ void dft_at(const typename Num<DF>::real* xr, const typename Num<DF>::real* xi, int k,
-                                       const float4* tw, typename Num<DF>::real& re, typename Num<DF>::real& im) {
-  using T = Num<DF>;
-  re = T::zero();
-  im = T::zero();
-  int j = 0;
-#pragma unroll
-  for (int s = 0; s < NIN; ++s) {
-    const float4 w = tw[j];
-    const float sh = INV ? w.z : -w.z, sl = INV ? w.w : -w.w;   // e^{i a} = c + i s (inverse), c - i s (forward)
-    T::mac(re, w.x, w.y, xr[s]);
-    T::mac(im, sh, sl, xr[s]);
-    if (!REAL_IN) {
-      T::mac(re, -sh, -sl, xi[s]);
-      T::mac(im, w.x, w.y, xi[s]);
-    }
-    j += k;
-    j -= j >= NM ? NM : 0;
+// Line transforms of NM = 2P - 1 points.  cos is even and sin odd about half
+// the line, so the forward transform of P nonzero inputs makes the outputs k
+// and NM - k from the same four sums, and the inverse, which keeps P outputs,
+// folds the inputs s and NM - s into their sum and difference first: half the
+// multiply-adds of the plain sums.
+// Twiddles: FP32 has cos and sin of 2 pi j / NM as constants of the unrolled
+// code (read from shared memory, one load per four multiply-adds, they held
+// the transforms at 30 % of the FP32 rate); double-float reads (cos hi, lo,
+// sin hi, lo) from shared memory.
+template <bool DF, int P>
+struct Twiddle;
+// cos x for |x| <= pi, by its Taylor series, at compile time.
+constexpr double series_cos(double x) {
+  double term = 1.0, sum = 1.0;
+  for (int k = 1; k < 40; ++k) {
+    term *= -x * x / ((2.0 * k - 1.0) * (2.0 * k));
+    sum += term;
   }
-  re = T::done(re);
-  im = T::done(im);
+  return sum;
+}
+template <int P>
+struct TwiddleTable {
+  float c[P] = {}, s[P] = {};
+  constexpr TwiddleTable() {
+    constexpr double pi = 3.14159265358979323846;
+    for (int j = 0; j < P; ++j) {
+      const double a = 2.0 * pi * j / (2 * P - 1);
+      c[j] = (float)series_cos(a);
+      s[j] = j ? (float)series_cos(a - 0.5 * pi) : 0.f;     // sin a
+    }
+  }
+};
+template <int P>
+struct Twiddle<false, P> {
+  static constexpr int NM = 2 * P - 1;
+  __device__ __forceinline__ Twiddle(const float4* __restrict__, const float4*) {}
+  // j in [0, NM)
+  __device__ __forceinline__ float4 at(int j) const {
+    constexpr TwiddleTable<P> t{};
+    return j < P ? make_float4(t.c[j], 0.f, t.s[j], 0.f) : make_float4(t.c[NM - j], 0.f, -t.s[NM - j], 0.f);
+  }
+};
+template <int P>
+struct Twiddle<true, P> {
+  const float4* tw;
+  __device__ __forceinline__ Twiddle(const float4* __restrict__, const float4* shared) : tw(shared) {}
+  __device__ __forceinline__ float4 at(int j) const { return tw[j]; }
+};
+
+// X_k = sum_{s < P} x_s e^{-2 pi i k s / NM}; emit(k, re, im) for k < NM, or for
+// real input (xi unused) k < P only.
+template <bool DF, int P, bool REAL, typename Emit>
+__device__ __forceinline__ void forward_line(const typename Num<DF>::real (&xr)[P],
+                                             const typename Num<DF>::real (&xi)[P], const Twiddle<DF, P>& tw,
+                                             Emit emit) {
+  using T = Num<DF>;
+  using real = typename T::real;
+  constexpr int NM = 2 * P - 1;
+  {
+    real re = xr[0], im = REAL ? T::zero() : xi[0];
+#pragma unroll
+    for (int s = 1; s < P; ++s) {
+      re = T::add(re, xr[s]);
+      if (!REAL) im = T::add(im, xi[s]);
+    }
+    emit(0, re, im);
+  }
+#pragma unroll(DF ? 1 : P)
+  for (int k = 1; k < P; ++k) {
+    real cr = T::zero(), ci = T::zero(), sr = T::zero(), si = T::zero();
+    T::mac(cr, 1.f, 0.f, xr[0]);
+    if (!REAL) T::mac(ci, 1.f, 0.f, xi[0]);
+    int j = 0;
+#pragma unroll
+    for (int s = 1; s < P; ++s) {
+      j += k;
+      j -= j >= NM ? NM : 0;
+      const float4 w = tw.at(j);
+      T::mac(cr, w.x, w.y, xr[s]);
+      T::mac(sr, w.z, w.w, xr[s]);
+      if (!REAL) {
+        T::mac(ci, w.x, w.y, xi[s]);
+        T::mac(si, w.z, w.w, xi[s]);
+      }
+    }
+    cr = T::done(cr);
+    sr = T::done(sr);
+    if (REAL) {
+      emit(k, cr, T::neg(sr));
+    } else {
+      ci = T::done(ci);
+      si = T::done(si);
+      emit(k, T::add(cr, si), T::add(ci, T::neg(sr)));
+      emit(NM - k, T::add(cr, T::neg(si)), T::add(ci, sr));
+    }
+  }
 }
 
+// y_z = sum_{s < NM} x_s e^{+2 pi i z s / NM}; emit(z, re, im) for z < P (ALL:
+// every z < NM).  xr, xi are used up.
+template <bool DF, int P, bool ALL = false, typename Emit>
+__device__ __forceinline__ void inverse_line(typename Num<DF>::real (&xr)[2 * P - 1],
+                                             typename Num<DF>::real (&xi)[2 * P - 1], const Twiddle<DF, P>& tw,
+                                             Emit emit) {
+  using T = Num<DF>;
+  using real = typename T::real;
+  constexpr int NM = 2 * P - 1;
+#pragma unroll
+  for (int s = 1; s < P; ++s) {                  // [s]: sum, [NM - s]: difference
+    const real ar = xr[s], ai = xi[s], br = xr[NM - s], bi = xi[NM - s];
+    xr[s] = T::add(ar, br);
+    xi[s] = T::add(ai, bi);
+    xr[NM - s] = T::add(ar, T::neg(br));
+    xi[NM - s] = T::add(ai, T::neg(bi));
+  }
+  {
+    real re = xr[0], im = xi[0];
+#pragma unroll
+    for (int s = 1; s < P; ++s) {
+      re = T::add(re, xr[s]);
+      im = T::add(im, xi[s]);
+    }
+    emit(0, re, im);
+  }
+#pragma unroll(DF ? 1 : P)
+  for (int z = 1; z < P; ++z) {
+    real cr = T::zero(), ci = T::zero(), sr = T::zero(), si = T::zero();
+    T::mac(cr, 1.f, 0.f, xr[0]);
+    T::mac(ci, 1.f, 0.f, xi[0]);
+    int j = 0;
+#pragma unroll
+    for (int s = 1; s < P; ++s) {
+      j += z;
+      j -= j >= NM ? NM : 0;
+      const float4 w = tw.at(j);
+      if (ALL) {
+        T::mac(cr, w.x, w.y, xr[s]);
+        T::mac(ci, w.x, w.y, xi[s]);
+        T::mac(si, w.z, w.w, xi[NM - s]);
+        T::mac(sr, w.z, w.w, xr[NM - s]);
+      } else {
+        T::mac(cr, w.x, w.y, xr[s]);
+        T::mac(ci, w.x, w.y, xi[s]);
+        T::mac(cr, -w.z, -w.w, xi[NM - s]);
+        T::mac(ci, w.z, w.w, xr[NM - s]);
+      }
+    }
+    cr = T::done(cr);
+    ci = T::done(ci);
+    if (ALL) {
+      sr = T::done(sr);
+      si = T::done(si);
+      emit(z, T::add(cr, T::neg(si)), T::add(ci, sr));
+      emit(NM - z, T::add(cr, si), T::add(ci, T::neg(sr)));
+    } else {
+      emit(z, cr, ci);
+    }
+  }
+}
+
+// The real points x < P of a half spectrum v[0..P-1]: Re v_0 + 2 sum Re(v_s e^{+2 pi i x s / NM}).
+template <bool DF, int P, typename Emit>
+__device__ __forceinline__ void inverse_real_line(const typename Num<DF>::real (&xr)[P],
+                                                  const typename Num<DF>::real (&xi)[P], const Twiddle<DF, P>& tw,
+                                                  Emit emit) {
+  using T = Num<DF>;
+  using real = typename T::real;
+  constexpr int NM = 2 * P - 1;
+#pragma unroll(DF ? 1 : P)
+  for (int x = 0; x < P; ++x) {
+    real a = T::zero();
+    int j = 0;
+#pragma unroll
+    for (int s = 1; s < P; ++s) {
+      j += x;
+      j -= j >= NM ? NM : 0;
+      const float4 w = tw.at(j);
+      T::mac(a, w.x, w.y, xr[s]);
+      T::mac(a, -w.z, -w.w, xi[s]);
+    }
+    emit(x, T::add(T::twice(T::done(a)), xr[0]));
+  }
+}
 
 // A stored value (FP32 or double-float) as the arithmetic's.
 template <bool DFA>

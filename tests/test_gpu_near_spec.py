@@ -1,0 +1,62 @@
+"""Near zone by spectral products (csrc/near_spec.cu) in the plain form, against
+the FP64 oracle: every leaf size it is built for, periodic (the tile's halo
+wraps onto itself at L = 2) and isolated (out-of-box leaves), orders below and
+above the leaf size.
+
+Tolerance: the plain form's 1e-6 (FP32 spectra of double-float transforms, 27
+products per sum; double-float throughout for 16-cell leaves)."""
+import numpy as np
+import pytest
+
+from oracle import fmm as ofmm
+from oracle import nonperiodic as npo
+from paper_2011_07099_gb300 import inputs
+from parity_util import assert_close, leaf_values
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def B():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2011_07099_gb300 import binding, build
+    build.build()
+    binding.lib()
+    return binding
+
+
+def _solve(B, rho, L, p, iso=False):
+    plan = B.Plan(rho.shape[0], L, p)
+    if iso:
+        B.fmm_plan_set_boundary(plan.handle, B.FMM_BOUNDARY_ISOLATED)
+    phi, acc = plan.solve(torch.from_numpy(rho).cuda())
+    torch.cuda.synchronize()
+    assert B.lib().fmm_plan_check(plan.handle) == B.FMM_OK
+    plan.close()
+    return phi.cpu().numpy(), acc.cpu().numpy()
+
+
+@pytest.mark.parametrize("S,L,p", [(4, 2, 1), (4, 2, 8), (4, 3, 3), (6, 2, 4), (6, 3, 7), (8, 2, 2), (8, 2, 8), (8, 3, 5),
+                                   (16, 2, 3), (16, 2, 8)])
+def test_near_zone_matches_oracle_at_sampled_leaves(B, S, L, p):
+    N = S << L
+    rho = inputs.plummer(N, n_clumps=6, seed=N + p, a_min=0.5, a_max=3.0)
+    phi, acc = _solve(B, rho, L, p)
+    n = 1 << L
+    leaves = np.array([[0, 0, 0], [n - 1, 0, n - 1], [1, n - 2, 2]])
+    ref = ofmm.solve_at(rho, L, p, leaves)
+    got = leaf_values(phi, acc, leaves, S)
+    assert_close(got[:, 0], ref[:, 0], 1e-6, f"phi S={S} L={L} p={p}")
+    assert_close(got[:, 1:], ref[:, 1:], 1e-6, f"g S={S} L={L} p={p}")
+
+
+@pytest.mark.parametrize("S,L,p", [(4, 2, 4), (6, 2, 3), (8, 2, 6), (4, 3, 2)])
+def test_near_zone_isolated_matches_oracle(B, S, L, p):
+    N = S << L
+    rho = inputs.plummer(N, n_clumps=4, seed=N, a_min=0.5, a_max=3.0)
+    phi, acc = _solve(B, rho, L, p, iso=True)
+    ophi, og = npo.solve_isolated(rho, L, p)
+    assert_close(phi, ophi, 1e-6, f"isolated phi S={S} L={L} p={p}")
+    assert_close(acc, og, 1e-6, f"isolated g S={S} L={L} p={p}")
