@@ -163,11 +163,12 @@ __global__ void __launch_bounds__(128) k_spec_fwd(const __grid_constant__ SpecAr
   using store = Num<DFS>;
   using real = typename T::real;
   using cplx = typename T::cplx;
-  constexpr int NM = Shape<P>::NM, NB = Shape<P>::NB, P3 = P * P * P, LANES = store::LANES;
+  constexpr int NM = Shape<P>::NM, NB = Shape<P>::NB, P3 = P * P * P, PS = Shape<P>::PS,
+                LANES = store::LANES;
   extern __shared__ float4 sm4[];
   __shared__ float4 tw[NM];
   cplx* t1 = reinterpret_cast<cplx*>(sm4);                 // [NB][z][y][kx]
-  cplx* t2 = t1 + NB * P3;                                 // [NB][z][ky][kx]
+  cplx* t2 = t1 + NB * P * P * PS;                         // [NB][z][ky][kx]
   real* in = reinterpret_cast<real*>(t2 + NB * P * NM * P);   // [NB][z][y][x]
   const int tid = threadIdx.x, nthr = blockDim.x;
   const SpecLevel& V = level_of(A, blockIdx.x);
@@ -175,17 +176,18 @@ __global__ void __launch_bounds__(128) k_spec_fwd(const __grid_constant__ SpecAr
   if (DFA && tid < NM) tw[tid] = __ldg(A.tw + tid);
   const Twiddle<DFA, P> wt(A.tw, tw);
   for (int i = tid; i < NB * P3; i += nthr) {
+    real& v = in[(i / P) * PS + i % P];
     if constexpr (DFS)
-      in[i] = V.M64 ? df_from_double(__ldg(V.M64 + node0 * P3 + i)) : make_float2(__ldg(V.M + node0 * P3 + i), 0.f);
+      v = V.M64 ? df_from_double(__ldg(V.M64 + node0 * P3 + i)) : make_float2(__ldg(V.M + node0 * P3 + i), 0.f);
     else
-      in[i] = widen<DFA>(__ldg(V.M + node0 * P3 + i));
+      v = widen<DFA>(__ldg(V.M + node0 * P3 + i));
   }
   __syncthreads();
   for (int l = tid; l < NB * P * P; l += nthr) {           // x: P reals -> P frequencies
     real x[P];
 #pragma unroll
-    for (int s = 0; s < P; ++s) x[s] = in[l * P + s];
-    forward_line<DFA, P, true>(x, x, wt, [&](int k, real re, real im) { t1[l * P + k] = T::pack(re, im); });
+    for (int s = 0; s < P; ++s) x[s] = in[l * PS + s];
+    forward_line<DFA, P, true>(x, x, wt, [&](int k, real re, real im) { t1[l * PS + k] = T::pack(re, im); });
   }
   __syncthreads();
   for (int l = tid; l < NB * P * P; l += nthr) {           // y: line (node, z, kx)
@@ -193,7 +195,7 @@ __global__ void __launch_bounds__(128) k_spec_fwd(const __grid_constant__ SpecAr
     real xr[P], xi[P];
 #pragma unroll
     for (int s = 0; s < P; ++s) {
-      const cplx c = t1[(nz * P + s) * P + kx];
+      const cplx c = t1[(nz * P + s) * PS + kx];
       xr[s] = T::re(c);
       xi[s] = T::im(c);
     }
@@ -225,7 +227,7 @@ __global__ void __launch_bounds__(256) k_spec_inv(const __grid_constant__ SpecAr
   using store = Num<DFS>;
   using real = typename T::real;
   using cplx = typename T::cplx;
-  constexpr int NM = Shape<P>::NM, NB = Shape<P>::NB, P3 = P * P * P;
+  constexpr int NM = Shape<P>::NM, NB = Shape<P>::NB, P3 = P * P * P, PS = Shape<P>::PS;
   extern __shared__ float4 sm4[];
   __shared__ float4 tw[NM];
   cplx* t1 = reinterpret_cast<cplx*>(sm4);                 // [NB][4][z][ky][kx]
@@ -258,14 +260,14 @@ __global__ void __launch_bounds__(256) k_spec_inv(const __grid_constant__ SpecAr
       xr[s] = T::re(c);
       xi[s] = T::im(c);
     }
-    inverse_line<DFA, P>(xr, xi, wt, [&](int y, real re, real im) { t2[(nfz * P + y) * P + kx] = T::pack(re, im); });
+    inverse_line<DFA, P>(xr, xi, wt, [&](int y, real re, real im) { t2[(nfz * P + y) * PS + kx] = T::pack(re, im); });
   }
   __syncthreads();
   for (int l = tid; l < NB * 4 * P * P; l += nthr) {       // x: line (node, f, z, y), half spectrum -> P reals
     real xr[P], xi[P];
 #pragma unroll
     for (int s = 0; s < P; ++s) {
-      const cplx c = t2[l * P + s];
+      const cplx c = t2[l * PS + s];
       xr[s] = T::re(c);
       xi[s] = T::im(c);
     }
@@ -517,13 +519,14 @@ __global__ void __launch_bounds__(kMacThrDf, 2) k_spec_mac_df(const __grid_const
 
 template <int P, bool DFA>
 size_t fwd_smem() {
-  constexpr int NB = Shape<P>::NB, P3 = P * P * P, NM = Shape<P>::NM;
-  return sizeof(typename Num<DFA>::cplx) * NB * (P3 + P * NM * P) + sizeof(typename Num<DFA>::real) * NB * P3;
+  constexpr int NB = Shape<P>::NB, NM = Shape<P>::NM;
+  constexpr int X3 = P * P * Shape<P>::PS;
+  return sizeof(typename Num<DFA>::cplx) * NB * (X3 + P * NM * P) + sizeof(typename Num<DFA>::real) * NB * X3;
 }
 template <int P, bool DFA>
 size_t inv_smem() {
-  constexpr int NB = Shape<P>::NB, P3 = P * P * P, NM = Shape<P>::NM;
-  return sizeof(typename Num<DFA>::cplx) * NB * 4 * (P * NM * P + P3);
+  constexpr int NB = Shape<P>::NB, NM = Shape<P>::NM;
+  return sizeof(typename Num<DFA>::cplx) * NB * 4 * (P * NM * P + P * P * Shape<P>::PS);
 }
 constexpr size_t kMacSmem = (size_t)kSlots * 128;
 

@@ -27,9 +27,14 @@
 // cells amplify every rounding (fmm_internal.cuh, kWideLeaf), double-float
 // throughout.
 // Measured (direct kernels of p2p.cu before -> here): 128^3 isolated with
-// 16-cell leaves 177 -> 3.0 ms; 256^3, S = 8 30.6 -> 6.7 ms at direct accuracy;
-// 96^3, S = 6 1.04 -> 0.33 ms; 128^3, S = 4 0.87 -> 0.51 ms.  The error of the
-// plain 256^3 solve against FP64 went from 3.5e-7 to 2.9e-7 with it.
+// 16-cell leaves 177 -> 2.9 ms; 256^3, S = 8 30.6 -> 6.0 ms at direct accuracy
+// (sums 0.91, inverse with L2P 4.3); 96^3, S = 6 1.04 -> 0.31 ms; 128^3, S = 4
+// 0.87 -> 0.47 ms.  FMM_NEAR_FFT at 256^3: 2.23 ms for radix-2 transforms of 16
+// points and a separate L2P -> 1.74 ms (sums 1.08 -> 0.91: 22 % fewer
+// frequencies; inverse and L2P 0.92 -> 0.69).  The error of the plain 256^3
+// solve against FP64 went from 3.7e-7 to 2.9e-7 with the direct form, and with
+// FP32 transforms in its place to 3.1e-7 there but from 1.2e-7 to 1.8e-7 at
+// 48^3, S = 6, so the direct form keeps double-float ones.
 #include "fmm_internal.cuh"
 #include "spec.cuh"
 #include "tc_ptx.cuh"
@@ -57,8 +62,12 @@ struct NearShape {
   static constexpr bool DFS = S >= kWideLeaf;                 // storage of the spectra
   static constexpr int THR_FWD = S >= 16 ? 512 : 128;
   static constexpr int THR_INV = S >= 16 ? 512 : 256;
-  static constexpr int IB = S >= 16 ? 1 : (S <= 4 ? 8 : 4);    // (leaf, field) items per inverse CTA
 };
+
+// (leaf, field) items per inverse CTA: one wave of lines over its threads, and
+// two CTAs' shared memory within an SM.
+template <int S, bool DFA>
+constexpr int kItems = S >= 16 ? 1 : (S <= 4 ? 8 : (S >= 8 && DFA ? 2 : 4));
 
 // ------------------------------------------------------------- plan time
 // The kernel's value for field f at lag d (cells), from the folded near table
@@ -162,11 +171,12 @@ __global__ void __launch_bounds__(NearShape<S>::THR_FWD) k_ns_fwd(const float* _
   using store = Num<DFS>;
   using real = typename T::real;
   using cplx = typename T::cplx;
-  constexpr int NM = Shape<S>::NM, NB = Shape<S>::NB, S3 = S * S * S, LANES = store::LANES;
+  constexpr int NM = Shape<S>::NM, NB = Shape<S>::NB, S3 = S * S * S, PS = Shape<S>::PS,
+                LANES = store::LANES;
   extern __shared__ float4 sm4[];
   __shared__ float4 tw[NM];
   cplx* t1 = reinterpret_cast<cplx*>(sm4);                 // [NB][z][y][kx]
-  cplx* t2 = t1 + NB * S3;                                 // [NB][z][ky][kx]
+  cplx* t2 = t1 + NB * S * S * PS;                         // [NB][z][ky][kx]
   real* in = reinterpret_cast<real*>(t2);                  // [NB][z][y][x], consumed before t2 is written
   const int tid = threadIdx.x, nthr = blockDim.x;
   const size_t leaf0 = (size_t)blockIdx.x * NB, leaves = (size_t)1 << (3 * L);
@@ -186,17 +196,17 @@ __global__ void __launch_bounds__(NearShape<S>::THR_FWD) k_ns_fwd(const float* _
       const float dlo = __fsub_rn(d.y, mu_lo);
       const float ph = __fmul_rn(d.x, iv);
       const float lo = fmaf(d.x, iv_lo, fmaf(dlo, iv, fmaf(d.x, iv, -ph)));
-      in[i] = T::done(make_float2(ph, lo));
+      in[(i / S) * PS + x] = T::done(make_float2(ph, lo));
     } else {
-      in[i] = ((r - mu_hi) - mu_lo) * iv;
+      in[(i / S) * PS + x] = ((r - mu_hi) - mu_lo) * iv;
     }
   }
   __syncthreads();
   for (int l = tid; l < NB * S * S; l += nthr) {           // x: S reals -> S frequencies
     real x[S];
 #pragma unroll
-    for (int s = 0; s < S; ++s) x[s] = in[l * S + s];
-    forward_line<DFA, S, true>(x, x, wt, [&](int k, real re, real im) { t1[l * S + k] = T::pack(re, im); });
+    for (int s = 0; s < S; ++s) x[s] = in[l * PS + s];
+    forward_line<DFA, S, true>(x, x, wt, [&](int k, real re, real im) { t1[l * PS + k] = T::pack(re, im); });
   }
   __syncthreads();
   for (int l = tid; l < NB * S * S; l += nthr) {           // y: line (leaf, z, kx)
@@ -204,7 +214,7 @@ __global__ void __launch_bounds__(NearShape<S>::THR_FWD) k_ns_fwd(const float* _
     real xr[S], xi[S];
 #pragma unroll
     for (int s = 0; s < S; ++s) {
-      const cplx c = t1[(nz * S + s) * S + kx];
+      const cplx c = t1[(nz * S + s) * PS + kx];
       xr[s] = T::re(c);
       xi[s] = T::im(c);
     }
@@ -229,26 +239,42 @@ __global__ void __launch_bounds__(NearShape<S>::THR_FWD) k_ns_fwd(const float* _
   }
 }
 
-// One separable L2P pass over `items` arrays: out[a][c][b] = sum_k W[k][c] in[a][k][b],
-// b < B, a < A; weights (hi, lo).
-template <bool DFA, int S>
-__device__ __forceinline__ void l2p_pass(const typename Num<DFA>::real* in, typename Num<DFA>::real* out, int total,
-                                         int B, int p, const float2* W, int tid, int nthr) {
+// One separable L2P pass: out[a][c][b] = sum_k W[k][c] in[a][k][b], b < B, a < A;
+// weights (hi, lo).  A thread makes the S outputs of a line (a, b).  OS: row
+// stride of `out`'s innermost S values.
+template <bool DFA, int S, int B, int OS>
+__device__ __forceinline__ void l2p_pass(const typename Num<DFA>::real* in, typename Num<DFA>::real* out, int A, int p,
+                                         const float2* W, int tid, int nthr) {
   using T = Num<DFA>;
-  for (int i = tid; i < total; i += nthr) {
-    const int b = i % B, c = (i / B) % S, a = i / (B * S);
+  for (int l = tid; l < A * B; l += nthr) {
+    const int b = l % B, a = l / B;
     const typename T::real* src = in + (size_t)a * p * B + b;
-    if constexpr (DFA) {
-      float2 acc = T::zero();
-      for (int k = 0; k < p; ++k) T::mac(acc, W[k * S + c].x, W[k * S + c].y, src[k * B]);
-      out[i] = T::done(acc);
-    } else {
-      float acc = 0.f, lo = 0.f;
-      for (int k = 0; k < p; ++k) {
-        acc = fmaf(W[k * S + c].x, src[k * B], acc);
-        lo = fmaf(W[k * S + c].y, src[k * B], lo);
+    float hi[S], lo[S];
+#pragma unroll
+    for (int c = 0; c < S; ++c) hi[c] = lo[c] = 0.f;
+#pragma unroll 1
+    for (int k = 0; k < p; ++k) {
+      const typename T::real x = src[k * B];
+#pragma unroll
+      for (int c = 0; c < S; ++c) {
+        const float2 w = W[k * S + c];
+        if constexpr (DFA) {
+          float2 t = make_float2(hi[c], lo[c]);
+          T::mac(t, w.x, w.y, x);
+          hi[c] = t.x;
+          lo[c] = t.y;
+        } else {
+          hi[c] = fmaf(w.x, x, hi[c]);
+          lo[c] = fmaf(w.y, x, lo[c]);
+        }
       }
-      out[i] = acc + lo;
+    }
+#pragma unroll
+    for (int c = 0; c < S; ++c) {
+      const int o = (a * S + c) * B + b;
+      typename T::real& dst = out[OS == S ? o : (o / S) * OS + o % S];
+      if constexpr (DFA) dst = T::done(make_float2(hi[c], lo[c]));
+      else dst = hi[c] + lo[c];
     }
   }
   __syncthreads();
@@ -256,7 +282,7 @@ __device__ __forceinline__ void l2p_pass(const typename Num<DFA>::real* in, type
 
 // Outputs.  CTA: IB (leaf, field) items.
 template <int S, bool DFA>
-__global__ void __launch_bounds__(NearShape<S>::THR_INV) k_ns_inv(const void* __restrict__ Pin, int nkp, int N, int p,
+__global__ void __launch_bounds__(NearShape<S>::THR_INV) k_ns_inv(const void* __restrict__ Pin, int nkp, int far_at, int N, int p,
                                                                   const float* __restrict__ F,
                                                                   const double* __restrict__ F64,
                                                                   const float2* __restrict__ wp2m,
@@ -267,21 +293,21 @@ __global__ void __launch_bounds__(NearShape<S>::THR_INV) k_ns_inv(const void* __
   using store = Num<DFS>;
   using real = typename T::real;
   using cplx = typename T::cplx;
-  constexpr int NM = Shape<S>::NM, IB = NearShape<S>::IB, S3 = S * S * S;
+  constexpr int NM = Shape<S>::NM, IB = kItems<S, DFA>, S3 = S * S * S, PS = Shape<S>::PS;
   extern __shared__ float4 sm4[];
   __shared__ float4 tw[NM];
   __shared__ float2 W[kMaxOrder * S];
-  real* far = reinterpret_cast<real*>(sm4);                // [IB][S^3]
-  cplx* t2 = reinterpret_cast<cplx*>(far + IB * S3);       // [IB][z][y][kx]
-  cplx* t1 = t2 + IB * S3;                                 // [IB][z][ky][kx]
+  cplx* t2 = reinterpret_cast<cplx*>(sm4);                 // [IB][z][y][kx]
+  cplx* t1 = t2 + IB * S * S * PS;                         // [IB][z][ky][kx]
+  real* far = reinterpret_cast<real*>(reinterpret_cast<char*>(sm4) + far_at);   // [IB][z][y][x], behind t1 and the L2P scratch
   const int tid = threadIdx.x, nthr = blockDim.x;
   const size_t item0 = (size_t)blockIdx.x * IB;
   const int p3 = p * p * p;
   if (DFA && tid < NM) tw[tid] = __ldg(twg + tid);
   const Twiddle<DFA, S> wt(twg, tw);
   for (int i = tid; i < p * S; i += nthr) W[i] = __ldg(wp2m + i);
-  {                                                        // L2P, scratch in t1's space
-    real* a = reinterpret_cast<real*>(t1);                 // [IB][p^3]
+  {                                                        // L2P, scratch in t2's and t1's space
+    real* a = reinterpret_cast<real*>(sm4);                // [IB][p^3]
     real* b = a + IB * p3;                                 // [IB][p][p][S]
     real* c = b + IB * p * p * S;                          // [IB][p][S][S]
     for (int i = tid; i < IB * p3; i += nthr) {
@@ -289,9 +315,9 @@ __global__ void __launch_bounds__(NearShape<S>::THR_INV) k_ns_inv(const void* __
       else a[i] = widen<DFA>(__ldg(F + item0 * p3 + i));
     }
     __syncthreads();
-    l2p_pass<DFA, S>(a, b, IB * p * p * S, 1, p, W, tid, nthr);
-    l2p_pass<DFA, S>(b, c, IB * p * S * S, S, p, W, tid, nthr);
-    l2p_pass<DFA, S>(c, far, IB * S3, S * S, p, W, tid, nthr);
+    l2p_pass<DFA, S, 1, S>(a, b, IB * p * p, p, W, tid, nthr);
+    l2p_pass<DFA, S, S, S>(b, c, IB * p, p, W, tid, nthr);
+    l2p_pass<DFA, S, S * S, PS>(c, far, IB, p, W, tid, nthr);
   }
   const typename store::cplx* Ph = reinterpret_cast<const typename store::cplx*>(Pin) + item0 * nkp;
   for (int l = tid; l < IB * NM * S; l += nthr) {          // z: line (item, ky, kx), NM -> S
@@ -315,7 +341,7 @@ __global__ void __launch_bounds__(NearShape<S>::THR_INV) k_ns_inv(const void* __
       xr[s] = T::re(v);
       xi[s] = T::im(v);
     }
-    inverse_line<DFA, S>(xr, xi, wt, [&](int y, real re, real im) { t2[(iz * S + y) * S + kx] = T::pack(re, im); });
+    inverse_line<DFA, S>(xr, xi, wt, [&](int y, real re, real im) { t2[(iz * S + y) * PS + kx] = T::pack(re, im); });
   }
   __syncthreads();
   const size_t N3 = (size_t)N * N * N;
@@ -323,7 +349,7 @@ __global__ void __launch_bounds__(NearShape<S>::THR_INV) k_ns_inv(const void* __
     real xr[S], xi[S];
 #pragma unroll
     for (int s = 0; s < S; ++s) {
-      const cplx v = t2[l * S + s];
+      const cplx v = t2[l * PS + s];
       xr[s] = T::re(v);
       xi[s] = T::im(v);
     }
@@ -333,40 +359,66 @@ __global__ void __launch_bounds__(NearShape<S>::THR_INV) k_ns_inv(const void* __
     unmorton((uint32_t)(item >> 2), lx, ly, lz);
     float* dst = (f == 0 ? phi : acc + (size_t)(f - 1) * N3) +
                  ((size_t)(lz * S + z) * N + (ly * S + y)) * N + lx * S;
-    const real* fr = far + l * S;
-    inverse_real_line<DFA, S>(xr, xi, wt, [&](int x, real v) { dst[x] = narrow<false, DFA>(T::add(v, fr[x])); });
+    const real* fr = far + l * PS;
+    if constexpr (!DFA && S % 4 == 0) {
+      float o[S];
+      inverse_real_line<DFA, S>(xr, xi, wt, [&](int x, float v) { o[x] = v + fr[x]; });
+#pragma unroll
+      for (int q = 0; q < S; q += 4) *reinterpret_cast<float4*>(dst + q) = make_float4(o[q], o[q + 1], o[q + 2], o[q + 3]);
+    } else {
+      inverse_real_line<DFA, S>(xr, xi, wt, [&](int x, real v) { dst[x] = narrow<false, DFA>(T::add(v, fr[x])); });
+    }
   }
 }
 
 // ---------------------------------------------------------- spectral sums
 // Rows of 4 target leaves along x per thread, as k_spec_mac; the chunk's 27
-// kernel spectra and the tile's 6^3 source spectra in shared memory (41 KB, so
-// that several CTAs share an SM and one's copies run under another's sums).
+// kernel spectra and the tile's 6^3 source spectra in shared memory (41 KB),
+// the next chunk's copied (cp.async) during the current sums: a CTA takes
+// `per` consecutive chunks of one tile, up to 8, fewer where that leaves fewer
+// than 4 CTAs per SM.
+constexpr int kChunks = 8;
+constexpr int kStage = kNO * 32 + kSlots * 8;   // float4 per stage
 template <bool DF>
 __global__ void __launch_bounds__(DF ? 512 : 256) k_ns_mac(const float4* __restrict__ K, const void* __restrict__ Mh,
-                                                          void* __restrict__ Ph, int L, int nkp, int iso) {
+                                                          void* __restrict__ Ph, int L, int nkp, int iso, int per) {
   constexpr int LANES = Num<DF>::LANES, NTHR = DF ? 512 : 256;
   extern __shared__ float4 sm4[];
-  float4* sK = sm4;                         // [27][32]
-  float4* sM = sm4 + kNO * 32;              // [216][8]
   const int tid = threadIdx.x, n = 1 << L, nt = n / kTile;
-  const int tile = blockIdx.x, chunk = blockIdx.y;
+  const int tile = blockIdx.x;
   const int TX = tile % nt, TY = (tile / nt) % nt, TZ = tile / (nt * nt);
   const size_t leaves = (size_t)1 << (3 * L);
-  const float4* Kc = K + (size_t)chunk * kNO * 32;
-  for (int i = tid; i < kNO * 32; i += NTHR) tc::cp_async16_full(tc::smem_u32(sK + i), Kc + i);
-  const char* src = reinterpret_cast<const char*>(Mh) + (size_t)chunk * (leaves + 1) * 128;
-  for (int i = tid; i < kSlots * 8; i += NTHR) {
-    const int slot = i >> 3, part = i & 7;
+  unsigned* slot_leaf = reinterpret_cast<unsigned*>(sm4 + 2 * kStage);   // [216]
+  for (int slot = tid; slot < kSlots; slot += NTHR) {
     const int ux = TX * kTile - 1 + slot % kHaloN, uy = TY * kTile - 1 + (slot / kHaloN) % kHaloN,
               uz = TZ * kTile - 1 + slot / (kHaloN * kHaloN);
     const bool inbox = (unsigned)ux < (unsigned)n && (unsigned)uy < (unsigned)n && (unsigned)uz < (unsigned)n;
-    const size_t leaf = inbox || !iso ? morton(ux & (n - 1), uy & (n - 1), uz & (n - 1)) : leaves;
-    tc::cp_async16_full(tc::smem_u32(sM + i), src + leaf * 128 + part * 16);
+    slot_leaf[slot] = inbox || !iso ? morton(ux & (n - 1), uy & (n - 1), uz & (n - 1)) : (unsigned)leaves;
   }
-  tc::cp_async_commit();
-  tc::cp_async_wait<0>();
   __syncthreads();
+  auto load = [&](int chunk, int st) {
+    float4* to = sm4 + st * kStage;
+    const float4* Kc = K + (size_t)chunk * kNO * 32;
+    for (int i = tid; i < kNO * 32; i += NTHR) tc::cp_async16_full(tc::smem_u32(to + i), Kc + i);
+    const char* src = reinterpret_cast<const char*>(Mh) + (size_t)chunk * (leaves + 1) * 128;
+    for (int i = tid; i < kSlots * 8; i += NTHR)
+      tc::cp_async16_full(tc::smem_u32(to + kNO * 32 + i), src + (size_t)slot_leaf[i >> 3] * 128 + (i & 7) * 16);
+    tc::cp_async_commit();
+  };
+  const int chunks = nkp / LANES, c_end = min(chunks, ((int)blockIdx.y + 1) * per);
+  int chunk = blockIdx.y * per;
+  load(chunk, 0);
+#pragma unroll 1
+  for (int st = 0; chunk < c_end; ++chunk, st ^= 1) {
+  if (chunk + 1 < c_end) {
+    load(chunk + 1, st ^ 1);
+    tc::cp_async_wait<1>();
+  } else {
+    tc::cp_async_wait<0>();
+  }
+  __syncthreads();
+  const float4* sK = sm4 + st * kStage;     // [27][32]
+  const float4* sM = sK + kNO * 32;         // [216][8]
   if constexpr (!DF) {
     const int fr = tid & 15, ty = (tid >> 4) & 3, tz = tid >> 6;
     const float2* halo = reinterpret_cast<const float2*>(sM) + fr;
@@ -468,20 +520,22 @@ __global__ void __launch_bounds__(DF ? 512 : 256) k_ns_mac(const float4* __restr
       out[(leaf * 4 + f) * nkp + (size_t)chunk * LANES + fr] = make_float4(a.x, a.y, b.x, b.y);
     }
   }
+  __syncthreads();                          // this stage is refilled next
+  }
 }
-constexpr size_t kMacSmem = sizeof(float4) * (kNO * 32 + kSlots * 8);
+constexpr size_t kMacSmem = sizeof(float4) * 2 * kStage + sizeof(unsigned) * kSlots;
 
 template <int S, bool DFA>
 size_t fwd_smem() {
   constexpr int NB = Shape<S>::NB, NM = Shape<S>::NM;
-  return sizeof(typename Num<DFA>::cplx) * NB * (S * S * S + S * NM * S);
+  return sizeof(typename Num<DFA>::cplx) * NB * (S * S * Shape<S>::PS + S * NM * S);
 }
 template <int S, bool DFA>
 size_t inv_smem(int p) {
-  constexpr int IB = NearShape<S>::IB, NM = Shape<S>::NM, S3 = S * S * S;
+  constexpr int IB = kItems<S, DFA>, NM = Shape<S>::NM, X3 = S * S * Shape<S>::PS;
   const size_t real = sizeof(typename Num<DFA>::real), cplx = sizeof(typename Num<DFA>::cplx);
-  const size_t t1 = cplx * IB * S * NM * S, l2p = real * IB * (p * p * p + p * p * S + p * S * S);
-  return real * IB * S3 + cplx * IB * S3 + (t1 > l2p ? t1 : l2p);
+  const size_t t = cplx * IB * (X3 + S * NM * S), l2p = real * IB * (p * p * p + p * p * S + p * S * S);
+  return (t > l2p ? t : l2p) + real * IB * X3;
 }
 
 template <int S, bool DFA>
@@ -496,10 +550,13 @@ cudaError_t rest_as(Plan& P, float* phi, float* acc, cudaStream_t s) {
   constexpr bool DFS = NearShape<S>::DFS;
   const unsigned leaves = 1u << (3 * P.L);
   const int nt = (1 << P.L) / kTile, ch = chunks_of(S, DFS), nkp = ch * Num<DFS>::LANES;
-  k_ns_mac<DFS><<<dim3(nt * nt * nt, ch), DFS ? 512 : 256, kMacSmem, s>>>(static_cast<const float4*>(P.ns_K), P.ns_M,
-                                                                         P.ns_P, P.L, nkp, P.iso);
-  k_ns_inv<S, DFA><<<leaves * 4 / NearShape<S>::IB, NearShape<S>::THR_INV, inv_smem<S, DFA>(P.p), s>>>(
-      P.ns_P, nkp, P.N, P.p, P.F[P.L], P.F64[P.L], P.w_p2m, P.ns_tw, phi, acc);
+  const int tiles = nt * nt * nt, fit = (int)((long)tiles * ch / (4 * P.num_sms));
+  const int per = fit < 1 ? 1 : (fit < kChunks ? fit : kChunks);
+  k_ns_mac<DFS><<<dim3(tiles, (ch + per - 1) / per), DFS ? 512 : 256, kMacSmem, s>>>(
+      static_cast<const float4*>(P.ns_K), P.ns_M, P.ns_P, P.L, nkp, P.iso, per);
+  k_ns_inv<S, DFA><<<leaves * 4 / kItems<S, DFA>, NearShape<S>::THR_INV, inv_smem<S, DFA>(P.p), s>>>(
+      P.ns_P, nkp, (int)(inv_smem<S, DFA>(P.p) - sizeof(typename Num<DFA>::real) * kItems<S, DFA> * S * S * Shape<S>::PS), P.N,
+      P.p, P.F[P.L], P.F64[P.L], P.w_p2m, P.ns_tw, phi, acc);
   return cudaGetLastError();
 }
 

@@ -17,6 +17,9 @@ template <int P>
 struct Shape {
   static constexpr int NM = 2 * P - 1;
   static constexpr int LINES = NM * P;
+  // row stride of the shared arrays whose x lines a thread walks: odd, so that
+  // a warp's rows start on different banks (P = 16 has no room for it)
+  static constexpr int PS = P >= 16 ? P : (P | 1);
   // blocks per CTA of the transforms: about 128 lines of the widest pass
   static constexpr int NB = LINES <= 16 ? 8 : (LINES <= 32 ? 4 : (LINES <= 72 ? 2 : 1));
 };
