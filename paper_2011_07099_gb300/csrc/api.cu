@@ -156,7 +156,12 @@ void free_plan(Plan* P) {
     cudaFree(P->Mbf_hi[l]);
     cudaFree(P->Apre[l]);
     delete static_cast<CUtensorMap*>(P->tmapB[l]);
+    cudaFree(P->stc_W[l]);
+    cudaFree(P->stc_scale[l]);
+    cudaFree(P->stc_B[l]);
+    delete static_cast<CUtensorMap*>(P->stc_map[l]);
   }
+  cudaFree(P->stc_amax);
   cudaFree(P->w_p2m);
   cudaFree(P->w_m2m);
   cudaFree(P->stage_in);
@@ -269,8 +274,10 @@ int retabulate(Plan& P) {
     }
   }
   if (P.ns_K && fmm::launch_near_spec_kernels(P, 0) != cudaSuccess) return FMM_ERR_CUDA;
-  for (int l = 2; l <= P.L; ++l)
+  for (int l = 2; l <= P.L; ++l) {
     if (P.spec_K[l] && fmm::launch_spec_kernels(P, l, 0) != cudaSuccess) return FMM_ERR_CUDA;
+    if (P.stc_W[l] && fmm::launch_stc_weights(P, l, 0) != cudaSuccess) return FMM_ERR_CUDA;
+  }
   if (P.tc_ready) {
     for (int l = fmm::kTcMinLevel; l <= P.L; ++l) {
       if (!P.Apre[l]) continue;
@@ -450,7 +457,7 @@ fmm_plan* fmm_plan_create(int N, int L, int order) {
       fmm::setup_m2l_tc(*P) != cudaSuccess || fmm::setup_learn() != cudaSuccess ||
       fmm::setup_learn_spec(*P) != cudaSuccess ||
       fmm::setup_downward(*P) != cudaSuccess || fmm::setup_p2p(*P) != cudaSuccess ||
-      fmm::setup_m2l_spec(*P) != cudaSuccess || retabulate(*P) != FMM_OK) {
+      fmm::setup_m2l_spec(*P) != cudaSuccess || fmm::setup_spec_tc(*P) != cudaSuccess || retabulate(*P) != FMM_OK) {
     free_plan(P);
     set_err(FMM_ERR_CUDA);
     return nullptr;
@@ -483,7 +490,24 @@ int prepare_tc(Plan& P) {
   const size_t E = 8 * P.p - 1;
   bool made = false;
   for (int l = fmm::tc_first_level(P); l <= P.L; ++l) {
-    if (P.Apre[l] || !fmm::tc_level(P, l)) continue;
+    if (fmm::spec_tc_level(P, l)) {
+      if (P.stc_map[l]) continue;
+      size_t nW, nB, nS;
+      fmm::stc_bytes(P, l, nW, nB, nS);
+      if ((!P.stc_amax && !dev_alloc(&P.stc_amax, (size_t)fmm::kMaxLevel + 1)) ||
+          (!P.stc_W[l] && cudaMalloc(&P.stc_W[l], nW) != cudaSuccess) ||
+          (!P.stc_B[l] && cudaMalloc(&P.stc_B[l], nB) != cudaSuccess) ||
+          (!P.stc_scale[l] && cudaMalloc(&P.stc_scale[l], nS) != cudaSuccess))
+        return FMM_ERR_ALLOC;
+      // the halo of the isolated problem stays zero
+      if (cudaMemset(P.stc_B[l], 0, nB) != cudaSuccess || fmm::launch_stc_weights(P, l, 0) != cudaSuccess)
+        return FMM_ERR_CUDA;
+      const int rc = fmm::make_stc_map(P, l);
+      if (rc != FMM_OK) return rc;
+      made = true;
+      continue;
+    }
+    if (P.Apre[l]) continue;
     const bool wide = fmm::tc_wide(P, l);   // wide modes: tiles from tab + tab_lo, no BF16 table
     if ((!wide && !P.tab_bf[l] && !dev_alloc(&P.tab_bf[l], E * E * E)) ||
         (!P.Mbf_hi[l] && cudaMalloc(&P.Mbf_hi[l], fmm::tc_bsplit_bytes(P.p, l, fmm::tc_splits(P, l))) != cudaSuccess) ||
@@ -537,6 +561,11 @@ int fmm_plan_set_boundary(fmm_plan* plan, int boundary) {
   P.offsets[2] = offs;
   P.n_off[2] = count;
   P.iso = iso;
+  for (int l = 2; l <= P.L; ++l) {      // the tensor cores' sources: a periodic halo, or zeros
+    size_t nW, nB, nS;
+    fmm::stc_bytes(P, l, nW, nB, nS);
+    if (P.stc_B[l]) FMM_CUDA_TRY(cudaMemset(P.stc_B[l], 0, nB));
+  }
   // the offset-range scratch of the coarse levels follows the list length
   const int rc = alloc_m2l_part(P);
   if (rc != FMM_OK) return set_err(rc);
@@ -858,10 +887,12 @@ int fmm_solve(fmm_plan* plan, const float* density, float* potential, float* acc
   for (int l = P.L - 1; l >= 2; --l) FMM_CUDA_TRY(fmm::launch_m2m(P, l, s));
   FMM_CUDA_TRY(mark(FMM_TIME_M2M, 1));
   FMM_CUDA_TRY(mark(FMM_TIME_M2L, 0));
-  auto on_spec = [&](int l) { return !fmm::fft_level(P, l) && !on_tc(l) && P.spec_K[l]; };
+  auto on_stc = [&](int l) { return !fmm::fft_level(P, l) && tc && fmm::spec_tc_level(P, l); };
+  auto on_spec = [&](int l) { return !fmm::fft_level(P, l) && !on_tc(l) && !on_stc(l) && P.spec_K[l]; };
   // one level on its own: FFT ablation, tensor cores or the dense CUDA-core kernels
   auto m2l_level = [&](int l, cudaStream_t q) -> cudaError_t {
     if (fmm::fft_level(P, l)) return fmm::launch_m2l_fft(P, l, q);
+    if (on_stc(l)) return fmm::launch_m2l_spec_tc(P, l, q);
     if (!on_tc(l)) return fmm::launch_m2l_fp32(P, l, q);
     const cudaError_t e = fmm::launch_split_bf16(P, l, q);
     return e != cudaSuccess ? e : fmm::launch_m2l_tc(P, l, P.prec, q);
@@ -871,14 +902,14 @@ int fmm_solve(fmm_plan* plan, const float* density, float* potential, float* acc
     // auxiliary stream: the double-float spectral levels and the rest
     bool side = false, main = false;
     for (int l = 2; l <= P.L; ++l) {
-      if (on_tc(l) || (on_spec(l) && !fmm::wide_level(P, l))) main = true;
+      if (on_tc(l) || on_stc(l) || (on_spec(l) && !fmm::wide_level(P, l))) main = true;
       else side = true;
     }
     const bool fork = side && main;
     cudaStream_t q = fork ? P.aux[0] : s;
     if (fork) FMM_CUDA_TRY(cudaEventRecord(P.fev[2], s));
     for (int l = P.L; l >= 2; --l)
-      if (on_tc(l)) FMM_CUDA_TRY(m2l_level(l, s));
+      if (on_tc(l) || on_stc(l)) FMM_CUDA_TRY(m2l_level(l, s));
     int f0 = P.L + 1, f1 = 1, d0 = P.L + 1, d1 = 1;   // spectral levels: wide_level and on_tc split them by depth
     for (int l = 2; l <= P.L; ++l) {
       if (!on_spec(l)) continue;
@@ -890,7 +921,7 @@ int fmm_solve(fmm_plan* plan, const float* density, float* potential, float* acc
     if (fork) FMM_CUDA_TRY(cudaStreamWaitEvent(q, P.fev[2], 0));
     if (d0 <= d1) FMM_CUDA_TRY(fmm::launch_m2l_spec(P, true, d0, d1, q));
     for (int l = 2; l <= P.L; ++l)
-      if (!on_tc(l) && !on_spec(l)) FMM_CUDA_TRY(m2l_level(l, q));
+      if (!on_tc(l) && !on_stc(l) && !on_spec(l)) FMM_CUDA_TRY(m2l_level(l, q));
     if (fork) {
       FMM_CUDA_TRY(cudaEventRecord(P.fev[3], q));
       FMM_CUDA_TRY(cudaStreamWaitEvent(s, P.fev[3], 0));

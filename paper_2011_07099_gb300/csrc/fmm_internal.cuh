@@ -101,6 +101,14 @@ struct Plan {
   void* spec_M[kMaxLevel + 1] = {};
   void* spec_P[kMaxLevel + 1] = {};
   float4* spec_tw = nullptr;
+  // the same products on the tensor cores (m2l_spec_tc.cu), levels the mixed
+  // forms take there: split weights and their scales, split source spectra,
+  // the tensor map (host CUtensorMap) and each level's largest mass sum
+  void* stc_W[kMaxLevel + 1] = {};
+  float* stc_scale[kMaxLevel + 1] = {};
+  void* stc_B[kMaxLevel + 1] = {};
+  void* stc_map[kMaxLevel + 1] = {};
+  float* stc_amax = nullptr;
   // tensor-core M2L (levels >= kTcMinLevel, allocated on the first mixed-precision solve)
   uint4* tab_bf[kMaxLevel + 1] = {};       // per table entry, per field: bf16 hi | bf16 lo << 16
   void* Mbf_hi[kMaxLevel + 1] = {};        // gridlet masses split into BF16 parts (2; 3 at bf16x6 levels), per parity class with a halo
@@ -197,20 +205,19 @@ inline int tc_first_level(const Plan& P) {
   return P.tc_min_level > wide_first ? P.tc_min_level : wide_first;
 }
 
-// The levels of the mixed forms that run the dense tensor-core contraction:
-// the wide ones (bf16x6; in double-float spectral products level 5 of 512^3
-// order 8 takes 74 ms against 94 ms, but the mixed form's results would then
-// differ from bf16x6's by its own 1e-3 of the rms at the cells around the
-// heaviest clumps), the low orders, and a level without spectral buffers.  From
-// kSpecOrder on the FP32 levels take the spectral products (m2l_spec.cu),
-// whose 16x (p = 6) to 36x (p = 8) fewer terms beat the tensor pipe's three
-// BF16 products per term: measured 256^3 p = 6 levels 4 + 5 4.78 -> 4.46 ms,
-// 512^3 p = 8 level 6 281 -> 77 ms; at p = 4 (5x fewer terms) the tensor
-// cores keep level 5 of 128^3 (0.83 against 1.30 ms).
-constexpr int kSpecOrder = 5;
-inline bool tc_level(const Plan& P, int l) {
-  return l >= tc_first_level(P) && (wide_level(P, l) || P.p < kSpecOrder || !P.spec_K[l]);
+// The levels of the mixed forms on the tensor cores.  Spectral products
+// (m2l_spec_tc.cu): the FP32-field levels of orders >= kSpecTcOrder.  Dense
+// contraction (m2l_tc.cu): the lower orders, whose gridlets make few
+// frequencies (p = 3: 75, at most half of a wave of CTAs); a level without
+// spectral buffers; and the wide levels (bf16x6; in double-float spectral
+// products level 5 of 512^3 order 8 takes 74 ms against 94 ms, but the mixed
+// form's results would then differ from bf16x6's by its own 1e-3 of the rms at
+// the cells around the heaviest clumps).
+constexpr int kSpecTcOrder = 4;
+inline bool spec_tc_level(const Plan& P, int l) {
+  return P.p >= kSpecTcOrder && l >= tc_first_level(P) && !wide_level(P, l) && P.spec_K[l];
 }
+inline bool tc_level(const Plan& P, int l) { return l >= tc_first_level(P) && !spec_tc_level(P, l); }
 
 cudaError_t setup_m2l_fp32(const Plan& P);
 // Number of offset ranges the FP32 M2L of a level is split into (1 = none).
@@ -243,6 +250,14 @@ size_t spec_source_bytes(const Plan& P, int level);
 size_t spec_target_bytes(const Plan& P, int level);
 cudaError_t setup_m2l_spec(const Plan& P);
 cudaError_t launch_spec_kernels(Plan& P, int level, cudaStream_t s);
+// Its tensor-core form (m2l_spec_tc.cu): buffer sizes of a level (weights,
+// source spectra, scales), the tensor map (FMM_* code), function attributes,
+// the plan-time weights (after the level's kernel spectra), the level's M2L.
+void stc_bytes(const Plan& P, int level, size_t& nW, size_t& nB, size_t& nS);
+int make_stc_map(Plan& P, int level);
+cudaError_t setup_spec_tc(const Plan& P);
+cudaError_t launch_stc_weights(Plan& P, int level, cudaStream_t s);
+cudaError_t launch_m2l_spec_tc(Plan& P, int level, cudaStream_t s);
 // FP32 spectra of `blocks` order-p gridlets, [chunk][blocks + 1][16].
 cudaError_t launch_spec_fwd(Plan& P, const float* src, void* dst, size_t blocks, cudaStream_t s);
 cudaError_t launch_m2l_spec(Plan& P, bool df, int l0, int l1, cudaStream_t s);

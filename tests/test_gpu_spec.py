@@ -1,19 +1,19 @@
-"""M2L by spectral products (csrc/m2l_spec.cu) against the FP64 oracle, through
-the C-ABI: every order it is built for, on trees whose levels take each of its
-kernels (level 2 periodic and isolated, double-float, row chains, FP32), with
-one cell per leaf and more.
+"""M2L by spectral products (csrc/m2l_spec.cu, on the tensor cores
+csrc/m2l_spec_tc.cu) against the FP64 oracle, through the C-ABI, on trees whose
+levels take each of its kernels (level 2 periodic and isolated, double-float,
+row chains, FP32, tensor cores), with one cell per leaf and more.
 
 Tolerance: the plain form's 1e-6 (FP32 spectra, sums over a plane's terms apart
 from the total, double-float transforms: rounding of ~1e-7 per level times the
-far field's cancellation of a few); the mixed form transforms in FP32 and keeps
-its bf16x3 bound 2e-5."""
+far field's cancellation of a few); the mixed form (FP16 pairs, 22 bits, FP32
+accumulation and transforms) keeps its bf16x3 bound 2e-5."""
 import numpy as np
 import pytest
 
 from oracle import fmm as ofmm
 from oracle import nonperiodic as npo
 from paper_2011_07099_gb300 import inputs
-from parity_util import assert_close
+from parity_util import assert_close, leaf_values
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -43,32 +43,94 @@ def _solve(B, rho, L, p, iso=False, prec=0, timing=False):
     return phi.cpu().numpy(), acc.cpu().numpy()
 
 
-@pytest.mark.parametrize("p", [2, 3, 4, 5, 6, 7, 8])
-@pytest.mark.parametrize("N,L", [(12, 2), (16, 3), (16, 4)])
-def test_spectral_m2l_matches_oracle(B, N, L, p):
+LEAVES = {2: [[0, 0, 0], [3, 1, 2]], 3: [[7, 0, 5]], 4: [[15, 0, 6]]}   # on the faces: every wrap is taken
+
+
+def _check(B, N, L, p, tol, iso=False, prec=0):
     rho = inputs.lognormal(N, sigma=0.8, seed=N + L + p)
-    phi, acc = _solve(B, rho, L, p)
-    ophi, og = ofmm.solve(rho, L, p)
-    assert_close(phi, ophi, 1e-6, f"phi {N}^3 L={L} p={p}")
-    assert_close(acc, og, 1e-6, f"g {N}^3 L={L} p={p}")
+    phi, acc = _solve(B, rho, L, p, iso, prec)
+    leaves = np.array(LEAVES[L])
+    ref = (npo.solve_isolated_at if iso else ofmm.solve_at)(rho, L, p, leaves)
+    got = leaf_values(phi, acc, leaves, N >> L)
+    what = f"{N}^3 L={L} p={p} iso={iso} prec={prec}"
+    assert_close(got[:, 0], ref[:, 0], tol, "phi " + what)
+    assert_close(got[:, 1:], ref[:, 1:], tol, "g " + what)
 
 
-@pytest.mark.parametrize("N,L,p", [(8, 2, 3), (16, 2, 6), (16, 3, 5), (16, 4, 6), (8, 3, 8)])
+# odd and even orders; p = 8 is in the full-size tests of the plain and the mixed form
+@pytest.mark.parametrize("N,L,p", [(12, 2, 5), (12, 2, 7), (16, 3, 4), (16, 4, 2), (16, 4, 3), (16, 4, 5), (16, 4, 6),
+                                   (16, 3, 7)])
+def test_spectral_m2l_matches_oracle(B, N, L, p):
+    _check(B, N, L, p, 1e-6)
+
+
+@pytest.mark.parametrize("N,L,p", [(8, 2, 3), (16, 2, 6), (16, 3, 5), (16, 4, 4)])
 def test_spectral_m2l_isolated_matches_oracle(B, N, L, p):
-    rho = inputs.lognormal(N, sigma=0.8, seed=N + p)
-    phi, acc = _solve(B, rho, L, p, iso=True)
-    ophi, og = npo.solve_isolated(rho, L, p)
-    assert_close(phi, ophi, 1e-6, f"isolated phi {N}^3 L={L} p={p}")
-    assert_close(acc, og, 1e-6, f"isolated g {N}^3 L={L} p={p}")
+    _check(B, N, L, p, 1e-6, iso=True)
 
 
-@pytest.mark.parametrize("N,L,p", [(32, 4, 5), (16, 4, 6), (32, 4, 7), (16, 4, 8)])
-def test_mixed_form_spectral_levels_match_oracle(B, N, L, p):
-    rho = inputs.lognormal(N, sigma=0.5, seed=N + L + p)
-    phi, acc = _solve(B, rho, L, p, prec=B.FMM_PREC_BF16X3)
-    ophi, og = ofmm.solve(rho, L, p)
-    assert_close(phi, ophi, 2e-5, f"mixed phi {N}^3 L={L} p={p}")
-    assert_close(acc, og, 2e-5, f"mixed g {N}^3 L={L} p={p}")
+# the tensor-core form: two parents per forward CTA (p <= 6) and one (p = 7),
+# periodic halo copies and the isolated problem's zeros
+@pytest.mark.parametrize("N,L,p,iso", [(16, 4, 4, False), (16, 4, 5, True), (16, 4, 6, False), (16, 4, 7, False),
+                                       (32, 5, 4, False)])
+def test_tensor_core_spectral_levels_match_oracle(B, N, L, p, iso):
+    LEAVES.setdefault(5, [[31, 0, 17]])
+    _check(B, N, L, p, 2e-5, iso=iso, prec=B.FMM_PREC_BF16X3)
+
+
+def test_tensor_core_form_follows_the_boundary(B):
+    # the periodic halo of an earlier solve must not leak into the isolated problem, nor zeros into the periodic one
+    N, L, p = 32, 4, 4
+    rho = torch.from_numpy(inputs.lognormal(N, sigma=0.8, seed=6)).cuda()
+    plan = B.Plan(N, L, p, precision=B.FMM_PREC_BF16X3)
+    out = []
+    for b in (B.FMM_BOUNDARY_PERIODIC, B.FMM_BOUNDARY_ISOLATED, B.FMM_BOUNDARY_PERIODIC, B.FMM_BOUNDARY_ISOLATED):
+        B.fmm_plan_set_boundary(plan.handle, b)
+        phi, acc = plan.solve(rho)
+        torch.cuda.synchronize()
+        out.append((phi, acc))
+    plan.close()
+    assert torch.equal(out[0][0], out[2][0]) and torch.equal(out[0][1], out[2][1])
+    fresh = B.Plan(N, L, p)
+    B.fmm_plan_set_boundary(fresh.handle, B.FMM_BOUNDARY_ISOLATED)
+    fresh.set_precision(B.FMM_PREC_BF16X3)
+    phi, acc = fresh.solve(rho)
+    torch.cuda.synchronize()
+    for k in (1, 3):
+        assert torch.equal(out[k][0], phi) and torch.equal(out[k][1], acc)
+    fresh.close()
+
+
+def test_tensor_core_scale_follows_the_field(B):
+    # the FP16 split is scaled by the level's largest mass sum: densities 1e12
+    # apart in size give the same solution up to rounding, and zeros give zeros
+    N, L, p = 32, 4, 4
+    rho = inputs.plummer(N, n_clumps=4, seed=3)
+    plan = B.Plan(N, L, p, precision=B.FMM_PREC_BF16X3)
+    ref = plan.solve(torch.from_numpy(rho).cuda())[0].double()
+    for s in (2.0 ** 40, 2.0 ** -40):
+        phi = plan.solve(torch.from_numpy((rho * np.float32(s)).astype(np.float32)).cuda())[0].double() / s
+        assert float((phi - ref).norm() / ref.norm()) < 1e-6
+    phi, acc = plan.solve(torch.full((N, N, N), 1.7, device="cuda"))
+    assert torch.all(phi == 0) and torch.all(acc == 0)
+    plan.close()
+
+
+def test_tensor_core_bounded_wait_expires_and_context_survives(B):
+    N, L, p = 32, 4, 4
+    rho = torch.from_numpy(inputs.lognormal(N, sigma=0.5, seed=2)).cuda()
+    plan = B.Plan(N, L, p, precision=B.FMM_PREC_BF16X3)
+    ref = [x.clone() for x in plan.solve(rho)]
+    B.fmm_plan_set_timeout_ms(plan.handle, 20)
+    B.fmm_plan_inject_fault(plan.handle, B.FMM_FAULT_TC_STALL)
+    plan.solve(rho)
+    assert B.lib().fmm_plan_check(plan.handle) == B.FMM_ERR_TIMEOUT
+    B.fmm_plan_inject_fault(plan.handle, B.FMM_FAULT_NONE)
+    B.fmm_plan_set_timeout_ms(plan.handle, 2000)
+    phi, acc = plan.solve(rho)
+    assert B.lib().fmm_plan_check(plan.handle) == B.FMM_OK
+    assert torch.equal(phi, ref[0]) and torch.equal(acc, ref[1])
+    plan.close()
 
 
 def test_levels_in_one_launch_equal_levels_one_by_one_bitwise(B):
@@ -80,7 +142,7 @@ def test_levels_in_one_launch_equal_levels_one_by_one_bitwise(B):
         assert np.array_equal(a[0], b[0]) and np.array_equal(a[1], b[1])
 
 
-@pytest.mark.parametrize("N,L,p", [(8, 2, 4), (8, 3, 3), (8, 3, 5), (16, 4, 2)])
+@pytest.mark.parametrize("N,L,p", [(8, 2, 5), (8, 3, 3), (8, 3, 2)])
 def test_spectral_table_gradient_matches_oracle_differences(B, N, L, p):
     # the loss is quadratic in the table values, so central differences of the
     # FP64 oracle are exact up to its rounding; entries at window edges
