@@ -867,17 +867,17 @@ int fmm_solve(fmm_plan* plan, const float* density, float* potential, float* acc
   FMM_CUDA_TRY(mark(FMM_TIME_MEAN, 1));
   const bool tc = P.prec != FMM_PREC_FP32 && P.tc_ready;
   auto on_tc = [&](int l) { return !fmm::fft_level(P, l) && tc && fmm::tc_level(P, l); };
-  // Untimed solves overlap independent stages: the near zone's source spectra
+  // Untimed solves overlap independent stages: the near zone's spectral sums
   // need only the density and its mean (second auxiliary stream, from the mean
-  // on); the M2L levels are independent of one another until the downward
+  // on), and fill what the small launches of the tree passes leave idle; the M2L levels are independent of one another until the downward
   // pass, so the double-float levels run on the first auxiliary stream beside
   // the FP32 and tensor-core levels on `s`.  Timed solves stay serial, so that
   // each stage's events bracket it alone.
-  const bool fwd_apart = !t && P.ns_K;
-  if (fwd_apart) {
+  const bool near_apart = !t && P.ns_K;
+  if (near_apart) {
     FMM_CUDA_TRY(cudaEventRecord(P.fev[0], s));
     FMM_CUDA_TRY(cudaStreamWaitEvent(P.aux[1], P.fev[0], 0));
-    FMM_CUDA_TRY(fmm::launch_near_spec_fwd(P, density, P.aux[1]));
+    FMM_CUDA_TRY(fmm::launch_near_spec_sums(P, density, P.aux[1]));
     FMM_CUDA_TRY(cudaEventRecord(P.fev[1], P.aux[1]));
   }
   FMM_CUDA_TRY(mark(FMM_TIME_P2M, 0));
@@ -938,8 +938,8 @@ int fmm_solve(fmm_plan* plan, const float* density, float* potential, float* acc
   for (int l = 2; l < P.L; ++l) FMM_CUDA_TRY(fmm::launch_l2l(P, l, s));
   FMM_CUDA_TRY(mark(FMM_TIME_L2L, 1));
   FMM_CUDA_TRY(mark(FMM_TIME_P2P, 0));
-  if (fwd_apart) FMM_CUDA_TRY(cudaStreamWaitEvent(s, P.fev[1], 0));
-  FMM_CUDA_TRY(fmm::launch_p2p(P, density, potential, accel, s, fwd_apart));
+  if (near_apart) FMM_CUDA_TRY(cudaStreamWaitEvent(s, P.fev[1], 0));
+  FMM_CUDA_TRY(fmm::launch_p2p(P, density, potential, accel, s, near_apart));
   FMM_CUDA_TRY(mark(FMM_TIME_P2P, 1));
   P.solved = 1;
   if (t) P.timed = 1;

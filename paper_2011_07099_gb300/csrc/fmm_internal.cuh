@@ -262,18 +262,18 @@ cudaError_t launch_m2l_spec_tc(Plan& P, int level, cudaStream_t s);
 cudaError_t launch_spec_fwd(Plan& P, const float* src, void* dst, size_t blocks, cudaStream_t s);
 cudaError_t launch_m2l_spec(Plan& P, bool df, int l0, int l1, cudaStream_t s);
 cudaError_t launch_l2l(Plan& P, int level, cudaStream_t s);       // F[level] -> F[level+1] (adds)
-// near_fwd_done: the near zone's source spectra were already taken (launch_near_spec_fwd).
+// near_sums_done: the near zone's spectral sums were already taken (launch_near_spec_sums).
 cudaError_t launch_p2p(Plan& P, const float* rho, float* phi, float* acc, cudaStream_t s,
-                       bool near_fwd_done = false);
+                       bool near_sums_done = false);
 // Near zone by spectral products (near_spec.cu): the leaf sizes it is built
 // for, its buffers (bytes), function attributes, the plan-time kernel spectra
-// (after every re-tabulation), the source spectra, and the sums with the
-// inverse transforms and L2P.
+// (after every re-tabulation), the spectral sums (which need the density only),
+// and the inverse transforms with L2P.
 bool near_spec_shape(const Plan& P);
 void near_spec_bytes(const Plan& P, size_t& nK, size_t& nM, size_t& nP);
 cudaError_t setup_near_spec(const Plan& P);
 cudaError_t launch_near_spec_kernels(Plan& P, cudaStream_t s);
-cudaError_t launch_near_spec_fwd(Plan& P, const float* rho, cudaStream_t s);
+cudaError_t launch_near_spec_sums(Plan& P, const float* rho, cudaStream_t s);
 cudaError_t launch_near_spec(Plan& P, float* phi, float* acc, cudaStream_t s);
 cudaError_t setup_m2l_tc(const Plan& P);
 cudaError_t setup_learn();

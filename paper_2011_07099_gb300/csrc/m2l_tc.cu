@@ -29,7 +29,7 @@
 //   warp 0      issues the MMAs (one thread);
 //   warp 1      one thread arms each stage's barrier with the stage's bytes
 //               and issues its bulk copies (A) and tensor loads (B);
-//   warps 2..5  drain TMEM (warps 2..9 in bf16x6): every G offsets
+//   warps 2..5  drain TMEM (warps 2..17 in bf16x6): every G offsets
 //               accumulate into a fresh TMEM partial, which the drain warps
 //               add into an FP32 total kept in TMEM while the issuer waits.  A single TMEM accumulator over
 //               all 189 p^3 terms drifts by ~1e-4 on the coherent, cancelling
@@ -47,7 +47,10 @@
 // lo hi); 128 targets per CTA (an 8 x 4 x 4 box of parents); every stage
 // accumulates into a fresh partial (two buffers, alternating), which the
 // drain adds into a double-float total by TwoSum; the level's FP64 local
-// field is written from hi + lo.  TMEM: partial 0 | partial 1 | hi | lo.
+// field is written from hi + lo.  TMEM: partial 0 | partial 1; the totals stay
+// in the drain threads' registers (one row and 32 columns each, 64 registers):
+// kept in TMEM, their loads and stores made a stage's drain 2390 clocks against
+// the 768 of its MMAs (512^3 order 8, level 5: 94 ms).
 // (A partial over a whole group of offsets cost 2.8e-5 at order 8: the
 // MMA's truncating accumulation, not the operand splits, dominated.)
 // Every wait is bounded; a timeout sets the plan's error word and later work
@@ -69,7 +72,6 @@ namespace {
 constexpr int kKC = 32;          // reduction indices per pipeline stage
 constexpr int kBX = 8, kBZ = 4;  // the targets' parents: an 8 x BY x 4 box
 constexpr int kHalo = 2;         // halo of the per-class source arrays (|(c - o - q)/2| <= 2)
-constexpr int kDrainMax = 256;   // drain threads: warps 2..5 (2..9 in bf16x6)
 constexpr uint32_t kTmemCols = 512;
 constexpr int kTileBytes = 128 * kKC * 2;     // one 128 x 32 BF16 tile of A
 
@@ -94,9 +96,9 @@ struct TcMode {
   static_assert(!WIDE || NT == 128, "the wide mode's TMEM layout needs 128 targets");
   static constexpr int BY = NT / (kBX * kBZ);
   static constexpr int TILEB = NT * kKC * 2;                           // one NT x 32 BF16 tile of B
-  // drain threads: bf16x6 adds a partial per stage into a double-float total,
-  // so two warps share each TMEM lane quadrant, one half of the columns each
-  static constexpr int DRAIN = WIDE ? 256 : 128;
+  // drain threads: bf16x6 adds a partial per stage into a double-float total
+  // in registers, so four warps share each TMEM lane quadrant, 32 columns each
+  static constexpr int DRAIN = WIDE ? 512 : 128;
   static constexpr int THREADS = 64 + DRAIN;
 };
 
@@ -121,7 +123,7 @@ __host__ __device__ constexpr int off_index(int ox, int oy, int oz) { return ((o
 constexpr int kOffSlots = 343;
 
 template <int P, int MODE, int NTT>
-__global__ void __launch_bounds__(64 + kDrainMax, 1)
+__global__ void __launch_bounds__(TcMode<MODE, NTT>::THREADS, 1)
 k_m2l_tc(const __grid_constant__ CUtensorMap tmapB, const uint8_t* __restrict__ Apre,
          const int8_t* __restrict__ offs, int n_off, int level, int group,
          float* __restrict__ F, double* __restrict__ F64, int* __restrict__ err, uint64_t kWaitNs, int stall) {
@@ -180,9 +182,8 @@ k_m2l_tc(const __grid_constant__ CUtensorMap tmapB, const uint8_t* __restrict__ 
   __syncthreads();
   tc::fence_after_sync();
   const uint32_t tmem = tmem_holder;
-  // TMEM columns: partial buffer(s) | total; bf16x6: partial 0 | partial 1 | total hi | total lo
+  // TMEM columns: partial buffer(s) | total (bf16x6: its total is in registers)
   const uint32_t t_tot = tmem + NB * kNT;
-  const uint32_t t_lo = tmem + (NB + 1) * kNT;
 
   if (warp == 0) {
     // ------------------------------------------------------------ MMA issuer
@@ -286,10 +287,41 @@ k_m2l_tc(const __grid_constant__ CUtensorMap tmapB, const uint8_t* __restrict__ 
     // ------------------------------------------------------------ drain warps
     const int q = warp & 3;                          // TMEM lane quadrant
     const uint32_t lanebase = (uint32_t)(q * 32) << 16;
-    // columns of this warp: all, or (bf16x6) one half
+    // columns of this warp: all, or (bf16x6) a quarter
     constexpr int CW = kNT * 128 / Md::DRAIN;
     const int cbeg = ((warp - 2) / 4) * CW, cend = cbeg + CW;
     bool ok = true;
+    // bf16x6: the double-float totals of this thread's row and columns, in registers
+    float th[Md::WIDE ? CW : 1], tl[Md::WIDE ? CW : 1];
+    if constexpr (Md::WIDE) {
+#pragma unroll
+      for (int k = 0; k < CW; ++k) th[k] = tl[k] = 0.f;
+#pragma unroll 1
+      for (int g = 0; g < n_units; ++g) {
+        const bool got = ok && tc::mbar_wait_bounded(&pfull[g % NB], (uint32_t)(g / NB) & 1u, kWaitNs);
+        ok = __all_sync(0xffffffffu, got);
+        if (!ok) break;
+        tc::fence_after_sync();
+        const uint32_t part = tmem + (uint32_t)((g % NB) * kNT) + lanebase + cbeg;
+#pragma unroll
+        for (int c0 = 0; c0 < CW; c0 += 16) {
+          uint32_t rp[16];
+          tc::tmem_ld16_nowait(part + c0, rp);
+          tc::tmem_wait_ld();
+          if (c0 + 16 == CW) {             // the partial is read: the issuer may refill it
+            tc::fence_before_sync();
+            tc::mbar_arrive(&pfree[g % NB]);
+          }
+          // (hi, lo) += partial by TwoSum, the error into lo
+#pragma unroll
+          for (int k = 0; k < 16; ++k) {
+            const float2 t = df_two_sum(th[c0 + k], __uint_as_float(rp[k]));
+            th[c0 + k] = t.x;
+            tl[c0 + k] = __fadd_rn(tl[c0 + k], t.y);
+          }
+        }
+      }
+    } else {
     for (int g = 0; g < n_units; ++g) {
       const bool got = ok && tc::mbar_wait_bounded(&pfull[g % NB], (uint32_t)(g / NB) & 1u, kWaitNs);
       ok = __all_sync(0xffffffffu, got);
@@ -297,57 +329,43 @@ k_m2l_tc(const __grid_constant__ CUtensorMap tmapB, const uint8_t* __restrict__ 
       tc::fence_after_sync();
       const uint32_t part = tmem + (uint32_t)((g % NB) * kNT);
       for (int c0 = cbeg; c0 < cend; c0 += 32) {
-        uint32_t rp[32], rt[32], rl[32];
+        uint32_t rp[32], rt[32];
         tc::tmem_ld32_nowait(part + lanebase + c0, rp);
         if (g > 0) tc::tmem_ld32_nowait(t_tot + lanebase + c0, rt);
-        if (Md::WIDE && g > 0) tc::tmem_ld32_nowait(t_lo + lanebase + c0, rl);
         tc::tmem_wait_ld();
-        if (Md::WIDE) {
-          // double-float total: (hi, lo) += partial by TwoSum, the error into lo
 #pragma unroll
-          for (int k = 0; k < 32; ++k) {
-            if (g == 0) {
-              rt[k] = rp[k];
-              rl[k] = 0u;
-            } else {
-              const float2 t = df_two_sum(__uint_as_float(rt[k]), __uint_as_float(rp[k]));
-              rt[k] = __float_as_uint(t.x);
-              rl[k] = __float_as_uint(__fadd_rn(__uint_as_float(rl[k]), t.y));
-            }
-          }
-          tc::tmem_st32(t_lo + lanebase + c0, rl);
-        } else {
-#pragma unroll
-          for (int k = 0; k < 32; ++k)
-            rt[k] = g == 0 ? rp[k] : __float_as_uint(__uint_as_float(rt[k]) + __uint_as_float(rp[k]));
-        }
+        for (int k = 0; k < 32; ++k)
+          rt[k] = g == 0 ? rp[k] : __float_as_uint(__uint_as_float(rt[k]) + __uint_as_float(rp[k]));
         tc::tmem_st32(t_tot + lanebase + c0, rt);
       }
       tc::tmem_wait_st();
       tc::fence_before_sync();
       tc::mbar_arrive(&pfree[g % NB]);
     }
+    }
     // final: F = total.  Target t of the tile is the child of parent
     // P0 + (t % 8, (t / 8) % 8, t / 64) at the CTA's child position.
     if (ok && n_off > 0 && __all_sync(0xffffffffu, atomicAdd(&s_err, 0) == 0)) {
       const int m = q * 32 + lane;
       const int gm = mt * 128 + m;
-      for (int c0 = cbeg; c0 < cend; c0 += 32) {
-        uint32_t rt[32], rl[32];
-        tc::tmem_ld32_nowait(t_tot + lanebase + c0, rt);
-        if (Md::WIDE) tc::tmem_ld32_nowait(t_lo + lanebase + c0, rl);
-        tc::tmem_wait_ld();
+      auto index_of = [&](int t) {
+        const uint32_t tx = 2u * (uint32_t)(P0x + t % kBX) + cx, ty = 2u * (uint32_t)(P0y + (t / kBX) % kBY) + cy,
+                       tz = 2u * (uint32_t)(P0z + t / (kBX * kBY)) + cz;
+        return (size_t)morton(tx, ty, tz) * 4 * P3 + gm;
+      };
+      if constexpr (Md::WIDE) {
         if (gm < 4 * P3) {
 #pragma unroll
-          for (int k = 0; k < 32; ++k) {
-            const int t = c0 + k;
-            const uint32_t tx = 2u * (uint32_t)(P0x + t % kBX) + cx, ty = 2u * (uint32_t)(P0y + (t / kBX) % kBY) + cy,
-                           tz = 2u * (uint32_t)(P0z + t / (kBX * kBY)) + cz;
-            const size_t o = (size_t)morton(tx, ty, tz) * 4 * P3 + gm;
-            if (Md::WIDE)
-              F64[o] = (double)__uint_as_float(rt[k]) + (double)__uint_as_float(rl[k]);
-            else
-              F[o] = __uint_as_float(rt[k]);
+          for (int k = 0; k < CW; ++k) F64[index_of(cbeg + k)] = df_to_double(make_float2(th[k], tl[k]));
+        }
+      } else {
+        for (int c0 = cbeg; c0 < cend; c0 += 32) {
+          uint32_t rt[32];
+          tc::tmem_ld32_nowait(t_tot + lanebase + c0, rt);
+          tc::tmem_wait_ld();
+          if (gm < 4 * P3) {
+#pragma unroll
+            for (int k = 0; k < 32; ++k) F[index_of(c0 + k)] = __uint_as_float(rt[k]);
           }
         }
       }

@@ -293,7 +293,7 @@ __global__ void __launch_bounds__(NearShape<S>::THR_INV) k_ns_inv(const void* __
   using store = Num<DFS>;
   using real = typename T::real;
   using cplx = typename T::cplx;
-  constexpr int NM = Shape<S>::NM, IB = kItems<S, DFA>, S3 = S * S * S, PS = Shape<S>::PS;
+  constexpr int NM = Shape<S>::NM, IB = kItems<S, DFA>, PS = Shape<S>::PS;
   extern __shared__ float4 sm4[];
   __shared__ float4 tw[NM];
   __shared__ float2 W[kMaxOrder * S];
@@ -545,15 +545,22 @@ cudaError_t fwd_as(Plan& P, const float* rho, cudaStream_t s) {
                                                                                             P.ns_tw, P.ns_M);
   return cudaGetLastError();
 }
-template <int S, bool DFA>
-cudaError_t rest_as(Plan& P, float* phi, float* acc, cudaStream_t s) {
+// The sums: like the source spectra they need the density only.
+template <int S>
+cudaError_t sums_as(Plan& P, cudaStream_t s) {
   constexpr bool DFS = NearShape<S>::DFS;
-  const unsigned leaves = 1u << (3 * P.L);
   const int nt = (1 << P.L) / kTile, ch = chunks_of(S, DFS), nkp = ch * Num<DFS>::LANES;
   const int tiles = nt * nt * nt, fit = (int)((long)tiles * ch / (4 * P.num_sms));
   const int per = fit < 1 ? 1 : (fit < kChunks ? fit : kChunks);
   k_ns_mac<DFS><<<dim3(tiles, (ch + per - 1) / per), DFS ? 512 : 256, kMacSmem, s>>>(
       static_cast<const float4*>(P.ns_K), P.ns_M, P.ns_P, P.L, nkp, P.iso, per);
+  return cudaGetLastError();
+}
+template <int S, bool DFA>
+cudaError_t rest_as(Plan& P, float* phi, float* acc, cudaStream_t s) {
+  constexpr bool DFS = NearShape<S>::DFS;
+  const unsigned leaves = 1u << (3 * P.L);
+  const int nkp = chunks_of(S, DFS) * Num<DFS>::LANES;
   k_ns_inv<S, DFA><<<leaves * 4 / kItems<S, DFA>, NearShape<S>::THR_INV, inv_smem<S, DFA>(P.p), s>>>(
       P.ns_P, nkp, (int)(inv_smem<S, DFA>(P.p) - sizeof(typename Num<DFA>::real) * kItems<S, DFA> * S * S * Shape<S>::PS), P.N,
       P.p, P.F[P.L], P.F64[P.L], P.w_p2m, P.ns_tw, phi, acc);
@@ -618,12 +625,15 @@ cudaError_t launch_near_spec_kernels(Plan& P, cudaStream_t s) {
   }
 }
 
-cudaError_t launch_near_spec_fwd(Plan& P, const float* rho, cudaStream_t s) {
+cudaError_t launch_near_spec_sums(Plan& P, const float* rho, cudaStream_t s) {
+  cudaError_t e;
   switch (P.S) {
-    case 4: return fwd_as<4, true>(P, rho, s);
-    case 6: return fwd_as<6, true>(P, rho, s);
-    case 8: return P.near_fft ? fwd_as<8, false>(P, rho, s) : fwd_as<8, true>(P, rho, s);
-    case 16: return fwd_as<16, true>(P, rho, s);
+    case 4: e = fwd_as<4, true>(P, rho, s); return e != cudaSuccess ? e : sums_as<4>(P, s);
+    case 6: e = fwd_as<6, true>(P, rho, s); return e != cudaSuccess ? e : sums_as<6>(P, s);
+    case 8:
+      e = P.near_fft ? fwd_as<8, false>(P, rho, s) : fwd_as<8, true>(P, rho, s);
+      return e != cudaSuccess ? e : sums_as<8>(P, s);
+    case 16: e = fwd_as<16, true>(P, rho, s); return e != cudaSuccess ? e : sums_as<16>(P, s);
     default: return cudaErrorInvalidValue;
   }
 }

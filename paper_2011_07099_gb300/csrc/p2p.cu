@@ -493,9 +493,9 @@ cudaError_t setup_p2p(const Plan& P) {
   }
 }
 
-cudaError_t launch_p2p(Plan& P, const float* rho, float* phi, float* acc, cudaStream_t s, bool near_fwd_done) {
+cudaError_t launch_p2p(Plan& P, const float* rho, float* phi, float* acc, cudaStream_t s, bool near_sums_done) {
   if (P.ns_K) {
-    const cudaError_t e = near_fwd_done ? cudaSuccess : launch_near_spec_fwd(P, rho, s);
+    const cudaError_t e = near_sums_done ? cudaSuccess : launch_near_spec_sums(P, rho, s);
     return e != cudaSuccess ? e : launch_near_spec(P, phi, acc, s);
   }
   switch (P.S) {
