@@ -4,98 +4,150 @@
 // transpose of the child's M2M matrix: Phi_child[q] = sum_r T_{r q} Phi_parent[r]
 // (Sec. 3 eq. fmm3).  With T the separable Lagrange matrix, that is the parent
 // field interpolated at the child's gridlet points.  The 8 children's points
-// form one uniform (2p)^3 mesh over the parent, so one CTA expands all four
-// fields of a parent onto that mesh and adds them to the children's fields
+// form one uniform (2p)^3 mesh over the parent, so a CTA expands a parent's
+// field onto that mesh, line by line, and adds it to the children's fields
 // (which already hold their own M2L result).
 #include "fmm_internal.cuh"
+#include "lines.cuh"
 
 namespace fmm {
 namespace {
 
-__global__ void k_l2l(const float* __restrict__ Fp, int p, const float2* __restrict__ w, float* __restrict__ Fc) {
-  extern __shared__ float2 sm2[];
-  const int K = 2 * p, p3 = p * p * p;
-  float2* W = sm2;                       // p*K  ([p][2p], used transposed)
-  float* in = reinterpret_cast<float*>(W + p * K);   // 4*p^3
-  float* t1 = in + 4 * p3;               // 4*p*p*K
-  float* t2 = t1 + 4 * p * p * K;        // 4*p*K*K
-  float* out = t2 + 4 * p * K * K;       // 4*K^3
+using lines::expand_line;
+using lines::expand_line_f;
+
+// Mesh index of child value i = (child c, q) of one field.
+template <int P>
+__device__ __forceinline__ int mesh_index(int i) {
+  constexpr int K = 2 * P, P3 = P * P * P;
+  const int c = i / P3, q = i % P3;
+  const int qx = q % P, qy = (q / P) % P, qz = q / (P * P);
+  return (((c >> 2) * P + qz) * K + ((c >> 1) & 1) * P + qy) * K + (c & 1) * P + qx;
+}
+
+// FP32: CTA per (parent, field).  A thread makes the 2p outputs of a line from
+// registers; the last pass goes through shared memory so that the children's
+// values are read and written along memory.  Measured at 256^3, p = 6 (level
+// 4 -> 5): 0.30 ms when each output was its own loop with two divisions.
+template <int P>
+__global__ void __launch_bounds__(128) k_l2l(const float* __restrict__ Fp, const float2* __restrict__ w,
+                                            float* __restrict__ Fc) {
+  constexpr int K = 2 * P, P3 = P * P * P;
+  __shared__ float2 W[P * K];            // [P][2P], used transposed
+  __shared__ float in[P3], t1[P * P * K], t2[P * K * K], out[K * K * K];
   const int tid = threadIdx.x, nthr = blockDim.x;
-  for (int i = tid; i < p * K; i += nthr) W[i] = w[i];
-  const float* src = Fp + (size_t)blockIdx.x * 4 * p3;
-  for (int i = tid; i < 4 * p3; i += nthr) in[i] = src[i];
+  const size_t parent = blockIdx.x >> 2;
+  const int f = blockIdx.x & 3;
+  for (int i = tid; i < P * K; i += nthr) W[i] = __ldg(w + i);
+  for (int i = tid; i < P3; i += nthr) in[i] = __ldg(Fp + (parent * 4 + f) * P3 + i);
   __syncthreads();
-  contract3(in, t1, t2, out, 4, p, K, W, K, true, tid, nthr);
-  float* dst = Fc + (size_t)blockIdx.x * 8 * 4 * p3;
-  for (int i = tid; i < 8 * 4 * p3; i += nthr) {
-    const int c = i / (4 * p3), rem = i % (4 * p3);
-    const int f = rem / p3, q = rem % p3;
-    const int qx = q % p, qy = (q / p) % p, qz = q / (p * p);
-    const int ux = (c & 1) * p + qx, uy = ((c >> 1) & 1) * p + qy, uz = (c >> 2) * p + qz;
-    dst[i] += out[((f * K + uz) * K + uy) * K + ux];
+  float a[K];
+  for (int l = tid; l < P * P; l += nthr) {                 // x: line (z, y)
+    expand_line_f<K>(in + l * P, 1, P, W, 1, K, a);
+#pragma unroll
+    for (int u = 0; u < K; ++u) t1[l * K + u] = a[u];
   }
+  __syncthreads();
+  for (int l = tid; l < P * K; l += nthr) {                 // y: line (z, ux)
+    const int ux = l % K, z = l / K;
+    expand_line_f<K>(t1 + z * P * K + ux, K, P, W, 1, K, a);
+#pragma unroll
+    for (int u = 0; u < K; ++u) t2[(z * K + u) * K + ux] = a[u];
+  }
+  __syncthreads();
+  for (int l = tid; l < K * K; l += nthr) {                 // z: line (uy, ux)
+    expand_line_f<K>(t2 + l, K * K, P, W, 1, K, a);
+#pragma unroll
+    for (int u = 0; u < K; ++u) out[u * K * K + l] = a[u];
+  }
+  __syncthreads();
+  for (int i = tid; i < 8 * P3; i += nthr)
+    Fc[((parent * 8 + i / P3) * 4 + f) * P3 + i % P3] += out[mesh_index<P>(i)];
 }
 
 // Variant for parents at the wide levels (the coarse levels 2 and 3; at
 // order >= 7 every level above the leaves): FP64 local fields, interpolated
-// in double-float (fmm_internal.cuh), one field
-// at a time (shared memory).  The child field is F64 (a coarse child, whose
-// FP32 copy is refreshed too) or the FP32 field of the first fine level, to
-// which the FP64 contribution is added before a single rounding.
-__global__ void k_l2l64(const double* __restrict__ Fp, int p, const float2* __restrict__ w,
-                        double* __restrict__ Fc64, float* __restrict__ Fc) {
+// in double-float (fmm_internal.cuh).  The child field is F64 (a coarse child,
+// whose FP32 copy is refreshed too) or the FP32 field of the first fine level,
+// to which the contribution is added in double-float before a single rounding
+// (in FP64, at 1/64 of the FP32 rate, these adds alone took 2.5 ms of the
+// 512^3 order-8 solve).
+template <int P>
+__global__ void __launch_bounds__(128) k_l2l64(const double* __restrict__ Fp, const float2* __restrict__ w,
+                                              double* __restrict__ Fc64, float* __restrict__ Fc) {
+  constexpr int K = 2 * P, P3 = P * P * P;
   extern __shared__ float2 smdf[];
-  const int K = 2 * p, p3 = p * p * p;
-  float2* W = smdf;                  // p*K  ([p][2p], used transposed)
-  float2* in = W + p * K;            // p^3
-  float2* t1 = in + p3;              // p*p*K
-  float2* t2 = t1 + p * p * K;       // p*K*K
-  float2* out = t2 + p * K * K;      // K^3
+  float2* W = smdf;                  // [P][2P], used transposed
+  float2* t1 = W + P * K;            // [z][y][ux]
+  float2* t2 = t1 + P * P * K;       // [z][uy][ux]
+  float2* out = t2 + P * K * K;      // [uz][uy][ux]
+  float2* in = out;                  // [z][y][x], consumed before `out` is written
   const int tid = threadIdx.x, nthr = blockDim.x;
-  for (int i = tid; i < p * K; i += nthr) W[i] = w[i];
-  for (int f = 0; f < 4; ++f) {
-    const double* src = Fp + ((size_t)blockIdx.x * 4 + f) * p3;
-    for (int i = tid; i < p3; i += nthr) in[i] = df_from_double(src[i]);
-    __syncthreads();
-    contract3_df(in, t1, t2, out, p, K, W, K, true, tid, nthr);
-    for (int i = tid; i < 8 * p3; i += nthr) {
-      const int c = i / p3, q = i % p3;
-      const int qx = q % p, qy = (q / p) % p, qz = q / (p * p);
-      const int ux = (c & 1) * p + qx, uy = ((c >> 1) & 1) * p + qy, uz = (c >> 2) * p + qz;
-      const size_t d = (((size_t)blockIdx.x * 8 + c) * 4 + f) * p3 + q;
-      const double v = df_to_double(out[(uz * K + uy) * K + ux]);
-      if (Fc64) {
-        const double t = Fc64[d] + v;
-        Fc64[d] = t;
-        Fc[d] = (float)t;
-      } else {
-        Fc[d] = (float)((double)Fc[d] + v);
-      }
-    }
-    __syncthreads();   // `in` and `out` are reused by the next field
+  const size_t parent = blockIdx.x >> 2;
+  const int f = blockIdx.x & 3;
+  for (int i = tid; i < P * K; i += nthr) W[i] = __ldg(w + i);
+  for (int i = tid; i < P3; i += nthr) in[i] = df_from_double(__ldg(Fp + (parent * 4 + f) * P3 + i));
+  __syncthreads();
+  float2 a[K];
+  for (int l = tid; l < P * P; l += nthr) {                 // x
+    expand_line<K>(in + l * P, 1, P, W, 1, K, a);
+#pragma unroll
+    for (int u = 0; u < K; ++u) t1[l * K + u] = a[u];
   }
+  __syncthreads();
+  for (int l = tid; l < P * K; l += nthr) {                 // y
+    const int ux = l % K, z = l / K;
+    expand_line<K>(t1 + z * P * K + ux, K, P, W, 1, K, a);
+#pragma unroll
+    for (int u = 0; u < K; ++u) t2[(z * K + u) * K + ux] = a[u];
+  }
+  __syncthreads();
+  for (int l = tid; l < K * K; l += nthr) {                 // z
+    expand_line<K>(t2 + l, K * K, P, W, 1, K, a);
+#pragma unroll
+    for (int u = 0; u < K; ++u) out[u * K * K + l] = a[u];
+  }
+  __syncthreads();
+  for (int i = tid; i < 8 * P3; i += nthr) {
+    const size_t d = ((parent * 8 + i / P3) * 4 + f) * P3 + i % P3;
+    const float2 v = out[mesh_index<P>(i)];
+    if (Fc64) {
+      const double t = Fc64[d] + df_to_double(v);
+      Fc64[d] = t;
+      Fc[d] = (float)t;
+    } else {
+      const float2 t = df_two_sum(Fc[d], v.x);
+      Fc[d] = __fadd_rn(t.x, __fadd_rn(t.y, v.y));
+    }
+  }
+}
+
+template <int P>
+size_t smem64() {
+  constexpr int K = 2 * P;
+  return sizeof(float2) * (P * K + P * P * K + P * K * K + K * K * K);
+}
+
+template <int P>
+cudaError_t setup_p() {
+  return cudaFuncSetAttribute(k_l2l64<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem64<P>());
+}
+
+template <int P>
+cudaError_t l2l_p(Plan& Pl, int level, cudaStream_t s) {
+  const unsigned blocks = 4u << (3 * level);
+  if (wide_level(Pl, level))
+    k_l2l64<P><<<blocks, 128, smem64<P>(), s>>>(Pl.F64[level], Pl.w_m2m,
+                                               wide_level(Pl, level + 1) ? Pl.F64[level + 1] : nullptr, Pl.F[level + 1]);
+  else
+    k_l2l<P><<<blocks, 128, 0, s>>>(Pl.F[level], Pl.w_m2m, Pl.F[level + 1]);
+  return cudaGetLastError();
 }
 
 }  // namespace
 
-cudaError_t setup_downward(const Plan& P) {
-  cudaError_t e = cudaFuncSetAttribute(k_l2l64, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(k_l2l, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-}
+cudaError_t setup_downward(const Plan& P) { FMM_BY_ORDER(P.p, setup_p, ()); }
 
-cudaError_t launch_l2l(Plan& P, int level, cudaStream_t s) {
-  const int p = P.p, K = 2 * p, p3 = p * p * p;
-  const size_t smem = sizeof(float2) * p * K + sizeof(float) * (4 * p3 + 4 * p * p * K + 4 * p * K * K + 4 * K * K * K);
-  const unsigned parents = 1u << (3 * level);
-  if (wide_level(P, level)) {
-    const size_t smem64 = sizeof(float2) * (p * K + p3 + p * p * K + p * K * K + K * K * K);
-    k_l2l64<<<parents, 256, smem64, s>>>(P.F64[level], p, P.w_m2m, wide_level(P, level + 1) ? P.F64[level + 1] : nullptr,
-                                         P.F[level + 1]);
-    return cudaGetLastError();
-  }
-  k_l2l<<<parents, 256, smem, s>>>(P.F[level], p, P.w_m2m, P.F[level + 1]);
-  return cudaGetLastError();
-}
+cudaError_t launch_l2l(Plan& P, int level, cudaStream_t s) { FMM_BY_ORDER(P.p, l2l_p, (P, level, s)); }
 
 }  // namespace fmm

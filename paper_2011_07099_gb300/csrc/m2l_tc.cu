@@ -304,17 +304,17 @@ k_m2l_tc(const __grid_constant__ CUtensorMap tmapB, const uint8_t* __restrict__ 
         tc::fence_after_sync();
         const uint32_t part = tmem + (uint32_t)((g % NB) * kNT) + lanebase + cbeg;
 #pragma unroll
-        for (int c0 = 0; c0 < CW; c0 += 16) {
-          uint32_t rp[16];
-          tc::tmem_ld16_nowait(part + c0, rp);
+        for (int c0 = 0; c0 < CW; c0 += 8) {
+          uint32_t rp[8];
+          tc::tmem_ld8_nowait(part + c0, rp);
           tc::tmem_wait_ld();
-          if (c0 + 16 == CW) {             // the partial is read: the issuer may refill it
+          if (c0 + 8 == CW) {             // the partial is read: the issuer may refill it
             tc::fence_before_sync();
             tc::mbar_arrive(&pfree[g % NB]);
           }
           // (hi, lo) += partial by TwoSum, the error into lo
 #pragma unroll
-          for (int k = 0; k < 16; ++k) {
+          for (int k = 0; k < 8; ++k) {
             const float2 t = df_two_sum(th[c0 + k], __uint_as_float(rp[k]));
             th[c0 + k] = t.x;
             tl[c0 + k] = __fadd_rn(tl[c0 + k], t.y);
