@@ -51,6 +51,7 @@ constexpr int kTile = 4;                  // target nodes per tile side
 constexpr int kHaloN = 8;                 // source nodes per halo side: T - 2 .. T + 5 of the tile's first node
 constexpr int kSlots = kHaloN * kHaloN * kHaloN;
 constexpr int kOff3 = 343;                // offsets o in [-3, 3]^3
+constexpr int kHalfN = 6;                 // source planes of half a tile
 
 // One level of a launch.
 struct SpecLevel {
@@ -374,18 +375,18 @@ __device__ __forceinline__ void mac_fp32(const float2* __restrict__ halo, const 
 // 4.1 of 5.8 cycles per instruction went to instruction fetch).
 // ROWS: the sums of one (oy, oz) row run as FP32 multiply-add chains (at most
 // 12 terms) and are then added to the double-float total, the low halves of
-// the operands gathered beside them: 3 instructions per product instead of
-// 12, for the level whose masses are FP32 (level 3 of orders < kWideOrder).
+// the kernel values gathered beside them: 2 instructions per product instead
+// of 12, for the level whose masses are FP32 (level 3 of orders < kWideOrder).
 template <int MODE, bool ROWS>
-__device__ __forceinline__ void mac_df(const float4* __restrict__ halo, const float4* __restrict__ K, int ty, int tz,
+__device__ __forceinline__ void mac_df(const float4* __restrict__ halo, const float4* __restrict__ K, int ty, int cz,
                                        float4 (&tot)[4]) {
-  const int cy = ty & 1, cz = tz & 1;
+  const int cy = ty & 1;
 #pragma unroll
   for (int j = 0; j < 4; ++j) tot[j] = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll 1
   for (int oz = -3; oz <= 3; ++oz) {
-    const int hz = tz + 2 - oz;
-    if (!allowed<MODE>(cz, oz) || hz < 0 || hz >= kHaloN) continue;
+    const int hz = cz + 2 - oz;                   // of the 6 source planes of this half tile
+    if (!allowed<MODE>(cz, oz) || hz < 0 || hz >= kHalfN) continue;
 #pragma unroll 1
     for (int oy = -3; oy <= 3; ++oy) {
       const int hy = ty + 2 - oy;
@@ -415,8 +416,8 @@ __device__ __forceinline__ void mac_df(const float4* __restrict__ halo, const fl
           if (ROWS) {
             part[j].x = fmaf(-q.z, m.z, fmaf(q.x, m.x, part[j].x));
             part[j].y = fmaf(q.z, m.x, fmaf(q.x, m.z, part[j].y));
-            tot[j].y = fmaf(-q.w, m.z, fmaf(-q.z, m.w, fmaf(q.y, m.x, fmaf(q.x, m.y, tot[j].y))));
-            tot[j].w = fmaf(q.w, m.x, fmaf(q.z, m.y, fmaf(q.y, m.z, fmaf(q.x, m.w, tot[j].w))));
+            tot[j].y = fmaf(-q.w, m.z, fmaf(q.y, m.x, tot[j].y));
+            tot[j].w = fmaf(q.w, m.x, fmaf(q.y, m.z, tot[j].w));
           } else {
             float2 re = make_float2(tot[j].x, tot[j].y), im = make_float2(tot[j].z, tot[j].w);
             Num<true>::mac(re, q.x, q.y, mr);
@@ -439,19 +440,20 @@ __device__ __forceinline__ void mac_df(const float4* __restrict__ halo, const fl
 }
 
 constexpr int kMacThr = 256;        // FP32: 16 frequencies x 16 rows
-constexpr int kMacThrDf = 512;      // double-float: 8 frequencies x 16 rows x 4 fields
+constexpr int kMacThrDf = 256;      // double-float: 8 frequencies x 8 rows x 4 fields
 
-// The tile's source spectra, 128 bytes per slot, into shared memory.
-__device__ __forceinline__ void load_halo(const SpecLevel& V, int iso, int tile, int chunk, float4* sm, int tid,
-                                          int nthr) {
+// The tile's source spectra (z planes z0 .. z0 + nz - 1 of the halo), 128 bytes
+// per slot, into shared memory.
+__device__ __forceinline__ void load_halo(const SpecLevel& V, int iso, int tile, int z0, int nz, int chunk, float4* sm,
+                                          int tid, int nthr) {
   const int n = 1 << V.level, nt = n / kTile;
   const int TX = tile % nt, TY = (tile / nt) % nt, TZ = tile / (nt * nt);
   const size_t nodes = (size_t)1 << (3 * V.level);
   const char* src = reinterpret_cast<const char*>(V.Mh) + (size_t)chunk * (nodes + 1) * 128;
-  for (int i = tid; i < kSlots * 8; i += nthr) {
+  for (int i = tid; i < nz * kHaloN * kHaloN * 8; i += nthr) {
     const int slot = i >> 3, part = i & 7;
     const int ux = TX * kTile - 2 + (slot & 7), uy = TY * kTile - 2 + ((slot >> 3) & 7),
-              uz = TZ * kTile - 2 + (slot >> 6);
+              uz = TZ * kTile - 2 + z0 + (slot >> 6);
     const bool inbox = (unsigned)ux < (unsigned)n && (unsigned)uy < (unsigned)n && (unsigned)uz < (unsigned)n;
     const size_t node = inbox || !iso ? morton(ux & (n - 1), uy & (n - 1), uz & (n - 1)) : nodes;
     tc::cp_async16_full(tc::smem_u32(sm + i), src + node * 128 + part * 16);
@@ -468,7 +470,7 @@ __global__ void __launch_bounds__(kMacThr, 2) k_spec_mac(const __grid_constant__
   const int nt = (1 << V.level) / kTile, tiles = nt * nt * nt;
   const int local = blockIdx.x - V.first, tile = local % tiles, chunk = local / tiles;
   const int TX = tile % nt, TY = (tile / nt) % nt, TZ = tile / (nt * nt);
-  load_halo(V, A.iso, tile, chunk, sm4, tid, kMacThr);
+  load_halo(V, A.iso, tile, 0, kHaloN, chunk, sm4, tid, kMacThr);
   // lane: frequency and the y half of the row; warp: child type (cy, cz) and the z half
   const int lane = tid & 31, warp = tid >> 5, fr = lane & 15;
   const int ty = (warp & 1) + 2 * (lane >> 4), tz = ((warp >> 1) & 1) + 2 * (warp >> 2);
@@ -484,28 +486,32 @@ __global__ void __launch_bounds__(kMacThr, 2) k_spec_mac(const __grid_constant__
   }
 }
 
-__global__ void __launch_bounds__(kMacThrDf, 2) k_spec_mac_df(const __grid_constant__ SpecArgs A) {
+// CTA: half a tile (2 target planes, 6 source planes), so that the few tiles
+// of levels 2 and 3 make CTAs enough to load the SMs evenly (32^3, p = 4: 225
+// whole tiles x chunks left one or two CTAs per SM).
+__global__ void __launch_bounds__(kMacThrDf, 4) k_spec_mac_df(const __grid_constant__ SpecArgs A) {
   extern __shared__ float4 sm4[];
   const int tid = threadIdx.x;
   const SpecLevel& V = level_of(A, blockIdx.x);
   const int nt = (1 << V.level) / kTile, tiles = nt * nt * nt;
-  const int local = blockIdx.x - V.first, tile = local % tiles, chunk = local / tiles;
+  const int local = blockIdx.x - V.first, zh = local & 1, tile = (local >> 1) % tiles, chunk = (local >> 1) / tiles;
   const int TX = tile % nt, TY = (tile / nt) % nt, TZ = tile / (nt * nt);
-  load_halo(V, A.iso, tile, chunk, sm4, tid, kMacThrDf);
-  // lane: frequency and the (y, z) half of the row; warp: child type (cy, cz) and field
-  const int lane = tid & 31, warp = tid >> 5, fr = lane & 7, sub = lane >> 3;
-  const int ty = (warp & 1) + 2 * (sub & 1), tz = ((warp >> 1) & 1) + 2 * (sub >> 1), f = warp >> 2;
+  load_halo(V, A.iso, tile, 2 * zh, kHalfN, chunk, sm4, tid, kMacThrDf);
+  // lane: frequency, y half of the row, low bit of the field; warp: child type (cy, cz), high bit of the field
+  const int lane = tid & 31, warp = tid >> 5, fr = lane & 7;
+  const int ty = (warp & 1) + 2 * ((lane >> 3) & 1), cz = (warp >> 1) & 1, f = 2 * (warp >> 2) + (lane >> 4);
+  const int tz = 2 * zh + cz;
   const float4* K = reinterpret_cast<const float4*>(V.K) + (size_t)chunk * kOff3 * 32 + f * 8 + fr;
   float4 tot[4];
   if (V.level > 2) {
     if (A.rows)
-      mac_df<0, true>(sm4 + fr, K, ty, tz, tot);
+      mac_df<0, true>(sm4 + fr, K, ty, cz, tot);
     else
-      mac_df<0, false>(sm4 + fr, K, ty, tz, tot);
+      mac_df<0, false>(sm4 + fr, K, ty, cz, tot);
   } else if (!A.iso) {
-    mac_df<1, false>(sm4 + fr, K, ty, tz, tot);
+    mac_df<1, false>(sm4 + fr, K, ty, cz, tot);
   } else {
-    mac_df<2, false>(sm4 + fr, K, ty, tz, tot);
+    mac_df<2, false>(sm4 + fr, K, ty, cz, tot);
   }
   float4* Ph = reinterpret_cast<float4*>(V.Ph);
 #pragma unroll
@@ -557,9 +563,9 @@ cudaError_t launch_as(Plan& Pl, int l0, int l1, cudaStream_t s) {
   int b = fill(Pl, DFS, l0, l1, A, [](int l) { return (1 << (3 * l)) / Shape<P>::NB; });
   if (!b) return cudaSuccess;
   k_spec_fwd<P, DFS, DFA><<<b, 128, fwd_smem<P, DFA>(), s>>>(A);
-  b = fill(Pl, DFS, l0, l1, A, [](int l) { return (1 << (3 * (l - 2))) * chunks_of(P, DFS); });
+  b = fill(Pl, DFS, l0, l1, A, [](int l) { return (1 << (3 * (l - 2))) * chunks_of(P, DFS) * (DFS ? 2 : 1); });
   if (DFS)
-    k_spec_mac_df<<<b, kMacThrDf, kMacSmem, s>>>(A);
+    k_spec_mac_df<<<b, kMacThrDf, kMacSmem * kHalfN / kHaloN, s>>>(A);
   else
     k_spec_mac<<<b, kMacThr, kMacSmem, s>>>(A);
   b = fill(Pl, DFS, l0, l1, A, [](int l) { return (1 << (3 * l)) / Shape<P>::NB; });
