@@ -16,7 +16,7 @@
 //
 // Kernels (each launch takes all levels of one arithmetic together, so a
 // small tree costs three launches and not three per level):
-//   k_spec_kernel  plan time: K^_o of every offset and field, FP64, rounded once
+//   k_spec_kernel  plan time: K^_o of every offset and field
 //   k_spec_fwd     per node: M^ of its gridlet, separable line DFTs
 //   k_spec_mac     per (tile of 4^3 target nodes, chunk of frequencies): the
 //                  189-offset sums of the 4 fields
@@ -86,80 +86,89 @@ __device__ __forceinline__ const SpecLevel& level_of(const SpecArgs& A, int bloc
 // K^[chunk][o][...]: FP32 as [2 field pairs][16] float4 (re, im of two
 // fields), double-float as [4 fields][8] float4 (re hi, re lo, im hi, im lo).
 // CTA (o, field): window values from the level table (hi + lo), three
-// separable passes in FP64; the inverse transform's 1/NM^3 is folded in.
+// separable passes in double-float (the spectra are stored as FP32 or as
+// double-float pairs; in FP64, at 1/64 of the FP32 rate, a level of order 6
+// took 0.37 ms); the inverse transform's 1/NM^3 is folded in.
 template <int P, bool DF>
-__global__ void __launch_bounds__(256) k_spec_kernel(const float4* __restrict__ tab, const float4* __restrict__ tab_lo,
-                                                     float* __restrict__ K) {
+__global__ void __launch_bounds__(128) k_spec_kernel(const float4* __restrict__ tab, const float4* __restrict__ tab_lo,
+                                                     const float4* __restrict__ twg, float* __restrict__ K) {
+  using T = Num<true>;
   constexpr int NM = Shape<P>::NM, HW = 4 * P - 1, E = 8 * P - 1, LANES = Num<DF>::LANES;
   const int o = blockIdx.x, f = blockIdx.y, tid = threadIdx.x;
   const int ox = o % 7 - 3, oy = (o / 7) % 7 - 3, oz = o / 49 - 3;
   if (abs(ox) <= 1 && abs(oy) <= 1 && abs(oz) <= 1) return;    // near nodes: never used
-  __shared__ double2 w[NM];
-  extern __shared__ double2 sd[];
-  double2* T1 = sd;                       // [z][y][kx]
-  double2* T2 = sd + NM * NM * P;         // [z][ky][kx]
-  if (tid < NM) {
-    double s, c;
-    sincospi(2.0 * tid / NM, &s, &c);
-    w[tid] = make_double2(c, -s);
-  }
+  __shared__ float4 tw[NM];
+  extern __shared__ float4 sm4[];
+  float4* T1 = sm4;                       // [z][y][kx]
+  float4* T2 = sm4 + NM * NM * P;         // [z][ky][kx]
+  if (tid < NM) tw[tid] = __ldg(twg + tid);
+  const Twiddle<true, P> wt(twg, tw);
   __syncthreads();
   auto lag = [](int v) { return v < P ? v : v - NM; };
-  for (int i = tid; i < NM * NM * P; i += blockDim.x) {
-    const int kx = i % P, vy = (i / P) % NM, vz = i / (P * NM);
+  for (int l = tid; l < NM * NM; l += blockDim.x) {            // x: line (vz, vy)
+    const int vy = l % NM, vz = l / NM;
     const size_t row = ((size_t)(oz * P + lag(vz) + HW) * E + (oy * P + lag(vy) + HW)) * E + ox * P + HW;
-    double re = 0.0, im = 0.0;
-    for (int vx = 0; vx < NM; ++vx) {
-      const float* a = reinterpret_cast<const float*>(tab + row + lag(vx));
-      const float* b = reinterpret_cast<const float*>(tab_lo + row + lag(vx));
-      const double v = (double)__ldg(a + f) + (double)__ldg(b + f);
-      const double2 t = w[(kx * vx) % NM];
-      re += v * t.x;
-      im += v * t.y;
-    }
-    T1[i] = make_double2(re, im);
+    float2 x[NM];
+#pragma unroll
+    for (int vx = 0; vx < NM; ++vx)
+      x[vx] = make_float2(__ldg(reinterpret_cast<const float*>(tab + row + lag(vx)) + f),
+                          __ldg(reinterpret_cast<const float*>(tab_lo + row + lag(vx)) + f));
+    spec::forward_real_full_line<true, P>(x, wt,
+                                          [&](int k, float2 re, float2 im) { T1[l * P + k] = T::pack(re, im); });
   }
   __syncthreads();
-  for (int i = tid; i < NM * NM * P; i += blockDim.x) {
-    const int kx = i % P, ky = (i / P) % NM, vz = i / (P * NM);
-    double re = 0.0, im = 0.0;
-    for (int vy = 0; vy < NM; ++vy) {
-      const double2 a = T1[(vz * NM + vy) * P + kx], t = w[(ky * vy) % NM];
-      re += a.x * t.x - a.y * t.y;
-      im += a.x * t.y + a.y * t.x;
+  for (int l = tid; l < NM * P; l += blockDim.x) {             // y: line (vz, kx)
+    const int kx = l % P, vz = l / P;
+    float2 xr[NM], xi[NM];
+#pragma unroll
+    for (int s = 0; s < NM; ++s) {
+      const float4 c = T1[(vz * NM + s) * P + kx];
+      xr[s] = T::re(c);
+      xi[s] = T::im(c);
     }
-    T2[i] = make_double2(re, im);
+    // the forward transform at k is the inverse one at NM - k
+    inverse_line<true, P, true>(xr, xi, wt, [&](int z, float2 re, float2 im) {
+      T2[(vz * NM + (z ? NM - z : 0)) * P + kx] = T::pack(re, im);
+    });
   }
   __syncthreads();
-  const double scale = 1.0 / ((double)NM * NM * NM);
-  for (int k = tid; k < NM * NM * P; k += blockDim.x) {
-    const int kx = k % P, ky = (k / P) % NM, kz = k / (P * NM);
-    double re = 0.0, im = 0.0;
-    for (int vz = 0; vz < NM; ++vz) {
-      const double2 a = T2[(vz * NM + ky) * P + kx], t = w[(kz * vz) % NM];
-      re += a.x * t.x - a.y * t.y;
-      im += a.x * t.y + a.y * t.x;
+  const float2 scale = df_from_double(1.0 / ((double)NM * NM * NM));
+  for (int q = tid; q < NM * P; q += blockDim.x) {             // z: line (ky, kx)
+    float2 xr[NM], xi[NM];
+#pragma unroll
+    for (int s = 0; s < NM; ++s) {
+      const float4 c = T2[s * NM * P + q];
+      xr[s] = T::re(c);
+      xi[s] = T::im(c);
     }
-    re *= scale;
-    im *= scale;
-    const size_t base = ((size_t)(k / LANES) * kOff3 + o) * (DF ? 16 : 8) * LANES;   // floats
-    const int l = k % LANES;
-    if (DF) {
-      const float2 a = df_from_double(re), b = df_from_double(im);
-      reinterpret_cast<float4*>(K + base)[f * LANES + l] = make_float4(a.x, a.y, b.x, b.y);
-    } else {
-      reinterpret_cast<float2*>(K + base)[((f / 2) * LANES + l) * 2 + (f & 1)] = make_float2((float)re, (float)im);
-    }
+    inverse_line<true, P, true>(xr, xi, wt, [&](int z, float2 re, float2 im) {
+      const int k = (z ? NM - z : 0) * NM * P + q;
+      float2 a = T::zero(), b = T::zero();
+      T::mac(a, scale.x, scale.y, re);
+      T::mac(b, scale.x, scale.y, im);
+      a = T::done(a);
+      b = T::done(b);
+      const size_t base = ((size_t)(k / LANES) * kOff3 + o) * (DF ? 16 : 8) * LANES;   // floats
+      const int l = k % LANES;
+      if (DF)
+        reinterpret_cast<float4*>(K + base)[f * LANES + l] = T::pack(a, b);
+      else
+        reinterpret_cast<float2*>(K + base)[((f / 2) * LANES + l) * 2 + (f & 1)] = make_float2(a.x, b.x);
+    });
   }
 }
 
 // ------------------------------------------------------------- transforms
+// Nodes per CTA of the inverse transforms (4 fields each).
+template <int P>
+constexpr int kInvNodes = P >= 5 ? 1 : (P == 4 ? 2 : (P == 3 ? 4 : 8));
+
 // DFS: double-float storage (the wide levels); DFA: double-float arithmetic
 // (always with DFS; with FP32 storage in the plain form, whose transforms then
 // round once, on store; the mixed forms transform in FP32).
 // Source spectra.  CTA: NB nodes; passes x, y, z through shared memory.
 template <int P, bool DFS, bool DFA>
-__global__ void __launch_bounds__(128) k_spec_fwd(const __grid_constant__ SpecArgs A) {
+__global__ void __launch_bounds__(Shape<P>::THR) k_spec_fwd(const __grid_constant__ SpecArgs A) {
   using T = Num<DFA>;
   using store = Num<DFS>;
   using real = typename T::real;
@@ -223,12 +232,12 @@ __global__ void __launch_bounds__(128) k_spec_fwd(const __grid_constant__ SpecAr
 
 // Local fields from the target spectra.  CTA: NB nodes, 4 fields each.
 template <int P, bool DFS, bool DFA>
-__global__ void __launch_bounds__(256) k_spec_inv(const __grid_constant__ SpecArgs A) {
+__global__ void __launch_bounds__(Shape<P>::threads(4 * kInvNodes<P>)) k_spec_inv(const __grid_constant__ SpecArgs A) {
   using T = Num<DFA>;
   using store = Num<DFS>;
   using real = typename T::real;
   using cplx = typename T::cplx;
-  constexpr int NM = Shape<P>::NM, NB = Shape<P>::NB, P3 = P * P * P, PS = Shape<P>::PS;
+  constexpr int NM = Shape<P>::NM, NB = kInvNodes<P>, P3 = P * P * P, PS = Shape<P>::PS;
   extern __shared__ float4 sm4[];
   __shared__ float4 tw[NM];
   cplx* t1 = reinterpret_cast<cplx*>(sm4);                 // [NB][4][z][ky][kx]
@@ -531,7 +540,7 @@ size_t fwd_smem() {
 }
 template <int P, bool DFA>
 size_t inv_smem() {
-  constexpr int NB = Shape<P>::NB, NM = Shape<P>::NM;
+  constexpr int NB = kInvNodes<P>, NM = Shape<P>::NM;
   return sizeof(typename Num<DFA>::cplx) * NB * 4 * (P * NM * P + P * P * Shape<P>::PS);
 }
 constexpr size_t kMacSmem = (size_t)kSlots * 128;
@@ -562,14 +571,14 @@ cudaError_t launch_as(Plan& Pl, int l0, int l1, cudaStream_t s) {
   SpecArgs A;
   int b = fill(Pl, DFS, l0, l1, A, [](int l) { return (1 << (3 * l)) / Shape<P>::NB; });
   if (!b) return cudaSuccess;
-  k_spec_fwd<P, DFS, DFA><<<b, 128, fwd_smem<P, DFA>(), s>>>(A);
+  k_spec_fwd<P, DFS, DFA><<<b, Shape<P>::THR, fwd_smem<P, DFA>(), s>>>(A);
   b = fill(Pl, DFS, l0, l1, A, [](int l) { return (1 << (3 * (l - 2))) * chunks_of(P, DFS) * (DFS ? 2 : 1); });
   if (DFS)
     k_spec_mac_df<<<b, kMacThrDf, kMacSmem * kHalfN / kHaloN, s>>>(A);
   else
     k_spec_mac<<<b, kMacThr, kMacSmem, s>>>(A);
-  b = fill(Pl, DFS, l0, l1, A, [](int l) { return (1 << (3 * l)) / Shape<P>::NB; });
-  k_spec_inv<P, DFS, DFA><<<b, 256, inv_smem<P, DFA>(), s>>>(A);
+  b = fill(Pl, DFS, l0, l1, A, [](int l) { return (1 << (3 * l)) / kInvNodes<P>; });
+  k_spec_inv<P, DFS, DFA><<<b, Shape<P>::threads(4 * kInvNodes<P>), inv_smem<P, DFA>(), s>>>(A);
   return cudaGetLastError();
 }
 
@@ -585,7 +594,7 @@ cudaError_t fwd_p(Plan& Pl, const float* src, void* dst, size_t blocks, cudaStre
   fill(Pl, false, 1, 0, A, [](int) { return 0; });
   A.n = 1;
   A.lev[0] = {src, nullptr, dst, nullptr, nullptr, nullptr, nullptr, 0, 0, blocks};
-  k_spec_fwd<P, false, false><<<(unsigned)(blocks / Shape<P>::NB), 128, fwd_smem<P, false>(), s>>>(A);
+  k_spec_fwd<P, false, false><<<(unsigned)(blocks / Shape<P>::NB), Shape<P>::THR, fwd_smem<P, false>(), s>>>(A);
   return cudaGetLastError();
 }
 
@@ -595,9 +604,9 @@ cudaError_t kernels_p(Plan& Pl, int l, cudaStream_t s) {
   const size_t smem = 2 * sizeof(double2) * NM * NM * P;
   const dim3 grid(kOff3, 4);
   if (wide_level(Pl, l))
-    k_spec_kernel<P, true><<<grid, 256, smem, s>>>(Pl.tab[l], Pl.tab_lo[l], static_cast<float*>(Pl.spec_K[l]));
+    k_spec_kernel<P, true><<<grid, 128, smem, s>>>(Pl.tab[l], Pl.tab_lo[l], Pl.spec_tw, static_cast<float*>(Pl.spec_K[l]));
   else
-    k_spec_kernel<P, false><<<grid, 256, smem, s>>>(Pl.tab[l], Pl.tab_lo[l], static_cast<float*>(Pl.spec_K[l]));
+    k_spec_kernel<P, false><<<grid, 128, smem, s>>>(Pl.tab[l], Pl.tab_lo[l], Pl.spec_tw, static_cast<float*>(Pl.spec_K[l]));
   return cudaGetLastError();
 }
 

@@ -15,13 +15,15 @@ namespace spec {
 
 template <int P>
 struct Shape {
+  static constexpr int threads(int blocks) { return (blocks * P * P + 31) / 32 * 32; }
   static constexpr int NM = 2 * P - 1;
-  static constexpr int LINES = NM * P;
   // row stride of the shared arrays whose x lines a thread walks: odd, so that
   // a warp's rows start on different banks (P = 16 has no room for it)
   static constexpr int PS = P >= 16 ? P : (P | 1);
-  // blocks per CTA of the transforms: about 128 lines of the widest pass
-  static constexpr int NB = LINES <= 16 ? 8 : (LINES <= 32 ? 4 : (LINES <= 72 ? 2 : 1));
+  // blocks per CTA of the forward transforms, and the threads: one round of the
+  // x and y lines (P^2 per block), just under two of the z lines (NM P)
+  static constexpr int NB = P >= 16 ? 1 : (P >= 7 ? 2 : (P >= 5 ? 4 : (P >= 3 ? 8 : 16)));
+  static constexpr int THR = threads(NB);
 };
 
 // ------------------------------------------------------------- arithmetic
@@ -253,6 +255,36 @@ __device__ __forceinline__ void inverse_real_line(const typename Num<DF>::real (
       T::mac(a, -w.z, -w.w, xi[s]);
     }
     emit(x, T::add(T::twice(T::done(a)), xr[0]));
+  }
+}
+
+// X_k = sum_{s < NM} x_s e^{-2 pi i k s / NM} of NM real values, k < P; xr is used up.
+template <bool DF, int P, typename Emit>
+__device__ __forceinline__ void forward_real_full_line(typename Num<DF>::real (&xr)[2 * P - 1], const Twiddle<DF, P>& tw,
+                                                       Emit emit) {
+  using T = Num<DF>;
+  using real = typename T::real;
+  constexpr int NM = 2 * P - 1;
+#pragma unroll
+  for (int s = 1; s < P; ++s) {
+    const real a = xr[s], b = xr[NM - s];
+    xr[s] = T::add(a, b);
+    xr[NM - s] = T::add(a, T::neg(b));
+  }
+#pragma unroll 1
+  for (int k = 0; k < P; ++k) {
+    real c = T::zero(), d = T::zero();
+    T::mac(c, 1.f, 0.f, xr[0]);
+    int j = 0;
+#pragma unroll
+    for (int s = 1; s < P; ++s) {
+      j += k;
+      j -= j >= NM ? NM : 0;
+      const float4 w = tw.at(j);
+      T::mac(c, w.x, w.y, xr[s]);
+      T::mac(d, -w.z, -w.w, xr[NM - s]);
+    }
+    emit(k, T::done(c), T::done(d));
   }
 }
 
