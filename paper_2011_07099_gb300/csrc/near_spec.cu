@@ -23,9 +23,8 @@
 //                the L2P far field (eq. fmm3 at the leaves), written once
 // Arithmetic: FP32 spectra and sums; the transforms in FP32 (FMM_NEAR_FFT) or,
 // where the plan asks for the direct sum's accuracy (FMM_NEAR_DIRECT), in
-// double-float with one rounding on store; with 16-cell leaves, whose edge
-// cells amplify every rounding (fmm_internal.cuh, kWideLeaf), double-float
-// throughout.
+// double-float with one rounding on store.  With 16-cell leaves the L2P reads
+// the FP64 local field (fmm_internal.cuh, kWideLeaf) in double-float.
 // Measured (direct kernels of p2p.cu before -> here): 128^3 isolated with
 // 16-cell leaves 177 -> 2.9 ms; 256^3, S = 8 30.6 -> 6.0 ms at direct accuracy
 // (sums 0.91, inverse with L2P 4.3); 96^3, S = 6 1.04 -> 0.31 ms; 128^3, S = 4
@@ -57,12 +56,9 @@ constexpr int kTile = 4;                    // target leaves per tile side
 constexpr int kHaloN = kTile + 2;
 constexpr int kSlots = kHaloN * kHaloN * kHaloN;
 
+// Leaves whose L2P reads the FP64 local field.
 template <int S>
-struct NearShape {
-  static constexpr bool DFS = S >= kWideLeaf;                 // storage of the spectra
-  static constexpr int THR_FWD = S >= 16 ? 512 : 128;
-  static constexpr int THR_INV = S >= 16 ? 512 : 256;
-};
+constexpr bool kWideField = S >= kWideLeaf;
 
 // (leaf, field) items per inverse CTA: one wave of lines over its threads, and
 // two CTAs' shared memory within an SM.
@@ -124,11 +120,11 @@ __global__ void __launch_bounds__(128) k_ns_planes(const float4* __restrict__ ta
   }
 }
 
-// The z transform, 1/NM^3, and the store K^[chunk][o][...] (layouts of
-// m2l_spec.cu: FP32 [2 field pairs][16] float4, double-float [4][8] float4).
-template <int S, bool DF>
+// The z transform, 1/NM^3, and the store K^[chunk][o][2 field pairs][16] float4
+// (re, im of two fields).
+template <int S>
 __global__ void __launch_bounds__(128) k_ns_lines(const double2* __restrict__ in, float* __restrict__ K) {
-  constexpr int NM = Shape<S>::NM, LANES = Num<DF>::LANES;
+  constexpr int NM = Shape<S>::NM, LANES = Num<false>::LANES;
   __shared__ double2 w[NM];
   const int o = blockIdx.y / 4, f = blockIdx.y % 4;
   if (threadIdx.x < NM) {
@@ -151,24 +147,18 @@ __global__ void __launch_bounds__(128) k_ns_lines(const double2* __restrict__ in
   im *= scale;
   const size_t base = ((size_t)(k / LANES) * kNO + o) * 128;   // floats
   const int l = k % LANES;
-  if (DF) {
-    const float2 a = df_from_double(re), b = df_from_double(im);
-    reinterpret_cast<float4*>(K + base)[f * LANES + l] = make_float4(a.x, a.y, b.x, b.y);
-  } else {
-    reinterpret_cast<float2*>(K + base)[((f / 2) * LANES + l) * 2 + (f & 1)] = make_float2((float)re, (float)im);
-  }
+  reinterpret_cast<float2*>(K + base)[((f / 2) * LANES + l) * 2 + (f & 1)] = make_float2((float)re, (float)im);
 }
 
 // ------------------------------------------------------------- transforms
 // Spectra of the leaves' masses m = (rho - mean) / N^3, NB leaves per CTA.
 template <int S, bool DFA>
-__global__ void __launch_bounds__(NearShape<S>::THR_FWD) k_ns_fwd(const float* __restrict__ rho,
+__global__ void __launch_bounds__(Shape<S>::THR) k_ns_fwd(const float* __restrict__ rho,
                                                                   const double* __restrict__ mean, int N, int L,
                                                                   const float4* __restrict__ twg,
                                                                   void* __restrict__ Mout) {
-  constexpr bool DFS = NearShape<S>::DFS;
   using T = Num<DFA>;
-  using store = Num<DFS>;
+  using store = Num<false>;
   using real = typename T::real;
   using cplx = typename T::cplx;
   constexpr int NM = Shape<S>::NM, NB = Shape<S>::NB, S3 = S * S * S, PS = Shape<S>::PS,
@@ -234,7 +224,7 @@ __global__ void __launch_bounds__(NearShape<S>::THR_FWD) k_ns_fwd(const float* _
     forward_line<DFA, S, false>(xr, xi, wt, [&](int kz, real re, real im) {
       const int k = kz * NM * S + q;
       Mh[((size_t)(k / LANES) * (leaves + 1) + leaf0 + nb) * LANES + k % LANES] =
-          store::pack(narrow<DFS, DFA>(re), narrow<DFS, DFA>(im));
+          store::pack(narrow<false, DFA>(re), narrow<false, DFA>(im));
     });
   }
 }
@@ -282,15 +272,14 @@ __device__ __forceinline__ void l2p_pass(const typename Num<DFA>::real* in, type
 
 // Outputs.  CTA: IB (leaf, field) items.
 template <int S, bool DFA>
-__global__ void __launch_bounds__(NearShape<S>::THR_INV) k_ns_inv(const void* __restrict__ Pin, int nkp, int far_at, int N, int p,
+__global__ void __launch_bounds__(Shape<S>::threads(kItems<S, DFA>)) k_ns_inv(const void* __restrict__ Pin, int nkp, int far_at, int N, int p,
                                                                   const float* __restrict__ F,
                                                                   const double* __restrict__ F64,
                                                                   const float2* __restrict__ wp2m,
                                                                   const float4* __restrict__ twg,
                                                                   float* __restrict__ phi, float* __restrict__ acc) {
-  constexpr bool DFS = NearShape<S>::DFS;
   using T = Num<DFA>;
-  using store = Num<DFS>;
+  using store = Num<false>;
   using real = typename T::real;
   using cplx = typename T::cplx;
   constexpr int NM = Shape<S>::NM, IB = kItems<S, DFA>, PS = Shape<S>::PS;
@@ -311,7 +300,7 @@ __global__ void __launch_bounds__(NearShape<S>::THR_INV) k_ns_inv(const void* __
     real* b = a + IB * p3;                                 // [IB][p][p][S]
     real* c = b + IB * p * p * S;                          // [IB][p][S][S]
     for (int i = tid; i < IB * p3; i += nthr) {
-      if constexpr (DFS) a[i] = df_from_double(__ldg(F64 + item0 * p3 + i));
+      if constexpr (kWideField<S>) a[i] = df_from_double(__ldg(F64 + item0 * p3 + i));
       else a[i] = widen<DFA>(__ldg(F + item0 * p3 + i));
     }
     __syncthreads();
@@ -372,17 +361,17 @@ __global__ void __launch_bounds__(NearShape<S>::THR_INV) k_ns_inv(const void* __
 }
 
 // ---------------------------------------------------------- spectral sums
-// Rows of 4 target leaves along x per thread, as k_spec_mac; the chunk's 27
-// kernel spectra and the tile's 6^3 source spectra in shared memory (41 KB),
+// Rows of 4 target leaves along x per thread, as k_spec_mac; the chunk's 14
+// kernel spectra and the tile's 6^3 source spectra in shared memory (35 KB),
 // the next chunk's copied (cp.async) during the current sums: a CTA takes
 // `per` consecutive chunks of one tile, up to 8, fewer where that leaves fewer
 // than 4 CTAs per SM.
 constexpr int kChunks = 8;
-constexpr int kStage = kNO * 32 + kSlots * 8;   // float4 per stage
-template <bool DF>
-__global__ void __launch_bounds__(DF ? 512 : 256) k_ns_mac(const float4* __restrict__ K, const void* __restrict__ Mh,
+constexpr int kKernels = kNO / 2 + 1;           // offsets 0..13: the others' kernels are their conjugates
+constexpr int kStage = kKernels * 32 + kSlots * 8;   // float4 per stage
+__global__ void __launch_bounds__(256) k_ns_mac(const float4* __restrict__ K, const void* __restrict__ Mh,
                                                           void* __restrict__ Ph, int L, int nkp, int iso, int per) {
-  constexpr int LANES = Num<DF>::LANES, NTHR = DF ? 512 : 256;
+  constexpr int LANES = Num<false>::LANES, NTHR = 256;
   extern __shared__ float4 sm4[];
   const int tid = threadIdx.x, n = 1 << L, nt = n / kTile;
   const int tile = blockIdx.x;
@@ -399,10 +388,10 @@ __global__ void __launch_bounds__(DF ? 512 : 256) k_ns_mac(const float4* __restr
   auto load = [&](int chunk, int st) {
     float4* to = sm4 + st * kStage;
     const float4* Kc = K + (size_t)chunk * kNO * 32;
-    for (int i = tid; i < kNO * 32; i += NTHR) tc::cp_async16_full(tc::smem_u32(to + i), Kc + i);
+    for (int i = tid; i < kKernels * 32; i += NTHR) tc::cp_async16_full(tc::smem_u32(to + i), Kc + i);
     const char* src = reinterpret_cast<const char*>(Mh) + (size_t)chunk * (leaves + 1) * 128;
     for (int i = tid; i < kSlots * 8; i += NTHR)
-      tc::cp_async16_full(tc::smem_u32(to + kNO * 32 + i), src + (size_t)slot_leaf[i >> 3] * 128 + (i & 7) * 16);
+      tc::cp_async16_full(tc::smem_u32(to + kKernels * 32 + i), src + (size_t)slot_leaf[i >> 3] * 128 + (i & 7) * 16);
     tc::cp_async_commit();
   };
   const int chunks = nkp / LANES, c_end = min(chunks, ((int)blockIdx.y + 1) * per);
@@ -417,9 +406,8 @@ __global__ void __launch_bounds__(DF ? 512 : 256) k_ns_mac(const float4* __restr
     tc::cp_async_wait<0>();
   }
   __syncthreads();
-  const float4* sK = sm4 + st * kStage;     // [27][32]
-  const float4* sM = sK + kNO * 32;         // [216][8]
-  if constexpr (!DF) {
+  const float4* sK = sm4 + st * kStage;     // [14][32]
+  const float4* sM = sK + kKernels * 32;    // [216][8]
     const int fr = tid & 15, ty = (tid >> 4) & 3, tz = tid >> 6;
     const float2* halo = reinterpret_cast<const float2*>(sM) + fr;
     float2 tot[4][4];
@@ -488,38 +476,6 @@ __global__ void __launch_bounds__(DF ? 512 : 256) k_ns_mac(const float4* __restr
 #pragma unroll
       for (int f = 0; f < 4; ++f) out[(leaf * 4 + f) * nkp + (size_t)chunk * LANES + fr] = tot[j][f];
     }
-  } else {
-    const int fr = tid & 7, ty = (tid >> 3) & 3, f = (tid >> 5) & 3, tz = tid >> 7;
-    const float4* halo = sM + fr;
-    float2 re[4], im[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) re[j] = im[j] = make_float2(0.f, 0.f);
-#pragma unroll 1
-    for (int row = 0; row < 9; ++row) {
-      const int oy = row % 3 - 1, oz = row / 3 - 1;
-      const float4* m0 = halo + ((tz + 1 + oz) * kHaloN + ty + 1 + oy) * kHaloN * LANES;
-#pragma unroll
-      for (int ox = -1; ox <= 1; ++ox) {
-        const float4 k = sK[(row * 3 + ox + 1) * 32 + f * 8 + fr];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const float4 v = m0[(j + 1 + ox) * LANES];
-          const float2 mr = make_float2(v.x, v.y), mi = make_float2(v.z, v.w);
-          Num<true>::mac(re[j], k.x, k.y, mr);
-          Num<true>::mac(im[j], k.x, k.y, mi);
-          Num<true>::mac(re[j], -k.z, -k.w, mi);
-          Num<true>::mac(im[j], k.z, k.w, mr);
-        }
-      }
-    }
-    float4* out = reinterpret_cast<float4*>(Ph);
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const size_t leaf = morton(TX * kTile + j, TY * kTile + ty, TZ * kTile + tz);
-      const float2 a = Num<true>::done(re[j]), b = Num<true>::done(im[j]);
-      out[(leaf * 4 + f) * nkp + (size_t)chunk * LANES + fr] = make_float4(a.x, a.y, b.x, b.y);
-    }
-  }
   __syncthreads();                          // this stage is refilled next
   }
 }
@@ -541,27 +497,25 @@ size_t inv_smem(int p) {
 template <int S, bool DFA>
 cudaError_t fwd_as(Plan& P, const float* rho, cudaStream_t s) {
   const unsigned leaves = 1u << (3 * P.L);
-  k_ns_fwd<S, DFA><<<leaves / Shape<S>::NB, NearShape<S>::THR_FWD, fwd_smem<S, DFA>(), s>>>(rho, P.d_mean, P.N, P.L,
+  k_ns_fwd<S, DFA><<<leaves / Shape<S>::NB, Shape<S>::THR, fwd_smem<S, DFA>(), s>>>(rho, P.d_mean, P.N, P.L,
                                                                                             P.ns_tw, P.ns_M);
   return cudaGetLastError();
 }
 // The sums: like the source spectra they need the density only.
 template <int S>
 cudaError_t sums_as(Plan& P, cudaStream_t s) {
-  constexpr bool DFS = NearShape<S>::DFS;
-  const int nt = (1 << P.L) / kTile, ch = chunks_of(S, DFS), nkp = ch * Num<DFS>::LANES;
+  const int nt = (1 << P.L) / kTile, ch = chunks_of(S, false), nkp = ch * Num<false>::LANES;
   const int tiles = nt * nt * nt, fit = (int)((long)tiles * ch / (4 * P.num_sms));
   const int per = fit < 1 ? 1 : (fit < kChunks ? fit : kChunks);
-  k_ns_mac<DFS><<<dim3(tiles, (ch + per - 1) / per), DFS ? 512 : 256, kMacSmem, s>>>(
-      static_cast<const float4*>(P.ns_K), P.ns_M, P.ns_P, P.L, nkp, P.iso, per);
+  k_ns_mac<<<dim3(tiles, (ch + per - 1) / per), 256, kMacSmem, s>>>(static_cast<const float4*>(P.ns_K), P.ns_M, P.ns_P,
+                                                                   P.L, nkp, P.iso, per);
   return cudaGetLastError();
 }
 template <int S, bool DFA>
 cudaError_t rest_as(Plan& P, float* phi, float* acc, cudaStream_t s) {
-  constexpr bool DFS = NearShape<S>::DFS;
   const unsigned leaves = 1u << (3 * P.L);
-  const int nkp = chunks_of(S, DFS) * Num<DFS>::LANES;
-  k_ns_inv<S, DFA><<<leaves * 4 / kItems<S, DFA>, NearShape<S>::THR_INV, inv_smem<S, DFA>(P.p), s>>>(
+  const int nkp = chunks_of(S, false) * Num<false>::LANES;
+  k_ns_inv<S, DFA><<<leaves * 4 / kItems<S, DFA>, Shape<S>::threads(kItems<S, DFA>), inv_smem<S, DFA>(P.p), s>>>(
       P.ns_P, nkp, (int)(inv_smem<S, DFA>(P.p) - sizeof(typename Num<DFA>::real) * kItems<S, DFA> * S * S * Shape<S>::PS), P.N,
       P.p, P.F[P.L], P.F64[P.L], P.w_p2m, P.ns_tw, phi, acc);
   return cudaGetLastError();
@@ -573,7 +527,7 @@ cudaError_t kernels_s(Plan& P, cudaStream_t s) {
   // the target spectra's space holds the half-transformed kernels meanwhile
   double2* scratch = static_cast<double2*>(P.ns_P);
   k_ns_planes<S><<<dim3(NM, kNO * 4), 128, 0, s>>>(P.near_tab, scratch);
-  k_ns_lines<S, NearShape<S>::DFS><<<dim3((NM * NM * S + 127) / 128, kNO * 4), 128, 0, s>>>(scratch,
+  k_ns_lines<S><<<dim3((NM * NM * S + 127) / 128, kNO * 4), 128, 0, s>>>(scratch,
                                                                                           static_cast<float*>(P.ns_K));
   return cudaGetLastError();
 }
@@ -585,13 +539,13 @@ cudaError_t opt_in(F* f, size_t bytes) {
 template <int S>
 cudaError_t setup_s() {
   cudaError_t e;
-  if constexpr (!NearShape<S>::DFS) {
+  if constexpr (!kWideField<S>) {
     if ((e = opt_in(k_ns_fwd<S, false>, fwd_smem<S, false>())) != cudaSuccess) return e;
     if ((e = opt_in(k_ns_inv<S, false>, inv_smem<S, false>(kMaxOrder))) != cudaSuccess) return e;
   }
   if ((e = opt_in(k_ns_fwd<S, true>, fwd_smem<S, true>())) != cudaSuccess) return e;
   if ((e = opt_in(k_ns_inv<S, true>, inv_smem<S, true>(kMaxOrder))) != cudaSuccess) return e;
-  return opt_in(k_ns_mac<NearShape<S>::DFS>, kMacSmem);
+  return opt_in(k_ns_mac, kMacSmem);
 }
 
 }  // namespace
@@ -599,7 +553,7 @@ cudaError_t setup_s() {
 bool near_spec_shape(const Plan& P) { return P.S == 4 || P.S == 6 || P.S == 8 || P.S == 16; }
 
 void near_spec_bytes(const Plan& P, size_t& nK, size_t& nM, size_t& nP) {
-  const size_t leaves = (size_t)1 << (3 * P.L), ch = chunks_of(P.S, P.S >= kWideLeaf);
+  const size_t leaves = (size_t)1 << (3 * P.L), ch = chunks_of(P.S, false);
   nK = ch * kNO * 512;
   nM = ch * (leaves + 1) * 128;
   nP = leaves * 4 * ch * 128;
