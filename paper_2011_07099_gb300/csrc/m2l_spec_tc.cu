@@ -208,25 +208,31 @@ __global__ void __launch_bounds__(256) k_stc_fwd(const float* __restrict__ M, in
       xi[s] = c.y;
     }
     const int px = px0 + ch / 8, child = ch % 8;
-    // this parent's place and, at the faces, its periodic copies in the halo
-    const bool ex = !iso && (px == 0 || px == nh - 1), ey = !iso && (py == 0 || py == nh - 1),
-               ez = !iso && (pz == 0 || pz == nh - 1);
+    __half2* dst = out + (child >> 2) * plane + (child & 3);
+    const size_t at = (((size_t)(pz + 1) * WY + py + 1) * WX + px + kXPad) * 4;
+    // the face parents' periodic copies in the halo, as distances along each axis
+    const ptrdiff_t ex = iso || (px > 0 && px < nh - 1) ? 0 : (px == 0 ? nh : -nh) * (ptrdiff_t)4;
+    const ptrdiff_t ey = iso || (py > 0 && py < nh - 1) ? 0 : (py == 0 ? nh : -nh) * (ptrdiff_t)(4 * WX);
+    const ptrdiff_t ez = iso || (pz > 0 && pz < nh - 1) ? 0 : (pz == 0 ? nh : -nh) * (ptrdiff_t)(4 * WX * WY);
+    const bool face = ex != 0 || ey != 0 || ez != 0;
     forward_line<false, P, false>(xr, xi, wt, [&](int kz, float re, float im) {
       re *= sm;
       im *= sm;
       const __half2 hi = __floats2half2_rn(re, im);
       const float2 back = __half22float2(hi);
       const __half2 lo = __floats2half2_rn(re - back.x, im - back.y);
-      __half2* dst = out + (size_t)(kz * NM * P + q) * 4 * plane + (child >> 2) * plane + (child & 3);
-      for (int cz = 0; cz <= (ez ? 1 : 0); ++cz)
-        for (int cy = 0; cy <= (ey ? 1 : 0); ++cy)
-          for (int cx = 0; cx <= (ex ? 1 : 0); ++cx) {
-            const int x = cx ? (px == 0 ? nh : -1) : px, y = cy ? (py == 0 ? nh : -1) : py,
-                      z = cz ? (pz == 0 ? nh : -1) : pz;
-            const size_t at = (((size_t)(z + 1) * WY + y + 1) * WX + x + kXPad) * 4;
-            dst[at] = hi;
-            dst[at + 2 * plane] = lo;
-          }
+      __half2* d = dst + (size_t)(kz * NM * P + q) * 4 * plane + at;
+      d[0] = hi;
+      d[2 * plane] = lo;
+      if (face) {
+#pragma unroll 1
+        for (int m = 1; m < 8; ++m) {
+          if (((m & 1) && !ex) || ((m & 2) && !ey) || ((m & 4) && !ez)) continue;
+          const ptrdiff_t o = (m & 1 ? ex : 0) + (m & 2 ? ey : 0) + (m & 4 ? ez : 0);
+          d[o] = hi;
+          d[o + 2 * (ptrdiff_t)plane] = lo;
+        }
+      }
     });
   }
 }
@@ -294,7 +300,7 @@ __device__ __forceinline__ void mma_f16(uint32_t d, uint64_t a, uint64_t b, uint
 
 __global__ void __launch_bounds__(kThr, 1)
 k_stc_mac(const __grid_constant__ CUtensorMap mapB, const uint8_t* __restrict__ W, const float* __restrict__ inv_w,
-          const float* __restrict__ amax, int nk, int level, float* __restrict__ Ph, int* __restrict__ err,
+          const float* __restrict__ amax, int nk, int parts, int level, float* __restrict__ Ph, int* __restrict__ err,
           uint64_t wait_ns, int stall) {
   // D FP32, A and B FP16 (format 0), both K-major, M = 128, N = 256
   constexpr uint32_t IDESC = (1u << 4) | ((uint32_t)(kN >> 3) << 17) | ((uint32_t)(kRows >> 4) << 24);
@@ -328,7 +334,9 @@ k_stc_mac(const __grid_constant__ CUtensorMap mapB, const uint8_t* __restrict__ 
   __syncthreads();
   tc::fence_after_sync();
   const uint32_t tmem = tmem_holder;
-  const int nmine = (int)blockIdx.x < nk ? (nk - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;   // frequencies of this CTA
+  // this CTA's units: unit v = (frequency v / parts, part v % parts of the boxes)
+  const int units = nk * parts, tpp = tiles / parts;
+  const int nmine = (int)blockIdx.x < units ? (units - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
 
   if (warp == 0) {
     // -------------------------------------------------------- MMA issuer
@@ -340,7 +348,7 @@ k_stc_mac(const __grid_constant__ CUtensorMap mapB, const uint8_t* __restrict__ 
           ok = false;
           break;
         }
-        for (int t = 0; t < tiles && ok; ++t, ++u) {
+        for (int t = 0; t < tpp && ok; ++t, ++u) {
           const uint32_t part = tmem + (uint32_t)((u & 1) * kN);
           if (u >= 2 && !tc::mbar_wait_bounded(&pfree[u & 1], (uint32_t)(u / 2 - 1) & 1u, wait_ns)) {
             ok = false;
@@ -380,7 +388,7 @@ k_stc_mac(const __grid_constant__ CUtensorMap mapB, const uint8_t* __restrict__ 
       bool ok = true;
       int it = 0, wloads = 0;
       for (int m = 0; m < nmine && ok; ++m) {
-        const int k = (int)blockIdx.x + m * (int)gridDim.x;
+        const int v = (int)blockIdx.x + m * (int)gridDim.x, k = v / parts, t0 = v % parts * tpp;
         if (m > 0 && !tc::mbar_wait_bounded(&wfree, (uint32_t)(m - 1) & 1u, wait_ns)) {
           ok = false;
           break;
@@ -389,7 +397,7 @@ k_stc_mac(const __grid_constant__ CUtensorMap mapB, const uint8_t* __restrict__ 
         for (int s = 0; s < kShifts; ++s)
           tc::bulk_g2s(sW + s * kWTile, W + (size_t)k * kWBytes + (size_t)s * kWTile, kWTile, &wfull);
         ++wloads;
-        for (int t = 0; t < tiles && ok; ++t) {
+        for (int t = t0; t < t0 + tpp && ok; ++t) {
           const int bx = (t % tx) * kBX, by = ((t / tx) % ty) * kBY, bz = t / (tx * ty) * kBZ;
           for (int g = 0; g < 9; ++g) {
             const int st = it % kStages, dy = g % 3, dz = g / 3;       // 0..2: the shift + the halo of 1
@@ -423,9 +431,9 @@ k_stc_mac(const __grid_constant__ CUtensorMap mapB, const uint8_t* __restrict__ 
     bool ok = true;
     int u = 0, turn = 0;
     for (int m = 0; m < nmine && ok; ++m) {
-      const int k = (int)blockIdx.x + m * (int)gridDim.x;
+      const int v = (int)blockIdx.x + m * (int)gridDim.x, k = v / parts, t0 = v % parts * tpp;
       const float sc = inv_m * __ldg(inv_w + (size_t)k * 4 + ((row >> 1) & 3));
-      for (int t = 0; t < tiles && ok; ++t, ++u) {
+      for (int t = t0; t < t0 + tpp && ok; ++t, ++u) {
         const int bx = (t % tx) * kBX, by = ((t / tx) % ty) * kBY, bz = t / (tx * ty) * kBZ;
         // the wait's outcome must be common to the 128 drain threads (they meet at a named barrier)
         const bool got = tc::mbar_wait_bounded(&pfull[u & 1], (uint32_t)(u / 2) & 1u, wait_ns);
@@ -503,9 +511,12 @@ cudaError_t launch_p(Plan& Pl, int level, cudaStream_t s) {
   k_stc_amax<<<blocks, 256, 0, s>>>(Pl.M[level], P * P * P, (int)nodes, amax);
   k_stc_fwd<P><<<(unsigned)(parents / StcShape<P>::PB), 256, stc_fwd_smem<P>(), s>>>(
       Pl.M[level], level, Pl.iso, amax, static_cast<__half2*>(Pl.stc_B[level]));
-  const unsigned grid = NK < Pl.num_sms ? NK : Pl.num_sms;
+  // few frequencies: halves of the boxes (196 frequencies of p = 4 are 1.3
+  // waves, rounded up to 2; 392 halves 2.6, to 1.5 frequencies' time); nh >= 8, so the tiles are even in number
+  const int parts = NK < 3 * Pl.num_sms ? 2 : 1;
+  const unsigned grid = NK * parts < Pl.num_sms ? NK * parts : Pl.num_sms;
   k_stc_mac<<<grid, kThr, kSmem, s>>>(*static_cast<const CUtensorMap*>(Pl.stc_map[level]),
-                                     static_cast<const uint8_t*>(Pl.stc_W[level]), Pl.stc_scale[level], amax, NK, level,
+                                     static_cast<const uint8_t*>(Pl.stc_W[level]), Pl.stc_scale[level], amax, NK, parts, level,
                                      static_cast<float*>(Pl.spec_P[level]), Pl.d_err, Pl.wait_ns, Pl.inject_stall);
   k_stc_inv<P><<<(unsigned)(nodes / StcShape<P>::NI), 256, stc_inv_smem<P>(), s>>>(
       static_cast<const float2*>(Pl.spec_P[level]), parents, Pl.F[level]);
