@@ -25,44 +25,56 @@ __device__ __forceinline__ int mesh_index(int i) {
   return (((c >> 2) * P + qz) * K + ((c >> 1) & 1) * P + qy) * K + (c & 1) * P + qx;
 }
 
-// FP32: CTA per (parent, field).  A thread makes the 2p outputs of a line from
-// registers; the last pass goes through shared memory so that the children's
-// values are read and written along memory.  Measured at 256^3, p = 6 (level
-// 4 -> 5): 0.30 ms when each output was its own loop with two divisions.
+// FP32: CTA per parent, all four fields (one field's passes have p^2, 2p^2 and
+// 4p^2 lines and would leave most threads idle).  A thread makes the 2p outputs
+// of a line from registers; the last pass goes through shared memory so that
+// the children's values are read and written along memory.  Measured at 256^3,
+// p = 6 (level 4 -> 5): 0.30 ms when each output was its own loop with two
+// divisions, 0.15 with a CTA per field.
 template <int P>
-__global__ void __launch_bounds__(128) k_l2l(const float* __restrict__ Fp, const float2* __restrict__ w,
-                                            float* __restrict__ Fc) {
-  constexpr int K = 2 * P, P3 = P * P * P;
-  __shared__ float2 W[P * K];            // [P][2P], used transposed
-  __shared__ float in[P3], t1[P * P * K], t2[P * K * K], out[K * K * K];
+constexpr int kL2lThr = (8 * P * P + 31) / 32 * 32 > 512 ? 512 : (8 * P * P + 31) / 32 * 32;
+
+template <int P>
+__global__ void __launch_bounds__(kL2lThr<P>) k_l2l(const float* __restrict__ Fp, const float2* __restrict__ w,
+                                                   float* __restrict__ Fc) {
+  constexpr int K = 2 * P, P3 = P * P * P, KS = K + 1, PR = P | 1;
+  extern __shared__ float2 smdf[];
+  float2* W = smdf;                                  // [P][2P], used transposed
+  float* in = reinterpret_cast<float*>(W + P * K);   // [f][z][y][x]
+  float* t1 = in + 4 * P * P * PR;                   // [f][z][y][ux]
+  float* t2 = t1 + 4 * P * P * KS;                   // [f][z][uy][ux]
+  float* out = t2 + 4 * P * K * K;                   // [f][uz][uy][ux]
   const int tid = threadIdx.x, nthr = blockDim.x;
-  const size_t parent = blockIdx.x >> 2;
-  const int f = blockIdx.x & 3;
+  const size_t parent = blockIdx.x;
   for (int i = tid; i < P * K; i += nthr) W[i] = __ldg(w + i);
-  for (int i = tid; i < P3; i += nthr) in[i] = __ldg(Fp + (parent * 4 + f) * P3 + i);
+  for (int i = tid; i < 4 * P3; i += nthr) in[(i / P) * PR + i % P] = __ldg(Fp + parent * 4 * P3 + i);
   __syncthreads();
   float a[K];
-  for (int l = tid; l < P * P; l += nthr) {                 // x: line (z, y)
-    expand_line_f<K>(in + l * P, 1, P, W, 1, K, a);
+  for (int l = tid; l < 4 * P * P; l += nthr) {             // x: line (f, z, y)
+    expand_line_f<K>(in + l * PR, 1, P, W, 1, K, a);
 #pragma unroll
-    for (int u = 0; u < K; ++u) t1[l * K + u] = a[u];
+    for (int u = 0; u < K; ++u) t1[l * KS + u] = a[u];
   }
   __syncthreads();
-  for (int l = tid; l < P * K; l += nthr) {                 // y: line (z, ux)
-    const int ux = l % K, z = l / K;
-    expand_line_f<K>(t1 + z * P * K + ux, K, P, W, 1, K, a);
+  for (int l = tid; l < 4 * P * K; l += nthr) {             // y: line (f, z, ux)
+    const int ux = l % K, fz = l / K;
+    expand_line_f<K>(t1 + fz * P * KS + ux, KS, P, W, 1, K, a);
 #pragma unroll
-    for (int u = 0; u < K; ++u) t2[(z * K + u) * K + ux] = a[u];
+    for (int u = 0; u < K; ++u) t2[(fz * K + u) * K + ux] = a[u];
   }
   __syncthreads();
-  for (int l = tid; l < K * K; l += nthr) {                 // z: line (uy, ux)
-    expand_line_f<K>(t2 + l, K * K, P, W, 1, K, a);
+  for (int l = tid; l < 4 * K * K; l += nthr) {             // z: line (f, uy, ux)
+    const int q = l % (K * K), f = l / (K * K);
+    expand_line_f<K>(t2 + f * P * K * K + q, K * K, P, W, 1, K, a);
 #pragma unroll
-    for (int u = 0; u < K; ++u) out[u * K * K + l] = a[u];
+    for (int u = 0; u < K; ++u) out[(f * K + u) * K * K + q] = a[u];
   }
   __syncthreads();
-  for (int i = tid; i < 8 * P3; i += nthr)
-    Fc[((parent * 8 + i / P3) * 4 + f) * P3 + i % P3] += out[mesh_index<P>(i)];
+  float* dst = Fc + parent * 32 * P3;
+  for (int i = tid; i < 32 * P3; i += nthr) {               // (child, f, q)
+    const int c = i / (4 * P3), fq = i % (4 * P3), f = fq / P3;
+    dst[i] += out[f * K * K * K + mesh_index<P>(c * P3 + fq % P3)];
+  }
 }
 
 // Variant for parents at the wide levels (the coarse levels 2 and 3; at
@@ -75,29 +87,29 @@ __global__ void __launch_bounds__(128) k_l2l(const float* __restrict__ Fp, const
 template <int P>
 __global__ void __launch_bounds__(128) k_l2l64(const double* __restrict__ Fp, const float2* __restrict__ w,
                                               double* __restrict__ Fc64, float* __restrict__ Fc) {
-  constexpr int K = 2 * P, P3 = P * P * P;
+  constexpr int K = 2 * P, P3 = P * P * P, KS = K + 1, PR = P | 1;
   extern __shared__ float2 smdf[];
   float2* W = smdf;                  // [P][2P], used transposed
-  float2* t1 = W + P * K;            // [z][y][ux]
-  float2* t2 = t1 + P * P * K;       // [z][uy][ux]
+  float2* t1 = W + P * K;            // [z][y][ux], odd row stride
+  float2* t2 = t1 + P * P * KS;       // [z][uy][ux]
   float2* out = t2 + P * K * K;      // [uz][uy][ux]
   float2* in = out;                  // [z][y][x], consumed before `out` is written
   const int tid = threadIdx.x, nthr = blockDim.x;
   const size_t parent = blockIdx.x >> 2;
   const int f = blockIdx.x & 3;
   for (int i = tid; i < P * K; i += nthr) W[i] = __ldg(w + i);
-  for (int i = tid; i < P3; i += nthr) in[i] = df_from_double(__ldg(Fp + (parent * 4 + f) * P3 + i));
+  for (int i = tid; i < P3; i += nthr) in[(i / P) * PR + i % P] = df_from_double(__ldg(Fp + (parent * 4 + f) * P3 + i));
   __syncthreads();
   float2 a[K];
   for (int l = tid; l < P * P; l += nthr) {                 // x
-    expand_line<K>(in + l * P, 1, P, W, 1, K, a);
+    expand_line<K>(in + l * PR, 1, P, W, 1, K, a);
 #pragma unroll
-    for (int u = 0; u < K; ++u) t1[l * K + u] = a[u];
+    for (int u = 0; u < K; ++u) t1[l * KS + u] = a[u];
   }
   __syncthreads();
   for (int l = tid; l < P * K; l += nthr) {                 // y
     const int ux = l % K, z = l / K;
-    expand_line<K>(t1 + z * P * K + ux, K, P, W, 1, K, a);
+    expand_line<K>(t1 + z * P * KS + ux, KS, P, W, 1, K, a);
 #pragma unroll
     for (int u = 0; u < K; ++u) t2[(z * K + u) * K + ux] = a[u];
   }
@@ -125,22 +137,30 @@ __global__ void __launch_bounds__(128) k_l2l64(const double* __restrict__ Fp, co
 template <int P>
 size_t smem64() {
   constexpr int K = 2 * P;
-  return sizeof(float2) * (P * K + P * P * K + P * K * K + K * K * K);
+  return sizeof(float2) * (P * K + P * P * (K + 1) + P * K * K + K * K * K);
+}
+
+template <int P>
+size_t smem32() {
+  constexpr int K = 2 * P;
+  return sizeof(float2) * P * K + sizeof(float) * 4 * (P * P * (P | 1) + P * P * (K + 1) + P * K * K + K * K * K);
 }
 
 template <int P>
 cudaError_t setup_p() {
+  const cudaError_t e = cudaFuncSetAttribute(k_l2l<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem32<P>());
+  if (e != cudaSuccess) return e;
   return cudaFuncSetAttribute(k_l2l64<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem64<P>());
 }
 
 template <int P>
 cudaError_t l2l_p(Plan& Pl, int level, cudaStream_t s) {
-  const unsigned blocks = 4u << (3 * level);
+  const unsigned parents = 1u << (3 * level);
   if (wide_level(Pl, level))
-    k_l2l64<P><<<blocks, 128, smem64<P>(), s>>>(Pl.F64[level], Pl.w_m2m,
+    k_l2l64<P><<<4 * parents, 128, smem64<P>(), s>>>(Pl.F64[level], Pl.w_m2m,
                                                wide_level(Pl, level + 1) ? Pl.F64[level + 1] : nullptr, Pl.F[level + 1]);
   else
-    k_l2l<P><<<blocks, 128, 0, s>>>(Pl.F[level], Pl.w_m2m, Pl.F[level + 1]);
+    k_l2l<P><<<parents, kL2lThr<P>, smem32<P>(), s>>>(Pl.F[level], Pl.w_m2m, Pl.F[level + 1]);
   return cudaGetLastError();
 }
 
