@@ -263,8 +263,9 @@ int alloc_m2l_part(Plan& P) {
 
 // Re-tabulate every table form from G_S1 plus the plan's corrections (MLP,
 // grid), synchronously.  Returns an FMM_* code.
-int retabulate(Plan& P) {
-  if (fmm::launch_tables(P, 0) != cudaSuccess) return FMM_ERR_CUDA;
+// near = false: a correction of the M2L tables only (the near zone keeps its table).
+int retabulate(Plan& P, bool near = true) {
+  if (fmm::launch_tables(P, near, 0) != cudaSuccess) return FMM_ERR_CUDA;
   if (P.fft) {   // the FFT form keeps the tables' spectra: rebuild them
     fmm::free_fft(P);
     if (P.m2l_fft) {
@@ -273,7 +274,7 @@ int retabulate(Plan& P) {
       if (rc != FMM_OK) return rc;
     }
   }
-  if (P.ns_K && fmm::launch_near_spec_kernels(P, 0) != cudaSuccess) return FMM_ERR_CUDA;
+  if (near && P.ns_K && fmm::launch_near_spec_kernels(P, 0) != cudaSuccess) return FMM_ERR_CUDA;
   for (int l = 2; l <= P.L; ++l) {
     if (P.spec_K[l] && fmm::launch_spec_kernels(P, l, 0) != cudaSuccess) return FMM_ERR_CUDA;
     if (P.stc_W[l] && fmm::launch_stc_weights(P, l, 0) != cudaSuccess) return FMM_ERR_CUDA;
@@ -742,7 +743,7 @@ int fmm_plan_set_correction(fmm_plan* plan, const float* weights, size_t n) {
   } else {
     P.has_corr = 0;
   }
-  return set_err(retabulate(P));
+  return set_err(retabulate(P, false));
 }
 
 int fmm_correction_grad(fmm_plan* plan, const float* density, const float* target_phi, const float* target_acc,
@@ -775,7 +776,7 @@ int fmm_plan_set_table_grid(fmm_plan* plan, const float* theta, size_t n) {
   } else {
     P.has_grid = 0;
   }
-  return set_err(retabulate(P));
+  return set_err(retabulate(P, false));
 }
 
 int fmm_table_grid_grad(fmm_plan* plan, const float* density, const float* target_phi, const float* target_acc,

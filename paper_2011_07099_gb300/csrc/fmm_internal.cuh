@@ -227,7 +227,7 @@ cudaError_t setup_p2p(const Plan& P);
 
 // ------------------------------------------------------------ kernel launchers
 // Each returns cudaGetLastError() after the launch.
-cudaError_t launch_tables(Plan& P, cudaStream_t s);
+cudaError_t launch_tables(Plan& P, bool near, cudaStream_t s);   // M2L tables, and the near table
 cudaError_t launch_mean(Plan& P, const float* rho, cudaStream_t s);
 // The same reduction into caller scratch (P.n_partials partials, 1 mean).
 cudaError_t launch_mean_into(const Plan& P, const float* rho, double* partials, double* mean, cudaStream_t s);

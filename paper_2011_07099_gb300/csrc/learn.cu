@@ -163,162 +163,188 @@ __global__ void k_table_grad(const float* __restrict__ lam, const float* __restr
 
 // ----------------------------------------------------------- MLP backward
 // Samples are the distinct network inputs of every level (learn_spec.cu) with
-// their folded upstream gradients.  One block of kBwdTile threads processes
-// tiles of kBwdTile samples (one per thread) and accumulates the parameter
-// gradient in shared memory (each thread owns a fixed set of parameters);
-// per-block partials are summed by k_grad_reduce.  Activation rows are padded
-// to 65 floats: a thread walks its own row, so rows 64 apart would put a
-// warp's 32 reads on one bank.  Measured at p = 6, L = 3: 16.4 ms for the
-// 830 600 table entries one by one.
+// their folded upstream gradients.  A block of 256 threads takes tiles of 64
+// samples: in the layer passes a thread holds 16 neurons of one sample (the
+// weights, four at a time, are broadcasts), in the weight gradients a 4 x 4
+// block of a layer's matrix summed over the tile's samples; activation rows are
+// padded to 65 floats, so that a warp's 32 rows start on different banks.
+// Per-block partials are summed by k_grad_reduce.  Measured at p = 6, L = 3,
+// one field: 16.4 ms for the 830 600 table entries one by one, 0.27 ms for
+// their distinct inputs with one thread per sample.
 constexpr int kBwdTile = 64;
-constexpr int kPerThread = (mlp::kParams + kBwdTile - 1) / kBwdTile;   // 138
+constexpr int kBwdThr = 256;
 constexpr int kRow = mlp::kH + 1;
 
-__global__ void __launch_bounds__(kBwdTile) k_mlp_backward(const float* __restrict__ w, const float* __restrict__ up,
-                                                          const uint32_t* __restrict__ samples, int ns, int lmax, int p,
-                                                          float* __restrict__ partials) {
+// acc[ii] = sum over j of W[(16 q + ii)][j] in[j], added in order of j.
+__device__ __forceinline__ void layer16(const float* __restrict__ W, const float* __restrict__ in, int q, float (&acc)[16]) {
+  for (int j = 0; j < mlp::kH; j += 4) {
+    const float h0 = in[j], h1 = in[j + 1], h2 = in[j + 2], h3 = in[j + 3];
+#pragma unroll
+    for (int ii = 0; ii < 16; ++ii) {
+      const float4 w = *reinterpret_cast<const float4*>(W + (16 * q + ii) * mlp::kH + j);
+      acc[ii] = fmaf(w.w, h3, fmaf(w.z, h2, fmaf(w.y, h1, fmaf(w.x, h0, acc[ii]))));
+    }
+  }
+}
+// acc[jj] = sum over i of W[i][16 q + jj] in[i].
+__device__ __forceinline__ void layer16_t(const float* __restrict__ W, const float* __restrict__ in, int q,
+                                          float (&acc)[16]) {
+  for (int i = 0; i < mlp::kH; ++i) {
+    const float g = in[i];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      const float4 w = *reinterpret_cast<const float4*>(W + i * mlp::kH + 16 * q + 4 * c);
+      acc[4 * c] = fmaf(w.x, g, acc[4 * c]);
+      acc[4 * c + 1] = fmaf(w.y, g, acc[4 * c + 1]);
+      acc[4 * c + 2] = fmaf(w.z, g, acc[4 * c + 2]);
+      acc[4 * c + 3] = fmaf(w.w, g, acc[4 * c + 3]);
+    }
+  }
+}
+// dW[4 a + x][4 b + y] += sum_s G[s][4 a + x] H[s][4 b + y], (a, b) = (tid / 16, tid % 16).
+__device__ __forceinline__ void outer16(const float* __restrict__ G, const float* __restrict__ H, int tid, float (&dW)[16]) {
+  const float *g0 = G + 4 * (tid >> 4), *h0 = H + 4 * (tid & 15);
+  for (int s = 0; s < kBwdTile; ++s) {
+    float g[4], h[4];
+#pragma unroll
+    for (int x = 0; x < 4; ++x) {
+      g[x] = g0[s * kRow + x];
+      h[x] = h0[s * kRow + x];
+    }
+#pragma unroll
+    for (int x = 0; x < 16; ++x) dW[x] = fmaf(g[x / 4], h[x % 4], dW[x]);
+  }
+}
+
+__global__ void __launch_bounds__(kBwdThr) k_mlp_backward(const float* __restrict__ w, const float* __restrict__ up,
+                                                         const uint32_t* __restrict__ samples, int ns, int lmax, int p,
+                                                         float* __restrict__ partials) {
   using namespace mlp;
-  extern __shared__ float smf[];
-  float* sw = smf;                               // kParams
-  float* X = sw + kParams;                       // tile x kIn
-  float* Z1 = X + kBwdTile * kIn;                // tile x kRow (pre-activations)
+  static_assert(kOffW2 % 4 == 0 && kOffW3 % 4 == 0, "float4 weight rows");
+  extern __shared__ float4 smf4[];
+  float* sw = reinterpret_cast<float*>(smf4);    // kParams (+ padding)
+  float* X = sw + (kParams + 3) / 4 * 4;         // tile x kIn
+  float* Z1 = X + kBwdTile * kIn;                // tile x kRow (pre-activations; Z3 then holds dz2)
   float* Z2 = Z1 + kBwdTile * kRow;
   float* Z3 = Z2 + kBwdTile * kRow;
   float* H1 = Z3 + kBwdTile * kRow;              // post-activations
   float* H2 = H1 + kBwdTile * kRow;
-  float* G = H2 + kBwdTile * kRow;               // tile x kRow (backprop buffer)
+  float* H3 = H2 + kBwdTile * kRow;
+  float* G = H3 + kBwdTile * kRow;               // dz3, then dz1
   float* GO = G + kBwdTile * kRow;               // tile (upstream gradient)
-  float* gacc = GO + kBwdTile;                   // kParams: this block's gradient
-  const int tid = threadIdx.x;
-  for (int i = tid; i < kParams; i += kBwdTile) {
-    sw[i] = w[i];
-    gacc[i] = 0.f;
-  }
+  const int tid = threadIdx.x, s = tid & 63, q = tid >> 6;
+  for (int i = tid; i < kParams; i += kBwdThr) sw[i] = w[i];
   const int total = (lmax - 1) * ns;
-  __syncthreads();
+  float d3[16] = {}, d2[16] = {}, dv = 0.f, dw1[2] = {0.f, 0.f}, db4 = 0.f;
   for (int base = blockIdx.x * kBwdTile; base < total; base += gridDim.x * kBwdTile) {
-    // forward for sample base + tid
-    {
+    __syncthreads();
+    if (tid < kBwdTile) {
       const int sidx = base + tid;
       float x[kIn] = {0.f, 0.f, 0.f, 0.f, 0.f};
       float go = 0.f;
       if (sidx < total) {
-        const uint32_t q = samples[sidx % ns];
+        const uint32_t v = samples[sidx % ns];
         const float inv = 1.f / (4.f * p);
-        x[0] = (int)((q >> 16) & 255) * inv;
-        x[1] = (int)((q >> 8) & 255) * inv;
-        x[2] = (int)(q & 255) * inv;
+        x[0] = (int)((v >> 16) & 255) * inv;
+        x[1] = (int)((v >> 8) & 255) * inv;
+        x[2] = (int)(v & 255) * inv;
         x[3] = (2 + sidx / ns) * 0.125f;
-        x[4] = (float)(q >> 24);
+        x[4] = (float)(v >> 24);
         go = up[sidx];
       }
       GO[tid] = go;
       for (int j = 0; j < kIn; ++j) X[tid * kIn + j] = x[j];
-      for (int i = 0; i < kH; ++i) {
-        float z = sw[kOffB1 + i];
-        for (int j = 0; j < kIn; ++j) z = fmaf(sw[kOffW1 + i * kIn + j], x[j], z);
-        Z1[tid * kRow + i] = z;
-        H1[tid * kRow + i] = gelu(z);
-      }
-      for (int i = 0; i < kH; ++i) {
-        float z = sw[kOffB2 + i];
-        for (int j = 0; j < kH; ++j) z = fmaf(sw[kOffW2 + i * kH + j], H1[tid * kRow + j], z);
-        Z2[tid * kRow + i] = z;
-        H2[tid * kRow + i] = gelu(z);
-      }
-      for (int i = 0; i < kH; ++i) {
-        float z = sw[kOffB3 + i];
-        for (int j = 0; j < kH; ++j) z = fmaf(sw[kOffW3 + i * kH + j], H2[tid * kRow + j], z);
-        Z3[tid * kRow + i] = z;
-        // dz3 = go * W4 * gelu'(z3)
-        G[tid * kRow + i] = go * sw[kOffW4 + i] * gelu_grad(z);
-      }
     }
     __syncthreads();
-    // parameter gradients of layers 3 and 4 (thread owns entries k*kBwdTile + tid)
-    for (int k = 0; k < kPerThread; ++k) {
-      const int q = k * kBwdTile + tid;
-      if (q >= kOffW3 && q < kOffB4 + 1) {
-        float a = 0.f;
-        if (q < kOffB3) {
-          const int i = (q - kOffW3) / kH, j = (q - kOffW3) % kH;
-          for (int s = 0; s < kBwdTile; ++s) a = fmaf(G[s * kRow + i], H2[s * kRow + j], a);
-        } else if (q < kOffW4) {
-          const int i = q - kOffB3;
-          for (int s = 0; s < kBwdTile; ++s) a += G[s * kRow + i];
-        } else if (q < kOffB4) {
-          const int i = q - kOffW4;
-          for (int s = 0; s < kBwdTile; ++s) a = fmaf(GO[s], gelu(Z3[s * kRow + i]), a);
-        } else {
-          for (int s = 0; s < kBwdTile; ++s) a += GO[s];
-        }
-        gacc[q] += a;
-      }
+    float a[16];
+#pragma unroll
+    for (int ii = 0; ii < 16; ++ii) {
+      const int i = 16 * q + ii;
+      float z = sw[kOffB1 + i];
+      for (int j = 0; j < kIn; ++j) z = fmaf(sw[kOffW1 + i * kIn + j], X[s * kIn + j], z);
+      Z1[s * kRow + i] = z;
+      H1[s * kRow + i] = gelu(z);
     }
     __syncthreads();
-    // dz2 = (W3^T dz3) * gelu'(z2), in place of Z3
-    {
-      float d2[kH];
-      for (int j = 0; j < kH; ++j) d2[j] = 0.f;
-      for (int i = 0; i < kH; ++i) {
-        const float g3 = G[tid * kRow + i];
-        for (int j = 0; j < kH; ++j) d2[j] = fmaf(sw[kOffW3 + i * kH + j], g3, d2[j]);
-      }
-      for (int j = 0; j < kH; ++j) Z3[tid * kRow + j] = d2[j] * gelu_grad(Z2[tid * kRow + j]);
+#pragma unroll
+    for (int ii = 0; ii < 16; ++ii) a[ii] = sw[kOffB2 + 16 * q + ii];
+    layer16(sw + kOffW2, H1 + s * kRow, q, a);
+#pragma unroll
+    for (int ii = 0; ii < 16; ++ii) {
+      Z2[s * kRow + 16 * q + ii] = a[ii];
+      H2[s * kRow + 16 * q + ii] = gelu(a[ii]);
     }
     __syncthreads();
-    for (int k = 0; k < kPerThread; ++k) {
-      const int q = k * kBwdTile + tid;
-      if (q >= kOffW2 && q < kOffW3) {
-        float a = 0.f;
-        if (q < kOffB2) {
-          const int i = (q - kOffW2) / kH, j = (q - kOffW2) % kH;
-          for (int s = 0; s < kBwdTile; ++s) a = fmaf(Z3[s * kRow + i], H1[s * kRow + j], a);
-        } else {
-          const int i = q - kOffB2;
-          for (int s = 0; s < kBwdTile; ++s) a += Z3[s * kRow + i];
-        }
-        gacc[q] += a;
-      }
+#pragma unroll
+    for (int ii = 0; ii < 16; ++ii) a[ii] = sw[kOffB3 + 16 * q + ii];
+    layer16(sw + kOffW3, H2 + s * kRow, q, a);
+    const float go = GO[s];
+#pragma unroll
+    for (int ii = 0; ii < 16; ++ii) {
+      const int i = 16 * q + ii;
+      H3[s * kRow + i] = gelu(a[ii]);
+      G[s * kRow + i] = go * sw[kOffW4 + i] * gelu_grad(a[ii]);   // dz3 = go W4 gelu'(z3)
     }
     __syncthreads();
-    // dz1 = (W2^T dz2) * gelu'(z1), into G
-    {
-      float d1[kH];
-      for (int j = 0; j < kH; ++j) d1[j] = 0.f;
-      for (int i = 0; i < kH; ++i) {
-        const float g2 = Z3[tid * kRow + i];
-        for (int j = 0; j < kH; ++j) d1[j] = fmaf(sw[kOffW2 + i * kH + j], g2, d1[j]);
-      }
-      for (int j = 0; j < kH; ++j) G[tid * kRow + j] = d1[j] * gelu_grad(Z1[tid * kRow + j]);
-    }
+    outer16(G, H2, tid, d3);
+    if (q == 0)                                    // b3
+      for (int t = 0; t < kBwdTile; ++t) dv += G[t * kRow + s];
+    else if (q == 1)                               // W4
+      for (int t = 0; t < kBwdTile; ++t) dv = fmaf(GO[t], H3[t * kRow + s], dv);
+    if (tid == 0)
+      for (int t = 0; t < kBwdTile; ++t) db4 += GO[t];
+#pragma unroll
+    for (int jj = 0; jj < 16; ++jj) a[jj] = 0.f;   // dz2 = (W3^T dz3) gelu'(z2)
+    layer16_t(sw + kOffW3, G + s * kRow, q, a);
+#pragma unroll
+    for (int jj = 0; jj < 16; ++jj) Z3[s * kRow + 16 * q + jj] = a[jj] * gelu_grad(Z2[s * kRow + 16 * q + jj]);
     __syncthreads();
-    for (int k = 0; k < kPerThread; ++k) {
-      const int q = k * kBwdTile + tid;
-      if (q < kOffW2) {
-        float a = 0.f;
-        if (q < kOffB1) {
-          const int i = q / kIn, j = q % kIn;
-          for (int s = 0; s < kBwdTile; ++s) a = fmaf(G[s * kRow + i], X[s * kIn + j], a);
-        } else {
-          const int i = q - kOffB1;
-          for (int s = 0; s < kBwdTile; ++s) a += G[s * kRow + i];
-        }
-        gacc[q] += a;
-      }
-    }
+    outer16(Z3, H1, tid, d2);
+    if (q == 2)                                    // b2
+      for (int t = 0; t < kBwdTile; ++t) dv += Z3[t * kRow + s];
+#pragma unroll
+    for (int jj = 0; jj < 16; ++jj) a[jj] = 0.f;   // dz1 = (W2^T dz2) gelu'(z1)
+    layer16_t(sw + kOffW2, Z3 + s * kRow, q, a);
+#pragma unroll
+    for (int jj = 0; jj < 16; ++jj) G[s * kRow + 16 * q + jj] = a[jj] * gelu_grad(Z1[s * kRow + 16 * q + jj]);
     __syncthreads();
+    if (q == 3)                                    // b1
+      for (int t = 0; t < kBwdTile; ++t) dv += G[t * kRow + s];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {                  // W1
+      const int e = tid + k * kBwdThr;
+      if (e < kH * kIn)
+        for (int t = 0; t < kBwdTile; ++t) dw1[k] = fmaf(G[t * kRow + e / kIn], X[t * kIn + e % kIn], dw1[k]);
+    }
   }
-  __syncthreads();
-  for (int q = tid; q < kParams; q += kBwdTile) partials[(size_t)blockIdx.x * kParams + q] = gacc[q];
+  float* out = partials + (size_t)blockIdx.x * kParams;
+#pragma unroll
+  for (int x = 0; x < 16; ++x) {
+    const int e = (4 * (tid >> 4) + x / 4) * kH + 4 * (tid & 15) + x % 4;
+    out[kOffW3 + e] = d3[x];
+    out[kOffW2 + e] = d2[x];
+  }
+  out[(q == 0 ? kOffB3 : (q == 1 ? kOffW4 : (q == 2 ? kOffB2 : kOffB1))) + s] = dv;
+#pragma unroll
+  for (int k = 0; k < 2; ++k)
+    if (tid + k * kBwdThr < kH * kIn) out[kOffW1 + tid + k * kBwdThr] = dw1[k];
+  if (tid == 0) out[kOffB4] = db4;
 }
 
-__global__ void k_grad_reduce(const float* __restrict__ partials, int nblocks, float* __restrict__ grad) {
-  for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < mlp::kParams; q += gridDim.x * blockDim.x) {
-    double a = 0.0;
-    for (int b = 0; b < nblocks; ++b) a += partials[(size_t)b * mlp::kParams + q];
-    grad[q] += (float)a;
-  }
+// grad += sum over the blocks of their partials (FP64): 32 parameters per
+// block, the partials dealt to 8 rows of threads.
+__global__ void __launch_bounds__(256) k_grad_reduce(const float* __restrict__ partials, int nblocks,
+                                                    float* __restrict__ grad) {
+  __shared__ double red[8][32];
+  const int q = blockIdx.x * 32 + threadIdx.x;
+  double a = 0.0;
+  if (q < mlp::kParams)
+    for (int b = threadIdx.y; b < nblocks; b += 8) a += partials[(size_t)b * mlp::kParams + q];
+  red[threadIdx.y][threadIdx.x] = a;
+  __syncthreads();
+  if (threadIdx.y || q >= mlp::kParams) return;
+  for (int r = 1; r < 8; ++r) a += red[r][threadIdx.x];
+  grad[q] += (float)a;
 }
 
 // ------------------------------------------------------------------ Adam
@@ -427,7 +453,7 @@ cudaError_t launch_adjoint_and_table_grad(Plan& P, const float* lam_cells, cudaS
 }
 
 size_t mlp_backward_smem() {
-  return sizeof(float) * (2 * mlp::kParams + kBwdTile * mlp::kIn + 6 * kBwdTile * kRow + kBwdTile);
+  return sizeof(float) * ((mlp::kParams + 3) / 4 * 4 + kBwdTile * mlp::kIn + 7 * kBwdTile * kRow + kBwdTile);
 }
 
 int mlp_backward_blocks(const Plan& P) { return 2 * P.num_sms; }
@@ -445,12 +471,13 @@ cudaError_t setup_learn() {
 cudaError_t launch_mlp_backward(Plan& P, const float* w, float* grad, cudaStream_t s) {
   cudaError_t e = launch_corr_fold(P, s);
   if (e != cudaSuccess) return e;
-  const int nb = mlp_backward_blocks(P);
-  k_mlp_backward<<<nb, kBwdTile, mlp_backward_smem(), s>>>(w, P.corr_up, P.corr_samples, P.n_corr, P.L, P.p,
-                                                          P.grad_partials);
+  const int tiles = ((P.L - 1) * P.n_corr + kBwdTile - 1) / kBwdTile;
+  const int nb = tiles < mlp_backward_blocks(P) ? tiles : mlp_backward_blocks(P);
+  k_mlp_backward<<<nb, kBwdThr, mlp_backward_smem(), s>>>(w, P.corr_up, P.corr_samples, P.n_corr, P.L, P.p,
+                                                         P.grad_partials);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  k_grad_reduce<<<(mlp::kParams + 255) / 256, 256, 0, s>>>(P.grad_partials, nb, grad);
+  k_grad_reduce<<<(mlp::kParams + 31) / 32, dim3(32, 8), 0, s>>>(P.grad_partials, nb, grad);
   return cudaGetLastError();
 }
 

@@ -226,22 +226,24 @@ __host__ __device__ inline uint32_t pack_sample(int cls, int a, int b, int c) {
 }
 
 // Upstream gradient of a sample: the table gradients of every entry that folds
-// onto it, each times the sign it is applied with, summed in FP64.
+// onto it, each times the sign it is applied with, summed in FP64.  Eight lanes
+// per sample share its up to 6 x 64 entries.
+constexpr int kFoldLanes = 8;
 __global__ void k_corr_fold(const float* __restrict__ dT_all, const uint32_t* __restrict__ samples, int ns, int p,
                             int lmax, float* __restrict__ up) {
   const int E = 8 * p - 1, HW = 4 * p - 1;
   const int total = (lmax - 1) * ns;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
+  const int sub = threadIdx.x % kFoldLanes, i = (blockIdx.x * blockDim.x + threadIdx.x) / kFoldLanes;
+  double sum = 0.0;
+  const bool valid = i < total;
+  if (valid) {
     const int level = 2 + i / ns;
     const uint32_t s = samples[i % ns];
     const int cls = s >> 24, v[3] = {(int)(s >> 16) & 255, (int)(s >> 8) & 255, (int)s & 255};
     const int period = (1 << level) * p;
     const float* dT = dT_all + (size_t)(level - 2) * E * E * E * 4;
-    double sum = 0.0;
-    if (cls && 2 * v[0] == period) {                          // half the box: sign 0
-      up[i] = 0.f;
-      continue;
-    }
+    // half the box: sign 0
+    if (!(cls && 2 * v[0] == period))
     for (int f = cls ? 1 : 0; f < (cls ? 4 : 1); ++f) {
       // arrangements of (a, b, c) on the axes: all distinct ones (G), or own on
       // axis f - 1 and the two distinct orders of (b, c)
@@ -276,20 +278,20 @@ __global__ void k_corr_fold(const float* __restrict__ dT_all, const uint32_t* __
             if (ok) pre[a][np[a]++] = cand[q];
           }
         }
-        for (int z = 0; z < np[2]; ++z)
-          for (int y = 0; y < np[1]; ++y)
-            for (int x = 0; x < np[0]; ++x) {
-              const int n[3] = {pre[0][x], pre[1][y], pre[2][z]};
-              if (!(n[0] | n[1] | n[2])) continue;
-              double sg = 1.0;
-              if (cls) sg = mlp::wrap_offset(n[f - 1], period) > 0 ? 1.0 : -1.0;
-              sum += sg * (double)__ldg(dT + (((size_t)(n[2] + HW) * E + n[1] + HW) * E + n[0] + HW) * 4 + f);
-            }
+        for (int e = sub; e < np[0] * np[1] * np[2]; e += kFoldLanes) {
+          const int n[3] = {pre[0][e % np[0]], pre[1][(e / np[0]) % np[1]], pre[2][e / (np[0] * np[1])]};
+          if (!(n[0] | n[1] | n[2])) continue;
+          double sg = 1.0;
+          if (cls) sg = mlp::wrap_offset(n[f - 1], period) > 0 ? 1.0 : -1.0;
+          sum += sg * (double)__ldg(dT + (((size_t)(n[2] + HW) * E + n[1] + HW) * E + n[0] + HW) * 4 + f);
+        }
       }
     }
     const double base = (double)(1 << level) * p;
-    up[i] = (float)(sum * mlp::kKappa * (cls ? base * base : base) / (4.0 * 3.14159265358979323846));
+    sum *= mlp::kKappa * (cls ? base * base : base) / (4.0 * 3.14159265358979323846);
   }
+  for (int o = kFoldLanes / 2; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+  if (valid && sub == 0) up[i] = (float)sum;
 }
 
 // The network at every distinct input of every level: one warp per sample, two
@@ -390,7 +392,7 @@ cudaError_t launch_corr_eval(Plan& P, cudaStream_t s) {
 
 cudaError_t launch_corr_fold(Plan& P, cudaStream_t s) {
   const int total = (P.L - 1) * P.n_corr;
-  k_corr_fold<<<(total + 127) / 128, 128, 0, s>>>(P.dT_all, P.corr_samples, P.n_corr, P.p, P.L, P.corr_up);
+  k_corr_fold<<<(total * kFoldLanes + 127) / 128, 128, 0, s>>>(P.dT_all, P.corr_samples, P.n_corr, P.p, P.L, P.corr_up);
   return cudaGetLastError();
 }
 

@@ -204,7 +204,7 @@ cudaError_t launch_tab_bf16(Plan& P, int level, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_tables(Plan& P, cudaStream_t s) {
+cudaError_t launch_tables(Plan& P, bool near, cudaStream_t s) {
   if (P.has_corr && plain_gs1(P)) {
     const cudaError_t e = launch_corr_eval(P, s);
     if (e != cudaSuccess) return e;
@@ -215,7 +215,7 @@ cudaError_t launch_tables(Plan& P, cudaStream_t s) {
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
-  k_tab_near<<<P.num_sms, 256, 0, s>>>(P.near_tab, P.S, P.N, spec_of(P), P.gmesh);
+  if (near) k_tab_near<<<P.num_sms, 256, 0, s>>>(P.near_tab, P.S, P.N, spec_of(P), P.gmesh);
   return cudaGetLastError();
 }
 
