@@ -415,9 +415,10 @@ int fmm_plan_copy_stage(fmm_plan* plan, int stage, int level, float* dst,
  *               sampled cells.
  *   stream      cudaStream_t as void*.  The call is synchronous: it returns
  *               after the work it enqueued on `stream` has finished.
- * Cost: samples x N^3 pair evaluations (on one GB300 0.14 s for 512 samples
- * at 256^3, 0.27 s for 1024); scratch of up to 10 MB is allocated and freed
- * by the call; the statement's density mean goes to that scratch too, so
+ * Cost: samples x N^3 pair evaluations (on one GB300 1.2 ms for 256 samples at
+ * 128^3); scratch of up to 6 MB is allocated by the first call (and by a later
+ * one with more samples) and kept by the plan; calls of several threads on one
+ * plan take turns.  The statement's density mean goes to that scratch too, so
  * the plan's mean stage (FMM_STAGE_MEAN) still holds the last solve's.  Do
  * not run it concurrently with a solve of the same plan.
  * Returns FMM_OK, FMM_ERR_ARG (NULL or misaligned pointers, samples out of

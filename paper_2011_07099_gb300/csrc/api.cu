@@ -162,6 +162,7 @@ void free_plan(Plan* P) {
     delete static_cast<CUtensorMap*>(P->stc_map[l]);
   }
   cudaFree(P->stc_amax);
+  cudaFree(P->es_scratch);
   cudaFree(P->w_p2m);
   cudaFree(P->w_m2m);
   cudaFree(P->stage_in);
@@ -1016,28 +1017,27 @@ int fmm_plan_error_stats(fmm_plan* plan, const float* density, const float* pote
     z ^= z >> 31;
     targets[(size_t)i] = z % n3;
   }
-  struct Scratch {
-    unsigned long long* targets = nullptr;
-    double* partials = nullptr;
-    double* sums = nullptr;
-    double* mean = nullptr;
-    ~Scratch() {
-      cudaFree(targets);
-      cudaFree(partials);
-      cudaFree(sums);
-      cudaFree(mean);
-    }
-  } d;
-  const size_t np = (size_t)fmm::error_stats_grid_x(P, samples) * samples * 4;
-  if (!dev_alloc(&d.targets, (size_t)samples) || !dev_alloc(&d.partials, np) || !dev_alloc(&d.sums, 4) ||
-      !dev_alloc(&d.mean, (size_t)P.n_partials + 1))
-    return set_err(FMM_ERR_ALLOC);
-  FMM_CUDA_TRY(cudaMemcpyAsync(d.targets, targets.data(), sizeof(unsigned long long) * samples,
+  // one plan-owned block, kept between calls: partials, mean, sums, targets.
+  // The call ends synchronised, so the lock covers every use of the block.
+  std::lock_guard<std::mutex> hold(P.es_lock);
+  const size_t np = (size_t)fmm::error_stats_grid_x(P, samples) * samples * 4, nm = (size_t)P.n_partials + 1,
+               ns = 4 + 4 * (size_t)samples, bytes = sizeof(double) * (np + nm + ns + (size_t)samples);
+  if (P.es_bytes < bytes) {
+    cudaFree(P.es_scratch);
+    P.es_scratch = nullptr;
+    P.es_bytes = 0;
+    if (cudaMalloc(&P.es_scratch, bytes) != cudaSuccess) return set_err(FMM_ERR_ALLOC);
+    P.es_bytes = bytes;
+  }
+  double* d_partials = static_cast<double*>(P.es_scratch);
+  double *d_mean = d_partials + np, *d_sums = d_mean + nm;
+  unsigned long long* d_targets = reinterpret_cast<unsigned long long*>(d_sums + ns);
+  FMM_CUDA_TRY(cudaMemcpyAsync(d_targets, targets.data(), sizeof(unsigned long long) * samples,
                                cudaMemcpyHostToDevice, s));
   FMM_CUDA_TRY(
-      fmm::launch_error_stats(P, density, potential, accel, d.targets, samples, d.partials, d.sums, d.mean, s));
+      fmm::launch_error_stats(P, density, potential, accel, d_targets, samples, d_partials, d_sums, d_mean, s));
   double sums[4] = {0.0, 0.0, 0.0, 0.0};
-  FMM_CUDA_TRY(cudaMemcpyAsync(sums, d.sums, sizeof(sums), cudaMemcpyDeviceToHost, s));
+  FMM_CUDA_TRY(cudaMemcpyAsync(sums, d_sums, sizeof(sums), cudaMemcpyDeviceToHost, s));
   FMM_CUDA_TRY(cudaStreamSynchronize(s));
   out[0] = sums[1] > 0.0 ? std::sqrt(sums[0] / sums[1]) : std::sqrt(sums[0]);
   out[1] = sums[3] > 0.0 ? std::sqrt(sums[2] / sums[3]) : std::sqrt(sums[2]);

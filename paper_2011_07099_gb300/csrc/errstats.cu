@@ -19,7 +19,7 @@ namespace fmm {
 namespace {
 
 constexpr int kEsThreads = 256;   // one target cell per thread
-constexpr int kEsChunk = 2048;    // source cells staged in shared memory per step
+constexpr int kEsChunk = 512;     // source cells staged in shared memory per step (128^3: 13.5 steps per CTA)
 
 // (s, c) += (mh + ml) g: exact product by FMA, TwoSum, the errors in c
 __device__ __forceinline__ void es_mac(float2& a, float mh, float ml, float g) {
@@ -118,50 +118,54 @@ __global__ void __launch_bounds__(kEsThreads) k_es_direct(const float* __restric
   }
 }
 
-// One block of 1024 threads: thread t sums target t's partials over the
-// blocks, compares with the given solution there, and the block reduces
-// sums[0..3] = (sum dPhi^2, sum Phi_ref^2, sum |dg|^2, sum |g_ref|^2).
-constexpr int kEsFinishThreads = 1024;
-
-__global__ void __launch_bounds__(kEsFinishThreads) k_es_finish(const double* __restrict__ partials, int nblocks,
-                                                                int T, const unsigned long long* __restrict__ targets,
-                                                                size_t n3, const float* __restrict__ phi,
-                                                                const float* __restrict__ acc,
-                                                                double* __restrict__ sums) {
-  __shared__ double red[4][kEsFinishThreads];
-  const int t = threadIdx.x;
-  double e[4] = {0.0, 0.0, 0.0, 0.0};
-  if (t < T) {
-    double ref[4] = {0.0, 0.0, 0.0, 0.0};
-    for (int b = 0; b < nblocks; ++b)
-      for (int f = 0; f < 4; ++f) ref[f] += partials[((size_t)b * T + t) * 4 + f];
-    const size_t i = targets[t];
-    const double dp = (double)phi[i] - ref[0];
-    e[0] = dp * dp;
-    e[1] = ref[0] * ref[0];
-    for (int c = 0; c < 3; ++c) {
-      const double dg = (double)acc[(size_t)c * n3 + i] - ref[1 + c];
-      e[2] += dg * dg;
-      e[3] += ref[1 + c] * ref[1 + c];
-    }
+// One warp per target: the sum of its partials over the blocks, compared with
+// the given solution there: terms[t] = (dPhi^2, Phi_ref^2, |dg|^2, |g_ref|^2).
+__global__ void __launch_bounds__(256) k_es_reduce(const double* __restrict__ partials, int nblocks, int T,
+                                                  const unsigned long long* __restrict__ targets, size_t n3,
+                                                  const float* __restrict__ phi, const float* __restrict__ acc,
+                                                  double* __restrict__ terms) {
+  const int lane = threadIdx.x & 31, t = blockIdx.x * 8 + (threadIdx.x >> 5);
+  if (t >= T) return;
+  double ref[4] = {0.0, 0.0, 0.0, 0.0};
+  for (int b = lane; b < nblocks; b += 32)
+    for (int f = 0; f < 4; ++f) ref[f] += partials[((size_t)b * T + t) * 4 + f];
+  for (int o = 16; o > 0; o >>= 1)
+    for (int f = 0; f < 4; ++f) ref[f] += __shfl_down_sync(0xffffffffu, ref[f], o);
+  if (lane) return;
+  const size_t i = targets[t];
+  const double dp = (double)phi[i] - ref[0];
+  double e[4] = {dp * dp, ref[0] * ref[0], 0.0, 0.0};
+  for (int c = 0; c < 3; ++c) {
+    const double dg = (double)acc[(size_t)c * n3 + i] - ref[1 + c];
+    e[2] += dg * dg;
+    e[3] += ref[1 + c] * ref[1 + c];
   }
-  for (int f = 0; f < 4; ++f) red[f][t] = e[f];
+  for (int f = 0; f < 4; ++f) terms[4 * (size_t)t + f] = e[f];
+}
+
+// sums[f] = sum over the targets of terms[t][f], one block.
+constexpr int kEsMaxSamples = 1024;
+__global__ void __launch_bounds__(256) k_es_finish(const double* __restrict__ terms, int T, double* __restrict__ sums) {
+  __shared__ double red[256];
+  const int f = threadIdx.x & 3;
+  double a = 0.0;
+  for (int t = threadIdx.x >> 2; t < T; t += 64) a += terms[4 * t + f];
+  red[threadIdx.x] = a;
   __syncthreads();
-  for (int h = kEsFinishThreads / 2; h > 0; h >>= 1) {
-    if (t < h)
-      for (int f = 0; f < 4; ++f) red[f][t] += red[f][t + h];
+  for (int h = 128; h >= 4; h >>= 1) {
+    if (threadIdx.x < h) red[threadIdx.x] += red[threadIdx.x + h];
     __syncthreads();
   }
-  if (t < 4) sums[t] = red[t][0];
+  if (threadIdx.x < 4) sums[threadIdx.x] = red[threadIdx.x];
 }
 
 }  // namespace
 
-int error_stats_max_samples() { return kEsFinishThreads; }
+int error_stats_max_samples() { return kEsMaxSamples; }
 
 int error_stats_grid_x(const Plan& P, int T) {
   const int gy = (T + kEsThreads - 1) / kEsThreads;
-  const int gx = (2 * P.num_sms + gy - 1) / gy;
+  const int gx = (4 * P.num_sms + gy - 1) / gy;
   return gx < 1 ? 1 : gx;
 }
 
@@ -178,7 +182,8 @@ cudaError_t launch_error_stats(Plan& P, const float* rho, const float* phi, cons
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   const size_t n3 = (size_t)P.N * P.N * P.N;
-  k_es_finish<<<1, kEsFinishThreads, 0, s>>>(partials, gx, T, targets, n3, phi, acc, sums);
+  k_es_reduce<<<(T + 7) / 8, 256, 0, s>>>(partials, gx, T, targets, n3, phi, acc, sums + 4);
+  k_es_finish<<<1, 256, 0, s>>>(sums + 4, T, sums);
   return cudaGetLastError();
 }
 

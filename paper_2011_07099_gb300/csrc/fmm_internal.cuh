@@ -3,6 +3,7 @@
 
 #include <cuda_runtime.h>
 #include <cstdint>
+#include <mutex>
 #include <cstddef>
 #include <vector>
 
@@ -165,6 +166,11 @@ struct Plan {
   cudaStream_t aux[2] = {};
   cudaEvent_t fev[4] = {};
 
+  // scratch of the error statement (targets, partials, sums, mean), grown on demand
+  void* es_scratch = nullptr;
+  size_t es_bytes = 0;
+  std::mutex es_lock;
+
   // per-stage timing: ev[2*k] / ev[2*k+1] bracket slot k
   int timing = 0;
   int timed = 0;
@@ -296,7 +302,7 @@ cudaError_t launch_mesh_green(int N, float* out, int sms, cudaStream_t s);
 cudaError_t launch_mesh_green_plan(const Plan& P, double* out, cudaStream_t s);
 // Sampled error against the direct periodic sum with G_S1 (errstats.cu):
 // targets T <= error_stats_max_samples(), partials error_stats_grid_x(P, T)
-// x T x 4 doubles, sums 4 doubles, mean_scratch P.n_partials + 1 doubles
+// x T x 4 doubles, sums 4 + 4 T doubles, mean_scratch P.n_partials + 1 doubles
 // (the density mean of the statement is its own, the plan's mean stage is
 // left as the last solve wrote it).
 int error_stats_max_samples();

@@ -117,3 +117,24 @@ def test_statement_of_a_solve_agrees_with_the_whole_mesh_error(B):
     e_phi, e_g = plan.error_stats(d, phi, acc, samples=1024, seed=5)
     plan.close()
     assert 0.5 < e_phi / full_phi < 2.0 and 0.5 < e_g / full_g < 2.0, (e_phi, full_phi, e_g, full_g)
+
+
+def test_statements_of_two_threads_on_one_plan_do_not_mix(B):
+    # the plan keeps the statement's scratch and grows it for the larger call:
+    # calls of several threads, on streams of their own, read what they read alone
+    from concurrent.futures import ThreadPoolExecutor
+    rho = _dev(inputs.lognormal(32, sigma=0.5, seed=3))
+    plan = B.Plan(32, 2, 4)
+    phi, acc = plan.solve(rho)
+    torch.cuda.synchronize()
+    sizes = [16, 1024, 100, 700] * 3
+    alone = [plan.error_stats(rho, phi, acc, samples=n, seed=n) for n in sizes]
+    fresh = B.Plan(32, 2, 4)
+
+    def one(n):
+        with torch.cuda.stream(torch.cuda.Stream()):
+            return fresh.error_stats(rho, phi, acc, samples=n, seed=n)
+    with ThreadPoolExecutor(4) as pool:
+        assert list(pool.map(one, sizes)) == alone
+    plan.close()
+    fresh.close()
