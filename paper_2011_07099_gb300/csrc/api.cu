@@ -320,8 +320,8 @@ int table_gradient(Plan& P, const float* density, const float* target_phi, const
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   const int rc = fmm_solve(reinterpret_cast<fmm_plan*>(&P), density, P.train_out, P.train_out + n3, stream);
   if (rc != FMM_OK) return rc;
-  if (fmm::launch_residual(P.train_out, P.train_out + n3, target_phi, target_acc, n3, w_phi, w_g, P.lam_cells, loss,
-                           P.num_sms, s) != cudaSuccess ||
+  if (fmm::launch_residual(P.train_out, P.train_out + n3, target_phi, target_acc, n3, w_phi, w_g, P.lam_cells,
+                           reinterpret_cast<double*>(P.grad_partials), loss, P.num_sms, s) != cudaSuccess ||
       fmm::launch_adjoint_and_table_grad(P, P.lam_cells, s) != cudaSuccess)
     return FMM_ERR_CUDA;
   return FMM_OK;

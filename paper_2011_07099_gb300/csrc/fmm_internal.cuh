@@ -292,7 +292,8 @@ cudaError_t launch_corr_fold(Plan& P, cudaStream_t s);
 void tg_bytes(const Plan& P, size_t& la, size_t& mh, size_t& gh, size_t& gl);
 cudaError_t launch_table_grad_spec(Plan& P, int level, cudaStream_t s);
 cudaError_t launch_residual(const float* phi, const float* acc, const float* tphi, const float* tacc, size_t n3,
-                            float w_phi, float w_g, float* lam, float* loss, int sms, cudaStream_t s);
+                            float w_phi, float w_g, float* lam, double* partials, float* loss, int sms,
+                            cudaStream_t s);   // partials: 4 * sms doubles
 cudaError_t launch_adjoint_and_table_grad(Plan& P, const float* lam_cells, cudaStream_t s);
 cudaError_t launch_mlp_backward(Plan& P, const float* w, float* grad, cudaStream_t s);
 int mlp_backward_blocks(const Plan& P);

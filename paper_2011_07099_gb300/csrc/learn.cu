@@ -20,10 +20,13 @@ namespace {
 
 // ------------------------------------------------------------ residual, loss
 // lam[f][i] = 2 w_f (out_f - target_f), f = Phi, g_x, g_y, g_z (SoA, N^3 each);
-// loss += sum w_f (out_f - target_f)^2.
-__global__ void k_residual(const float* __restrict__ phi, const float* __restrict__ acc, const float* __restrict__ tphi,
+// partials[block] = the block's share of sum w_f (out_f - target_f)^2, added to
+// the loss in block order by k_loss_add: one rounding per field, where an
+// FP32 atomic per warp (4864 of them) drifted by 1e-6 from run to run.
+__global__ void __launch_bounds__(256) k_residual(const float* __restrict__ phi, const float* __restrict__ acc, const float* __restrict__ tphi,
                            const float* __restrict__ tacc, size_t n3, float w_phi, float w_g, float* __restrict__ lam,
-                           float* __restrict__ loss) {
+                           double* __restrict__ partials) {
+  __shared__ double warps[8];
   double part = 0.0;
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < 4 * n3; i += (size_t)gridDim.x * blockDim.x) {
     const bool isphi = i < n3;
@@ -33,7 +36,20 @@ __global__ void k_residual(const float* __restrict__ phi, const float* __restric
     part += (double)w * d * d;
   }
   for (int o = 16; o > 0; o >>= 1) part += __shfl_down_sync(0xffffffffu, part, o);
-  if ((threadIdx.x & 31) == 0) atomicAdd(loss, (float)part);
+  if ((threadIdx.x & 31) == 0) warps[threadIdx.x >> 5] = part;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < 8; ++w) part += warps[w];
+    partials[blockIdx.x] = part;
+  }
+}
+
+// *loss += sum of the n partials (one warp).
+__global__ void k_loss_add(const double* __restrict__ partials, int n, float* __restrict__ loss) {
+  double a = 0.0;
+  for (int i = threadIdx.x; i < n; i += 32) a += partials[i];
+  for (int o = 16; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
+  if (threadIdx.x == 0) atomicAdd(loss, (float)a);
 }
 
 // --------------------------------------------------------- adjoint of L2P
@@ -414,8 +430,10 @@ cudaError_t launch_mesh_green_plan(const Plan& P, double* out, cudaStream_t s) {
 
 // --------------------------------------------------------------- launchers
 cudaError_t launch_residual(const float* phi, const float* acc, const float* tphi, const float* tacc, size_t n3,
-                            float w_phi, float w_g, float* lam, float* loss, int sms, cudaStream_t s) {
-  k_residual<<<4 * sms, 256, 0, s>>>(phi, acc, tphi, tacc, n3, w_phi, w_g, lam, loss);
+                            float w_phi, float w_g, float* lam, double* partials, float* loss, int sms,
+                            cudaStream_t s) {
+  k_residual<<<4 * sms, 256, 0, s>>>(phi, acc, tphi, tacc, n3, w_phi, w_g, lam, partials);
+  k_loss_add<<<1, 32, 0, s>>>(partials, 4 * sms, loss);
   return cudaGetLastError();
 }
 

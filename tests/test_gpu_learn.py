@@ -292,3 +292,22 @@ def test_training_against_pm_gk_gains_on_held_out_fields(B):
     assert after[0] < 0.8 * before[0] and after[1] < before[1]
     plain.close()
     tr.plan.close()
+
+
+@pytest.mark.parametrize("N,L", [(8, 2), (24, 3)])
+def test_loss_is_the_fp64_sum_of_the_residuals(B, N, L):
+    # FP32 residuals, summed in FP64, rounded once and added to the loss: two
+    # roundings of 2^-24, so 2^-22 holds; the loss passed in is kept
+    plan = B.Plan(N, L, 3)
+    rho = torch.from_numpy(inputs.lognormal(N, sigma=0.5, seed=4)).cuda()
+    phi, acc = plan.solve(rho)
+    g = torch.Generator(device="cuda").manual_seed(5)
+    tphi, tacc = (x + x.abs().mean() * torch.randn(x.shape, generator=g, device="cuda") for x in (phi, acc))
+    grad = torch.zeros(B.FMM_MLP_PARAMS, dtype=torch.float32, device="cuda")
+    loss = torch.full((1,), 0.5, dtype=torch.float32, device="cuda")
+    B.fmm_plan_set_correction_inference(plan.handle, B.FMM_INFER_FP32)
+    B.fmm_plan_set_correction(plan.handle, torch.zeros(B.FMM_MLP_PARAMS, dtype=torch.float32, device="cuda"))
+    B.fmm_correction_grad(plan.handle, rho, tphi, tacc, 2.0, 0.25, grad, loss)
+    want = 0.5 + 2.0 * float(((phi - tphi).double() ** 2).sum()) + 0.25 * float(((acc - tacc).double() ** 2).sum())
+    assert abs(float(loss.item()) - want) <= 2.0 ** -22 * want
+    plan.close()
