@@ -186,6 +186,14 @@ bool dev_alloc(T** ptr, size_t count) {
 // allocation fails (the dense kernels need ~20 times less memory), keeps the
 // dense contraction.
 constexpr size_t kSpecMaxBytes = (size_t)64 << 30;
+// ... and, from 1 GB up, at most a quarter of the memory that is free: a plan
+// that fits with the dense forms leaves the caller room with these.
+bool spectra_fit(size_t bytes) {
+  if (bytes > kSpecMaxBytes) return false;
+  if (bytes < ((size_t)1 << 30)) return true;
+  size_t free_b = 0, total = 0;
+  return cudaMemGetInfo(&free_b, &total) != cudaSuccess || bytes <= free_b / 4;
+}
 
 // (cos, sin) of 2 pi j / (2 points - 1) as (hi, lo) FP32 pairs.
 int make_twiddles(int points, float4** out) {
@@ -202,11 +210,11 @@ int make_twiddles(int points, float4** out) {
 
 // Buffers of the near zone's spectral products (near_spec.cu) for the leaf
 // sizes it is built for; without them the direct kernels run.
-int alloc_near_spec(Plan& P, size_t limit) {
+int alloc_near_spec(Plan& P, bool asked) {
   if (P.ns_K || !fmm::near_spec_shape(P)) return FMM_OK;
   size_t nK, nM, nP;
   fmm::near_spec_bytes(P, nK, nM, nP);
-  if (nK + nM + nP > limit) return FMM_OK;
+  if (!asked && !spectra_fit(nK + nM + nP)) return FMM_OK;
   if (!P.ns_tw) {
     const int rc = make_twiddles(P.S, &P.ns_tw);
     if (rc != FMM_OK) return rc;
@@ -231,7 +239,7 @@ int alloc_spec(Plan& P) {
   for (int l = 2; l <= P.L; ++l) {
     const size_t nk = fmm::spec_kernel_bytes(P, l), ns = fmm::spec_source_bytes(P, l),
                  nt = fmm::spec_target_bytes(P, l);
-    if (nk + ns + nt > kSpecMaxBytes) continue;
+    if (!spectra_fit(nk + ns + nt)) continue;
     if (cudaMalloc(&P.spec_K[l], nk) != cudaSuccess || cudaMalloc(&P.spec_M[l], ns) != cudaSuccess ||
         cudaMalloc(&P.spec_P[l], nt) != cudaSuccess) {
       cudaFree(P.spec_K[l]);
@@ -306,7 +314,7 @@ int table_gradient(Plan& P, const float* density, const float* target_phi, const
     if (!ok) return FMM_ERR_ALLOC;
     size_t la, mh, gh, gl;
     fmm::tg_bytes(P, la, mh, gh, gl);
-    if (P.p >= 2 && la + mh + gh + gl <= kSpecMaxBytes &&
+    if (P.p >= 2 && spectra_fit(la + mh + gh + gl) &&
         (cudaMalloc(&P.tg_mh, mh) != cudaSuccess || cudaMalloc(&P.tg_gh, gh) != cudaSuccess ||
          cudaMalloc(&P.tg_gl, gl) != cudaSuccess || cudaMalloc(&P.tg_la, la) != cudaSuccess)) {
       for (void** b : {&P.tg_la, &P.tg_mh, &P.tg_gh, &P.tg_gl}) {   // no room: the direct sums
@@ -448,7 +456,7 @@ fmm_plan* fmm_plan_create(int N, int L, int order) {
     for (int l = 2; l <= L && fok; ++l)
       if (fmm::wide_level(*P, l)) fok = dev_alloc(&P->F64[l], ((size_t)1 << (3 * l)) * 4 * p3);
     int rc = fok ? alloc_spec(*P) : FMM_ERR_ALLOC;
-    if (rc == FMM_OK) rc = alloc_near_spec(*P, kSpecMaxBytes);
+    if (rc == FMM_OK) rc = alloc_near_spec(*P, false);
     if (rc != FMM_OK || alloc_m2l_part(*P) != FMM_OK) {
       free_plan(P);
       set_err(rc != FMM_OK ? rc : FMM_ERR_ALLOC);
@@ -625,7 +633,7 @@ int fmm_plan_set_near_algorithm(fmm_plan* plan, int algorithm) {
   }
   if (P.S != 8) return set_err(FMM_ERR_UNSUPPORTED);
   if (!P.ns_K) {   // over the default limit at plan creation: the caller asks for it
-    const int rc = alloc_near_spec(P, ~(size_t)0);
+    const int rc = alloc_near_spec(P, true);
     if (rc != FMM_OK || !P.ns_K) return set_err(rc != FMM_OK ? rc : FMM_ERR_ALLOC);
     FMM_CUDA_TRY(fmm::launch_near_spec_kernels(P, 0));
   }
