@@ -4,7 +4,7 @@
 One step = one full solve (mean removal, P2M, M2M, M2L at every level, L2L,
 L2P and the near-zone sum) of a seeded synthetic 256^3 density field,
 order p = 6, with the input already resident in HBM.  The timed form is the
-mixed-precision one (tensor-core bf16x3 M2L at levels >= 4); the plain FP32
+mixed-precision one (tensor-core M2L at levels >= 4); the plain FP32
 form is timed on the same field in the same run, and the result's error
 against PM is stated twice: by the library (fmm_plan_error_stats, exact at
 256 sampled cells) and, with the CPU baseline, over every cell by the FP64
@@ -138,23 +138,8 @@ def workload_density(n, field):
     return inputs.lognormal(n, sigma=0.5, seed=5000 + field)
 
 
-# DRAM bytes (read + write) of one k_p2p launch, from an ncu capture of the
-# current kernel at 256^3, p = 6, L = 5 (dram__bytes_read.sum +
-# dram__bytes_write.sum); not measured in this run
-P2P_TRAFFIC = {(256, 5, 6): 419.3e6}
-# DRAM bytes (read + write) of one launch of the tensor-core M2L at the leaf
-# level and of the three near-zone FFT kernels together, from ncu captures
-# of the current kernels at 256^3 p=6 (profiles/); None where not captured
-M2L_TC_TRAFFIC = {(256, 5, 6): 1603.3e6}
-M2L_TC_TRAFFIC_SOURCE = ("ncu capture of the current k_m2l_tc at 256^3 p=6, level 5 (dram__bytes read 1503.1 MB + "
-                         "write 100.2 MB), not measured in this run")
-NEAR_FFT_TRAFFIC = {(256, 5, 6): 6942.5e6}
-NEAR_FFT_TRAFFIC_SOURCE = ("ncu capture of the current k_nz_fwd + k_nz_mac + k_nz_l2p + k_nz_inv at 256^3 p=6 "
-                           "(dram__bytes read+write summed), not measured in this run")
-P2P_TRAFFIC_SOURCE = ("ncu capture of the current k_p2p at 256^3 p=6 (dram__bytes read 197.6 MB + write 221.7 MB), "
-                      "not measured in this run")
-
-
+# DRAM bytes of the leaf stage and of the leaf level's M2L are not captured in
+# this run; the spectra each writes and reads back once are stated instead
 def measure_fp32_peak(B, dev, stream, reps=40):
     """The FP32 CUDA-core peak of this device, measured: the library's FMA
     probe (dependent FMA chains only, 2 CTAs of 1024 threads per SM), each
@@ -188,30 +173,36 @@ def measure_fp32_peak(B, dev, stream, reps=40):
                    f"median of {reps}"}
 
 
-def p2p_flops(N, L):
+def near_flops(N, L, fields=4):
+    """Arithmetic of the near zone by spectral products per solve: with leaves
+    of S cells, transforms on (2S - 1)^3 points of which NK = (2S - 1)^2 S
+    frequencies are kept; per leaf the sums (27 offsets x 4 fields x NK, 8 flop
+    per complex multiply-add), the forward transform of the masses and the
+    four inverse transforms to the S^3 cells, by lines."""
     S = N >> L
-    return (8 ** L) * (S ** 3) * 27 * (S ** 3) * 8.0      # 4 FMA per pair
+    M = 2 * S - 1
+    mac = 27 * fields * M * M * S * 8
+    fwd = 4 * S * S * S * S + 8 * S * S * M * S + 8 * S * M * M * S   # x (real), y, z passes
+    inv = 8 * S * M * S * M + 8 * S * S * S * M + 4 * S * S * S * S
+    return float(8 ** L * (mac + fwd + fields * inv))
 
 
-def m2l_flops(L, p):
-    tot = 0.0
-    for lev in range(2, L + 1):
-        n_off = 37 if lev == 2 else 189
-        tot += 2.0 * 4 * p ** 3 * p ** 3 * n_off * 8 ** lev
-    return tot
+def near_bytes(N, L, fields=4):
+    """Source spectra and the fields' target spectra, each written and read once (FP32 complex)."""
+    S = N >> L
+    return 8.0 ** L * 2 * (1 + fields) * 8 * (2 * S - 1) ** 2 * S
 
 
-def near_fft_flops(N, L, p):
-    """Arithmetic of the near zone by FFT per solve, counted as the kernels do
-    it (direct DFTs per axis, 8-cell leaves, 16^3 padded transforms): the
-    spectral sums (27 offsets x 4 fields x 2304 frequencies, 8 flop per complex
-    multiply-add), the forward transform of the masses and the four inverse
-    transforms that keep only the leaf's cells."""
-    leaves = 8 ** L
-    mac = 27 * 4 * 2304 * 8
-    fwd = 2 * (64 * 9 * 8 * 2 + 8 * 16 * 9 * 8 * 4 + 16 * 16 * 9 * 8 * 4)        # FMA x 2 per axis pass
-    inv = 4 * 2 * (8 * 16 * 9 * 16 * 4 + 8 * 8 * 9 * 16 * 4 + 512 * 8 * 2)   # per field, 4 fields
-    return float(leaves * (mac + fwd + inv))
+def m2l_spectral_flops(lev, p, fields=4):
+    """The spectral sums of one M2L level: per node and frequency 189 (level 2:
+    37) offsets x 4 fields, 8 flop per complex multiply-add."""
+    return 8.0 ** lev * (37 if lev == 2 else 189) * fields * 8 * (2 * p - 1) ** 2 * p
+
+
+def m2l_tensor_flops(lev, p):
+    """The tensor-core form executes, per frequency and parent, 27 x 16 x 128
+    multiply-adds on both FP16 parts of the sources."""
+    return 8.0 ** (lev - 1) * (2 * p - 1) ** 2 * p * 2 * 2.0 * 27 * 16 * 128
 
 
 def cpu_baseline():
@@ -270,14 +261,15 @@ def learned_correction(args):
 
 
 def near_fft_used(args):
-    """The near zone by FFT (Sec. 3's doubled-grid convolution) needs 8-cell leaves."""
+    """The near zone's FP32 transforms (--near fft) are the form of 8-cell leaves."""
     return args.near == "fft" and (args.n >> args.L) == 8
 
 
 def headline_config(args, learned, ws):
     """The `config` object of the headline workload; both arms print it."""
     n, L, p = args.n, args.L, args.p
-    near = "near zone by FFT on the doubled grid" if near_fft_used(args) else "near zone by direct sum"
+    near = ("near zone by FFT on the doubled grid" if near_fft_used(args)
+            else "near zone at the direct sum's accuracy")
     return {"workload": f"{n}^3 lognormal sigma=0.5 (seeded), order p={p}, L={L} (S={n >> L}), "
                         f"M2L levels>=4 {args.precision}, levels 2-3 extended-precision CUDA-core, {near}"
                         + (", learned table correction" if learned else ""),
@@ -369,40 +361,54 @@ def device_check(B, plan):
 
 
 def launches_per_solve(L, tc, p=6, near_fft=False):
-    # mean (2) + P2M + M2M per level + M2L per level + L2L per level + P2P
-    # (four kernels with the near zone by FFT: forward, sums, L2P, inverse);
-    # M2L of the coarse levels (2-3, and every level above the leaves at
-    # order >= 7) adds the FP64 range-sum kernel, tensor-core levels the
-    # BF16 split kernel
+    # the library's dense forms (M2L by dense sums, the near zone by pairs): mean
+    # (2) + P2M + M2M per level + M2L per level + L2L per level + near zone (1;
+    # by FFT 4); M2L of the coarse levels (2-3, and every level above the leaves
+    # at order >= 7) adds the range sums, tensor-core levels the split.  The
+    # spectral forms launch more; this is the least a solve launches, for the
+    # case that the profiler counts none (profiled_launches).
     wide = lambda lev: lev <= 3 or (p >= 7 and lev < L)
     tc_first = max(4, L) if p >= 7 else 4
     m2l = sum(2 if (wide(lev) or (tc and lev >= tc_first)) else 1 for lev in range(2, L + 1))
     return 2 + 1 + (L - 2) + m2l + (L - 2) + (4 if near_fft else 1)
 
 
-def solve_roofline(n, L, p, tc, ms, peaks, fp32_tflops, near_fft=False):
-    """Ideal time of the whole solve (each step at its own bound: FP32 FMA,
-    BF16 tensor (executed products), HBM bytes) against the measured step.
-    With the near zone by FFT its term is the larger of its arithmetic at the
-    FP32 peak and its spectra's HBM round trips (source spectra written and
-    read, target spectra written and read: 2 x (18 + 74) KB per leaf)."""
+def profiled_launches(solve):
+    """Kernels of this library in one call of `solve`, as the CUDA profiler
+    lists them (all are named fmm::...::k_*; copies and fills do not count).
+    The first profile of a process may see nothing, so two are taken."""
+    import torch
+    from torch.profiler import ProfilerActivity, profile
+    n = 0
+    for _ in range(2):
+        try:
+            with profile(activities=[ProfilerActivity.CUDA]) as prof:
+                solve()
+                torch.cuda.synchronize()
+            n = sum(1 for e in prof.events() if "fmm::" in e.name and "k_" in e.name)
+        except RuntimeError:   # another profiler holds the device: no count
+            n = 0
+    return n
+
+
+def solve_roofline(n, L, p, tc, ms, peaks, fp32_tflops):
+    """Ideal time of the whole solve, each step at its own bound (FP32 FMA,
+    FP16 tensor at the BF16 rate, HBM bytes), against the measured step.  The
+    near zone and each M2L level take the larger of their arithmetic and of
+    their spectra's one round trip through HBM."""
     fp32 = fp32_tflops * 1e12
-    bf16 = peaks.get("bf16_tflops_sustained", 1700.0) * 1e12
+    f16 = peaks.get("bf16_tflops_sustained", 1700.0) * 1e12
     hbm = peaks.get("hbm_gbs", 6500.0) * 1e9
     p3 = p ** 3
     tc_first = max(4, L) if p >= 7 else 4
-    if near_fft:
-        near = max(near_fft_flops(n, L, p) / fp32, (8 ** L) * 2 * (18432 + 73728) / peaks.get("hbm_gbs", 6500.0) / 1e9)
-        t = {"near_fft": near, "m2l_cuda_cores": 0.0, "m2l_tensor": 0.0}
-    else:
-        t = {"p2p": p2p_flops(n, L) / fp32, "m2l_cuda_cores": 0.0, "m2l_tensor": 0.0}
+    t = {"near": max(near_flops(n, L) / fp32, near_bytes(n, L) / hbm), "m2l_cuda_cores": 0.0, "m2l_tensor": 0.0}
     for lev in range(2, L + 1):
-        f = 2.0 * 4 * p3 * p3 * (37 if lev == 2 else 189) * 8 ** lev
+        spectra = 8.0 ** lev * 2 * 5 * 8 * (2 * p - 1) ** 2 * p / hbm
         if tc and lev >= tc_first:
-            t["m2l_tensor"] += 3 * f / bf16
+            t["m2l_tensor"] += max(m2l_tensor_flops(lev, p) / f16, spectra)
         else:
-            t["m2l_cuda_cores"] += f / fp32
-    bytes_ = 4 * n ** 3 * 2 + 4 * p3 * 8 ** L                              # mean + P2M
+            t["m2l_cuda_cores"] += max(m2l_spectral_flops(lev, p) / fp32, spectra)
+    bytes_ = 4 * n ** 3 * 2 + 4 * p3 * 8 ** L + 16 * n ** 3                # mean + P2M + the outputs
     bytes_ += sum(9 * 4 * p3 * 8 ** lev for lev in range(2, L))          # M2M
     bytes_ += sum(4 * 4 * p3 * 8 ** lev * 17 for lev in range(2, L))     # L2L (parent + children read/write)
     t["hbm_passes"] = bytes_ / hbm
@@ -545,42 +551,24 @@ def run_ours(args):
     peaks, src = _peaks()
     fma = measure_fp32_peak(B, dev, stream)
     fp32_peak = fma["tflops"]
-    dominant = max(names, key=lambda k: stage_ms[k])
-    roof_p2p = roof_near = None
-    if near_fft:
-        near_ach = near_fft_flops(n, L, p) / (stage_ms["p2p_l2p"] / 1000.0) / 1e12
-        roof_near = {"kernel": "k_nz_fwd + k_nz_mac + k_nz_l2p + k_nz_inv (near zone by FFT and L2P; the whole stage)",
-                     "bound": "alu", "achieved": near_ach, "peak": fp32_peak, "unit": "TFLOP/s",
-                     "frac": near_ach / fp32_peak, "traffic": NEAR_FFT_TRAFFIC.get((n, L, p)),
-                     "traffic_source": NEAR_FFT_TRAFFIC_SOURCE if NEAR_FFT_TRAFFIC.get((n, L, p)) else None,
-                     "peak_source": "measured (of measured): " + fma["how"]}
-    else:
-        p2p_ach = p2p_flops(n, L) / (stage_ms["p2p_l2p"] / 1000.0) / 1e12
-        traffic = P2P_TRAFFIC.get((n, L, p))
-        roof_p2p = {"kernel": "k_p2p (fused L2P + near-zone sum)", "bound": "alu", "achieved": p2p_ach,
-                    "peak": fp32_peak, "unit": "TFLOP/s", "frac": p2p_ach / fp32_peak,
-                    "traffic": traffic, "traffic_source": P2P_TRAFFIC_SOURCE if traffic else None,
-                    "peak_source": "measured (of measured): " + fma["how"], "fp32_probe": fma}
+    near_s = stage_ms["p2p_l2p"] / 1000.0
+    near_ach = near_flops(n, L) / near_s / 1e12
+    roof_near = {"kernel": "k_ns_fwd + k_ns_mac + k_ns_inv (near zone by spectral products and L2P; the whole stage)",
+                 "bound": "alu", "achieved": near_ach, "peak": fp32_peak, "unit": "TFLOP/s",
+                 "frac": near_ach / fp32_peak, "traffic": None, "spectra_bytes": near_bytes(n, L),
+                 "hbm_frac": near_bytes(n, L) / near_s / (peaks.get("hbm_gbs", 6500.0) * 1e9),
+                 "peak_source": "measured (of measured): " + fma["how"], "fp32_probe": fma}
     roof_m2l = None
     if tc:
-        # the leaf level's launch: the longest single launch of the mixed forms
         tc_ms = stage_ms[f"m2l_level{L}"]
-        alg = 2.0 * 4 * p ** 3 * p ** 3 * 189 * 8 ** L
-        ach = alg / (tc_ms / 1000.0) / 1e12
+        ach = m2l_tensor_flops(L, p) / (tc_ms / 1000.0) / 1e12
         peak = peaks.get("bf16_tflops_sustained", 1700.0)
-        traffic = M2L_TC_TRAFFIC.get((n, L, p))
-        roof_m2l = {"kernel": f"k_m2l_tc (level {L}, one launch)", "bound": "tensor",
-                    "achieved": ach, "peak": peak, "unit": "TFLOP/s", "frac": ach / peak, "traffic": traffic,
-                    "traffic_source": M2L_TC_TRAFFIC_SOURCE if traffic else None,
-                    "executed_tflops": ach * (3 if prec == B.FMM_PREC_BF16X3 else 1),
-                    "executed_frac": ach * (3 if prec == B.FMM_PREC_BF16X3 else 1) / peak,
-                    "peak_source": f"bf16_tflops_sustained ({src}, of measured); achieved counts the algorithmic "
-                                   "contraction (2 x 4p^3 x p^3 x 189 flop per node), bf16x3 executes 3 MMAs per "
-                                   "product"}
-    if near_fft:
-        roof = roof_m2l if roof_m2l is not None else roof_near
-    else:
-        roof = roof_p2p if (dominant == "p2p_l2p" or roof_m2l is None) else roof_m2l
+        roof_m2l = {"kernel": f"k_stc_amax + k_stc_fwd + k_stc_mac + k_stc_inv (level {L}, the whole level)",
+                    "bound": "hbm/latency", "achieved": ach, "peak": peak, "unit": "TFLOP/s", "frac": ach / peak,
+                    "traffic": None,
+                    "peak_source": f"bf16_tflops_sustained ({src}, of measured); achieved counts the executed FP16 "
+                                   "products of the spectral sums over the level's transforms and sums together"}
+    roof = roof_near if (roof_m2l is None or stage_ms["p2p_l2p"] >= stage_ms[f"m2l_level{L}"]) else roof_m2l
 
     # end to end through the public host-buffer entry point
     hin = torch.from_numpy(rho_host).pin_memory()
@@ -593,6 +581,8 @@ def run_ours(args):
         B.fmm_solve_host(plan.handle, hin, hphi, hacc, stream)
     e2e_s = (time.perf_counter() - t0) / e2e_steps
     checks["e2e"] = device_check(B, plan)
+    launches = (profiled_launches(lambda: plan.solve(rho, phi, acc)) if rank == 0 else 0) or launches_per_solve(
+        L, tc, p, near_fft)
     plan.close()
 
     if rank != 0:
@@ -609,17 +599,16 @@ def run_ours(args):
         "config": dict(headline_config(args, learned, ws), tc_tiles=tc_tiles),
         "stage_ms": stage_ms,
         "stage_ms_source": "two solves with the library's stage timing on, which runs the stages one after another; "
-                           "the timed steps overlap the CUDA-core M2L levels and the near zone's forward transform "
-                           "with the tensor-core levels",
+                           "the timed steps overlap the near zone's transform and sums with the tree passes and the "
+                           "coarse M2L levels with the tensor-core ones",
         "wall_s": wall,
         "roofline": roof,
-        "roofline_p2p": roof_p2p,
-        "roofline_near_fft": roof_near,
+        "roofline_near": roof_near,
         "roofline_m2l": roof_m2l,
         "e2e": {"value": ws * n ** 3 / e2e_s, "unit": UNIT, "h2d_bytes_per_step": 4 * n ** 3,
                 "d2h_bytes_per_step": 16 * n ** 3},
-        "gpu_launches": launches_per_solve(L, tc, p, near_fft) * args.steps,
-        "solve_roofline": solve_roofline(n, L, p, tc, ms, peaks, fp32_peak, near_fft),
+        "gpu_launches": launches * args.steps,
+        "solve_roofline": solve_roofline(n, L, p, tc, ms, peaks, fp32_peak),
         "clocks": clocks,
         "error_statement": statement,
         "device_checks": checks,
@@ -743,7 +732,7 @@ def run_full512(args):
             "ms_per_step": out["mixed_bf16x3"]["ms_per_step"], "higher_is_better": True, "scaling": "weak",
             "vs_baseline": None, "dtype": "bf16x3", "data": "synthetic",
             "config": {"workload": "512^3, p=8, L=6 (S=8), 1 + lognormal(sigma=1.5) + 4096 Plummer clumps; mixed form: "
-                                   "bf16x3 leaf-level M2L, bf16x6 level 5 (FP64 fields), double-float levels 2-4"
+                                   "tensor-core leaf-level M2L, bf16x6 level 5 (FP64 fields), double-float levels 2-4"
                                    + (", near zone by FFT" if args.near == "fft" else ""),
                        "forms": out}, "clocks": clk.summary()}
     print(json.dumps(line), flush=True)
