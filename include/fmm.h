@@ -54,6 +54,10 @@ typedef struct fmm_plan fmm_plan;
                                tcgen05 tensor cores, BF16 operands, FP32
                                accumulation in TMEM                           */
 #define FMM_PREC_BF16X3  2  /* as BF16 with split products hi*hi+hi*lo+lo*hi */
+/* From order 4 the tensor-core levels of both mixed forms run the spectral
+ * products on FP16 hi + lo operands (all four products), which are closer to
+ * FP64 than either BF16 form; the dense BF16 contractions above run below
+ * that order and where a level's spectra have no room (FMM_M2L_DENSE). */
 
 /* ---- plan lifecycle -------------------------------------------------- */
 
@@ -82,7 +86,7 @@ void fmm_plan_destroy(fmm_plan* plan);
  * Steps (Sec. 2, Sec. 3 eqs. fmm1-fmm3): mean removal and P2M at the leaves,
  * M2M up to level 2, M2L over the interaction zone at every level 2..L
  * (37 periodic nodes at level 2, 189 below) with G_S1, L2L down the tree,
- * and at each leaf L2P plus the direct near-zone sum over its 27 periodic
+ * and at each leaf L2P plus the near-zone sum over its 27 periodic
  * neighbour leaves.  Buffers must not overlap.  Returns FMM_ERR_ARG for NULL
  * or misaligned pointers, FMM_ERR_CUDA if a launch fails.  The return value
  * covers the enqueueing only: a bounded device-side wait of the tensor-core
@@ -107,15 +111,15 @@ int fmm_solve_host(fmm_plan* plan, const float* density_host,
  * FMM_PREC_BF16 / FMM_PREC_BF16X3 apply to levels >= 4 (see
  * fmm_plan_set_tc_min_level).  In every mode the coarse levels, whose
  * long-range sums cancel most, run on the CUDA cores in extended precision:
- * level 2 in double-float (error-free products and sums), level 3 with split
- * tables, both reduced in FP64 into FP64 local fields.  At order >= 7 every
+ * levels 2 and 3 in double-float (error-free products and sums) into FP64
+ * local fields.  At order >= 7 every
  * level above the leaves keeps FP64 local fields: in the tensor-core modes
  * levels >= 5 of them run "bf16x6" (both operands split in three BF16 parts,
  * six products, partials of each 32-deep stage added into a double-float
  * total, written in FP64), the coarser ones the double-float CUDA-core
  * kernel, and the leaf level the selected mode.  The first tensor-core
- * selection allocates and tabulates the split BF16 tables, translation tiles
- * and multipole buffers (synchronous).  Order 1 ignores the tensor-core
+ * selection allocates and tabulates the kernel tiles and source buffers
+ * (synchronous).  Order 1 ignores the tensor-core
  * modes.  FMM_ERR_ARG for an unknown mode. */
 int fmm_plan_set_precision(fmm_plan* plan, int mode);
 
@@ -165,8 +169,11 @@ int fmm_plan_set_green_mesh(fmm_plan* plan, const double* mesh, size_t n);
 int fmm_plan_mesh_green(const fmm_plan* plan, double* out, void* stream);
 
 /* How M2L evaluates eq. fmm2 at the fine levels.  FMM_M2L_DENSE (default):
- * the dense contraction per offset (CUDA cores or, in the mixed forms, the
- * tensor cores).  FMM_M2L_FFT: the HPM form of Sec. 2, as an ablation: per
+ * the sum per offset, on the CUDA cores or, in the mixed forms, the tensor
+ * cores, as products of node spectra on (2 order - 1)^3 points; the spectra
+ * are allocated with the plan, per level, if they take at most 64 GiB and,
+ * from 1 GB up, a quarter of the free memory; without them (and at order 1)
+ * the dense contractions run.  FMM_M2L_FFT: the HPM form of Sec. 2, as an ablation: per
  * parent, the gridlet masses of its neighbours' children on a zero-padded
  * (8 order)^3 grid, one FFT convolution with the level table (cuFFT, FP32),
  * and the 27 near nodes' terms subtracted by direct sums; used at the levels
@@ -179,18 +186,20 @@ int fmm_plan_mesh_green(const fmm_plan* plan, double* out, void* stream);
 int fmm_plan_set_m2l_algorithm(fmm_plan* plan, int algorithm);
 
 /* How the leaf stage evaluates the near zone (Sec. 2, part 3 of the
- * potential).  FMM_NEAR_DIRECT (default): the direct sum over the 27
- * neighbour leaves.  FMM_NEAR_FFT: the same sum by FFT convolution under
- * non-periodic boundary conditions on a doubled grid, the approach Sec. 3
- * takes for the near zone of a regular grid: per pair of neighbour leaves
- * the 8^3 masses zero-padded to 16^3, the 27 x 4 kernel spectra of the near
- * table (FP64, rounded once), FP32 transforms and products; the inverse
- * transforms add the near field to the leaf's L2P far field.  Needs 8-cell
- * leaves (N = 8 * 2^L);
- * FMM_ERR_UNSUPPORTED otherwise.  Allocates the spectra (synchronous;
- * 2^(3L) x 92 KB: 3.0 GB at 256^3, L = 5) and computes the kernel spectra,
- * again after every re-tabulation.  FMM_NEAR_DIRECT frees them.  FMM_ERR_ARG
- * for an unknown value, FMM_ERR_ALLOC if the spectra do not fit. */
+ * potential).  FMM_NEAR_DIRECT (default): the sum over the 27 neighbour
+ * leaves at the accuracy of the direct sum.  FMM_NEAR_FFT: the same sum with
+ * FP32 transforms throughout.  Both run, for leaves of S = 4, 6, 8 or 16
+ * cells, as convolutions under non-periodic boundary conditions on a padded
+ * grid, the approach Sec. 3 takes for the near zone of a regular grid: per
+ * pair of neighbour leaves the S^3 masses zero-padded to (2 S - 1)^3, the
+ * 27 x 4 kernel spectra of the near table (FP64, rounded once), FP32 products;
+ * FMM_NEAR_DIRECT transforms in double-float.  Other leaves sum directly, as
+ * do plans whose spectra had no room at creation (same limits as
+ * FMM_M2L_DENSE; 2^(3L) x 72 KB for S = 8: 2.4 GB at 256^3, L = 5).
+ * FMM_NEAR_FFT needs 8-cell leaves (N = 8 * 2^L), FMM_ERR_UNSUPPORTED
+ * otherwise, and allocates the spectra if the plan has none (synchronous).
+ * FMM_NEAR_DIRECT keeps them.  FMM_ERR_ARG for an unknown value, FMM_ERR_ALLOC
+ * if the spectra do not fit. */
 #define FMM_NEAR_DIRECT 0
 #define FMM_NEAR_FFT    1
 int fmm_plan_set_near_algorithm(fmm_plan* plan, int algorithm);
@@ -210,7 +219,7 @@ int fmm_plan_set_timeout_ms(fmm_plan* plan, int ms);
 #define FMM_FAULT_TC_STALL 1
 int fmm_plan_inject_fault(fmm_plan* plan, int kind);
 
-/* Tensor-core M2L: number of interaction offsets (1..189) accumulated in one
+/* Dense tensor-core M2L: number of interaction offsets (1..189) accumulated in one
  * TMEM partial sum before it is added to the compensated FP32 total on the
  * CUDA cores.  Smaller is more accurate, larger is faster; default 2.
  * FMM_ERR_ARG outside 1..189. */
@@ -232,7 +241,7 @@ int fmm_plan_set_m2l_group(fmm_plan* plan, int offsets_per_partial);
  * (synchronously).  FMM_ERR_ARG outside 4..9. */
 int fmm_plan_set_tc_min_level(fmm_plan* plan, int level);
 
-/* Tensor-core tile of one level: targets per CTA, 256 (default: an
+/* Dense tensor-core M2L, tile of one level: targets per CTA, 256 (default: an
  * 8 x 8 x 4 box of parents, MMA N = 256) or 128 (8 x 4 x 4, N = 128: twice
  * the CTAs, for levels whose 256-target grid leaves SMs idle).  The results
  * do not depend on it (each target's sums run in the same order).  The bf16x6

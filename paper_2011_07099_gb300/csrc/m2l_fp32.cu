@@ -1,4 +1,5 @@
-// M2L on CUDA cores in FP32 (the plain form).
+// M2L on CUDA cores by dense sums: order 1, and levels whose spectra
+// (m2l_spec.cu) have no room.
 //
 // Eq. fmm2 (Sec. 3): for a target node T at level l and every source node S
 // of its interaction zone (the children of the parent's neighbours that are

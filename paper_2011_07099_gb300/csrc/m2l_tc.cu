@@ -1,4 +1,6 @@
-// M2L on the tcgen05 tensor cores (BF16 operands, FP32 accumulation in TMEM).
+// Dense M2L on the tcgen05 tensor cores (BF16 operands, FP32 accumulation in
+// TMEM): the wide levels >= 5 of orders >= 7 (bf16x6), and the other mixed
+// levels where m2l_spec_tc.cu does not run (low orders, no room for spectra).
 //
 // Eq. fmm2 (Sec. 3) over a level is, for the targets T of one child type c
 // (all of which share the interaction list IL(c), Sec. 2 Fig. fmm), the dense

@@ -1,5 +1,7 @@
 // Leaf stage: L2P plus the near-zone direct sum (P2P), fused, writing the
-// final potential and acceleration of every cell.
+// final potential and acceleration of every cell.  Runs for leaves of 1, 2 and
+// 3 cells, where 27 S^3 pairs per cell are fewer operations than spectra
+// (near_spec.cu), and where a plan's spectra have no room.
 //
 // Far field (eq. fmm3 at the leaves): the leaf's local field interpolated at
 // its cell centres by the transpose of the P2M matrix.
