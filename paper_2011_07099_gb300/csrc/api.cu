@@ -879,10 +879,11 @@ int fmm_solve(fmm_plan* plan, const float* density, float* potential, float* acc
   auto on_tc = [&](int l) { return !fmm::fft_level(P, l) && tc && fmm::tc_level(P, l); };
   // Untimed solves overlap independent stages: the near zone's spectral sums
   // need only the density and its mean (second auxiliary stream, from the mean
-  // on), and fill what the small launches of the tree passes leave idle; the M2L levels are independent of one another until the downward
-  // pass, so the double-float levels run on the first auxiliary stream beside
-  // the FP32 and tensor-core levels on `s`.  Timed solves stay serial, so that
-  // each stage's events bracket it alone.
+  // on), and fill what the small launches of the tree passes leave idle; the
+  // M2L levels are independent of one another until the downward pass, so the
+  // double-float levels run on the first auxiliary stream beside the FP32 and
+  // tensor-core levels on `s`.  Timed solves stay serial, so that each stage's
+  // events bracket it alone.
   const bool near_apart = !t && P.ns_K;
   if (near_apart) {
     FMM_CUDA_TRY(cudaEventRecord(P.fev[0], s));

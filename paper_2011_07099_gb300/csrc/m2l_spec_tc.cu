@@ -546,18 +546,22 @@ int make_stc_map(Plan& P, int level) {
       return FMM_ERR_CUDA;
     encode = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn);
   }
-  if (!P.stc_map[level]) P.stc_map[level] = new (std::nothrow) CUtensorMap;
-  if (!P.stc_map[level]) return FMM_ERR_ALLOC;
+  CUtensorMap* map = new (std::nothrow) CUtensorMap;
+  if (!map) return FMM_ERR_ALLOC;
   const cuuint64_t nh = (cuuint64_t)1 << (level - 1), WX = nh + 2 * kXPad, WY = nh + 2;
   const cuuint64_t dims[4] = {WX * 8, WY, WY, (cuuint64_t)nk_of(P.p) * 4};
   const cuuint64_t strides[3] = {WX * 16, WX * 16 * WY, WX * 16 * WY * WY};
   const cuuint32_t box[4] = {(kBX + 2) * 8, kBY, kBZ, 4};
   const cuuint32_t estr[4] = {1, 1, 1, 1};
-  const CUresult r = encode(static_cast<CUtensorMap*>(P.stc_map[level]), CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 4,
-                            P.stc_B[level], dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                            CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-                            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  return r == CUDA_SUCCESS ? FMM_OK : FMM_ERR_CUDA;
+  const CUresult r = encode(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 4, P.stc_B[level], dims, strides, box, estr,
+                            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+                            CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  if (r != CUDA_SUCCESS) {      // a level with a map counts as prepared: keep none that failed
+    delete map;
+    return FMM_ERR_CUDA;
+  }
+  P.stc_map[level] = map;
+  return FMM_OK;
 }
 
 cudaError_t setup_spec_tc(const Plan& P) {
