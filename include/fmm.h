@@ -57,7 +57,7 @@ typedef struct fmm_plan fmm_plan;
 /* From order 4 the tensor-core levels of both mixed forms run the spectral
  * products on FP16 hi + lo operands (all four products), which are closer to
  * FP64 than either BF16 form; the dense BF16 contractions above run below
- * that order and where a level's spectra have no room (FMM_M2L_DENSE). */
+ * that order and where a level's spectra have no room. */
 
 /* ---- plan lifecycle -------------------------------------------------- */
 
@@ -212,11 +212,14 @@ int fmm_plan_set_near_algorithm(fmm_plan* plan, int algorithm);
  * are not valid. */
 int fmm_plan_set_timeout_ms(fmm_plan* plan, int ms);
 
-/* Test hook for the failure path (no GPU fault is involved):
+/* Test hook for the failure paths (no GPU fault is involved):
  * FMM_FAULT_TC_STALL makes the tensor-core MMA issuer of later solves do
- * nothing, so the dependent bounded waits expire; FMM_FAULT_NONE clears it. */
+ * nothing, so the dependent bounded waits expire; FMM_FAULT_ALLOC(n), n in
+ * 0..255, makes the n-th device allocation of later calls on the plan fail,
+ * once (counted from 0); FMM_FAULT_NONE clears either. */
 #define FMM_FAULT_NONE     0
 #define FMM_FAULT_TC_STALL 1
+#define FMM_FAULT_ALLOC(n) (256 + (n))
 int fmm_plan_inject_fault(fmm_plan* plan, int kind);
 
 /* Dense tensor-core M2L: number of interaction offsets (1..189) accumulated in one

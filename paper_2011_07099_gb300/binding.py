@@ -30,6 +30,7 @@ FMM_INFER_FP32 = 1
 
 FMM_FAULT_NONE = 0
 FMM_FAULT_TC_STALL = 1
+FMM_FAULT_ALLOC = 256       # + n: the n-th allocation of later calls fails
 
 FMM_BOUNDARY_PERIODIC = 0
 FMM_BOUNDARY_ISOLATED = 1

@@ -176,10 +176,26 @@ void free_plan(Plan* P) {
   delete P;
 }
 
+// Device memory.  An allocation that fails is the caller's to report: CUDA's
+// record of it is cleared, so that no later launch reads it as its own error.
+bool dev_alloc_bytes(void** ptr, size_t bytes) {
+  if (cudaMalloc(ptr, bytes) == cudaSuccess) return true;
+  (void)cudaGetLastError();
+  *ptr = nullptr;
+  return false;
+}
 template <typename T>
 bool dev_alloc(T** ptr, size_t count) {
-  return cudaMalloc(reinterpret_cast<void**>(ptr), sizeof(T) * count) == cudaSuccess;
+  return dev_alloc_bytes(reinterpret_cast<void**>(ptr), sizeof(T) * count);
 }
+// The same for a plan in use, whose allocation FMM_FAULT_ALLOC names asks for
+// more than any device holds.
+template <typename T>
+bool plan_alloc(Plan& P, T** ptr, size_t count) {
+  const bool fail = P.fail_alloc >= 0 && P.fail_alloc-- == 0;
+  return dev_alloc(ptr, fail ? ((size_t)1 << 60) / sizeof(T) : count);
+}
+bool plan_alloc(Plan& P, void** ptr, size_t bytes) { return plan_alloc(P, reinterpret_cast<char**>(ptr), bytes); }
 
 // Buffers of the spectral M2L (m2l_spec.cu) for every level of orders >= 2
 // whose spectra take at most kSpecMaxBytes; a level that has none, or whose
@@ -286,11 +302,11 @@ int retabulate(Plan& P, bool near = true) {
   if (near && P.ns_K && fmm::launch_near_spec_kernels(P, 0) != cudaSuccess) return FMM_ERR_CUDA;
   for (int l = 2; l <= P.L; ++l) {
     if (P.spec_K[l] && fmm::launch_spec_kernels(P, l, 0) != cudaSuccess) return FMM_ERR_CUDA;
-    if (P.stc_W[l] && fmm::launch_stc_weights(P, l, 0) != cudaSuccess) return FMM_ERR_CUDA;
+    if (P.stc_map[l] && fmm::launch_stc_weights(P, l, 0) != cudaSuccess) return FMM_ERR_CUDA;
   }
   if (P.tc_ready) {
     for (int l = fmm::kTcMinLevel; l <= P.L; ++l) {
-      if (!P.Apre[l]) continue;
+      if (!P.tmapB[l]) continue;
       if ((!fmm::tc_wide(P, l) && fmm::launch_tab_bf16(P, l, 0) != cudaSuccess) ||
           fmm::launch_build_a(P, l, 0) != cudaSuccess)
         return FMM_ERR_CUDA;
@@ -493,35 +509,53 @@ int fmm_plan_get_shape(const fmm_plan* plan, int* N, int* L, int* order, int* S)
 }
 
 namespace {
-// Tensor-core M2L buffers: split tables, split multipoles and the translation
-// tiles of every level from the first tensor-core level down to the leaves
-// (levels that already have them are kept).  Tabulated once, synchronously.
+// A level of the spectral tensor-core form: split weights and sources, their
+// scales and the tensor map, all of them or none (FMM_* code).
+int prepare_stc(Plan& P, int l) {
+  size_t nW, nB, nS;
+  fmm::stc_bytes(P, l, nW, nB, nS);
+  int rc = FMM_ERR_ALLOC;
+  if ((P.stc_amax || plan_alloc(P, &P.stc_amax, (size_t)fmm::kMaxLevel + 1)) && plan_alloc(P, &P.stc_W[l], nW) &&
+      plan_alloc(P, &P.stc_B[l], nB) && plan_alloc(P, &P.stc_scale[l], nS / sizeof(float))) {
+    // the halo of the isolated problem stays zero
+    rc = cudaMemset(P.stc_B[l], 0, nB) == cudaSuccess && fmm::launch_stc_weights(P, l, 0) == cudaSuccess
+             ? fmm::make_stc_map(P, l)
+             : FMM_ERR_CUDA;
+  }
+  if (rc != FMM_OK) {
+    cudaFree(P.stc_W[l]);
+    cudaFree(P.stc_B[l]);
+    cudaFree(P.stc_scale[l]);
+    P.stc_W[l] = P.stc_B[l] = nullptr;
+    P.stc_scale[l] = nullptr;
+  }
+  return rc;
+}
+
+// Tensor-core M2L buffers of every level from the first tensor-core level down
+// to the leaves (levels that already have them are kept): the spectral form's
+// or, where that has no room or does not run, the dense contraction's split
+// tables, split multipoles and translation tiles.  A level counts as prepared
+// once it has its tensor map, which is made last.  Tabulated once, synchronously.
 int prepare_tc(Plan& P) {
   const size_t E = 8 * P.p - 1;
   bool made = false;
   for (int l = fmm::tc_first_level(P); l <= P.L; ++l) {
     if (fmm::spec_tc_level(P, l)) {
       if (P.stc_map[l]) continue;
-      size_t nW, nB, nS;
-      fmm::stc_bytes(P, l, nW, nB, nS);
-      if ((!P.stc_amax && !dev_alloc(&P.stc_amax, (size_t)fmm::kMaxLevel + 1)) ||
-          (!P.stc_W[l] && cudaMalloc(&P.stc_W[l], nW) != cudaSuccess) ||
-          (!P.stc_B[l] && cudaMalloc(&P.stc_B[l], nB) != cudaSuccess) ||
-          (!P.stc_scale[l] && cudaMalloc(&P.stc_scale[l], nS) != cudaSuccess))
-        return FMM_ERR_ALLOC;
-      // the halo of the isolated problem stays zero
-      if (cudaMemset(P.stc_B[l], 0, nB) != cudaSuccess || fmm::launch_stc_weights(P, l, 0) != cudaSuccess)
-        return FMM_ERR_CUDA;
-      const int rc = fmm::make_stc_map(P, l);
-      if (rc != FMM_OK) return rc;
-      made = true;
-      continue;
+      const int rc = prepare_stc(P, l);
+      if (rc == FMM_OK) {
+        made = true;
+        continue;
+      }
+      if (rc != FMM_ERR_ALLOC) return rc;
+      P.stc_off[l] = true;                  // no room: spec_tc_level is false from here on
     }
-    if (P.Apre[l]) continue;
+    if (P.tmapB[l]) continue;
     const bool wide = fmm::tc_wide(P, l);   // wide modes: tiles from tab + tab_lo, no BF16 table
-    if ((!wide && !P.tab_bf[l] && !dev_alloc(&P.tab_bf[l], E * E * E)) ||
-        (!P.Mbf_hi[l] && cudaMalloc(&P.Mbf_hi[l], fmm::tc_bsplit_bytes(P.p, l, fmm::tc_splits(P, l))) != cudaSuccess) ||
-        cudaMalloc(&P.Apre[l], fmm::tc_apre_bytes(P.p, fmm::tc_splits(P, l))) != cudaSuccess)
+    if ((!wide && !P.tab_bf[l] && !plan_alloc(P, &P.tab_bf[l], E * E * E)) ||
+        (!P.Mbf_hi[l] && !plan_alloc(P, &P.Mbf_hi[l], fmm::tc_bsplit_bytes(P.p, l, fmm::tc_splits(P, l)))) ||
+        (!P.Apre[l] && !plan_alloc(P, &P.Apre[l], fmm::tc_apre_bytes(P.p, fmm::tc_splits(P, l)))))
       return FMM_ERR_ALLOC;
     if ((!wide && fmm::launch_tab_bf16(P, l, 0) != cudaSuccess) || fmm::launch_build_a(P, l, 0) != cudaSuccess)
       return FMM_ERR_CUDA;
@@ -648,8 +682,11 @@ int fmm_plan_set_timeout_ms(fmm_plan* plan, int ms) {
 }
 
 int fmm_plan_inject_fault(fmm_plan* plan, int kind) {
-  if (!plan || (kind != FMM_FAULT_NONE && kind != FMM_FAULT_TC_STALL)) return set_err(FMM_ERR_ARG);
-  reinterpret_cast<Plan*>(plan)->inject_stall = kind == FMM_FAULT_TC_STALL ? 1 : 0;
+  const bool alloc = kind >= FMM_FAULT_ALLOC(0) && kind <= FMM_FAULT_ALLOC(255);
+  if (!plan || (kind != FMM_FAULT_NONE && kind != FMM_FAULT_TC_STALL && !alloc)) return set_err(FMM_ERR_ARG);
+  Plan& P = *reinterpret_cast<Plan*>(plan);
+  P.inject_stall = kind == FMM_FAULT_TC_STALL ? 1 : 0;
+  P.fail_alloc = alloc ? kind - FMM_FAULT_ALLOC(0) : -1;
   return set_err(FMM_OK);
 }
 
@@ -662,11 +699,16 @@ int fmm_plan_set_m2l_group(fmm_plan* plan, int offsets_per_partial) {
 int fmm_plan_set_tc_min_level(fmm_plan* plan, int level) {
   if (!plan || level < fmm::kTcMinLevel || level > fmm::kMaxLevel + 1) return set_err(FMM_ERR_ARG);
   Plan& P = *reinterpret_cast<Plan*>(plan);
+  const int was_level = P.tc_min_level, was_set = P.tc_min_set;
   P.tc_min_level = level;
   P.tc_min_set = 1;
   if (P.tc_ready) {   // a lower first level needs its tiles now
     const int rc = prepare_tc(P);
-    if (rc != FMM_OK) return set_err(rc);
+    if (rc != FMM_OK) {   // a level without them must not run
+      P.tc_min_level = was_level;
+      P.tc_min_set = was_set;
+      return set_err(rc);
+    }
   }
   return set_err(FMM_OK);
 }

@@ -109,6 +109,7 @@ struct Plan {
   float* stc_scale[kMaxLevel + 1] = {};
   void* stc_B[kMaxLevel + 1] = {};
   void* stc_map[kMaxLevel + 1] = {};
+  bool stc_off[kMaxLevel + 1] = {};        // no room for them: the level's dense contraction runs
   float* stc_amax = nullptr;
   // tensor-core M2L (levels >= kTcMinLevel, allocated on the first mixed-precision solve)
   uint4* tab_bf[kMaxLevel + 1] = {};       // per table entry, per field: bf16 hi | bf16 lo << 16
@@ -157,6 +158,7 @@ struct Plan {
   int has_grid = 0;
   uint64_t wait_ns = 2000000000ull;        // limit of every bounded device-side wait
   int inject_stall = 0;                    // test hook: tensor-core MMA issuer stalls
+  int fail_alloc = -1;                     // test hook: the plan's allocation, counted from now, that fails (-1: none)
   int tc_ready = 0;
   int* d_err = nullptr;                    // device error word (bounded waits that gave up)
   int n_off[kMaxLevel + 1] = {};
@@ -221,7 +223,7 @@ inline int tc_first_level(const Plan& P) {
 // the cells around the heaviest clumps).
 constexpr int kSpecTcOrder = 4;
 inline bool spec_tc_level(const Plan& P, int l) {
-  return P.p >= kSpecTcOrder && l >= tc_first_level(P) && !wide_level(P, l) && P.spec_K[l];
+  return P.p >= kSpecTcOrder && l >= tc_first_level(P) && !wide_level(P, l) && P.spec_K[l] && !P.stc_off[l];
 }
 inline bool tc_level(const Plan& P, int l) { return l >= tc_first_level(P) && !spec_tc_level(P, l); }
 

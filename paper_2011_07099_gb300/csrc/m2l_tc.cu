@@ -594,19 +594,25 @@ int make_tc_map(Plan& P, int level) {
       return FMM_ERR_CUDA;
     encode = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn);
   }
-  if (!P.tmapB[level]) P.tmapB[level] = new (std::nothrow) CUtensorMap;
-  if (!P.tmapB[level]) return FMM_ERR_ALLOC;
+  CUtensorMap* map = static_cast<CUtensorMap*>(P.tmapB[level]);
+  if (!map) map = new (std::nothrow) CUtensorMap;
+  if (!map) return FMM_ERR_ALLOC;
   const cuuint64_t kp = (cuuint64_t)tc_padded_k(P.p), W = (cuuint64_t)(1 << (level - 1)) + 2 * kHalo;
   const cuuint64_t dims[5] = {kp, W, W, W, (cuuint64_t)(8 * tc_splits(P, level))};
   const cuuint64_t strides[4] = {kp * 2, kp * 2 * W, kp * 2 * W * W, kp * 2 * W * W * W};
   const cuuint32_t box[5] = {(cuuint32_t)kKC, (cuuint32_t)kBX, (cuuint32_t)(tc_targets(P, level) / (kBX * kBZ)),
                              (cuuint32_t)kBZ, 1};
   const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
-  const CUresult r = encode(static_cast<CUtensorMap*>(P.tmapB[level]), CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5,
+  const CUresult r = encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5,
                             P.Mbf_hi[level], dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
                             CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  return r == CUDA_SUCCESS ? FMM_OK : FMM_ERR_CUDA;
+  if (r != CUDA_SUCCESS) {      // a level with a map counts as prepared: keep none that failed
+    if (!P.tmapB[level]) delete map;
+    return FMM_ERR_CUDA;
+  }
+  P.tmapB[level] = map;
+  return FMM_OK;
 }
 
 cudaError_t launch_build_a(Plan& P, int level, cudaStream_t s) {

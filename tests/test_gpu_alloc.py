@@ -1,0 +1,76 @@
+"""Calls on a plan whose device allocations fail, through the C-ABI and the
+host-side hook FMM_FAULT_ALLOC (the n-th allocation asks for more than any
+device holds): the call falls back or reports FMM_ERR_ALLOC, and the plan then
+solves as it did, with no half-made buffers."""
+import numpy as np
+import pytest
+
+from oracle import fmm as ofmm
+from paper_2011_07099_gb300 import inputs
+from parity_util import assert_close
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+TOL_BF16X3 = 2e-5      # the dense form's bound, as in test_gpu_tensor.py
+
+
+@pytest.fixture(scope="module")
+def B():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2011_07099_gb300 import binding, build
+    build.build()
+    binding.lib()
+    return binding
+
+
+def _solve(B, plan, d):
+    phi, acc = plan.solve(d)
+    torch.cuda.synchronize()
+    assert B.lib().fmm_plan_check(plan.handle) == B.FMM_OK
+    return phi.cpu().numpy(), acc.cpu().numpy()
+
+
+@pytest.mark.parametrize("n", [0, 1, 2, 3])
+def test_a_level_without_room_for_its_tensor_core_spectra_runs_dense(B, n):
+    # the level's allocations, in order: largest mass sums, split weights, split
+    # sources, scales.  The mixed form then runs the dense contraction there,
+    # and a later re-tabulation reaches no missing buffer.
+    N, L, p = 32, 4, 4
+    rho = inputs.lognormal(N, sigma=0.5, seed=9)
+    d = torch.from_numpy(rho).cuda()
+    plan = B.Plan(N, L, p)
+    B.fmm_plan_inject_fault(plan.handle, B.FMM_FAULT_ALLOC + n)
+    plan.set_precision(B.FMM_PREC_BF16X3)
+    got = _solve(B, plan, d)
+    ophi, og = ofmm.solve(rho, L, p)
+    assert_close(got[0], ophi, TOL_BF16X3, f"allocation {n} phi")
+    assert_close(got[1], og, TOL_BF16X3, f"allocation {n} g")
+    theta = torch.zeros(B.fmm_plan_table_grid_size(plan.handle))
+    B.fmm_plan_set_table_grid(plan.handle, theta)          # a zero correction: the same tables again
+    again = _solve(B, plan, d)
+    assert np.array_equal(got[0], again[0]) and np.array_equal(got[1], again[1])
+    plan.close()
+
+
+@pytest.mark.parametrize("n", [0, 1, 2])
+def test_a_first_level_that_cannot_be_prepared_is_not_taken(B, n):
+    # order 2: the dense form's BF16 table, sources and tiles of level 4
+    N, L, p = 32, 5, 2
+    d = torch.from_numpy(inputs.lognormal(N, sigma=0.5, seed=3)).cuda()
+    plan = B.Plan(N, L, p)
+    B.fmm_plan_set_tc_min_level(plan.handle, 5)
+    plan.set_precision(B.FMM_PREC_BF16X3)
+    ref = _solve(B, plan, d)
+    B.fmm_plan_inject_fault(plan.handle, B.FMM_FAULT_ALLOC + n)
+    assert B.lib().fmm_plan_set_tc_min_level(plan.handle, 4) == B.FMM_ERR_ALLOC
+    got = _solve(B, plan, d)                               # level 5 alone, as before
+    assert np.array_equal(got[0], ref[0]) and np.array_equal(got[1], ref[1])
+    B.fmm_plan_set_tc_min_level(plan.handle, 4)            # and with room
+    fresh = B.Plan(N, L, p)
+    fresh.set_precision(B.FMM_PREC_BF16X3)
+    a, b = _solve(B, plan, d), _solve(B, fresh, d)
+    assert np.array_equal(a[0], b[0]) and np.array_equal(a[1], b[1])
+    plan.close()
+    fresh.close()
