@@ -111,6 +111,22 @@ std::vector<int8_t> isolated_level2_offsets() {
   return out;
 }
 
+// Training buffers (alloc_train).
+void free_train(Plan& P) {
+  for (void** b : {&P.tg_la, &P.tg_mh, &P.tg_gh, &P.tg_gl}) {
+    cudaFree(*b);
+    *b = nullptr;
+  }
+  for (float** b : {&P.train_out, &P.lam_cells, &P.dT_all, &P.grad_partials}) {
+    cudaFree(*b);
+    *b = nullptr;
+  }
+  for (int l = 0; l <= fmm::kMaxLevel; ++l) {
+    cudaFree(P.lam[l]);
+    P.lam[l] = P.dT[l] = nullptr;
+  }
+}
+
 void free_plan(Plan* P) {
   if (!P) return;
   cudaFree(P->d_partials);
@@ -139,18 +155,10 @@ void free_plan(Plan* P) {
   cudaFree(P->corr_samples);
   cudaFree(P->corr_val);
   cudaFree(P->corr_up);
-  cudaFree(P->tg_la);
-  cudaFree(P->tg_mh);
-  cudaFree(P->tg_gh);
-  cudaFree(P->tg_gl);
-  cudaFree(P->train_out);
-  cudaFree(P->lam_cells);
-  cudaFree(P->dT_all);
-  cudaFree(P->grad_partials);
+  free_train(*P);
   cudaFree(P->grid);
   cudaFree(P->gmesh);
   fmm::free_fft(*P);
-  for (int l = 0; l <= fmm::kMaxLevel; ++l) cudaFree(P->lam[l]);
   for (int l = 0; l <= fmm::kMaxLevel; ++l) {
     cudaFree(P->tab_bf[l]);
     cudaFree(P->Mbf_hi[l]);
@@ -315,31 +323,41 @@ int retabulate(Plan& P, bool near = true) {
   return cudaDeviceSynchronize() == cudaSuccess ? FMM_OK : FMM_ERR_CUDA;
 }
 
-// Training buffers (first use) and one forward solve, cell residual and
-// adjoint sweep down to the table gradients P.dT of every level; the loss is
-// added to `loss`.  Returns an FMM_* code.
+// Training buffers, all of them or none (FMM_* code); the scratch of the
+// spectral table gradient where it has room.
+int alloc_train(Plan& P) {
+  const size_t n3 = (size_t)P.N * P.N * P.N, p3 = (size_t)P.p * P.p * P.p, E = 8 * P.p - 1;
+  bool ok = plan_alloc(P, &P.train_out, 4 * n3) && plan_alloc(P, &P.lam_cells, 4 * n3) &&
+            plan_alloc(P, &P.dT_all, (size_t)(P.L - 1) * E * E * E * 4) &&
+            plan_alloc(P, &P.grad_partials, (size_t)fmm::mlp_backward_blocks(P) * fmm::mlp::kParams);
+  for (int l = 2; l <= P.L && ok; ++l) ok = plan_alloc(P, &P.lam[l], ((size_t)1 << (3 * l)) * 4 * p3);
+  if (!ok) {
+    free_train(P);
+    return FMM_ERR_ALLOC;
+  }
+  size_t la, mh, gh, gl;
+  fmm::tg_bytes(P, la, mh, gh, gl);
+  if (P.p >= 2 && spectra_fit(la + mh + gh + gl) &&
+      !(plan_alloc(P, &P.tg_mh, mh) && plan_alloc(P, &P.tg_gh, gh) && plan_alloc(P, &P.tg_gl, gl) &&
+        plan_alloc(P, &P.tg_la, la))) {
+    for (void** b : {&P.tg_la, &P.tg_mh, &P.tg_gh, &P.tg_gl}) {   // no room: the direct sums
+      cudaFree(*b);
+      *b = nullptr;
+    }
+  }
+  for (int l = 2; l <= P.L; ++l) P.dT[l] = P.dT_all + (size_t)(l - 2) * E * E * E * 4;
+  return FMM_OK;
+}
+
+// One forward solve, cell residual and adjoint sweep down to the table
+// gradients P.dT of every level; the loss is added to `loss`.  Returns an
+// FMM_* code.
 int table_gradient(Plan& P, const float* density, const float* target_phi, const float* target_acc, float w_phi,
                    float w_g, float* loss, void* stream) {
   const size_t n3 = (size_t)P.N * P.N * P.N;
-  const size_t p3 = (size_t)P.p * P.p * P.p, E = 8 * P.p - 1;
   if (!P.train_out) {
-    bool ok = dev_alloc(&P.train_out, 4 * n3) && dev_alloc(&P.lam_cells, 4 * n3) &&
-              dev_alloc(&P.dT_all, (size_t)(P.L - 1) * E * E * E * 4) &&
-              dev_alloc(&P.grad_partials, (size_t)fmm::mlp_backward_blocks(P) * fmm::mlp::kParams);
-    for (int l = 2; l <= P.L && ok; ++l) ok = dev_alloc(&P.lam[l], ((size_t)1 << (3 * l)) * 4 * p3);
-    if (!ok) return FMM_ERR_ALLOC;
-    size_t la, mh, gh, gl;
-    fmm::tg_bytes(P, la, mh, gh, gl);
-    if (P.p >= 2 && spectra_fit(la + mh + gh + gl) &&
-        (cudaMalloc(&P.tg_mh, mh) != cudaSuccess || cudaMalloc(&P.tg_gh, gh) != cudaSuccess ||
-         cudaMalloc(&P.tg_gl, gl) != cudaSuccess || cudaMalloc(&P.tg_la, la) != cudaSuccess)) {
-      for (void** b : {&P.tg_la, &P.tg_mh, &P.tg_gh, &P.tg_gl}) {   // no room: the direct sums
-        cudaFree(*b);
-        *b = nullptr;
-      }
-      (void)cudaGetLastError();
-    }
-    for (int l = 2; l <= P.L; ++l) P.dT[l] = P.dT_all + (size_t)(l - 2) * E * E * E * 4;
+    const int rc = alloc_train(P);
+    if (rc != FMM_OK) return rc;
   }
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   const int rc = fmm_solve(reinterpret_cast<fmm_plan*>(&P), density, P.train_out, P.train_out + n3, stream);

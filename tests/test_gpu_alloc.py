@@ -74,3 +74,36 @@ def test_a_first_level_that_cannot_be_prepared_is_not_taken(B, n):
     assert np.array_equal(a[0], b[0]) and np.array_equal(a[1], b[1])
     plan.close()
     fresh.close()
+
+
+@pytest.mark.parametrize("n", range(9))
+def test_training_buffers_are_made_all_or_none(B, n):
+    # the call's allocations, in order: solve outputs, residual, table
+    # gradients, network partials, one adjoint (level 2); then the four of the
+    # spectral table gradient, without which the direct sums run
+    N, L, p = 8, 2, 3
+    rho = torch.from_numpy(inputs.lognormal(N, sigma=0.8, seed=2)).cuda()
+    tphi, tg = torch.randn((N, N, N), device="cuda"), torch.randn((3, N, N, N), device="cuda")
+
+    def gradient(plan, fault=None):
+        grad = torch.zeros(B.fmm_plan_table_grid_size(plan.handle), device="cuda")
+        loss = torch.zeros(1, device="cuda")
+        if fault is not None:
+            B.fmm_plan_inject_fault(plan.handle, B.FMM_FAULT_ALLOC + fault)
+        ptr = lambda t: t.data_ptr()
+        rc = B.lib().fmm_table_grid_grad(plan.handle, ptr(rho), ptr(tphi), ptr(tg), 1.0, 1.0, ptr(grad), ptr(loss), 0)
+        torch.cuda.synchronize()
+        return rc, grad.double(), float(loss)
+
+    fresh, plan = B.Plan(N, L, p), B.Plan(N, L, p)
+    rc, want, want_loss = gradient(fresh)
+    assert rc == B.FMM_OK
+    rc, got, _ = gradient(plan, n)
+    assert rc == (B.FMM_ERR_ALLOC if n < 5 else B.FMM_OK)
+    if n < 5:
+        rc, got, loss = gradient(plan)
+        assert rc == B.FMM_OK and loss == want_loss
+    # FP32 sums of ~1e4 terms in another order: 1e-5 of the gradient
+    assert float((got - want).norm() / want.norm()) < 1e-5
+    plan.close()
+    fresh.close()
