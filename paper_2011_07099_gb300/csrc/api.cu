@@ -280,7 +280,9 @@ int alloc_spec(Plan& P) {
   return FMM_OK;
 }
 
-// Scratch for the offset-range partials of the dense wide levels.
+// Scratch for the offset-range partials of the dense wide levels, which
+// follows the length of their interaction lists; the old one is given up only
+// once there is a new one.
 int alloc_m2l_part(Plan& P) {
   size_t part = 0;
   const size_t p3 = (size_t)P.p * P.p * P.p;
@@ -289,9 +291,11 @@ int alloc_m2l_part(Plan& P) {
     const size_t need = 2 * (size_t)fmm::m2l_fp32_splits(P, l) * ((size_t)1 << (3 * l)) * 4 * p3;
     if (need > part) part = need;
   }
+  float* fresh = nullptr;
+  if (part && !plan_alloc(P, &fresh, part)) return FMM_ERR_ALLOC;
   cudaFree(P.m2l_part);
-  P.m2l_part = nullptr;
-  return !part || dev_alloc(&P.m2l_part, part) ? FMM_OK : FMM_ERR_ALLOC;
+  P.m2l_part = fresh;
+  return FMM_OK;
 }
 
 // Re-tabulate every table form from G_S1 plus the plan's corrections (MLP,
@@ -614,23 +618,24 @@ int fmm_plan_set_boundary(fmm_plan* plan, int boundary) {
     all.insert(all.end(), o.begin(), o.end());
   }
   int8_t* offs = nullptr;
-  if (!dev_alloc(&offs, all.size())) return set_err(FMM_ERR_ALLOC);
-  if (cudaMemcpy(offs, all.data(), all.size(), cudaMemcpyHostToDevice) != cudaSuccess) {
+  if (!plan_alloc(P, &offs, all.size())) return set_err(FMM_ERR_ALLOC);
+  const int was = P.n_off[2];
+  P.n_off[2] = count;
+  const int rc = cudaMemcpy(offs, all.data(), all.size(), cudaMemcpyHostToDevice) == cudaSuccess ? alloc_m2l_part(P)
+                                                                                                  : FMM_ERR_CUDA;
+  if (rc != FMM_OK) {                   // the plan keeps its boundary
+    P.n_off[2] = was;
     cudaFree(offs);
-    return set_err(FMM_ERR_CUDA);
+    return set_err(rc);
   }
   cudaFree(P.offsets[2]);
   P.offsets[2] = offs;
-  P.n_off[2] = count;
   P.iso = iso;
   for (int l = 2; l <= P.L; ++l) {      // the tensor cores' sources: a periodic halo, or zeros
     size_t nW, nB, nS;
     fmm::stc_bytes(P, l, nW, nB, nS);
     if (P.stc_B[l]) FMM_CUDA_TRY(cudaMemset(P.stc_B[l], 0, nB));
   }
-  // the offset-range scratch of the coarse levels follows the list length
-  const int rc = alloc_m2l_part(P);
-  if (rc != FMM_OK) return set_err(rc);
   return set_err(retabulate(P));
 }
 

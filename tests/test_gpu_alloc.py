@@ -6,6 +6,7 @@ import numpy as np
 import pytest
 
 from oracle import fmm as ofmm
+from oracle import nonperiodic as npo
 from paper_2011_07099_gb300 import inputs
 from parity_util import assert_close
 
@@ -107,3 +108,24 @@ def test_training_buffers_are_made_all_or_none(B, n):
     assert float((got - want).norm() / want.norm()) < 1e-5
     plan.close()
     fresh.close()
+
+
+@pytest.mark.parametrize("n", [0, 1])
+def test_a_boundary_that_cannot_be_set_is_not_taken(B, n):
+    # order 1 runs the dense sums: the new interaction list, then the scratch
+    # of its offset ranges
+    N, L, p = 8, 3, 1
+    rho = inputs.lognormal(N, sigma=0.5, seed=4)
+    d = torch.from_numpy(rho).cuda()
+    plan = B.Plan(N, L, p)
+    ref = _solve(B, plan, d)
+    B.fmm_plan_inject_fault(plan.handle, B.FMM_FAULT_ALLOC + n)
+    assert B.lib().fmm_plan_set_boundary(plan.handle, B.FMM_BOUNDARY_ISOLATED) == B.FMM_ERR_ALLOC
+    got = _solve(B, plan, d)
+    assert np.array_equal(got[0], ref[0]) and np.array_equal(got[1], ref[1])
+    B.fmm_plan_set_boundary(plan.handle, B.FMM_BOUNDARY_ISOLATED)
+    got = _solve(B, plan, d)
+    ophi, og = npo.solve_isolated(rho, L, p)
+    assert_close(got[0], ophi, 1e-6, "isolated phi")
+    assert_close(got[1], og, 1e-6, "isolated g")
+    plan.close()
