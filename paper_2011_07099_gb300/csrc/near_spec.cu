@@ -34,6 +34,10 @@
 // solve against FP64 went from 3.7e-7 to 2.9e-7 with the direct form, and with
 // FP32 transforms in its place to 3.1e-7 there but from 1.2e-7 to 1.8e-7 at
 // 48^3, S = 6, so the direct form keeps double-float ones.
+// FP32 inverse transforms sum from the highest frequency down (spec.cuh,
+// RISING).  FMM_NEAR_FFT against FP64, 64^3, S = 8, p = 6, potential: radix-2 of
+// 16 points 1.96e-7 (lognormal), 1.62e-7 (clumps); 15-term lines from frequency
+// 0 up 2.28e-7, 1.93e-7; rising 1.86e-7, 1.35e-7, at 256^3 for 0.2 % of a solve.
 #include "fmm_internal.cuh"
 #include "spec.cuh"
 #include "tc_ptx.cuh"
@@ -318,7 +322,7 @@ __global__ void __launch_bounds__(Shape<S>::threads(kItems<S, DFA>)) k_ns_inv(co
       xr[s] = widen<DFA>(store::re(v));
       xi[s] = widen<DFA>(store::im(v));
     }
-    inverse_line<DFA, S>(xr, xi, wt, [&](int z, real re, real im) { t1[(it * S + z) * NM * S + q] = T::pack(re, im); });
+    inverse_line<DFA, S, false, !DFA>(xr, xi, wt, [&](int z, real re, real im) { t1[(it * S + z) * NM * S + q] = T::pack(re, im); });
   }
   __syncthreads();
   for (int l = tid; l < IB * S * S; l += nthr) {           // y: line (item, z, kx), NM -> S
@@ -330,7 +334,7 @@ __global__ void __launch_bounds__(Shape<S>::threads(kItems<S, DFA>)) k_ns_inv(co
       xr[s] = T::re(v);
       xi[s] = T::im(v);
     }
-    inverse_line<DFA, S>(xr, xi, wt, [&](int y, real re, real im) { t2[(iz * S + y) * PS + kx] = T::pack(re, im); });
+    inverse_line<DFA, S, false, !DFA>(xr, xi, wt, [&](int y, real re, real im) { t2[(iz * S + y) * PS + kx] = T::pack(re, im); });
   }
   __syncthreads();
   const size_t N3 = (size_t)N * N * N;
@@ -351,11 +355,11 @@ __global__ void __launch_bounds__(Shape<S>::threads(kItems<S, DFA>)) k_ns_inv(co
     const real* fr = far + l * PS;
     if constexpr (!DFA && S % 4 == 0) {
       float o[S];
-      inverse_real_line<DFA, S>(xr, xi, wt, [&](int x, float v) { o[x] = v + fr[x]; });
+      inverse_real_line<DFA, S, !DFA>(xr, xi, wt, [&](int x, float v) { o[x] = v + fr[x]; });
 #pragma unroll
       for (int q = 0; q < S; q += 4) *reinterpret_cast<float4*>(dst + q) = make_float4(o[q], o[q + 1], o[q + 2], o[q + 3]);
     } else {
-      inverse_real_line<DFA, S>(xr, xi, wt, [&](int x, real v) { dst[x] = narrow<false, DFA>(T::add(v, fr[x])); });
+      inverse_real_line<DFA, S, !DFA>(xr, xi, wt, [&](int x, real v) { dst[x] = narrow<false, DFA>(T::add(v, fr[x])); });
     }
   }
 }

@@ -174,7 +174,11 @@ __device__ __forceinline__ void forward_line(const typename Num<DF>::real (&xr)[
 
 // y_z = sum_{s < NM} x_s e^{+2 pi i z s / NM}; emit(z, re, im) for z < P (ALL:
 // every z < NM).  xr, xi are used up.
-template <bool DF, int P, bool ALL = false, typename Emit>
+// RISING: the sums run from the highest frequency down to 0.  The spectrum of a
+// near field falls off, so the terms then grow along the sum and most of its
+// FP32 roundings are of a small running value; the constant term last costs one
+// addition per output (FMM_NEAR_FFT: near_spec.cu).
+template <bool DF, int P, bool ALL = false, bool RISING = false, typename Emit>
 __device__ __forceinline__ void inverse_line(typename Num<DF>::real (&xr)[2 * P - 1],
                                              typename Num<DF>::real (&xi)[2 * P - 1], const Twiddle<DF, P>& tw,
                                              Emit emit) {
@@ -190,9 +194,10 @@ __device__ __forceinline__ void inverse_line(typename Num<DF>::real (&xr)[2 * P 
     xi[NM - s] = T::add(ai, T::neg(bi));
   }
   {
-    real re = xr[0], im = xi[0];
+    real re = xr[RISING ? P - 1 : 0], im = xi[RISING ? P - 1 : 0];
 #pragma unroll
-    for (int s = 1; s < P; ++s) {
+    for (int i = 1; i < P; ++i) {
+      const int s = RISING ? P - 1 - i : i;
       re = T::add(re, xr[s]);
       im = T::add(im, xi[s]);
     }
@@ -201,12 +206,15 @@ __device__ __forceinline__ void inverse_line(typename Num<DF>::real (&xr)[2 * P 
 #pragma unroll(DF ? 1 : P)
   for (int z = 1; z < P; ++z) {
     real cr = T::zero(), ci = T::zero(), sr = T::zero(), si = T::zero();
-    T::mac(cr, 1.f, 0.f, xr[0]);
-    T::mac(ci, 1.f, 0.f, xi[0]);
-    int j = 0;
+    if (!RISING) {
+      T::mac(cr, 1.f, 0.f, xr[0]);
+      T::mac(ci, 1.f, 0.f, xi[0]);
+    }
+    int j = RISING ? P * z % NM : 0;
 #pragma unroll
-    for (int s = 1; s < P; ++s) {
-      j += z;
+    for (int i = 1; i < P; ++i) {
+      const int s = RISING ? P - i : i;
+      j += RISING ? NM - z : z;
       j -= j >= NM ? NM : 0;
       const float4 w = tw.at(j);
       if (ALL) {
@@ -220,6 +228,10 @@ __device__ __forceinline__ void inverse_line(typename Num<DF>::real (&xr)[2 * P 
         T::mac(cr, -w.z, -w.w, xi[NM - s]);
         T::mac(ci, w.z, w.w, xr[NM - s]);
       }
+    }
+    if (RISING) {
+      T::mac(cr, 1.f, 0.f, xr[0]);
+      T::mac(ci, 1.f, 0.f, xi[0]);
     }
     cr = T::done(cr);
     ci = T::done(ci);
@@ -235,7 +247,7 @@ __device__ __forceinline__ void inverse_line(typename Num<DF>::real (&xr)[2 * P 
 }
 
 // The real points x < P of a half spectrum v[0..P-1]: Re v_0 + 2 sum Re(v_s e^{+2 pi i x s / NM}).
-template <bool DF, int P, typename Emit>
+template <bool DF, int P, bool RISING = false, typename Emit>
 __device__ __forceinline__ void inverse_real_line(const typename Num<DF>::real (&xr)[P],
                                                   const typename Num<DF>::real (&xi)[P], const Twiddle<DF, P>& tw,
                                                   Emit emit) {
@@ -245,10 +257,11 @@ __device__ __forceinline__ void inverse_real_line(const typename Num<DF>::real (
 #pragma unroll(DF ? 1 : P)
   for (int x = 0; x < P; ++x) {
     real a = T::zero();
-    int j = 0;
+    int j = RISING ? P * x % NM : 0;
 #pragma unroll
-    for (int s = 1; s < P; ++s) {
-      j += x;
+    for (int i = 1; i < P; ++i) {
+      const int s = RISING ? P - i : i;
+      j += RISING ? NM - x : x;
       j -= j >= NM ? NM : 0;
       const float4 w = tw.at(j);
       T::mac(a, w.x, w.y, xr[s]);

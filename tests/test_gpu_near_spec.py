@@ -60,3 +60,22 @@ def test_near_zone_isolated_matches_oracle(B, S, L, p):
     ophi, og = npo.solve_isolated(rho, L, p)
     assert_close(phi, ophi, 1e-6, f"isolated phi S={S} L={L} p={p}")
     assert_close(acc, og, 1e-6, f"isolated g S={S} L={L} p={p}")
+
+
+@pytest.mark.parametrize("N,L,p,phi_bound,g_bound", [(64, 3, 6, 1.63e-7, 1.57e-7), (32, 2, 4, 2.33e-7, 1.68e-7)])
+def test_fp32_transforms_round_no_more_than_radix_2_ones(B, N, L, p, phi_bound, g_bound):
+    # FMM_NEAR_FFT against FMM_NEAR_DIRECT, clumped fields, mean of three: the
+    # bounds are what radix-2 FP32 transforms of 16 points differ by from the
+    # sums over pairs on the same fields
+    err = []
+    for seed in (1, 2, 3):
+        d = torch.from_numpy(inputs.plummer(N, n_clumps=16, seed=seed)).cuda()
+        plan = B.Plan(N, L, p)
+        direct = plan.solve(d)
+        B.fmm_plan_set_near_algorithm(plan.handle, B.FMM_NEAR_FFT)
+        fft = plan.solve(d)
+        torch.cuda.synchronize()
+        err.append([float((a.double() - b.double()).norm() / a.double().norm()) for a, b in zip(direct, fft)])
+        plan.close()
+    phi, g = np.mean(err, axis=0)
+    assert phi <= phi_bound and g <= g_bound, (phi, g)
