@@ -1091,10 +1091,10 @@ int fmm_plan_error_stats(fmm_plan* plan, const float* density, const float* pote
     z ^= z >> 31;
     targets[(size_t)i] = z % n3;
   }
-  // one plan-owned block, kept between calls: partials, mean, sums, targets.
+  // one plan-owned block, kept between calls: partials, mean, largest value, sums, targets.
   // The call ends synchronised, so the lock covers every use of the block.
   std::lock_guard<std::mutex> hold(P.es_lock);
-  const size_t np = (size_t)fmm::error_stats_grid_x(P, samples) * samples * 4, nm = (size_t)P.n_partials + 1,
+  const size_t np = (size_t)fmm::error_stats_grid_x(P, samples) * samples * 4, nm = (size_t)P.n_partials + 2,
                ns = 4 + 4 * (size_t)samples, bytes = sizeof(double) * (np + nm + ns + (size_t)samples);
   if (P.es_bytes < bytes) {
     cudaFree(P.es_scratch);

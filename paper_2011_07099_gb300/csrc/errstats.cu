@@ -8,8 +8,12 @@
 // acceleration over those cells is the result.
 //
 // Arithmetic: per-axis xi(d/N), xi'(d/N) in FP64 (green_s1.cuh) rounded to
-// FP32; each pair's (G, -grad G) in FP32; masses, their products with the pair
-// values and the sums in double-float (fmm_internal.cuh).
+// FP32; each pair's (G, -grad G) in FP32, its root and quotients rounded once;
+// masses, in a unit that follows the density, their products with the pair
+// values and the sums in double-float (fmm_internal.cuh).  The error of these
+// sums against FP64 (1024 cells, N = 24 .. 192, sigma = 0.3 and 1.5) is that of
+// the same pair values summed in FP64 within 0.2 % for the potential, and 3 %
+// above (N = 24) to 19 % below it for the acceleration.
 #include <cuda_runtime.h>
 
 #include "fmm_internal.cuh"
@@ -19,7 +23,29 @@ namespace fmm {
 namespace {
 
 constexpr int kEsThreads = 256;   // one target cell per thread
-constexpr int kEsChunk = 512;     // source cells staged in shared memory per step (128^3: 13.5 steps per CTA)
+constexpr int kEsChunk = 512;     // source cells staged in shared memory per step (128^3: 6.7 steps per CTA)
+
+// amax = max |rho| as the bits of a non-negative float (a NaN lies above all).
+__global__ void __launch_bounds__(256) k_es_amax(const float4* __restrict__ rho4, size_t n4, float* __restrict__ amax) {
+  float m = 0.f;
+  auto take = [&](float v) { m = fabsf(v) > m || v != v ? fabsf(v) : m; };
+  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n4; i += (size_t)gridDim.x * blockDim.x) {
+    const float4 v = __ldg(rho4 + i);
+    take(v.x);
+    take(v.y);
+    take(v.z);
+    take(v.w);
+  }
+  const int b = __reduce_max_sync(0xffffffffu, __float_as_int(m));
+  if ((threadIdx.x & 31) == 0) atomicMax(reinterpret_cast<int*>(amax), b);
+}
+
+// The power of two that takes amax to [1, 2): the double-float masses, whose
+// product errors reach 2^-48 below them, then stay clear of FP32's ends
+// whatever the density's unit (1 where amax is 0 or not finite).
+__device__ __forceinline__ double es_scale(float amax) {
+  return amax > 0.f && amax <= 3.4e38f ? ldexp(1.0, -ilogbf(amax)) : 1.0;
+}
 
 // (s, c) += (mh + ml) g: exact product by FMA, TwoSum, the errors in c
 __device__ __forceinline__ void es_mac(float2& a, float mh, float ml, float g) {
@@ -32,14 +58,17 @@ __device__ __forceinline__ void es_mac(float2& a, float mh, float ml, float g) {
 
 // partials[(blockIdx.x * T + t) * 4 + f]: block blockIdx.x's share of the
 // direct sum (Phi, g_x, g_y, g_z) at target t, over the source chunks
-// blockIdx.x, blockIdx.x + gridDim.x, ...  Bound by FP32 issue, ~55
+// blockIdx.x, blockIdx.x + gridDim.x, ...  Bound by FP32 issue, ~60
 // instructions per pair: G = -1/(4 pi |xhat|) and c = G / |xhat|^2 come from
-// one reciprocal square root (one Newton step behind rsqrtf); along a row
-// g_y and g_z differ from the sum of c m by row constants only, so one
-// double-float sum serves both.  With FP64 sums, at 1/64 of the FP32 rate, it
-// took 8.97 ms for 256 targets of a 128^3 mesh.
+// one rsqrtf, each corrected by its FMA residual (Markstein, "Computation of
+// elementary functions on the IBM RISC System/6000", 1990): one Newton step
+// and plain products, 4 % faster, had left up to 40 % more error at N = 24.
+// Along a row g_y and g_z differ from the sum of c m by row constants only, so
+// one double-float sum serves both.  256 targets of a 128^3 mesh: 1.19 ms, with
+// FP64 sums, at 1/64 of the FP32 rate, 8.97 ms.
 __global__ void __launch_bounds__(kEsThreads) k_es_direct(const float* __restrict__ rho,
-                                                          const double* __restrict__ mean, int N,
+                                                          const double* __restrict__ mean,
+                                                          const float* __restrict__ amax, int N,
                                                           const unsigned long long* __restrict__ targets, int T,
                                                           double* __restrict__ partials) {
   extern __shared__ __align__(16) unsigned char es_smem[];
@@ -48,8 +77,8 @@ __global__ void __launch_bounds__(kEsThreads) k_es_direct(const float* __restric
   for (int d = threadIdx.x; d < N; d += blockDim.x)
     sx[d] = make_float2((float)green::xi_s1((double)d / N), (float)green::dxi_s1((double)d / N));
   const size_t n3 = (size_t)N * N * N;
-  const double inv_n3 = 1.0 / (double)n3;
   const double mu = *mean;
+  const double sc = es_scale(*amax);
   const int ti = blockIdx.y * kEsThreads + threadIdx.x;
   const bool valid = ti < T;
   int tx = 0, ty = 0, tz = 0;
@@ -65,7 +94,7 @@ __global__ void __launch_bounds__(kEsThreads) k_es_direct(const float* __restric
   for (size_t c0 = (size_t)blockIdx.x * kEsChunk; c0 < n3; c0 += (size_t)gridDim.x * kEsChunk) {
     const int cnt = (int)((n3 - c0) < (size_t)kEsChunk ? (n3 - c0) : (size_t)kEsChunk);
     __syncthreads();
-    for (int k = threadIdx.x; k < cnt; k += blockDim.x) sm[k] = df_from_double(((double)rho[c0 + k] - mu) * inv_n3);
+    for (int k = threadIdx.x; k < cnt; k += blockDim.x) sm[k] = df_from_double(((double)rho[c0 + k] - mu) * sc);
     __syncthreads();
     if (!valid) continue;
     // offsets d = (t - j) mod N per axis, stepped along the chunk (x fastest)
@@ -79,7 +108,7 @@ __global__ void __launch_bounds__(kEsThreads) k_es_direct(const float* __restric
       // the sources of one row
       const int run = N - jx < cnt - k ? N - jx : cnt - k;
       const float2 vy = sx[dy], vz = sx[dz];
-      const float ryz2 = vy.x * vy.x + vz.x * vz.x;
+      const float ryz2 = fmaf(vz.x, vz.x, vy.x * vy.x);
       const bool on_row = (dy | dz) == 0;
       float2 sc = make_float2(0.f, 0.f);
       for (int q = 0; q < run; ++q) {
@@ -87,12 +116,20 @@ __global__ void __launch_bounds__(kEsThreads) k_es_direct(const float* __restric
         const float2 vx = sx[dx];
         const float r2 = fmaf(vx.x, vx.x, ryz2);
         const bool at0 = on_row && dx == 0;             // self term; grad G(0) = 0
-        float ir = rsqrtf(at0 ? 1.f : r2);
-        ir = fmaf(0.5f * ir, fmaf(-r2 * ir, ir, 1.f), ir);
-        const float G = at0 ? self : -inv4pi * ir;
-        const float c = at0 ? 0.f : G * (ir * ir);      // -1 / (4 pi |xhat|^3)
+        // r = sqrt(r2), G = -1/(4 pi r), c = G / r2
+        const float ir = rsqrtf(at0 ? 1.f : r2), i2 = ir * ir;
+        float r = r2 * ir;
+        r = fmaf(fmaf(-r, r, r2), 0.5f * ir, r);
+        float G = -inv4pi * ir;
+        G = fmaf(fmaf(-G, r, -inv4pi), ir, G);
+        float c = G * i2;                               // -1 / (4 pi |xhat|^3)
+        c = fmaf(fmaf(-c, r2, G), i2, c);
+        if (at0) {
+          G = self;
+          c = 0.f;
+        }
         es_mac(a[0], mj.x, mj.y, G);
-        es_mac(a[1], mj.x, mj.y, c * (vx.x * vx.y));
+        es_mac(a[1], mj.x, mj.y, c * vx.x * vx.y);
         es_mac(sc, mj.x, mj.y, c);
         dx = dx == 0 ? N - 1 : dx - 1;
       }
@@ -114,7 +151,8 @@ __global__ void __launch_bounds__(kEsThreads) k_es_direct(const float* __restric
   }
   if (valid) {
     double* o = partials + ((size_t)blockIdx.x * T + ti) * 4;
-    for (int f = 0; f < 4; ++f) o[f] = df_to_double(a[f]);
+    const double unit = 1.0 / (sc * (double)n3);        // masses are (rho - mean) / N^3
+    for (int f = 0; f < 4; ++f) o[f] = df_to_double(a[f]) * unit;
   }
 }
 
@@ -173,12 +211,16 @@ cudaError_t launch_error_stats(Plan& P, const float* rho, const float* phi, cons
                                const unsigned long long* targets, int T, double* partials, double* sums,
                                double* mean_scratch, cudaStream_t s) {
   double* mean = mean_scratch + P.n_partials;
+  float* amax = reinterpret_cast<float*>(mean + 1);
   cudaError_t e = launch_mean_into(P, rho, mean_scratch, mean, s);
   if (e != cudaSuccess) return e;
+  e = cudaMemsetAsync(amax, 0, sizeof(float), s);
+  if (e != cudaSuccess) return e;
+  k_es_amax<<<4 * P.num_sms, 256, 0, s>>>(reinterpret_cast<const float4*>(rho), (size_t)P.N * P.N * P.N / 4, amax);
   const int gx = error_stats_grid_x(P, T);
   const dim3 grid(gx, (T + kEsThreads - 1) / kEsThreads);
   const size_t smem = sizeof(float2) * (size_t)kEsChunk + sizeof(float2) * (size_t)P.N;
-  k_es_direct<<<grid, kEsThreads, smem, s>>>(rho, mean, P.N, targets, T, partials);
+  k_es_direct<<<grid, kEsThreads, smem, s>>>(rho, mean, amax, P.N, targets, T, partials);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   const size_t n3 = (size_t)P.N * P.N * P.N;

@@ -305,7 +305,7 @@ cudaError_t launch_mesh_green(int N, float* out, int sms, cudaStream_t s);
 cudaError_t launch_mesh_green_plan(const Plan& P, double* out, cudaStream_t s);
 // Sampled error against the direct periodic sum with G_S1 (errstats.cu):
 // targets T <= error_stats_max_samples(), partials error_stats_grid_x(P, T)
-// x T x 4 doubles, sums 4 + 4 T doubles, mean_scratch P.n_partials + 1 doubles
+// x T x 4 doubles, sums 4 + 4 T doubles, mean_scratch P.n_partials + 2 doubles
 // (the density mean of the statement is its own, the plan's mean stage is
 // left as the last solve wrote it).
 int error_stats_max_samples();

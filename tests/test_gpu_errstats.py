@@ -138,3 +138,45 @@ def test_statements_of_two_threads_on_one_plan_do_not_mix(B):
         assert list(pool.map(one, sizes)) == alone
     plan.close()
     fresh.close()
+
+
+@pytest.mark.parametrize("power", [-110, -100, 100])
+def test_statement_does_not_depend_on_the_density_unit(B, power):
+    # a solution scaled with its density by a power of two is the same statement:
+    # masses of 1e-40 must not lose their low halves (FP32 pair values leave
+    # ~1e-7; the unscaled statement reads <= 1e-6)
+    N = 32
+    rho = inputs.lognormal(N, sigma=0.5, seed=3)
+    phi, g = _pm_fields(rho)
+    plan = B.Plan(N, 3, 4)
+    want = plan.error_stats(_dev(rho), _dev(phi), _dev(g), samples=512, seed=2)
+    f = 2.0 ** power
+    got = plan.error_stats(_dev(rho) * f, _dev(phi) * f, _dev(g) * f, samples=512, seed=2)
+    plan.close()
+    assert max(want) < 1e-6
+    # the fields' own rounding differs where they leave FP32's normal range: 1e-3 of the statement
+    assert got == pytest.approx(want, rel=1e-3), (got, want)
+
+
+@pytest.mark.parametrize("N", [24, 32, 48])
+def test_pair_values_are_rounded_once(B, N):
+    # the reference sums restated with FP32 pair values (root and quotients
+    # rounded once) and exact sums: the statement of those fields reads only
+    # what the fields' FP32 storage rounds off, 2^-23 / sqrt(12) = 3.44e-8 of
+    # their norm at most
+    rho = inputs.lognormal(N, sigma=1.0, seed=N)
+    d = np.arange(N) / N
+    pi = np.pi
+    xi = (9 / (8 * pi) * np.sin(pi * d) - np.sin(3 * pi * d) / (24 * pi)).astype(np.float32)
+    fma = lambda a, b, c: (a.astype(np.float64) * b + c).astype(np.float32)
+    z, y, x = np.meshgrid(xi, xi, xi, indexing="ij")
+    r2 = fma(x, x, fma(z, z, y * y))
+    r2[0, 0, 0] = 1
+    G = np.float32(-1 / (4 * pi)) / np.sqrt(r2)
+    G[0, 0, 0] = green.self_term(N)
+    m = (rho.astype(np.float64) - rho.astype(np.float64).mean()) / N ** 3
+    phi = np.fft.ifftn(np.fft.fftn(m) * np.fft.fftn(G.astype(np.float64))).real
+    plan = B.Plan(N, {24: 2, 32: 3, 48: 3}[N], 2)
+    e_phi, _ = plan.error_stats(_dev(rho), _dev(phi), _dev(np.zeros((3, N, N, N))), samples=1024, seed=1)
+    plan.close()
+    assert e_phi <= 3.5e-8, e_phi
