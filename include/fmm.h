@@ -170,10 +170,9 @@ int fmm_plan_mesh_green(const fmm_plan* plan, double* out, void* stream);
 
 /* How M2L evaluates eq. fmm2 at the fine levels.  FMM_M2L_DENSE (default):
  * the sum per offset, on the CUDA cores or, in the mixed forms, the tensor
- * cores, as products of node spectra on (2 order - 1)^3 points; the spectra
- * are allocated with the plan, per level, if they take at most 64 GiB and,
- * from 1 GB up, a quarter of the free memory; without them (and at order 1)
- * the dense contractions run.  FMM_M2L_FFT: the HPM form of Sec. 2, as an ablation: per
+ * cores, as products of node spectra on (2 order - 1)^3 points; where the
+ * spectra have no room (fmm_plan_set_spectra_limit) and at order 1 the dense
+ * contractions run.  FMM_M2L_FFT: the HPM form of Sec. 2, as an ablation: per
  * parent, the gridlet masses of its neighbours' children on a zero-padded
  * (8 order)^3 grid, one FFT convolution with the level table (cuFFT, FP32),
  * and the 27 near nodes' terms subtracted by direct sums; used at the levels
@@ -194,15 +193,38 @@ int fmm_plan_set_m2l_algorithm(fmm_plan* plan, int algorithm);
  * pair of neighbour leaves the S^3 masses zero-padded to (2 S - 1)^3, the
  * 27 x 4 kernel spectra of the near table (FP64, rounded once), FP32 products;
  * FMM_NEAR_DIRECT transforms in double-float.  Other leaves sum directly, as
- * do plans whose spectra had no room at creation (same limits as
- * FMM_M2L_DENSE; 2^(3L) x 72 KB for S = 8: 2.4 GB at 256^3, L = 5).
+ * do plans whose spectra have no room (fmm_plan_set_spectra_limit; 2^(3L) x
+ * 72 KB for S = 8: 2.4 GB at 256^3, L = 5).
  * FMM_NEAR_FFT needs 8-cell leaves (N = 8 * 2^L), FMM_ERR_UNSUPPORTED
- * otherwise, and allocates the spectra if the plan has none (synchronous).
- * FMM_NEAR_DIRECT keeps them.  FMM_ERR_ARG for an unknown value, FMM_ERR_ALLOC
+ * otherwise, and allocates the spectra if the plan has none, whatever the
+ * limit (synchronous).  FMM_NEAR_DIRECT keeps them within it.  FMM_ERR_ARG for an unknown value, FMM_ERR_ALLOC
  * if the spectra do not fit. */
 #define FMM_NEAR_DIRECT 0
 #define FMM_NEAR_FFT    1
 int fmm_plan_set_near_algorithm(fmm_plan* plan, int algorithm);
+
+/* The spectral forms of M2L (orders >= 2), of the near zone (leaves of 4, 6, 8
+ * and 16 cells) and of the training step keep spectra on the device; where
+ * those have no room the dense kernels run, which round differently.  By
+ * default a plan's spectra take at most 96 GB and no more than the memory that
+ * stays free beside them when they are made, so the forms can depend on what
+ * else the device holds then.  fmm_plan_set_spectra_limit sets the limit in
+ * bytes instead (0: dense kernels everywhere; SIZE_MAX: the default again) and
+ * makes the plan's spectra anew, synchronously; FMM_NEAR_FFT's are kept, the
+ * training step's are made on its next use.  FMM_ERR_ALLOC where the buffers of
+ * the forms that follow cannot be made: solves then return that code until the
+ * call succeeds.
+ * fmm_plan_get_forms tells what runs: forms[0] the near zone (DENSE: sums over
+ * pairs), forms[l] the M2L of level l in the present precision and algorithm,
+ * for l < n; *spectra (may be NULL) the bytes held. */
+#define FMM_FORM_NONE        0   /* no such level */
+#define FMM_FORM_DENSE       1   /* dense sums on the CUDA cores */
+#define FMM_FORM_SPECTRAL    2   /* spectral products on the CUDA cores */
+#define FMM_FORM_DENSE_TC    3   /* dense contraction on the tensor cores */
+#define FMM_FORM_SPECTRAL_TC 4   /* spectral products on the tensor cores */
+#define FMM_FORM_FFT         5   /* FMM_M2L_FFT */
+int fmm_plan_set_spectra_limit(fmm_plan* plan, size_t bytes);
+int fmm_plan_get_forms(const fmm_plan* plan, int* forms, int n, size_t* spectra);
 
 /* Limit of every bounded device-side wait (pipeline barriers of the
  * tensor-core M2L), in milliseconds, 1..600000; default 2000.  A wait that

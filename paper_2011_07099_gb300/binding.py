@@ -48,6 +48,8 @@ FMM_STAGE_MULTIPOLE = 0
 FMM_STAGE_LOCAL = 1
 FMM_STAGE_MEAN = 2
 
+FMM_FORM_NONE, FMM_FORM_DENSE, FMM_FORM_SPECTRAL, FMM_FORM_DENSE_TC, FMM_FORM_SPECTRAL_TC, FMM_FORM_FFT = range(6)
+
 # every symbol include/fmm.h declares, with (restype, argtypes)
 _VP, _FP, _I, _SZ = ctypes.c_void_p, ctypes.c_void_p, ctypes.c_int, ctypes.c_size_t
 SIGNATURES = {
@@ -76,6 +78,8 @@ SIGNATURES = {
     "fmm_plan_set_green_mesh": (_I, [_VP, _FP, _SZ]),
     "fmm_plan_set_m2l_algorithm": (_I, [_VP, _I]),
     "fmm_plan_set_near_algorithm": (_I, [_VP, _I]),
+    "fmm_plan_set_spectra_limit": (_I, [_VP, _SZ]),
+    "fmm_plan_get_forms": (_I, [_VP, ctypes.POINTER(_I), _I, ctypes.POINTER(_SZ)]),
     "fmm_plan_set_tc_tile": (_I, [_VP, _I, _I]),
     "fmm_plan_autotune_tiles": (_I, [_VP, _VP, ctypes.POINTER(ctypes.c_int), _I, _VP]),
     "fmm_batch_set_near_algorithm": (_I, [_VP, _I]),
@@ -246,6 +250,21 @@ def fmm_plan_set_m2l_algorithm(plan, algorithm):
 
 def fmm_plan_set_near_algorithm(plan, algorithm):
     _check(lib().fmm_plan_set_near_algorithm(plan, int(algorithm)), "fmm_plan_set_near_algorithm")
+
+
+def fmm_plan_set_spectra_limit(plan, nbytes):
+    """nbytes: the most the plan's spectra may take (0: dense kernels), or None for the default rule."""
+    n = 2 ** (8 * ctypes.sizeof(_SZ)) - 1 if nbytes is None else int(nbytes)
+    _check(lib().fmm_plan_set_spectra_limit(plan, n), "fmm_plan_set_spectra_limit")
+
+
+def fmm_plan_get_forms(plan):
+    """(forms, bytes): FMM_FORM_* of the near zone ([0]) and of the M2L of every level, and the spectra's bytes."""
+    L, n = ctypes.c_int(), _SZ(0)
+    _check(lib().fmm_plan_get_shape(plan, None, ctypes.byref(L), None, None), "fmm_plan_get_shape")
+    out = (ctypes.c_int * (L.value + 1))()
+    _check(lib().fmm_plan_get_forms(plan, out, L.value + 1, ctypes.byref(n)), "fmm_plan_get_forms")
+    return list(out), int(n.value)
 
 
 def fmm_plan_set_tc_tile(plan, level, targets):

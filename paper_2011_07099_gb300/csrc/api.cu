@@ -127,6 +127,30 @@ void free_train(Plan& P) {
   }
 }
 
+void free_near_spec(Plan& P) {
+  for (void** b : {&P.ns_K, &P.ns_M, &P.ns_P}) {
+    cudaFree(*b);
+    *b = nullptr;
+  }
+}
+
+// A level's spectra: of the CUDA cores and, without them or alone, of the tensor cores.
+void free_stc(Plan& P, int l) {
+  for (void** b : {&P.stc_W[l], &P.stc_B[l], reinterpret_cast<void**>(&P.stc_scale[l])}) {
+    cudaFree(*b);
+    *b = nullptr;
+  }
+  delete static_cast<CUtensorMap*>(P.stc_map[l]);
+  P.stc_map[l] = nullptr;
+}
+void free_spec(Plan& P, int l) {
+  free_stc(P, l);
+  for (void** b : {&P.spec_K[l], &P.spec_M[l], &P.spec_P[l]}) {
+    cudaFree(*b);
+    *b = nullptr;
+  }
+}
+
 void free_plan(Plan* P) {
   if (!P) return;
   cudaFree(P->d_partials);
@@ -140,15 +164,11 @@ void free_plan(Plan* P) {
     cudaFree(P->F64[l]);
     cudaFree(P->M64[l]);
     cudaFree(P->offsets[l]);
-    cudaFree(P->spec_K[l]);
-    cudaFree(P->spec_M[l]);
-    cudaFree(P->spec_P[l]);
+    free_spec(*P, l);
   }
   cudaFree(P->spec_tw);
   cudaFree(P->near_tab);
-  cudaFree(P->ns_K);
-  cudaFree(P->ns_M);
-  cudaFree(P->ns_P);
+  free_near_spec(*P);
   cudaFree(P->ns_tw);
   cudaFree(P->d_err);
   cudaFree(P->corr_w);
@@ -164,10 +184,6 @@ void free_plan(Plan* P) {
     cudaFree(P->Mbf_hi[l]);
     cudaFree(P->Apre[l]);
     delete static_cast<CUtensorMap*>(P->tmapB[l]);
-    cudaFree(P->stc_W[l]);
-    cudaFree(P->stc_scale[l]);
-    cudaFree(P->stc_B[l]);
-    delete static_cast<CUtensorMap*>(P->stc_map[l]);
   }
   cudaFree(P->stc_amax);
   cudaFree(P->es_scratch);
@@ -205,18 +221,45 @@ bool plan_alloc(Plan& P, T** ptr, size_t count) {
 }
 bool plan_alloc(Plan& P, void** ptr, size_t bytes) { return plan_alloc(P, reinterpret_cast<char**>(ptr), bytes); }
 
-// Buffers of the spectral M2L (m2l_spec.cu) for every level of orders >= 2
-// whose spectra take at most kSpecMaxBytes; a level that has none, or whose
-// allocation fails (the dense kernels need ~20 times less memory), keeps the
-// dense contraction.
-constexpr size_t kSpecMaxBytes = (size_t)64 << 30;
-// ... and, from 1 GB up, at most a quarter of the memory that is free: a plan
-// that fits with the dense forms leaves the caller room with these.
-bool spectra_fit(size_t bytes) {
-  if (bytes > kSpecMaxBytes) return false;
-  if (bytes < ((size_t)1 << 30)) return true;
+// Spectra are optional: the dense kernels need ~20 times less memory.  A plan
+// holds at most what its caller allows (fmm_plan_set_spectra_limit) or, by
+// default, kSpecMaxBytes and no more than the memory that stays free beside
+// them, counted over all its sets of buffers: the M2L levels (m2l_spec.cu,
+// m2l_spec_tc.cu), the near zone (near_spec.cu), the training step
+// (learn_spec.cu).  A set that has no room, or whose allocation fails, is left
+// out and its dense kernels run.
+constexpr size_t kSpecMaxBytes = (size_t)96 << 30;
+
+size_t spectra_bytes(const Plan& P) {
+  size_t sum = 0, a, b, c, d;
+  for (int l = 2; l <= P.L; ++l) {
+    if (P.spec_K[l]) sum += fmm::spec_kernel_bytes(P, l) + fmm::spec_source_bytes(P, l) + fmm::spec_target_bytes(P, l);
+    if (P.stc_map[l]) {
+      fmm::stc_bytes(P, l, a, b, c);
+      sum += a + b + c;
+    }
+  }
+  if (P.ns_K) {
+    fmm::near_spec_bytes(P, a, b, c);
+    sum += a + b + c;
+  }
+  if (P.tg_la) {
+    fmm::tg_bytes(P, a, b, c, d);
+    sum += a + b + c + d;
+  }
+  return sum;
+}
+
+bool spectra_fit(const Plan& P, size_t bytes) {
+  const size_t held = spectra_bytes(P), want = held + bytes;
+  if (P.spec_limit != SIZE_MAX) return want <= P.spec_limit;
+  if (want > kSpecMaxBytes) return false;
   size_t free_b = 0, total = 0;
-  return cudaMemGetInfo(&free_b, &total) != cudaSuccess || bytes <= free_b / 4;
+  if (cudaMemGetInfo(&free_b, &total) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return true;
+  }
+  return want <= (free_b + held) / 2;
 }
 
 // (cos, sin) of 2 pi j / (2 points - 1) as (hi, lo) FP32 pairs.
@@ -233,44 +276,38 @@ int make_twiddles(int points, float4** out) {
 }
 
 // Buffers of the near zone's spectral products (near_spec.cu) for the leaf
-// sizes it is built for; without them the direct kernels run.
+// sizes it is built for; `asked`: the caller names them (FMM_NEAR_FFT), so the
+// limit does not apply.
 int alloc_near_spec(Plan& P, bool asked) {
   if (P.ns_K || !fmm::near_spec_shape(P)) return FMM_OK;
   size_t nK, nM, nP;
   fmm::near_spec_bytes(P, nK, nM, nP);
-  if (!asked && !spectra_fit(nK + nM + nP)) return FMM_OK;
+  if (!asked && !spectra_fit(P, nK + nM + nP)) return FMM_OK;
   if (!P.ns_tw) {
     const int rc = make_twiddles(P.S, &P.ns_tw);
     if (rc != FMM_OK) return rc;
   }
-  if (cudaMalloc(&P.ns_M, nM) != cudaSuccess || cudaMalloc(&P.ns_P, nP) != cudaSuccess ||
-      cudaMalloc(&P.ns_K, nK) != cudaSuccess) {
-    cudaFree(P.ns_K);
-    cudaFree(P.ns_M);
-    cudaFree(P.ns_P);
-    P.ns_K = P.ns_M = P.ns_P = nullptr;
-    (void)cudaGetLastError();
+  if (!plan_alloc(P, &P.ns_M, nM) || !plan_alloc(P, &P.ns_P, nP) || !plan_alloc(P, &P.ns_K, nK)) {
+    free_near_spec(P);
     return FMM_OK;
   }
   // the padding frequencies, and the all-zero spectrum of out-of-box leaves
   return cudaMemset(P.ns_K, 0, nK) == cudaSuccess && cudaMemset(P.ns_M, 0, nM) == cudaSuccess ? FMM_OK : FMM_ERR_CUDA;
 }
 
+// Buffers of the spectral M2L for every level of orders >= 2, the coarse first.
 int alloc_spec(Plan& P) {
   if (P.p < 2) return FMM_OK;
-  const int rc = make_twiddles(P.p, &P.spec_tw);
-  if (rc != FMM_OK) return rc;
+  if (!P.spec_tw) {
+    const int rc = make_twiddles(P.p, &P.spec_tw);
+    if (rc != FMM_OK) return rc;
+  }
   for (int l = 2; l <= P.L; ++l) {
     const size_t nk = fmm::spec_kernel_bytes(P, l), ns = fmm::spec_source_bytes(P, l),
                  nt = fmm::spec_target_bytes(P, l);
-    if (!spectra_fit(nk + ns + nt)) continue;
-    if (cudaMalloc(&P.spec_K[l], nk) != cudaSuccess || cudaMalloc(&P.spec_M[l], ns) != cudaSuccess ||
-        cudaMalloc(&P.spec_P[l], nt) != cudaSuccess) {
-      cudaFree(P.spec_K[l]);
-      cudaFree(P.spec_M[l]);
-      cudaFree(P.spec_P[l]);
-      P.spec_K[l] = P.spec_M[l] = P.spec_P[l] = nullptr;
-      (void)cudaGetLastError();
+    if (!spectra_fit(P, nk + ns + nt)) continue;
+    if (!plan_alloc(P, &P.spec_M[l], ns) || !plan_alloc(P, &P.spec_P[l], nt) || !plan_alloc(P, &P.spec_K[l], nk)) {
+      free_spec(P, l);
       continue;
     }
     // the padding frequencies, and the all-zero spectrum of out-of-box nodes
@@ -296,6 +333,16 @@ int alloc_m2l_part(Plan& P) {
   cudaFree(P.m2l_part);
   P.m2l_part = fresh;
   return FMM_OK;
+}
+
+// How the M2L of level l runs in the plan's present settings (FMM_FORM_*).
+int m2l_form(const Plan& P, int l) {
+  if (fmm::fft_level(P, l)) return FMM_FORM_FFT;
+  if (P.prec != FMM_PREC_FP32 && P.tc_ready) {
+    if (fmm::spec_tc_level(P, l)) return FMM_FORM_SPECTRAL_TC;
+    if (fmm::tc_level(P, l)) return FMM_FORM_DENSE_TC;
+  }
+  return P.spec_K[l] ? FMM_FORM_SPECTRAL : FMM_FORM_DENSE;
 }
 
 // Re-tabulate every table form from G_S1 plus the plan's corrections (MLP,
@@ -341,7 +388,7 @@ int alloc_train(Plan& P) {
   }
   size_t la, mh, gh, gl;
   fmm::tg_bytes(P, la, mh, gh, gl);
-  if (P.p >= 2 && spectra_fit(la + mh + gh + gl) &&
+  if (P.p >= 2 && spectra_fit(P, la + mh + gh + gl) &&
       !(plan_alloc(P, &P.tg_mh, mh) && plan_alloc(P, &P.tg_gh, gh) && plan_alloc(P, &P.tg_gl, gl) &&
         plan_alloc(P, &P.tg_la, la))) {
     for (void** b : {&P.tg_la, &P.tg_mh, &P.tg_gh, &P.tg_gl}) {   // no room: the direct sums
@@ -537,20 +584,14 @@ int prepare_stc(Plan& P, int l) {
   size_t nW, nB, nS;
   fmm::stc_bytes(P, l, nW, nB, nS);
   int rc = FMM_ERR_ALLOC;
-  if ((P.stc_amax || plan_alloc(P, &P.stc_amax, (size_t)fmm::kMaxLevel + 1)) && plan_alloc(P, &P.stc_W[l], nW) &&
-      plan_alloc(P, &P.stc_B[l], nB) && plan_alloc(P, &P.stc_scale[l], nS / sizeof(float))) {
+  if (spectra_fit(P, nW + nB + nS) && (P.stc_amax || plan_alloc(P, &P.stc_amax, (size_t)fmm::kMaxLevel + 1)) &&
+      plan_alloc(P, &P.stc_W[l], nW) && plan_alloc(P, &P.stc_B[l], nB) && plan_alloc(P, &P.stc_scale[l], nS / sizeof(float))) {
     // the halo of the isolated problem stays zero
     rc = cudaMemset(P.stc_B[l], 0, nB) == cudaSuccess && fmm::launch_stc_weights(P, l, 0) == cudaSuccess
              ? fmm::make_stc_map(P, l)
              : FMM_ERR_CUDA;
   }
-  if (rc != FMM_OK) {
-    cudaFree(P.stc_W[l]);
-    cudaFree(P.stc_B[l]);
-    cudaFree(P.stc_scale[l]);
-    P.stc_W[l] = P.stc_B[l] = nullptr;
-    P.stc_scale[l] = nullptr;
-  }
+  if (rc != FMM_OK) free_stc(P, l);
   return rc;
 }
 
@@ -600,6 +641,39 @@ int fmm_plan_set_precision(fmm_plan* plan, int mode) {
     if (rc != FMM_OK) return set_err(rc);
   }
   P.prec = mode;
+  return set_err(FMM_OK);
+}
+
+int fmm_plan_set_spectra_limit(fmm_plan* plan, size_t bytes) {
+  if (!plan) return set_err(FMM_ERR_ARG);
+  Plan& P = *reinterpret_cast<Plan*>(plan);
+  FMM_CUDA_TRY(cudaDeviceSynchronize());
+  P.spec_limit = bytes;
+  // every set again within the limit; the training step's on its next use.
+  // Until all is made the plan solves nothing (P.unmade).
+  for (int l = 2; l <= P.L; ++l) {
+    free_spec(P, l);
+    P.stc_off[l] = false;
+  }
+  free_near_spec(P);
+  free_train(P);
+  int rc = alloc_spec(P);
+  if (rc == FMM_OK) rc = alloc_near_spec(P, P.near_fft != 0);
+  if (rc == FMM_OK && P.near_fft && !P.ns_K) rc = FMM_ERR_ALLOC;
+  if (rc == FMM_OK) rc = alloc_m2l_part(P);
+  if (rc == FMM_OK && P.tc_ready) rc = prepare_tc(P);
+  if (rc == FMM_OK) rc = retabulate(P);
+  P.unmade = rc;
+  return set_err(rc);
+}
+
+int fmm_plan_get_forms(const fmm_plan* plan, int* forms, int n, size_t* spectra) {
+  if (!plan || n < 0 || (n > 0 && !forms)) return set_err(FMM_ERR_ARG);
+  const Plan& P = *reinterpret_cast<const Plan*>(plan);
+  for (int l = 0; l < n; ++l)
+    forms[l] = l == 0 ? (P.ns_K ? FMM_FORM_SPECTRAL : FMM_FORM_DENSE)
+                      : (l >= 2 && l <= P.L ? m2l_form(P, l) : FMM_FORM_NONE);
+  if (spectra) *spectra = spectra_bytes(P);
   return set_err(FMM_OK);
 }
 
@@ -686,6 +760,7 @@ int fmm_plan_set_near_algorithm(fmm_plan* plan, int algorithm) {
   if (algorithm == FMM_NEAR_DIRECT) {
     if (cudaDeviceSynchronize() != cudaSuccess) return set_err(FMM_ERR_CUDA);
     P.near_fft = 0;
+    if (P.spec_limit != SIZE_MAX && spectra_bytes(P) > P.spec_limit) free_near_spec(P);
     return set_err(FMM_OK);
   }
   if (P.S != 8) return set_err(FMM_ERR_UNSUPPORTED);
@@ -929,6 +1004,7 @@ int fmm_solve(fmm_plan* plan, const float* density, float* potential, float* acc
   if (!plan || !density || !potential || !accel) return set_err(FMM_ERR_ARG);
   if (!aligned16(density) || !aligned16(potential) || !aligned16(accel)) return set_err(FMM_ERR_ARG);
   Plan& P = *reinterpret_cast<Plan*>(plan);
+  if (P.unmade != FMM_OK) return set_err(P.unmade);
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   const bool t = P.timing != 0;
   auto mark = [&](int slot, int end) -> cudaError_t {
@@ -940,8 +1016,6 @@ int fmm_solve(fmm_plan* plan, const float* density, float* potential, float* acc
   else
     FMM_CUDA_TRY(fmm::launch_mean(P, density, s));
   FMM_CUDA_TRY(mark(FMM_TIME_MEAN, 1));
-  const bool tc = P.prec != FMM_PREC_FP32 && P.tc_ready;
-  auto on_tc = [&](int l) { return !fmm::fft_level(P, l) && tc && fmm::tc_level(P, l); };
   // Untimed solves overlap independent stages: the near zone's spectral sums
   // need only the density and its mean (second auxiliary stream, from the mean
   // on), and fill what the small launches of the tree passes leave idle; the
@@ -963,13 +1037,14 @@ int fmm_solve(fmm_plan* plan, const float* density, float* potential, float* acc
   for (int l = P.L - 1; l >= 2; --l) FMM_CUDA_TRY(fmm::launch_m2m(P, l, s));
   FMM_CUDA_TRY(mark(FMM_TIME_M2M, 1));
   FMM_CUDA_TRY(mark(FMM_TIME_M2L, 0));
-  auto on_stc = [&](int l) { return !fmm::fft_level(P, l) && tc && fmm::spec_tc_level(P, l); };
-  auto on_spec = [&](int l) { return !fmm::fft_level(P, l) && !on_tc(l) && !on_stc(l) && P.spec_K[l]; };
+  auto on_tensor = [&](int l) { return m2l_form(P, l) == FMM_FORM_SPECTRAL_TC || m2l_form(P, l) == FMM_FORM_DENSE_TC; };
+  auto on_spec = [&](int l) { return m2l_form(P, l) == FMM_FORM_SPECTRAL; };
   // one level on its own: FFT ablation, tensor cores or the dense CUDA-core kernels
   auto m2l_level = [&](int l, cudaStream_t q) -> cudaError_t {
-    if (fmm::fft_level(P, l)) return fmm::launch_m2l_fft(P, l, q);
-    if (on_stc(l)) return fmm::launch_m2l_spec_tc(P, l, q);
-    if (!on_tc(l)) return fmm::launch_m2l_fp32(P, l, q);
+    const int form = m2l_form(P, l);
+    if (form == FMM_FORM_FFT) return fmm::launch_m2l_fft(P, l, q);
+    if (form == FMM_FORM_SPECTRAL_TC) return fmm::launch_m2l_spec_tc(P, l, q);
+    if (form == FMM_FORM_DENSE) return fmm::launch_m2l_fp32(P, l, q);
     const cudaError_t e = fmm::launch_split_bf16(P, l, q);
     return e != cudaSuccess ? e : fmm::launch_m2l_tc(P, l, P.prec, q);
   };
@@ -978,15 +1053,15 @@ int fmm_solve(fmm_plan* plan, const float* density, float* potential, float* acc
     // auxiliary stream: the double-float spectral levels and the rest
     bool side = false, main = false;
     for (int l = 2; l <= P.L; ++l) {
-      if (on_tc(l) || on_stc(l) || (on_spec(l) && !fmm::wide_level(P, l))) main = true;
+      if (on_tensor(l) || (on_spec(l) && !fmm::wide_level(P, l))) main = true;
       else side = true;
     }
     const bool fork = side && main;
     cudaStream_t q = fork ? P.aux[0] : s;
     if (fork) FMM_CUDA_TRY(cudaEventRecord(P.fev[2], s));
     for (int l = P.L; l >= 2; --l)
-      if (on_tc(l) || on_stc(l)) FMM_CUDA_TRY(m2l_level(l, s));
-    int f0 = P.L + 1, f1 = 1, d0 = P.L + 1, d1 = 1;   // spectral levels: wide_level and on_tc split them by depth
+      if (on_tensor(l)) FMM_CUDA_TRY(m2l_level(l, s));
+    int f0 = P.L + 1, f1 = 1, d0 = P.L + 1, d1 = 1;   // spectral levels: wide_level and on_tensor split them by depth
     for (int l = 2; l <= P.L; ++l) {
       if (!on_spec(l)) continue;
       int &lo = fmm::wide_level(P, l) ? d0 : f0, &hi = fmm::wide_level(P, l) ? d1 : f1;
@@ -997,7 +1072,7 @@ int fmm_solve(fmm_plan* plan, const float* density, float* potential, float* acc
     if (fork) FMM_CUDA_TRY(cudaStreamWaitEvent(q, P.fev[2], 0));
     if (d0 <= d1) FMM_CUDA_TRY(fmm::launch_m2l_spec(P, true, d0, d1, q));
     for (int l = 2; l <= P.L; ++l)
-      if (!on_tc(l) && !on_stc(l) && !on_spec(l)) FMM_CUDA_TRY(m2l_level(l, q));
+      if (!on_tensor(l) && !on_spec(l)) FMM_CUDA_TRY(m2l_level(l, q));
     if (fork) {
       FMM_CUDA_TRY(cudaEventRecord(P.fev[3], q));
       FMM_CUDA_TRY(cudaStreamWaitEvent(s, P.fev[3], 0));

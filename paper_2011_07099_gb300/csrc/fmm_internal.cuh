@@ -102,6 +102,10 @@ struct Plan {
   void* spec_M[kMaxLevel + 1] = {};
   void* spec_P[kMaxLevel + 1] = {};
   float4* spec_tw = nullptr;
+  // the caller's limit on all optional spectra (SIZE_MAX: the default rule), and
+  // the error of a limit whose buffers could not be made (no solve until then)
+  size_t spec_limit = SIZE_MAX;
+  int unmade = FMM_OK;
   // the same products on the tensor cores (m2l_spec_tc.cu), levels the mixed
   // forms take there: split weights and their scales, split source spectra,
   // the tensor map (host CUtensorMap) and each level's largest mass sum

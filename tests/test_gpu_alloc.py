@@ -129,3 +129,46 @@ def test_a_boundary_that_cannot_be_set_is_not_taken(B, n):
     assert_close(got[0], ophi, 1e-6, "isolated phi")
     assert_close(got[1], og, 1e-6, "isolated g")
     plan.close()
+
+
+def test_spectra_limit_sets_the_forms_and_is_undone_bitwise(B):
+    N, L, p = 64, 4, 4
+    d = torch.from_numpy(inputs.lognormal(N, sigma=0.5, seed=7)).cuda()
+    plan = B.Plan(N, L, p, precision=B.FMM_PREC_BF16X3)
+    forms, held = B.fmm_plan_get_forms(plan.handle)
+    S, D, T, C = B.FMM_FORM_SPECTRAL, B.FMM_FORM_DENSE, B.FMM_FORM_DENSE_TC, B.FMM_FORM_SPECTRAL_TC
+    assert forms == [S, B.FMM_FORM_NONE, S, S, C] and held > 0
+    ref = _solve(B, plan, d)
+    B.fmm_plan_set_spectra_limit(plan.handle, 0)
+    assert B.fmm_plan_get_forms(plan.handle) == ([D, B.FMM_FORM_NONE, D, D, T], 0)
+    dense = _solve(B, plan, d)
+    assert_close(dense[0], ref[0], 2e-5, "dense against spectral phi")
+    B.fmm_plan_set_near_algorithm(plan.handle, B.FMM_NEAR_DIRECT)
+    assert B.fmm_plan_get_forms(plan.handle)[1] == 0
+    for limit in (6 << 20, 1 << 25):                # level 2 fits (5.4 MB); levels 2 and 3 (18 MB)
+        B.fmm_plan_set_spectra_limit(plan.handle, limit)
+        f, b = B.fmm_plan_get_forms(plan.handle)
+        assert 0 < b <= limit and f[2] == S and f[0] == D, (f, b)
+    B.fmm_plan_set_spectra_limit(plan.handle, None)
+    assert B.fmm_plan_get_forms(plan.handle) == (forms, held)
+    got = _solve(B, plan, d)
+    assert np.array_equal(got[0], ref[0]) and np.array_equal(got[1], ref[1])
+    plan.close()
+
+
+def test_a_limit_whose_buffers_cannot_be_made_stops_the_solves(B):
+    # the scratch of the dense coarse levels is the only allocation of the limit 0 in the plain form
+    N, L, p = 16, 3, 4
+    d = torch.from_numpy(inputs.lognormal(N, sigma=0.5, seed=8)).cuda()
+    plan, fresh = B.Plan(N, L, p), B.Plan(N, L, p)
+    B.fmm_plan_inject_fault(plan.handle, B.FMM_FAULT_ALLOC + 0)
+    assert B.lib().fmm_plan_set_spectra_limit(plan.handle, 0) == B.FMM_ERR_ALLOC
+    with pytest.raises(B.FMMError) as e:
+        plan.solve(d)
+    assert e.value.code == B.FMM_ERR_ALLOC
+    for pl in (plan, fresh):
+        B.fmm_plan_set_spectra_limit(pl.handle, 0)
+    a, b = _solve(B, plan, d), _solve(B, fresh, d)
+    assert np.array_equal(a[0], b[0]) and np.array_equal(a[1], b[1])
+    plan.close()
+    fresh.close()
