@@ -270,7 +270,8 @@ int make_stc_map(Plan& P, int level);
 cudaError_t setup_spec_tc(const Plan& P);
 cudaError_t launch_stc_weights(Plan& P, int level, cudaStream_t s);
 cudaError_t launch_m2l_spec_tc(Plan& P, int level, cudaStream_t s);
-// FP32 spectra of `blocks` order-p gridlets, [chunk][blocks + 1][16].
+// FP32 spectra of `blocks` order-p gridlets, [chunk][blocks + 1][16], transformed
+// in double-float.
 cudaError_t launch_spec_fwd(Plan& P, const float* src, void* dst, size_t blocks, cudaStream_t s);
 cudaError_t launch_m2l_spec(Plan& P, bool df, int l0, int l1, cudaStream_t s);
 cudaError_t launch_l2l(Plan& P, int level, cudaStream_t s);       // F[level] -> F[level+1] (adds)

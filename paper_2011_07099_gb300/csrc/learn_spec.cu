@@ -9,8 +9,7 @@
 //   g^_o(k) = sum_T lam^_T(k) conj(M^_{T-o}(k)),
 // one complex multiply-add per frequency and field where the direct sum over
 // (r, d) takes p^6 / NK times as many.  Measured at 64^3, p = 6 (levels 2 + 3,
-// 8 fields): 224 ms for the direct sums; the whole training step of 8 fields
-// 381 -> 15.5 ms with both changes of this file.
+// 8 fields): 224 ms for the direct sums, 2.3 ms here.
 //
 // Correction.  The network sees a table entry only through the sorted absolute
 // components of its (nearest-image) offset, so the (8p-1)^3 x 4 entries of a
@@ -31,10 +30,12 @@ using spec::inverse_line;
 using spec::Num;
 using spec::Shape;
 using spec::Twiddle;
+using spec::widen;
 
 constexpr int kOff3 = 343;
 constexpr int kLn = 16;                 // frequencies per chunk (FP32)
 constexpr int kTgGroups = 8;            // target rows in flight per CTA
+constexpr int kTgChain = 32;            // steps (of two targets) per FP32 chain
 
 // Offsets a child at position c of its parent takes, per axis.
 template <int MODE>   // 0: levels >= 3; 1: level 2, periodic
@@ -45,12 +46,33 @@ __device__ __forceinline__ constexpr bool allowed(int c, int o) {
 // CTA: one row of offsets (oy, oz; the 7 ox) x one chunk of 16 frequencies.
 // Lane: a frequency; the 8 groups of 16 lanes walk the (z, y) rows of targets,
 // two targets (one parent's x pair) per step, whose 6 sources along x serve
-// both.  56 sums per thread, added over the groups at the end.  Bound by the
-// FP32 pipe (192 multiply-adds per 14 eight-byte loads from L1/L2).
+// both.  56 sums per thread; every kTgChain steps they are added to the group's
+// totals in shared memory, so that the FP32 chains do not grow with the level;
+// the groups are added at the end.  Bound by the FP32 pipe (192 multiply-adds
+// per 14 eight-byte loads from L1/L2).
+// Error of the table gradient against FP64, relative, at the leaf level: direct
+// sums 7.0e-8 to 7.9e-8 (128^3, L = 5, p = 4), 6.6e-8 to 7.8e-8 (192^3, L = 6,
+// p = 3); with one chain per group and FP32 transforms 1.4e-7 to 1.7e-7, 3.3e-7
+// to 3.6e-7; with these chains and double-float transforms, rounded on store,
+// 6.2e-8 to 7.9e-8, 6.6e-8 to 7.7e-8.  The training step of 8 fields at 64^3,
+// p = 6 takes 7.4 ms with them, 6.6 without.
 template <int MODE>
 __device__ __forceinline__ void tg_rows(const float2* __restrict__ La, const float2* __restrict__ Mh, int level, int oy,
-                                        int oz, int grp, float2 (&acc)[7][4]) {
+                                        int oz, int grp, float2 (*tot)[kLn]) {
   const int n = 1 << level;
+  float2 acc[7][4];
+  auto flush = [&](bool first) {
+#pragma unroll
+    for (int i = 0; i < 7; ++i)
+#pragma unroll
+      for (int f = 0; f < 4; ++f) {
+        float2& t = tot[i * 4 + f][0];
+        t = first ? make_float2(0.f, 0.f) : make_float2(t.x + acc[i][f].x, t.y + acc[i][f].y);
+        acc[i][f] = make_float2(0.f, 0.f);
+      }
+  };
+  flush(true);
+  int steps = 0;
   const bool near = oy >= -1 && oy <= 1 && oz >= -1 && oz <= 1;
   for (int r = grp; r < n * n; r += kTgGroups) {
     const int y = r % n, z = r / n;
@@ -82,8 +104,13 @@ __device__ __forceinline__ void tg_rows(const float2* __restrict__ La, const flo
           }
         }
       }
+      if (++steps == kTgChain) {
+        flush(false);
+        steps = 0;
+      }
     }
   }
+  flush(false);
 }
 
 __global__ void __launch_bounds__(kLn* kTgGroups) k_tg_mac(const float2* __restrict__ La, const float2* __restrict__ Mh,
@@ -93,20 +120,12 @@ __global__ void __launch_bounds__(kLn* kTgGroups) k_tg_mac(const float2* __restr
   const size_t nodes = (size_t)1 << (3 * level);
   La += (size_t)chunk * (4 * nodes + 1) * kLn + fr;
   Mh += (size_t)chunk * (nodes + 1) * kLn + fr;
-  float2 acc[7][4];
-#pragma unroll
-  for (int i = 0; i < 7; ++i)
-#pragma unroll
-    for (int f = 0; f < 4; ++f) acc[i][f] = make_float2(0.f, 0.f);
-  if (level > 2)
-    tg_rows<0>(La, Mh, level, oy, oz, grp, acc);
-  else
-    tg_rows<1>(La, Mh, level, oy, oz, grp, acc);
   __shared__ float2 red[kTgGroups][28][kLn];
-#pragma unroll
-  for (int i = 0; i < 7; ++i)
-#pragma unroll
-    for (int f = 0; f < 4; ++f) red[grp][i * 4 + f][fr] = acc[i][f];
+  float2(*tot)[kLn] = reinterpret_cast<float2(*)[kLn]>(&red[grp][0][fr]);   // this thread's column
+  if (level > 2)
+    tg_rows<0>(La, Mh, level, oy, oz, grp, tot);
+  else
+    tg_rows<1>(La, Mh, level, oy, oz, grp, tot);
   __syncthreads();
   for (int q = grp; q < 28; q += kTgGroups) {
     float2 v = red[0][q][fr];
@@ -120,62 +139,68 @@ __global__ void __launch_bounds__(kLn* kTgGroups) k_tg_mac(const float2* __restr
 }
 
 // Lags g_o(d) of one (offset, field): CTA, three separable inverse passes over
-// all NM points of each axis.  out [o][f][dz][dy][dx], index d mod NM.
+// all NM points of each axis, in double-float with one rounding at the end.
+// out [o][f][dz][dy][dx], index d mod NM.
+template <int P>
+size_t inv_smem() {
+  return 2 * sizeof(float4) * Shape<P>::NM * Shape<P>::NM * P;
+}
 template <int P>
 __global__ void __launch_bounds__(128) k_tg_inv(const float2* __restrict__ G, int nkp, const float4* __restrict__ twg,
                                                float* __restrict__ out) {
+  using T = Num<true>;
   constexpr int NM = Shape<P>::NM;
-  extern __shared__ float2 sg[];
+  extern __shared__ float4 sg[];
   __shared__ float4 tw[NM];
-  float2* t1 = sg;                        // [z][ky][kx]
-  float2* t2 = sg + NM * NM * P;          // [z][y][kx]
+  float4* t1 = sg;                        // [z][ky][kx]
+  float4* t2 = sg + NM * NM * P;          // [z][y][kx]
   const int tid = threadIdx.x, o = blockIdx.x / 4;
   const int ox = o % 7 - 3, oy = (o / 7) % 7 - 3, oz = o / 49 - 3;
   if (abs(ox) <= 1 && abs(oy) <= 1 && abs(oz) <= 1) return;   // near nodes: never gathered
   if (tid < NM) tw[tid] = __ldg(twg + tid);
   __syncthreads();
   const float2* src = G + (size_t)blockIdx.x * nkp;
-  const Twiddle<false, P> wt(twg, nullptr);
+  const Twiddle<true, P> wt(twg, tw);
   for (int q = tid; q < NM * P; q += blockDim.x) {
-    float xr[NM], xi[NM];
+    float2 xr[NM], xi[NM];
 #pragma unroll
     for (int s = 0; s < NM; ++s) {
       const float2 c = __ldg(src + s * NM * P + q);
-      xr[s] = c.x;
-      xi[s] = c.y;
+      xr[s] = widen<true>(c.x);
+      xi[s] = widen<true>(c.y);
     }
-    inverse_line<false, P, true>(xr, xi, wt,
-                                 [&](int z, float re, float im) { t1[z * NM * P + q] = make_float2(re, im); });
+    inverse_line<true, P, true>(xr, xi, wt, [&](int z, float2 re, float2 im) { t1[z * NM * P + q] = T::pack(re, im); });
   }
   __syncthreads();
   for (int q = tid; q < NM * P; q += blockDim.x) {            // line (z, kx)
     const int kx = q % P, z = q / P;
-    float xr[NM], xi[NM];
+    float2 xr[NM], xi[NM];
 #pragma unroll
     for (int s = 0; s < NM; ++s) {
-      const float2 c = t1[(z * NM + s) * P + kx];
-      xr[s] = c.x;
-      xi[s] = c.y;
+      const float4 c = t1[(z * NM + s) * P + kx];
+      xr[s] = T::re(c);
+      xi[s] = T::im(c);
     }
-    inverse_line<false, P, true>(xr, xi, wt,
-                                 [&](int y, float re, float im) { t2[(z * NM + y) * P + kx] = make_float2(re, im); });
+    inverse_line<true, P, true>(xr, xi, wt,
+                                [&](int y, float2 re, float2 im) { t2[(z * NM + y) * P + kx] = T::pack(re, im); });
   }
   __syncthreads();
-  const float scale = 1.f / (float)(NM * NM * NM);
+  const float2 scale = df_from_double(1.0 / ((double)NM * NM * NM));
   for (int i = tid; i < NM * NM * NM; i += blockDim.x) {
     const int x = i % NM;
-    const float2* v = t2 + (i / NM) * P;
-    float a = 0.f;
+    const float4* v = t2 + (i / NM) * P;
+    float2 a = T::zero(), g = T::zero();
     int j = x;
 #pragma unroll
     for (int s = 1; s < P; ++s) {
       const float4 w = tw[j];
-      a = fmaf(w.x, v[s].x, a);
-      a = fmaf(-w.z, v[s].y, a);
+      T::mac(a, w.x, w.y, T::re(v[s]));
+      T::mac(a, -w.z, -w.w, T::im(v[s]));
       j += x;
       j -= j >= NM ? NM : 0;
     }
-    out[(size_t)blockIdx.x * NM * NM * NM + i] = fmaf(2.f, a, v[0].x) * scale;
+    T::mac(g, scale.x, scale.y, T::add(T::twice(T::done(a)), T::re(v[0])));
+    out[(size_t)blockIdx.x * NM * NM * NM + i] = g.x + g.y;
   }
 }
 
@@ -212,8 +237,7 @@ __global__ void k_tg_gather(const float* __restrict__ g, int p, int level, float
 
 template <int P>
 cudaError_t inv_p(const float2* G, int nkp, const float4* tw, float* out, cudaStream_t s) {
-  constexpr int NM = Shape<P>::NM;
-  k_tg_inv<P><<<kOff3 * 4, 128, 2 * sizeof(float2) * NM * NM * P, s>>>(G, nkp, tw, out);
+  k_tg_inv<P><<<kOff3 * 4, 128, inv_smem<P>(), s>>>(G, nkp, tw, out);
   return cudaGetLastError();
 }
 
@@ -401,10 +425,8 @@ cudaError_t setup_learn_spec(const Plan& P) {
   if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(k_corr_eval<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)eval_smem());
   if (e != cudaSuccess) return e;
-  const size_t inv = 2 * sizeof(float2) * (2 * P.p - 1) * (2 * P.p - 1) * P.p;
-  switch (P.p) {
-    case 7: return cudaFuncSetAttribute(k_tg_inv<7>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)inv);
-    case 8: return cudaFuncSetAttribute(k_tg_inv<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)inv);
+  switch (P.p) {                          // above 48 KB
+    case 8: return cudaFuncSetAttribute(k_tg_inv<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)inv_smem<8>());
     default: return cudaSuccess;
   }
 }

@@ -594,7 +594,7 @@ cudaError_t fwd_p(Plan& Pl, const float* src, void* dst, size_t blocks, cudaStre
   fill(Pl, false, 1, 0, A, [](int) { return 0; });
   A.n = 1;
   A.lev[0] = {src, nullptr, dst, nullptr, nullptr, nullptr, nullptr, 0, 0, blocks};
-  k_spec_fwd<P, false, false><<<(unsigned)(blocks / Shape<P>::NB), Shape<P>::THR, fwd_smem<P, false>(), s>>>(A);
+  k_spec_fwd<P, false, true><<<(unsigned)(blocks / Shape<P>::NB), Shape<P>::THR, fwd_smem<P, true>(), s>>>(A);
   return cudaGetLastError();
 }
 

@@ -151,3 +151,22 @@ def test_direct_table_gradient_of_a_periodic_plan_matches_oracle_differences(B, 
             fd = (olearn.grid_loss(tp_, rho, L, p, tphi, tg, w_phi, w_g)
                   - olearn.grid_loss(tm_, rho, L, p, tphi, tg, w_phi, w_g)) / (2 * h)
             assert abs(got[i] - fd) <= 1e-3 * np.abs(blk).max(), (lev, f, a, got[i], fd, np.abs(blk).max())
+
+
+@pytest.mark.parametrize("N,L,p", [(128, 6, 2), (96, 5, 3), (64, 3, 6)])
+def test_spectral_table_gradient_rounds_like_the_direct_one_at_depth(B, N, L, p):
+    # FP32 spectra and chains of 128 terms leave ~1e-7 of the leaf level's
+    # gradient against FP64, as the direct sums do: 2e-7 between the two.  (One
+    # FP32 chain over a level of 2^6 nodes per axis left 3.2e-7.)
+    rho = torch.from_numpy(inputs.lognormal(N, sigma=0.8, seed=N)).cuda()
+    zero = torch.zeros((4, N, N, N), device="cuda")
+    G3, out = 4 * (4 * p) ** 3, []
+    for plan in (B.Plan(N, L, p), _plan(B, N, L, p)):
+        grad = torch.zeros(B.fmm_plan_table_grid_size(plan.handle), device="cuda")
+        loss = torch.zeros(1, device="cuda")
+        B.fmm_table_grid_grad(plan.handle, rho, zero[0].contiguous(), zero[1:].contiguous(), 1.0, 1e-3, grad, loss)
+        torch.cuda.synchronize()
+        out.append(grad[-G3:].double())
+        plan.close()
+    err = float((out[0] - out[1]).norm() / out[1].norm())
+    assert err < 2e-7, err
