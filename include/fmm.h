@@ -246,7 +246,7 @@ int fmm_plan_inject_fault(fmm_plan* plan, int kind);
 
 /* Dense tensor-core M2L: number of interaction offsets (1..189) accumulated in one
  * TMEM partial sum before it is added to the compensated FP32 total on the
- * CUDA cores.  Smaller is more accurate, larger is faster; default 2.
+ * CUDA cores.  Smaller is more accurate, larger is faster; default 4.
  * FMM_ERR_ARG outside 1..189. */
 int fmm_plan_set_m2l_group(fmm_plan* plan, int offsets_per_partial);
 
@@ -277,8 +277,10 @@ int fmm_plan_set_tc_tile(fmm_plan* plan, int level, int targets);
  * times each tensor-core level's M2L with both tiles (stage-timed solves of
  * `density`, one warm-up and the faster of two, enqueued on `stream`; the
  * plan's precision must already be set), keeps the faster per level, and
- * writes the chosen targets per CTA to tiles[l] for l < n (0 for levels not
- * on the tensor cores; n may be 0).  Allocates scratch outputs for its
+ * writes the targets per CTA to tiles[l] for l < n (0 for levels not on the
+ * tensor cores; n may be 0).  Levels on the spectral form have no tile
+ * (fmm_plan_get_forms): they keep their setting, and where no level runs the
+ * dense contraction nothing is solved.  Allocates scratch outputs for its
  * solves (4 N^3 floats) and synchronises.  FMM_ERR_ARG for NULL or
  * misaligned pointers, FMM_ERR_ALLOC, FMM_ERR_CUDA. */
 int fmm_plan_autotune_tiles(fmm_plan* plan, const float* density, int* tiles, int n, void* stream);

@@ -829,9 +829,13 @@ int fmm_plan_autotune_tiles(fmm_plan* plan, const float* density, int* tiles, in
   Plan& P = *reinterpret_cast<Plan*>(plan);
   const bool tc = P.prec != FMM_PREC_FP32 && P.tc_ready;
   const size_t n3 = (size_t)P.N * P.N * P.N;
-  if (tc) {
+  // levels whose kernel has a tile: the dense contraction's, but for bf16x6
+  auto tiled = [&](int l) { return m2l_form(P, l) == FMM_FORM_DENSE_TC && !fmm::tc_wide(P, l); };
+  bool any = false;
+  for (int l = 2; l <= P.L; ++l) any = any || tiled(l);
+  if (any) {
     float* out = nullptr;
-    if (cudaMalloc(&out, sizeof(float) * 4 * n3) != cudaSuccess) return set_err(FMM_ERR_ALLOC);
+    if (!dev_alloc(&out, 4 * n3)) return set_err(FMM_ERR_ALLOC);
     const int was_timing = P.timing;
     int rc = fmm_plan_set_timing(plan, 1);
     float best[fmm::kMaxLevel + 1] = {};
@@ -839,7 +843,7 @@ int fmm_plan_autotune_tiles(fmm_plan* plan, const float* density, int* tiles, in
     for (int c = 0; c < 2 && rc == FMM_OK; ++c) {
       const int t = c == 0 ? 256 : 128;
       for (int l = fmm::tc_first_level(P); l <= P.L && rc == FMM_OK; ++l)
-        if (!fmm::tc_wide(P, l)) rc = fmm_plan_set_tc_tile(plan, l, t);
+        if (tiled(l)) rc = fmm_plan_set_tc_tile(plan, l, t);
       float ms[FMM_TIME_SLOTS];
       float lev[fmm::kMaxLevel + 1];
       for (int l = 0; l <= fmm::kMaxLevel; ++l) lev[l] = 1e30f;
@@ -856,7 +860,7 @@ int fmm_plan_autotune_tiles(fmm_plan* plan, const float* density, int* tiles, in
         }
     }
     for (int l = fmm::tc_first_level(P); l <= P.L && rc == FMM_OK; ++l)
-      if (!fmm::tc_wide(P, l)) rc = fmm_plan_set_tc_tile(plan, l, pick[l]);
+      if (tiled(l)) rc = fmm_plan_set_tc_tile(plan, l, pick[l]);
     fmm_plan_set_timing(plan, was_timing);
     cudaFree(out);
     if (rc != FMM_OK) return set_err(rc);

@@ -170,3 +170,22 @@ def test_spectral_table_gradient_rounds_like_the_direct_one_at_depth(B, N, L, p)
         plan.close()
     err = float((out[0] - out[1]).norm() / out[1].norm())
     assert err < 2e-7, err
+
+
+def test_tile_autotuner_times_only_levels_that_have_a_tile(B):
+    N, L, p = 64, 5, 4
+    rho = torch.from_numpy(inputs.lognormal(N, sigma=0.5, seed=12)).cuda()
+    plan = B.Plan(N, L, p, precision=B.FMM_PREC_BF16X3)       # levels 4 and 5 on the spectral form
+    B.fmm_plan_autotune_tiles(plan.handle, rho)
+    with pytest.raises(B.FMMError):                          # no solve was timed
+        B.fmm_plan_stage_times(plan.handle)
+    plan.close()
+    plan = _plan(B, N, L, p, prec=B.FMM_PREC_BF16X3)
+    before = plan.solve(rho)
+    tiles = B.fmm_plan_autotune_tiles(plan.handle, rho)
+    assert tiles[3] == 0 and tiles[4] in (128, 256) and tiles[5] in (128, 256)
+    assert B.fmm_plan_stage_times(plan.handle)[B.FMM_TIME_M2L] > 0
+    after = plan.solve(rho)
+    torch.cuda.synchronize()
+    assert all(torch.equal(a, b) for a, b in zip(before, after))
+    plan.close()
