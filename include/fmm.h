@@ -191,7 +191,7 @@ int fmm_plan_set_m2l_algorithm(fmm_plan* plan, int algorithm);
  * cells, as convolutions under non-periodic boundary conditions on a padded
  * grid, the approach Sec. 3 takes for the near zone of a regular grid: per
  * pair of neighbour leaves the S^3 masses zero-padded to (2 S - 1)^3, the
- * 27 x 4 kernel spectra of the near table (FP64, rounded once), FP32 products;
+ * kernel spectra of the near table (double-float, rounded once), FP32 products;
  * FMM_NEAR_DIRECT transforms in double-float.  Other leaves sum directly, as
  * do plans whose spectra have no room (fmm_plan_set_spectra_limit; 2^(3L) x
  * 72 KB for S = 8: 2.4 GB at 256^3, L = 5).

@@ -260,6 +260,7 @@ void free_fft(Plan& P);
 size_t spec_kernel_bytes(const Plan& P, int level);
 size_t spec_source_bytes(const Plan& P, int level);
 size_t spec_target_bytes(const Plan& P, int level);
+cudaError_t launch_clear_blocks(char* to, size_t stride, size_t n, cudaStream_t s);   // n x 128 bytes of zeros
 cudaError_t setup_m2l_spec(const Plan& P);
 cudaError_t launch_spec_kernels(Plan& P, int level, cudaStream_t s);
 // Its tensor-core form (m2l_spec_tc.cu): buffer sizes of a level (weights,

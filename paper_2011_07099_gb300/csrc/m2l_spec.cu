@@ -532,6 +532,12 @@ __global__ void __launch_bounds__(kMacThrDf, 4) k_spec_mac_df(const __grid_const
   }
 }
 
+// 128 bytes of zeros at `to`, to + stride, ... (n of them).
+__global__ void k_clear_blocks(char* __restrict__ to, size_t stride, size_t n) {
+  const size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+  if (i < n * 8) *reinterpret_cast<float4*>(to + i / 8 * stride + i % 8 * 16) = make_float4(0.f, 0.f, 0.f, 0.f);
+}
+
 template <int P, bool DFA>
 size_t fwd_smem() {
   constexpr int NB = Shape<P>::NB, NM = Shape<P>::NM;
@@ -632,6 +638,11 @@ cudaError_t setup_p() {
 }
 
 }  // namespace
+
+cudaError_t launch_clear_blocks(char* to, size_t stride, size_t n, cudaStream_t s) {
+  k_clear_blocks<<<(unsigned)((n * 8 + 127) / 128), 128, 0, s>>>(to, stride, n);
+  return cudaGetLastError();
+}
 
 size_t spec_kernel_bytes(const Plan& P, int l) {
   const bool df = wide_level(P, l);

@@ -15,7 +15,7 @@
 // against 27 x 4 x 262 144 at S = 8.
 //
 // Kernels
-//   k_ns_planes, k_ns_lines  plan time: the 27 x 4 kernel spectra in FP64, rounded once
+//   k_ns_planes, k_ns_lines  plan time: the kernel spectra, double-float rounded once
 //   k_ns_fwd     per leaf: the spectrum of its masses
 //   k_ns_mac     per (tile of 4^3 target leaves, chunk of frequencies): the
 //                27-term sums of the 4 fields
@@ -55,7 +55,7 @@ using spec::Shape;
 using spec::Twiddle;
 using spec::widen;
 
-constexpr int kNO = 27;
+constexpr int kKernels = 14;                // offsets 0..13 of 27: the others' kernels are their conjugates
 constexpr int kTile = 4;                    // target leaves per tile side
 constexpr int kHaloN = kTile + 2;
 constexpr int kSlots = kHaloN * kHaloN * kHaloN;
@@ -70,88 +70,94 @@ template <int S, bool DFA>
 constexpr int kItems = S >= 16 ? 1 : (S <= 4 ? 8 : (S >= 8 && DFA ? 2 : 4));
 
 // ------------------------------------------------------------- plan time
+// Kernel spectra of the offsets 0..13 (kKernels) only: Phi's kernel is even and
+// g's odd, so the opposite offsets' are their conjugates up to sign (k_ns_mac).
+// Line transforms in double-float, rounded once on store.  With all 27 offsets
+// in FP64, at 1/64 of the FP32 rate, the plan of the isolated 128^3 solve (16-
+// cell leaves) took 4.7 ms to create; 1.6 this way.
+//
 // The kernel's value for field f at lag d (cells), from the folded near table
 // (|d_i| in [0, 2S-1]); the gradient fields take the sign of their own
 // component as the direct sum does, and vanish where that component is 0.
-__device__ __forceinline__ double near_value(const float4* __restrict__ tab, int S, int f, int dx, int dy, int dz) {
+__device__ __forceinline__ float near_value(const float4* __restrict__ tab, int S, int f, int dx, int dy, int dz) {
   const int TD = 2 * S;
   const int ax = dx < 0 ? -dx : dx, ay = dy < 0 ? -dy : dy, az = dz < 0 ? -dz : dz;
-  const float4 t = __ldg(tab + (az * TD + ay) * TD + ax);
-  switch (f) {
-    case 0: return (double)t.x;
-    case 1: return dx > 0 ? (double)t.y : (dx < 0 ? -(double)t.y : 0.0);
-    case 2: return dy > 0 ? (double)t.z : (dy < 0 ? -(double)t.z : 0.0);
-    default: return dz > 0 ? (double)t.w : (dz < 0 ? -(double)t.w : 0.0);
-  }
+  const float v = __ldg(reinterpret_cast<const float*>(tab + (az * TD + ay) * TD + ax) + f);
+  const int own = f == 1 ? dx : (f == 2 ? dy : dz);
+  return f == 0 || own > 0 ? v : (own < 0 ? -v : 0.f);
 }
 
-// CTA (z lag, offset x field): the x and y transforms of one lag plane.
+// CTA (z lag, offset x field): the x and y transforms of one lag plane, a line
+// per thread.  out [offset x field][z lag][ky][kx].
+constexpr int kPlaneThr = 32;
 template <int S>
-__global__ void __launch_bounds__(128) k_ns_planes(const float4* __restrict__ tab, double2* __restrict__ out) {
+__global__ void __launch_bounds__(kPlaneThr) k_ns_planes(const float4* __restrict__ tab, const float4* __restrict__ twg,
+                                                         float4* __restrict__ out) {
+  using T = Num<true>;
   constexpr int NM = Shape<S>::NM;
-  __shared__ double2 w[NM];
-  __shared__ double2 T1[NM * S];
+  static_assert(NM <= kPlaneThr, "a thread per x line");
+  __shared__ float4 tw[NM];
+  __shared__ float4 t1[NM * S];           // [y][kx]
   const int vz = blockIdx.x, of = blockIdx.y, o = of / 4, f = of % 4, tid = threadIdx.x;
   const int ox = o % 3 - 1, oy = (o / 3) % 3 - 1, oz = o / 9 - 1;
-  if (tid < NM) {
-    double s, c;
-    sincospi(2.0 * tid / NM, &s, &c);
-    w[tid] = make_double2(c, -s);
-  }
+  if (tid < NM) tw[tid] = __ldg(twg + tid);
   __syncthreads();
+  const Twiddle<true, S> wt(twg, tw);
   auto lag = [](int v) { return v < S ? v : v - NM; };
-  for (int i = tid; i < NM * S; i += blockDim.x) {
-    const int kx = i % S, vy = i / S;
-    double re = 0.0, im = 0.0;
-    for (int vx = 0; vx < NM; ++vx) {
-      const double a = near_value(tab, S, f, lag(vx) - S * ox, lag(vy) - S * oy, lag(vz) - S * oz);
-      const double2 t = w[(kx * vx) % NM];
-      re += a * t.x;
-      im += a * t.y;
-    }
-    T1[i] = make_double2(re, im);
+  if (tid < NM) {                         // x: line y lag = tid
+    float2 x[NM];
+#pragma unroll
+    for (int vx = 0; vx < NM; ++vx)
+      x[vx] = widen<true>(near_value(tab, S, f, lag(vx) - S * ox, lag(tid) - S * oy, lag(vz) - S * oz));
+    spec::forward_real_full_line<true, S>(x, wt,
+                                          [&](int k, float2 re, float2 im) { t1[tid * S + k] = T::pack(re, im); });
   }
   __syncthreads();
-  for (int i = tid; i < NM * S; i += blockDim.x) {
-    const int kx = i % S, ky = i / S;
-    double re = 0.0, im = 0.0;
-    for (int vy = 0; vy < NM; ++vy) {
-      const double2 a = T1[vy * S + kx], t = w[(ky * vy) % NM];
-      re += a.x * t.x - a.y * t.y;
-      im += a.x * t.y + a.y * t.x;
+  if (tid < S) {                          // y: line kx = tid
+    float2 xr[NM], xi[NM];
+#pragma unroll
+    for (int v = 0; v < NM; ++v) {
+      const float4 c = t1[v * S + tid];
+      xr[v] = T::re(c);
+      xi[v] = T::im(c);
     }
-    out[((size_t)of * NM + vz) * NM * S + i] = make_double2(re, im);
+    // the forward transform at k is the inverse one at NM - k
+    inverse_line<true, S, true>(xr, xi, wt, [&](int y, float2 re, float2 im) {
+      out[(((size_t)of * NM + vz) * NM + (y ? NM - y : 0)) * S + tid] = T::pack(re, im);
+    });
   }
 }
 
-// The z transform, 1/NM^3, and the store K^[chunk][o][2 field pairs][16] float4
-// (re, im of two fields).
+// The z transform, 1/NM^3, and the store K^[chunk][offset][2 field pairs][16]
+// float4 (re, im of two fields); a line (ky, kx) per thread.
 template <int S>
-__global__ void __launch_bounds__(128) k_ns_lines(const double2* __restrict__ in, float* __restrict__ K) {
+__global__ void __launch_bounds__(128) k_ns_lines(const float4* __restrict__ in, const float4* __restrict__ twg,
+                                                  float* __restrict__ K) {
+  using T = Num<true>;
   constexpr int NM = Shape<S>::NM, LANES = Num<false>::LANES;
-  __shared__ double2 w[NM];
+  __shared__ float4 tw[NM];
   const int o = blockIdx.y / 4, f = blockIdx.y % 4;
-  if (threadIdx.x < NM) {
-    double s, c;
-    sincospi(2.0 * threadIdx.x / NM, &s, &c);
-    w[threadIdx.x] = make_double2(c, -s);
-  }
+  if (threadIdx.x < NM) tw[threadIdx.x] = __ldg(twg + threadIdx.x);
   __syncthreads();
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= NM * NM * S) return;
-  const int q = k % (NM * S), kz = k / (NM * S);
-  double re = 0.0, im = 0.0;
-  for (int vz = 0; vz < NM; ++vz) {
-    const double2 a = in[((size_t)blockIdx.y * NM + vz) * NM * S + q], t = w[(kz * vz) % NM];
-    re += a.x * t.x - a.y * t.y;
-    im += a.x * t.y + a.y * t.x;
+  const Twiddle<true, S> wt(twg, tw);
+  const int q = blockIdx.x * blockDim.x + threadIdx.x;
+  if (q >= NM * S) return;
+  float2 xr[NM], xi[NM];
+#pragma unroll
+  for (int v = 0; v < NM; ++v) {
+    const float4 c = __ldg(in + ((size_t)blockIdx.y * NM + v) * NM * S + q);
+    xr[v] = T::re(c);
+    xi[v] = T::im(c);
   }
-  const double scale = 1.0 / ((double)NM * NM * NM);
-  re *= scale;
-  im *= scale;
-  const size_t base = ((size_t)(k / LANES) * kNO + o) * 128;   // floats
-  const int l = k % LANES;
-  reinterpret_cast<float2*>(K + base)[((f / 2) * LANES + l) * 2 + (f & 1)] = make_float2((float)re, (float)im);
+  const float2 scale = df_from_double(1.0 / ((double)NM * NM * NM));
+  inverse_line<true, S, true>(xr, xi, wt, [&](int z, float2 re, float2 im) {
+    const int k = (z ? NM - z : 0) * NM * S + q, l = k % LANES;
+    float2 a = T::zero(), b = T::zero();
+    T::mac(a, scale.x, scale.y, re);
+    T::mac(b, scale.x, scale.y, im);
+    const size_t base = ((size_t)(k / LANES) * kKernels + o) * 128;   // floats
+    reinterpret_cast<float2*>(K + base)[((f / 2) * LANES + l) * 2 + (f & 1)] = make_float2(a.x + a.y, b.x + b.y);
+  });
 }
 
 // ------------------------------------------------------------- transforms
@@ -371,7 +377,6 @@ __global__ void __launch_bounds__(Shape<S>::threads(kItems<S, DFA>)) k_ns_inv(co
 // `per` consecutive chunks of one tile, up to 8, fewer where that leaves fewer
 // than 4 CTAs per SM.
 constexpr int kChunks = 8;
-constexpr int kKernels = kNO / 2 + 1;           // offsets 0..13: the others' kernels are their conjugates
 constexpr int kStage = kKernels * 32 + kSlots * 8;   // float4 per stage
 __global__ void __launch_bounds__(256) k_ns_mac(const float4* __restrict__ K, const void* __restrict__ Mh,
                                                           void* __restrict__ Ph, int L, int nkp, int iso, int per) {
@@ -391,7 +396,7 @@ __global__ void __launch_bounds__(256) k_ns_mac(const float4* __restrict__ K, co
   __syncthreads();
   auto load = [&](int chunk, int st) {
     float4* to = sm4 + st * kStage;
-    const float4* Kc = K + (size_t)chunk * kNO * 32;
+    const float4* Kc = K + (size_t)chunk * kKernels * 32;
     for (int i = tid; i < kKernels * 32; i += NTHR) tc::cp_async16_full(tc::smem_u32(to + i), Kc + i);
     const char* src = reinterpret_cast<const char*>(Mh) + (size_t)chunk * (leaves + 1) * 128;
     for (int i = tid; i < kSlots * 8; i += NTHR)
@@ -529,10 +534,9 @@ template <int S>
 cudaError_t kernels_s(Plan& P, cudaStream_t s) {
   constexpr int NM = Shape<S>::NM;
   // the target spectra's space holds the half-transformed kernels meanwhile
-  double2* scratch = static_cast<double2*>(P.ns_P);
-  k_ns_planes<S><<<dim3(NM, kNO * 4), 128, 0, s>>>(P.near_tab, scratch);
-  k_ns_lines<S><<<dim3((NM * NM * S + 127) / 128, kNO * 4), 128, 0, s>>>(scratch,
-                                                                                          static_cast<float*>(P.ns_K));
+  float4* scratch = static_cast<float4*>(P.ns_P);
+  k_ns_planes<S><<<dim3(NM, kKernels * 4), kPlaneThr, 0, s>>>(P.near_tab, P.ns_tw, scratch);
+  k_ns_lines<S><<<dim3((NM * S + 127) / 128, kKernels * 4), 128, 0, s>>>(scratch, P.ns_tw, static_cast<float*>(P.ns_K));
   return cudaGetLastError();
 }
 
@@ -558,7 +562,7 @@ bool near_spec_shape(const Plan& P) { return P.S == 4 || P.S == 6 || P.S == 8 ||
 
 void near_spec_bytes(const Plan& P, size_t& nK, size_t& nM, size_t& nP) {
   const size_t leaves = (size_t)1 << (3 * P.L), ch = chunks_of(P.S, false);
-  nK = ch * kNO * 512;
+  nK = ch * kKernels * 512;
   nM = ch * (leaves + 1) * 128;
   nP = leaves * 4 * ch * 128;
 }

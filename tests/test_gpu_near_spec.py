@@ -79,3 +79,16 @@ def test_fp32_transforms_round_no_more_than_radix_2_ones(B, N, L, p, phi_bound, 
         plan.close()
     phi, g = np.mean(err, axis=0)
     assert phi <= phi_bound and g <= g_bound, (phi, g)
+
+
+@pytest.mark.parametrize("S", [4, 6, 8, 16])
+def test_a_plan_holds_the_kernel_spectra_of_half_the_offsets(B, S):
+    # order 1 has no M2L spectra: 14 of the 27 offsets' kernels (the others are
+    # their conjugates), 4 fields of 16 complex values per chunk of 16
+    # frequencies; the leaves' spectra and one of zeros; the targets' 4 fields
+    L = 2
+    plan = B.Plan(S << L, L, 1)
+    _, held = B.fmm_plan_get_forms(plan.handle)
+    plan.close()
+    chunks, leaves = -(-(2 * S - 1) ** 2 * S // 16), 8 ** L
+    assert held == chunks * (14 * 512 + (leaves + 1) * 128 + leaves * 4 * 128)
