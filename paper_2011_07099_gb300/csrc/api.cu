@@ -1188,7 +1188,7 @@ int fmm_plan_error_stats(fmm_plan* plan, const float* density, const float* pote
     cudaFree(P.es_scratch);
     P.es_scratch = nullptr;
     P.es_bytes = 0;
-    if (cudaMalloc(&P.es_scratch, bytes) != cudaSuccess) return set_err(FMM_ERR_ALLOC);
+    if (!plan_alloc(P, &P.es_scratch, bytes)) return set_err(FMM_ERR_ALLOC);
     P.es_bytes = bytes;
   }
   double* d_partials = static_cast<double*>(P.es_scratch);

@@ -172,3 +172,20 @@ def test_a_limit_whose_buffers_cannot_be_made_stops_the_solves(B):
     assert np.array_equal(a[0], b[0]) and np.array_equal(a[1], b[1])
     plan.close()
     fresh.close()
+
+
+def test_a_statement_without_scratch_leaves_no_error_behind(B):
+    # CUDA keeps a failed allocation's error until it is read: the next solve must not report it
+    N, L, p = 16, 2, 3
+    d = torch.from_numpy(inputs.lognormal(N, sigma=0.5, seed=5)).cuda()
+    plan = B.Plan(N, L, p)
+    phi, acc = plan.solve(d)
+    B.fmm_plan_inject_fault(plan.handle, B.FMM_FAULT_ALLOC + 0)
+    with pytest.raises(B.FMMError) as e:
+        plan.error_stats(d, phi, acc, samples=32, seed=1)
+    assert e.value.code == B.FMM_ERR_ALLOC
+    again = plan.solve(d)
+    torch.cuda.synchronize()
+    assert torch.equal(again[0], phi) and torch.equal(again[1], acc)
+    assert max(plan.error_stats(d, phi, acc, samples=32, seed=1)) < 1.0
+    plan.close()
