@@ -1115,9 +1115,8 @@ int fmm_solve_host(fmm_plan* plan, const float* density_host, float* potential_h
   if (!plan || !density_host || !potential_host || !accel_host) return set_err(FMM_ERR_ARG);
   Plan& P = *reinterpret_cast<Plan*>(plan);
   const size_t n3 = (size_t)P.N * P.N * P.N;
-  if (!P.stage_in) {
-    if (!dev_alloc(&P.stage_in, n3) || !dev_alloc(&P.stage_out, 4 * n3)) return set_err(FMM_ERR_ALLOC);
-  }
+  if ((!P.stage_in && !plan_alloc(P, &P.stage_in, n3)) || (!P.stage_out && !plan_alloc(P, &P.stage_out, 4 * n3)))
+    return set_err(FMM_ERR_ALLOC);
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   FMM_CUDA_TRY(cudaMemcpyAsync(P.stage_in, density_host, n3 * sizeof(float), cudaMemcpyHostToDevice, s));
   int rc = fmm_solve(plan, P.stage_in, P.stage_out, P.stage_out + n3, stream);

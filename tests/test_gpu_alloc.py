@@ -189,3 +189,19 @@ def test_a_statement_without_scratch_leaves_no_error_behind(B):
     assert torch.equal(again[0], phi) and torch.equal(again[1], acc)
     assert max(plan.error_stats(d, phi, acc, samples=32, seed=1)) < 1.0
     plan.close()
+
+
+@pytest.mark.parametrize("n", [0, 1])
+def test_host_staging_is_made_on_the_next_call(B, n):
+    N, L, p = 16, 2, 3
+    host = torch.from_numpy(inputs.lognormal(N, sigma=0.5, seed=5))
+    phi, acc = torch.empty((N, N, N)), torch.empty((3, N, N, N))
+    plan = B.Plan(N, L, p)
+    ref = _solve(B, plan, host.cuda())
+    B.fmm_plan_inject_fault(plan.handle, B.FMM_FAULT_ALLOC + n)
+    with pytest.raises(B.FMMError) as e:
+        B.fmm_solve_host(plan.handle, host, phi, acc)
+    assert e.value.code == B.FMM_ERR_ALLOC
+    B.fmm_solve_host(plan.handle, host, phi, acc)
+    assert np.array_equal(phi.numpy(), ref[0]) and np.array_equal(acc.numpy(), ref[1])
+    plan.close()
