@@ -82,6 +82,7 @@ def m2l_forms(N, L, p, density, steps=5):
                             ("dense_bf16x3", B.FMM_PREC_BF16X3, B.FMM_M2L_DENSE),
                             ("fft_fp32", B.FMM_PREC_FP32, B.FMM_M2L_FFT)):
         plan = B.Plan(N, L, p)
+        B.fmm_plan_set_spectra_limit(plan.handle, 0)     # the contractions themselves, not their spectral products
         if prec != B.FMM_PREC_FP32:
             plan.set_precision(prec)
         B.fmm_plan_set_m2l_algorithm(plan.handle, alg)

@@ -189,3 +189,17 @@ def test_tile_autotuner_times_only_levels_that_have_a_tile(B):
     torch.cuda.synchronize()
     assert all(torch.equal(a, b) for a, b in zip(before, after))
     plan.close()
+
+
+def test_m2l_ablation_times_the_dense_contractions(B, monkeypatch):
+    from paper_2011_07099_gb300 import ablation
+    seen, solve = [], B.Plan.solve
+
+    def recorded(self, *a, **k):
+        seen.append(tuple(B.fmm_plan_get_forms(self.handle)[0][2:]))
+        return solve(self, *a, **k)
+    monkeypatch.setattr(B.Plan, "solve", recorded)
+    d = torch.from_numpy(inputs.lognormal(32, sigma=0.5, seed=1)).cuda()
+    rows = ablation.m2l_forms(32, 4, 4, d, steps=1)
+    D, T, F = B.FMM_FORM_DENSE, B.FMM_FORM_DENSE_TC, B.FMM_FORM_FFT
+    assert list(dict.fromkeys(seen)) == [(D, D, D), (D, D, T), (D, D, F)] and len(rows) == 3
