@@ -63,6 +63,10 @@ void destroy_batch(fmm_batch* b) {
   delete b;
 }
 
+// In every key of the level cache; changed with the M2L or near-zone kernels,
+// whose times decide the leaf size.
+constexpr const char* kTuneKernels = "spectral";
+
 std::string gpu_name() {
   int dev = 0;
   cudaDeviceProp prop;
@@ -111,8 +115,9 @@ extern "C" {
 
 int fmm_autotune_levels(int N, int order, int precision, const char* cache_path, int* L_out, float* ms_out) {
   if (N < 4 || order < 1 || order > fmm::kMaxOrder || !L_out) return fmm::set_last_error(FMM_ERR_ARG);
+  // kTuneKernels names the kernels that were timed: entries of others are not taken
   const std::string key = gpu_name() + "|N=" + std::to_string(N) + "|p=" + std::to_string(order) +
-                          "|prec=" + std::to_string(precision);
+                          "|prec=" + std::to_string(precision) + "|" + kTuneKernels;
   int L = 0;
   float ms = 0.f;
   if (cache_lookup(cache_path, key, &L, &ms)) {

@@ -108,3 +108,14 @@ def test_batch_with_autotuned_levels(B, monkeypatch, tmp_path):
     for n, l in zip(Ns, batch.levels):
         assert n % (1 << l) == 0 and l >= 3
     batch.close()
+
+
+def test_level_cache_entries_of_other_kernels_are_not_taken(B, tmp_path):
+    # an entry without the kernels' tag: tuned before the spectral forms
+    path = tmp_path / "tune.jsonl"
+    key = f"{torch.cuda.get_device_name()}|N=32|p=2|prec=0"
+    path.write_text('{"key": "%s", "L": 7, "ms": 0.001}\n' % key)
+    L, ms = B.fmm_autotune_levels(32, 2, B.FMM_PREC_FP32, str(path))
+    assert L in (3, 4) and ms > 0.001
+    assert B.fmm_autotune_levels(32, 2, B.FMM_PREC_FP32, str(path))[0] == L        # its own entry is
+    assert len(path.read_text().splitlines()) == 2
