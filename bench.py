@@ -174,16 +174,19 @@ def measure_fp32_peak(B, dev, stream, reps=40):
 
 
 def near_flops(N, L, fields=4):
-    """Arithmetic of the near zone by spectral products per solve: with leaves
-    of S cells, transforms on (2S - 1)^3 points of which NK = (2S - 1)^2 S
-    frequencies are kept; per leaf the sums (27 offsets x 4 fields x NK, 8 flop
-    per complex multiply-add), the forward transform of the masses and the
-    four inverse transforms to the S^3 cells, by lines."""
+    """Arithmetic the near zone by spectral products executes per solve: with
+    leaves of S cells, transforms on (2S - 1)^3 points of which NK =
+    (2S - 1)^2 S frequencies are kept.  Sums: per leaf and frequency the leaf's
+    own kernel and 13 pairs of opposite offsets, whose kernels are conjugate.
+    Lines of the forward transform of the masses and of the four inverse ones
+    to the S^3 cells: the symmetric halves of a line share their sums."""
     S = N >> L
-    M = 2 * S - 1
-    mac = 27 * fields * M * M * S * 8
-    fwd = 4 * S * S * S * S + 8 * S * S * M * S + 8 * S * M * M * S   # x (real), y, z passes
-    inv = 8 * S * M * S * M + 8 * S * S * S * M + 4 * S * S * S * S
+    M, h = 2 * S - 1, S - 1
+    mac = M * M * S * (13 * (4 + 8 * fields) + 6 * fields)
+    line_real, line_fwd = h + 4 * h * h, 2 * h + h * (8 * h + 4)
+    line_inv, line_cells = 6 * h + h * (8 * h + 2), S * (4 * h + 2)
+    fwd = S * S * line_real + S * S * line_fwd + M * S * line_fwd          # x, y, z passes
+    inv = M * S * line_inv + S * S * line_inv + S * S * line_cells
     return float(8 ** L * (mac + fwd + fields * inv))
 
 
@@ -361,16 +364,32 @@ def device_check(B, plan):
 
 
 def launches_per_solve(L, tc, p=6, near_fft=False):
-    # the library's dense forms (M2L by dense sums, the near zone by pairs): mean
+    # the library's dense forms (spectra limit 0; M2L by dense sums, the near zone by pairs): mean
     # (2) + P2M + M2M per level + M2L per level + L2L per level + near zone (1;
     # by FFT 4); M2L of the coarse levels (2-3, and every level above the leaves
-    # at order >= 7) adds the range sums, tensor-core levels the split.  The
-    # spectral forms launch more; this is the least a solve launches, for the
-    # case that the profiler counts none (profiled_launches).
+    # at order >= 7) adds the range sums, tensor-core levels the split
     wide = lambda lev: lev <= 3 or (p >= 7 and lev < L)
     tc_first = max(4, L) if p >= 7 else 4
     m2l = sum(2 if (wide(lev) or (tc and lev >= tc_first)) else 1 for lev in range(2, L + 1))
     return 2 + 1 + (L - 2) + m2l + (L - 2) + (4 if near_fft else 1)
+
+
+def launches_of_forms(forms, p, S):
+    """Kernels an untimed periodic solve launches in the forms its plan runs
+    (fmm_plan_get_forms: [0] the near zone, [l] the M2L of level l), for the
+    case that the profiler counts none (profiled_launches): mean (2), P2M, M2M
+    and L2L per level, near zone (spectral: source spectra, sums, inverse) and
+    M2L: the spectral levels of one arithmetic share three launches, spectral
+    tensor-core levels take four each (scale, spectra, products, inverse),
+    dense ones one and their split or range sums."""
+    from paper_2011_07099_gb300 import binding as B
+    L = len(forms) - 1
+    wide = lambda lev: lev <= 3 or (p >= 7 and lev < L) or S >= 16
+    spectral = {wide(lev) for lev in range(2, L + 1) if forms[lev] == B.FMM_FORM_SPECTRAL}
+    each = {B.FMM_FORM_SPECTRAL_TC: 4, B.FMM_FORM_DENSE_TC: 2}
+    m2l = 3 * len(spectral) + sum(each.get(forms[lev], 2 if wide(lev) else 1) for lev in range(2, L + 1)
+                                  if forms[lev] != B.FMM_FORM_SPECTRAL)
+    return 2 + 1 + 2 * (L - 2) + m2l + (3 if forms[0] == B.FMM_FORM_SPECTRAL else 1)
 
 
 def profiled_launches(solve):
@@ -460,8 +479,12 @@ def run_ours(args):
     near_fft = near_fft_used(args)
     if near_fft:
         B.fmm_plan_set_near_algorithm(plan.handle, B.FMM_NEAR_FFT)
-    # the tensor-core tile of each level, autotuned at plan time (outside the timed region)
+    # the tile of each level on the dense tensor-core contraction, autotuned at
+    # plan time (outside the timed region); none where all run spectral products
     tc_tiles = B.fmm_plan_autotune_tiles(plan.handle, rho)[:L + 1] if tc else None
+    m2l_forms, _ = B.fmm_plan_get_forms(plan.handle)
+    if tc:
+        tc_tiles = [t if f == B.FMM_FORM_DENSE_TC else 0 for t, f in zip(tc_tiles, m2l_forms)]
     with ClockSampler(dev.index) as clk:
         step_ms, stage, wall = _time_solves(B, plan, rho, phi, acc, args.steps, args.warmup, l2_flush, stream,
                                             barrier)
@@ -581,8 +604,8 @@ def run_ours(args):
         B.fmm_solve_host(plan.handle, hin, hphi, hacc, stream)
     e2e_s = (time.perf_counter() - t0) / e2e_steps
     checks["e2e"] = device_check(B, plan)
-    launches = (profiled_launches(lambda: plan.solve(rho, phi, acc)) if rank == 0 else 0) or launches_per_solve(
-        L, tc, p, near_fft)
+    launches = (profiled_launches(lambda: plan.solve(rho, phi, acc)) if rank == 0 else 0) or launches_of_forms(
+        m2l_forms, p, n >> L)
     plan.close()
 
     if rank != 0:

@@ -18,3 +18,15 @@ def test_launch_count_claim_matches_the_profiled_launch_list():
     assert bench.launches_per_solve(5, True, 6, near_fft=True) == 21
     assert bench.launches_per_solve(5, True, 6) == 18
     assert bench.launches_per_solve(5, False, 6) == 16
+
+
+def test_launch_count_of_the_forms_that_run():
+    import bench
+    from paper_2011_07099_gb300 import binding as B
+    S, D, T, C, N = (B.FMM_FORM_SPECTRAL, B.FMM_FORM_DENSE, B.FMM_FORM_DENSE_TC, B.FMM_FORM_SPECTRAL_TC,
+                     B.FMM_FORM_NONE)
+    # 256^3 p = 6: mean 2, P2M, M2M 3, levels 2-3 spectral 3, levels 4-5 on the tensor cores 8, L2L 3, near 3
+    assert bench.launches_of_forms([S, N, S, S, C, C], 6, 8) == 23
+    assert bench.launches_of_forms([S, N, S, S, S, S], 6, 8) == 18          # plain: FP32 and double-float spectra
+    assert bench.launches_of_forms([D, N, D, D, T, T], 6, 8) == bench.launches_per_solve(5, True, 6)
+    assert bench.launches_of_forms([D, N, D, D, D, D], 6, 8) == bench.launches_per_solve(5, False, 6)
