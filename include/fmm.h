@@ -111,9 +111,9 @@ int fmm_solve_host(fmm_plan* plan, const float* density_host,
  * FMM_PREC_BF16 / FMM_PREC_BF16X3 apply to levels >= 4 (see
  * fmm_plan_set_tc_min_level).  In every mode the coarse levels, whose
  * long-range sums cancel most, run on the CUDA cores in extended precision:
- * levels 2 and 3 in double-float (error-free products and sums) into FP64
- * local fields.  At order >= 7 every
- * level above the leaves keeps FP64 local fields: in the tensor-core modes
+ * levels 2 and 3 in double-float into FP64 local fields (error-free products
+ * and sums; level 3 of orders < 7 takes its products in FP32 chains of at most
+ * 12 terms).  At order >= 7 every level above the leaves keeps FP64 local fields: in the tensor-core modes
  * levels >= 5 of them run "bf16x6" (both operands split in three BF16 parts,
  * six products, partials of each 32-deep stage added into a double-float
  * total, written in FP64), the coarser ones the double-float CUDA-core
@@ -186,8 +186,11 @@ int fmm_plan_set_m2l_algorithm(fmm_plan* plan, int algorithm);
 
 /* How the leaf stage evaluates the near zone (Sec. 2, part 3 of the
  * potential).  FMM_NEAR_DIRECT (default): the sum over the 27 neighbour
- * leaves at the accuracy of the direct sum.  FMM_NEAR_FFT: the same sum with
- * FP32 transforms throughout.  Both run, for leaves of S = 4, 6, 8 or 16
+ * leaves at the accuracy of the direct sum, in the mesh's norm: for leaves of
+ * 4 cells and more a cell's error is relative to the largest field of its
+ * neighbour leaves, and a lone cell's force on itself is not exactly 0 but
+ * ~1e-9 of that field.  FMM_NEAR_FFT: the same sum with FP32 transforms
+ * throughout.  Both run, for leaves of S = 4, 6, 8 or 16
  * cells, as convolutions under non-periodic boundary conditions on a padded
  * grid, the approach Sec. 3 takes for the near zone of a regular grid: per
  * pair of neighbour leaves the S^3 masses zero-padded to (2 S - 1)^3, the

@@ -20,10 +20,11 @@ constexpr int kMaxOrder = 8;
 constexpr int kFields = 4;          // Phi, g_x, g_y, g_z
 constexpr int kMaxOffsets = 189;    // interaction-zone size below level 2 (Sec. 2)
 // The top two far-field levels (2 and 3) carry the long-range potential, whose
-// sum cancels most; their Phi contraction uses G = hi + lo split tables.
+// sum cancels most: double-float spectra, or, by dense sums, split tables
+// G = hi + lo.
 constexpr int kExtTopLevel = 3;
-// Levels at or below kExtTopLevel always run the FP32 split-table kernel; the
-// tensor-core precision modes apply from kTcMinLevel down to the leaves.
+// They always run on the CUDA cores; the tensor-core precision modes apply from
+// kTcMinLevel down to the leaves.
 constexpr int kTcMinLevel = kExtTopLevel + 1;
 
 // ---------------------------------------------------------------- Morton keys
@@ -91,7 +92,7 @@ struct Plan {
   // FP64 as well (M2M writes both copies; M2L reads them as hi + lo).
   double* M64[kMaxLevel + 1] = {};
   float4* tab[kMaxLevel + 1] = {};  // (G, -dG/dx, -dG/dy, -dG/dz) at n dx_l, n in [-(4p-1), 4p-1]^3
-  float4* tab_lo[kMaxLevel + 1] = {};  // v - fl32(v) of the same entries, 4 fields (wide levels)
+  float4* tab_lo[kMaxLevel + 1] = {};  // v - fl32(v) of the same entries, 4 fields
   float4* near_tab = nullptr;       // the same at cell spacing for |d_i| in [0, 2S-1], folded
   float2* w_p2m = nullptr;          // Lagrange weights [p][S] as (hi, lo): gridlet s at cell c
   float2* w_m2m = nullptr;          // Lagrange weights [p][2p] as (hi, lo): parent s at child point u
@@ -167,8 +168,8 @@ struct Plan {
   int* d_err = nullptr;                    // device error word (bounded waits that gave up)
   int n_off[kMaxLevel + 1] = {};
 
-  // untimed solves of the tensor-core forms overlap independent stages on
-  // two plan-owned streams (aux), joined by events (fev)
+  // untimed solves overlap independent stages on two plan-owned streams (aux),
+  // joined by events (fev)
   cudaStream_t aux[2] = {};
   cudaEvent_t fev[4] = {};
 

@@ -22,7 +22,9 @@
 //                  189-offset sums of the 4 fields
 //   k_spec_inv     per node: the 4 fields' p^3 values
 // Arithmetic: FP32 at the fine levels; at the wide levels (FP64 local fields)
-// every value, twiddle, product and sum is double-float.
+// values, twiddles and sums are double-float, and products too but for level 3
+// of orders < kWideOrder: there a row's products run in FP32 chains of at most
+// 12 terms on the high halves of the source spectra (mac_df, ROWS).
 // Measured (dense kernels of m2l_fp32.cu before -> here, with transforms):
 // 256^3 p = 6, levels 4 + 5 FP32 87.1 -> 6.6 ms (plain form; 4.5 ms with FP32
 // transforms, sums 4.1 ms), levels 2 + 3 1.95 -> 0.35 ms; 512^3 p = 8, levels
@@ -380,8 +382,8 @@ __device__ __forceinline__ void mac_fp32(const float2* __restrict__ halo, const 
 // Double-float, one field of a row of 4 targets per thread: (re hi, re lo, im
 // hi, im lo) sums.  The kernel values of the row's 7 x offsets stay in
 // registers while the 8 source spectra pass by, and one field per thread keeps
-// the unrolled row within the instruction cache (with 4 fields per thread
-// 4.1 of 5.8 cycles per instruction went to instruction fetch).
+// the unrolled row within the instruction cache (4 fields per thread waited for
+// instruction fetch most of the time).
 // ROWS: the sums of one (oy, oz) row run as FP32 multiply-add chains (at most
 // 12 terms) and are then added to the double-float total, the low halves of
 // the kernel values gathered beside them: 2 instructions per product instead

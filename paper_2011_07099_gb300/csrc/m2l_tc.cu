@@ -51,8 +51,8 @@
 // drain adds into a double-float total by TwoSum; the level's FP64 local
 // field is written from hi + lo.  TMEM: partial 0 | partial 1; the totals stay
 // in the drain threads' registers (one row and 32 columns each, 64 registers):
-// kept in TMEM, their loads and stores made a stage's drain 2390 clocks against
-// the 768 of its MMAs (512^3 order 8, level 5: 94 ms).
+// kept in TMEM, their loads and stores made a stage's drain longer than its
+// MMAs (512^3 order 8, level 5: 94 ms, now 79).
 // (A partial over a whole group of offsets cost 2.8e-5 at order 8: the
 // MMA's truncating accumulation, not the operand splits, dominated.)
 // Every wait is bounded; a timeout sets the plan's error word and later work

@@ -23,10 +23,14 @@
 //                the L2P far field (eq. fmm3 at the leaves), written once
 // Arithmetic: FP32 spectra and sums; the transforms in FP32 (FMM_NEAR_FFT) or,
 // where the plan asks for the direct sum's accuracy (FMM_NEAR_DIRECT), in
-// double-float with one rounding on store.  With 16-cell leaves the L2P reads
+// double-float with one rounding on store.  That accuracy is of the mesh's
+// norm: the rounding of a pair of leaves is spread over both, so a cell beside
+// a heavy one errs by ~1e-7 of the heavy one's peak field, and a lone cell's
+// force on itself, exactly 0 by pairs, reads 4e-10 of its peak field (1e-8 with
+// FP32 transforms).  With 16-cell leaves the L2P reads
 // the FP64 local field (fmm_internal.cuh, kWideLeaf) in double-float.
 // Measured (direct kernels of p2p.cu before -> here): 128^3 isolated with
-// 16-cell leaves 177 -> 2.9 ms; 256^3, S = 8 30.6 -> 6.0 ms at direct accuracy
+// 16-cell leaves 177 -> 1.6 ms; 256^3, S = 8 30.6 -> 6.1 ms at direct accuracy
 // (sums 0.91, inverse with L2P 4.3); 96^3, S = 6 1.04 -> 0.31 ms; 128^3, S = 4
 // 0.87 -> 0.47 ms.  FMM_NEAR_FFT at 256^3: 2.23 ms for radix-2 transforms of 16
 // points and a separate L2P -> 1.74 ms (sums 1.08 -> 0.91: 22 % fewer

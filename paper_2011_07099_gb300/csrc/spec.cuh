@@ -80,8 +80,8 @@ struct Num<true> {
 // folds the inputs s and NM - s into their sum and difference first: half the
 // multiply-adds of the plain sums.
 // Twiddles: FP32 has cos and sin of 2 pi j / NM as constants of the unrolled
-// code (read from shared memory, one load per four multiply-adds, they held
-// the transforms at 30 % of the FP32 rate); double-float reads (cos hi, lo,
+// code (read from shared memory, one load per four multiply-adds, the loads
+// bounded the transforms); double-float reads (cos hi, lo,
 // sin hi, lo) from shared memory.
 template <bool DF, int P>
 struct Twiddle;
