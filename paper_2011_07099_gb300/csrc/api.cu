@@ -4,6 +4,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <initializer_list>
 #include <new>
 #include <set>
 #include <tuple>
@@ -111,12 +112,15 @@ std::vector<int8_t> isolated_level2_offsets() {
   return out;
 }
 
+// Frees a set of buffers that set_alloc made: the first owns the memory.
+void free_set(std::initializer_list<void**> parts) {
+  cudaFree(**parts.begin());
+  for (void** p : parts) *p = nullptr;
+}
+
 // Training buffers (alloc_train).
 void free_train(Plan& P) {
-  for (void** b : {&P.tg_la, &P.tg_mh, &P.tg_gh, &P.tg_gl}) {
-    cudaFree(*b);
-    *b = nullptr;
-  }
+  free_set({&P.tg_la, &P.tg_mh, &P.tg_gh, &P.tg_gl});
   for (float** b : {&P.train_out, &P.lam_cells, &P.dT_all, &P.grad_partials}) {
     cudaFree(*b);
     *b = nullptr;
@@ -127,28 +131,17 @@ void free_train(Plan& P) {
   }
 }
 
-void free_near_spec(Plan& P) {
-  for (void** b : {&P.ns_K, &P.ns_M, &P.ns_P}) {
-    cudaFree(*b);
-    *b = nullptr;
-  }
-}
+void free_near_spec(Plan& P) { free_set({&P.ns_K, &P.ns_M, &P.ns_P}); }
 
 // A level's spectra: of the CUDA cores and, without them or alone, of the tensor cores.
 void free_stc(Plan& P, int l) {
-  for (void** b : {&P.stc_W[l], &P.stc_B[l], reinterpret_cast<void**>(&P.stc_scale[l])}) {
-    cudaFree(*b);
-    *b = nullptr;
-  }
+  free_set({&P.stc_W[l], &P.stc_B[l], &P.stc_scale[l], &P.stc_amax[l]});
   delete static_cast<CUtensorMap*>(P.stc_map[l]);
   P.stc_map[l] = nullptr;
 }
 void free_spec(Plan& P, int l) {
   free_stc(P, l);
-  for (void** b : {&P.spec_K[l], &P.spec_M[l], &P.spec_P[l]}) {
-    cudaFree(*b);
-    *b = nullptr;
-  }
+  free_set({&P.spec_K[l], &P.spec_M[l], &P.spec_P[l]});
 }
 
 void free_plan(Plan* P) {
@@ -169,7 +162,6 @@ void free_plan(Plan* P) {
   cudaFree(P->spec_tw);
   cudaFree(P->near_tab);
   free_near_spec(*P);
-  cudaFree(P->ns_tw);
   cudaFree(P->d_err);
   cudaFree(P->corr_w);
   cudaFree(P->corr_samples);
@@ -185,7 +177,6 @@ void free_plan(Plan* P) {
     cudaFree(P->Apre[l]);
     delete static_cast<CUtensorMap*>(P->tmapB[l]);
   }
-  cudaFree(P->stc_amax);
   cudaFree(P->es_scratch);
   cudaFree(P->w_p2m);
   cudaFree(P->w_m2m);
@@ -221,6 +212,25 @@ bool plan_alloc(Plan& P, T** ptr, size_t count) {
 }
 bool plan_alloc(Plan& P, void** ptr, size_t bytes) { return plan_alloc(P, reinterpret_cast<char**>(ptr), bytes); }
 
+// A set of buffers in one allocation (free_set), all of them or none: an
+// allocation takes 30 to 60 us and a plan has up to 11 sets.
+struct Part {
+  void** at;
+  size_t bytes;
+};
+bool set_alloc(Plan& P, std::initializer_list<Part> parts) {
+  auto rounded = [](size_t n) { return (n + 255) / 256 * 256; };
+  size_t total = 0;
+  for (const Part& p : parts) total += rounded(p.bytes);
+  char* base = nullptr;
+  if (!plan_alloc(P, &base, total)) return false;
+  for (const Part& p : parts) {
+    *p.at = base;
+    base += rounded(p.bytes);
+  }
+  return true;
+}
+
 // Spectra are optional: the dense kernels need ~20 times less memory.  A plan
 // holds at most what its caller allows (fmm_plan_set_spectra_limit) or, by
 // default, kSpecMaxBytes and no more than the memory that stays free beside
@@ -250,78 +260,60 @@ size_t spectra_bytes(const Plan& P) {
   return sum;
 }
 
-bool spectra_fit(const Plan& P, size_t bytes) {
-  const size_t held = spectra_bytes(P), want = held + bytes;
-  if (P.spec_limit != SIZE_MAX) return want <= P.spec_limit;
-  if (want > kSpecMaxBytes) return false;
+// The most bytes of spectra the plan may hold now; held and free memory change
+// by the same amount while its sets are made, so one look serves them all.
+size_t spectra_room(const Plan& P) {
+  if (P.spec_limit != SIZE_MAX) return P.spec_limit;
   size_t free_b = 0, total = 0;
   if (cudaMemGetInfo(&free_b, &total) != cudaSuccess) {
     (void)cudaGetLastError();
-    return true;
+    return kSpecMaxBytes;
   }
-  return want <= (free_b + held) / 2;
+  return std::min(kSpecMaxBytes, (free_b + spectra_bytes(P)) / 2);
 }
+bool spectra_fit(const Plan& P, size_t room, size_t bytes) { return spectra_bytes(P) + bytes <= room; }
 
-// (cos, sin) of 2 pi j / (2 points - 1) as (hi, lo) FP32 pairs.
-int make_twiddles(int points, float4** out) {
-  const int nm = 2 * points - 1;
-  std::vector<float4> tw((size_t)nm);
-  for (int j = 0; j < nm; ++j) {
-    const double a = 2.0 * 3.14159265358979323846 * j / nm, c = std::cos(a), s = std::sin(a);
-    tw[j] = make_float4((float)c, (float)(c - (double)(float)c), (float)s, (float)(s - (double)(float)s));
+// (cos, sin) of 2 pi j / (2 points - 1) as (hi, lo) FP32 pairs, for gridlets
+// (points = order) and for leaves (points = S).
+int make_twiddles(Plan& P) {
+  std::vector<float4> tw;
+  for (int points : {P.p, P.S}) {
+    const int nm = 2 * points - 1;
+    for (int j = 0; j < nm; ++j) {
+      const double a = 2.0 * 3.14159265358979323846 * j / nm, c = std::cos(a), s = std::sin(a);
+      tw.push_back(make_float4((float)c, (float)(c - (double)(float)c), (float)s, (float)(s - (double)(float)s)));
+    }
   }
-  if (!dev_alloc(out, tw.size())) return FMM_ERR_ALLOC;
-  return cudaMemcpy(*out, tw.data(), tw.size() * sizeof(float4), cudaMemcpyHostToDevice) == cudaSuccess ? FMM_OK
-                                                                                                      : FMM_ERR_CUDA;
-}
-
-// Zeros where spectra are read but never written: the padding frequencies of
-// the last chunk, and the spectrum of out-of-box blocks behind each chunk's
-// `blocks` (128 bytes a block; filling all of 512^3, order 8 took 2 ms).
-cudaError_t clear_spectra(void* K, size_t nK, void* M, size_t nM, size_t blocks) {
-  const size_t chunk = (blocks + 1) * 128, chunks = nM / chunk, kc = nK / chunks;
-  char *k = static_cast<char*>(K), *m = static_cast<char*>(M);
-  cudaError_t e = cudaMemset(k + nK - kc, 0, kc);
-  if (e == cudaSuccess) e = cudaMemset(m + nM - chunk, 0, chunk);
-  return e == cudaSuccess ? fmm::launch_clear_blocks(m + blocks * 128, chunk, chunks, 0) : e;
+  if (!dev_alloc(&P.spec_tw, tw.size())) return FMM_ERR_ALLOC;
+  P.ns_tw = P.spec_tw + 2 * P.p - 1;
+  return cudaMemcpy(P.spec_tw, tw.data(), tw.size() * sizeof(float4), cudaMemcpyHostToDevice) == cudaSuccess
+             ? FMM_OK
+             : FMM_ERR_CUDA;
 }
 
 // Buffers of the near zone's spectral products (near_spec.cu) for the leaf
-// sizes it is built for; `asked`: the caller names them (FMM_NEAR_FFT), so the
-// limit does not apply.
-int alloc_near_spec(Plan& P, bool asked) {
+// sizes it is built for.
+int alloc_near_spec(Plan& P, size_t room) {
   if (P.ns_K || !fmm::near_spec_shape(P)) return FMM_OK;
   size_t nK, nM, nP;
   fmm::near_spec_bytes(P, nK, nM, nP);
-  if (!asked && !spectra_fit(P, nK + nM + nP)) return FMM_OK;
-  if (!P.ns_tw) {
-    const int rc = make_twiddles(P.S, &P.ns_tw);
-    if (rc != FMM_OK) return rc;
-  }
-  if (!plan_alloc(P, &P.ns_M, nM) || !plan_alloc(P, &P.ns_P, nP) || !plan_alloc(P, &P.ns_K, nK)) {
-    free_near_spec(P);
+  if (!spectra_fit(P, room, nK + nM + nP) || !set_alloc(P, {{&P.ns_K, nK}, {&P.ns_M, nM}, {&P.ns_P, nP}}))
     return FMM_OK;
-  }
-  const size_t leaves = (size_t)1 << (3 * P.L);
-  return clear_spectra(P.ns_K, nK, P.ns_M, nM, leaves) == cudaSuccess ? FMM_OK : FMM_ERR_CUDA;
+  return fmm::launch_clear_spectra(P.ns_K, nK, P.ns_M, nM, (size_t)1 << (3 * P.L), 0) == cudaSuccess ? FMM_OK
+                                                                                                     : FMM_ERR_CUDA;
 }
 
 // Buffers of the spectral M2L for every level of orders >= 2, the coarse first.
-int alloc_spec(Plan& P) {
+int alloc_spec(Plan& P, size_t room) {
   if (P.p < 2) return FMM_OK;
-  if (!P.spec_tw) {
-    const int rc = make_twiddles(P.p, &P.spec_tw);
-    if (rc != FMM_OK) return rc;
-  }
   for (int l = 2; l <= P.L; ++l) {
     const size_t nk = fmm::spec_kernel_bytes(P, l), ns = fmm::spec_source_bytes(P, l),
                  nt = fmm::spec_target_bytes(P, l);
-    if (!spectra_fit(P, nk + ns + nt)) continue;
-    if (!plan_alloc(P, &P.spec_M[l], ns) || !plan_alloc(P, &P.spec_P[l], nt) || !plan_alloc(P, &P.spec_K[l], nk)) {
-      free_spec(P, l);
+    if (!spectra_fit(P, room, nk + ns + nt) ||
+        !set_alloc(P, {{&P.spec_K[l], nk}, {&P.spec_M[l], ns}, {&P.spec_P[l], nt}}))
       continue;
-    }
-    if (clear_spectra(P.spec_K[l], nk, P.spec_M[l], ns, (size_t)1 << (3 * l)) != cudaSuccess) return FMM_ERR_CUDA;
+    if (fmm::launch_clear_spectra(P.spec_K[l], nk, P.spec_M[l], ns, (size_t)1 << (3 * l), 0) != cudaSuccess)
+      return FMM_ERR_CUDA;
   }
   return FMM_OK;
 }
@@ -397,14 +389,8 @@ int alloc_train(Plan& P) {
   }
   size_t la, mh, gh, gl;
   fmm::tg_bytes(P, la, mh, gh, gl);
-  if (P.p >= 2 && spectra_fit(P, la + mh + gh + gl) &&
-      !(plan_alloc(P, &P.tg_mh, mh) && plan_alloc(P, &P.tg_gh, gh) && plan_alloc(P, &P.tg_gl, gl) &&
-        plan_alloc(P, &P.tg_la, la))) {
-    for (void** b : {&P.tg_la, &P.tg_mh, &P.tg_gh, &P.tg_gl}) {   // no room: the direct sums
-      cudaFree(*b);
-      *b = nullptr;
-    }
-  }
+  if (P.p >= 2 && spectra_fit(P, spectra_room(P), la + mh + gh + gl))   // else the direct sums
+    (void)set_alloc(P, {{&P.tg_la, la}, {&P.tg_mh, mh}, {&P.tg_gh, gh}, {&P.tg_gl, gl}});
   for (int l = 2; l <= P.L; ++l) P.dT[l] = P.dT_all + (size_t)(l - 2) * E * E * E * 4;
   return FMM_OK;
 }
@@ -549,8 +535,10 @@ fmm_plan* fmm_plan_create(int N, int L, int order) {
     bool fok = true;
     for (int l = 2; l <= L && fok; ++l)
       if (fmm::wide_level(*P, l)) fok = dev_alloc(&P->F64[l], ((size_t)1 << (3 * l)) * 4 * p3);
-    int rc = fok ? alloc_spec(*P) : FMM_ERR_ALLOC;
-    if (rc == FMM_OK) rc = alloc_near_spec(*P, false);
+    int rc = fok ? make_twiddles(*P) : FMM_ERR_ALLOC;
+    const size_t room = spectra_room(*P);
+    if (rc == FMM_OK) rc = alloc_spec(*P, room);
+    if (rc == FMM_OK) rc = alloc_near_spec(*P, room);
     if (rc != FMM_OK || alloc_m2l_part(*P) != FMM_OK) {
       free_plan(P);
       set_err(rc != FMM_OK ? rc : FMM_ERR_ALLOC);
@@ -589,12 +577,12 @@ int fmm_plan_get_shape(const fmm_plan* plan, int* N, int* L, int* order, int* S)
 namespace {
 // A level of the spectral tensor-core form: split weights and sources, their
 // scales and the tensor map, all of them or none (FMM_* code).
-int prepare_stc(Plan& P, int l) {
+int prepare_stc(Plan& P, int l, size_t room) {
   size_t nW, nB, nS;
   fmm::stc_bytes(P, l, nW, nB, nS);
   int rc = FMM_ERR_ALLOC;
-  if (spectra_fit(P, nW + nB + nS) && (P.stc_amax || plan_alloc(P, &P.stc_amax, (size_t)fmm::kMaxLevel + 1)) &&
-      plan_alloc(P, &P.stc_W[l], nW) && plan_alloc(P, &P.stc_B[l], nB) && plan_alloc(P, &P.stc_scale[l], nS / sizeof(float))) {
+  if (spectra_fit(P, room, nW + nB + nS) &&
+      set_alloc(P, {{&P.stc_W[l], nW}, {&P.stc_B[l], nB}, {&P.stc_scale[l], nS}, {&P.stc_amax[l], sizeof(float)}})) {
     // the halo of the isolated problem stays zero (fmm_plan_set_boundary clears it too)
     rc = (!P.iso || cudaMemset(P.stc_B[l], 0, nB) == cudaSuccess) && fmm::launch_stc_weights(P, l, 0) == cudaSuccess
              ? fmm::make_stc_map(P, l)
@@ -610,12 +598,12 @@ int prepare_stc(Plan& P, int l) {
 // tables, split multipoles and translation tiles.  A level counts as prepared
 // once it has its tensor map, which is made last.  Tabulated once, synchronously.
 int prepare_tc(Plan& P) {
-  const size_t E = 8 * P.p - 1;
+  const size_t E = 8 * P.p - 1, room = spectra_room(P);
   bool made = false;
   for (int l = fmm::tc_first_level(P); l <= P.L; ++l) {
     if (fmm::spec_tc_level(P, l)) {
       if (P.stc_map[l]) continue;
-      const int rc = prepare_stc(P, l);
+      const int rc = prepare_stc(P, l, room);
       if (rc == FMM_OK) {
         made = true;
         continue;
@@ -666,8 +654,9 @@ int fmm_plan_set_spectra_limit(fmm_plan* plan, size_t bytes) {
   }
   free_near_spec(P);
   free_train(P);
-  int rc = alloc_spec(P);
-  if (rc == FMM_OK) rc = alloc_near_spec(P, P.near_fft != 0);
+  const size_t room = spectra_room(P);
+  int rc = alloc_spec(P, room);
+  if (rc == FMM_OK) rc = alloc_near_spec(P, P.near_fft ? SIZE_MAX : room);
   if (rc == FMM_OK && P.near_fft && !P.ns_K) rc = FMM_ERR_ALLOC;
   if (rc == FMM_OK) rc = alloc_m2l_part(P);
   if (rc == FMM_OK && P.tc_ready) rc = prepare_tc(P);
@@ -774,7 +763,7 @@ int fmm_plan_set_near_algorithm(fmm_plan* plan, int algorithm) {
   }
   if (P.S != 8) return set_err(FMM_ERR_UNSUPPORTED);
   if (!P.ns_K) {   // over the default limit at plan creation: the caller asks for it
-    const int rc = alloc_near_spec(P, true);
+    const int rc = alloc_near_spec(P, SIZE_MAX);
     if (rc != FMM_OK || !P.ns_K) return set_err(rc != FMM_OK ? rc : FMM_ERR_ALLOC);
     FMM_CUDA_TRY(fmm::launch_near_spec_kernels(P, 0));
   }

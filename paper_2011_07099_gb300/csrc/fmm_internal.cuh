@@ -111,11 +111,11 @@ struct Plan {
   // forms take there: split weights and their scales, split source spectra,
   // the tensor map (host CUtensorMap) and each level's largest mass sum
   void* stc_W[kMaxLevel + 1] = {};
-  float* stc_scale[kMaxLevel + 1] = {};
+  void* stc_scale[kMaxLevel + 1] = {};
   void* stc_B[kMaxLevel + 1] = {};
   void* stc_map[kMaxLevel + 1] = {};
   bool stc_off[kMaxLevel + 1] = {};        // no room for them: the level's dense contraction runs
-  float* stc_amax = nullptr;
+  void* stc_amax[kMaxLevel + 1] = {};
   // tensor-core M2L (levels >= kTcMinLevel, allocated on the first mixed-precision solve)
   uint4* tab_bf[kMaxLevel + 1] = {};       // per table entry, per field: bf16 hi | bf16 lo << 16
   void* Mbf_hi[kMaxLevel + 1] = {};        // gridlet masses split into BF16 parts (2; 3 at bf16x6 levels), per parity class with a halo
@@ -261,7 +261,10 @@ void free_fft(Plan& P);
 size_t spec_kernel_bytes(const Plan& P, int level);
 size_t spec_source_bytes(const Plan& P, int level);
 size_t spec_target_bytes(const Plan& P, int level);
-cudaError_t launch_clear_blocks(char* to, size_t stride, size_t n, cudaStream_t s);   // n x 128 bytes of zeros
+// Zeros where spectra are read but never written: the padding frequencies of the
+// last chunk of K and M, and the spectrum of out-of-box blocks behind each
+// chunk's `blocks` in M.
+cudaError_t launch_clear_spectra(void* K, size_t nK, void* M, size_t nM, size_t blocks, cudaStream_t s);
 cudaError_t setup_m2l_spec(const Plan& P);
 cudaError_t launch_spec_kernels(Plan& P, int level, cudaStream_t s);
 // Its tensor-core form (m2l_spec_tc.cu): buffer sizes of a level (weights,

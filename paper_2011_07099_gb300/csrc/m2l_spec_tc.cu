@@ -503,7 +503,7 @@ template <int P>
 cudaError_t launch_p(Plan& Pl, int level, cudaStream_t s) {
   constexpr int NK = StcShape<P>::NK;
   const size_t nodes = (size_t)1 << (3 * level), parents = nodes / 8;
-  float* amax = Pl.stc_amax + level;
+  float* amax = static_cast<float*>(Pl.stc_amax[level]);
   cudaError_t e = cudaMemsetAsync(amax, 0, sizeof(float), s);
   if (e != cudaSuccess) return e;
   const size_t want = (nodes + 63) / 64;            // 8 nodes per warp at least
@@ -516,7 +516,8 @@ cudaError_t launch_p(Plan& Pl, int level, cudaStream_t s) {
   const int parts = NK < 3 * Pl.num_sms ? 2 : 1;
   const unsigned grid = NK * parts < Pl.num_sms ? NK * parts : Pl.num_sms;
   k_stc_mac<<<grid, kThr, kSmem, s>>>(*static_cast<const CUtensorMap*>(Pl.stc_map[level]),
-                                     static_cast<const uint8_t*>(Pl.stc_W[level]), Pl.stc_scale[level], amax, NK, parts, level,
+                                     static_cast<const uint8_t*>(Pl.stc_W[level]),
+                                     static_cast<const float*>(Pl.stc_scale[level]), amax, NK, parts, level,
                                      static_cast<float*>(Pl.spec_P[level]), Pl.d_err, Pl.wait_ns, Pl.inject_stall);
   k_stc_inv<P><<<(unsigned)(nodes / StcShape<P>::NI), 256, stc_inv_smem<P>(), s>>>(
       static_cast<const float2*>(Pl.spec_P[level]), parents, Pl.F[level]);
@@ -577,7 +578,7 @@ cudaError_t setup_spec_tc(const Plan& P) {
 
 cudaError_t launch_stc_weights(Plan& P, int level, cudaStream_t s) {
   k_stc_weights<<<nk_of(P.p), 256, 0, s>>>(static_cast<const float*>(P.spec_K[level]),
-                                          static_cast<uint8_t*>(P.stc_W[level]), P.stc_scale[level]);
+                                          static_cast<uint8_t*>(P.stc_W[level]), static_cast<float*>(P.stc_scale[level]));
   return cudaGetLastError();
 }
 
