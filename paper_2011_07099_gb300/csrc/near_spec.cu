@@ -78,7 +78,7 @@ constexpr int kItems = S >= 16 ? 1 : (S <= 4 ? 8 : (S >= 8 && DFA ? 2 : 4));
 // g's odd, so the opposite offsets' are their conjugates up to sign (k_ns_mac).
 // Line transforms in double-float, rounded once on store.  With all 27 offsets
 // in FP64, at 1/64 of the FP32 rate, the plan of the isolated 128^3 solve (16-
-// cell leaves) took 4.7 ms to create; 1.6 this way.
+// cell leaves) took 4.7 ms to create; 1.4 with these.
 //
 // The kernel's value for field f at lag d (cells), from the folded near table
 // (|d_i| in [0, 2S-1]); the gradient fields take the sign of their own
