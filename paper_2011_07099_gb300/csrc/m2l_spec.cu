@@ -326,7 +326,8 @@ __device__ __forceinline__ void mac_fp32(const float2* __restrict__ halo, const 
     const int hz = tz + 2 - oz;
     if (!allowed<MODE>(cz, oz) || hz < 0 || hz >= kHaloN) continue;
     // a plane's sums stay apart from the total: the running FP32 sums are no
-    // longer than one plane's terms
+    // longer than one plane's terms.  (A stage per row as well took 10 % off the
+    // error of 32^3, p = 2 .. 4 and 7 % more time of this kernel.)
     float2 acc[4][4];
 #pragma unroll
     for (int j = 0; j < 4; ++j)
